@@ -1,14 +1,17 @@
 """Python binding of the B200 residual-VQ KV-cache library.
 
 Argument marshalling only: every function below forwards to the C entry point
-of the same name in ``librvq_b200.so`` (declared in ``include/rvq.h``).  PyTorch
-supplies device memory and streams; all arithmetic runs in the CUDA kernels.
-There is no CPU fallback: if the library is missing or fails to load, importing
-this package raises.
+of the same name in ``librvq_b200.so`` (declared in ``include/rvq.h``); the calls
+that launch kernels go through ``_native.so`` (``csrc/binding.cpp``), which turns
+tensors into addresses and finds the current stream.  PyTorch supplies device
+memory and streams; all arithmetic runs in the CUDA kernels.  There is no CPU
+fallback: if a library is missing or fails to load, importing this package raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -98,6 +101,19 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 
+
+def _load_native():
+    path = os.path.join(_HERE, "_native.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: run `python paper_2410_15704_b200/build.py`")
+    loader = importlib.machinery.ExtensionFileLoader("_native", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_native", loader))
+    loader.exec_module(module)
+    return module
+
+
+_native = _load_native()
+
 EXPORTS = ("rvq_attention_workspace_bytes", "rvq_attention_decode", "rvq_selftest_encode_timeout", "rvq_rope_table", "rvq_decode_rope", "rvq_learn_step", "rvq_kmeans_workspace_bytes", "rvq_kmeans_init", "rvq_encode_stats", "rvq_ema_update_static", "rvq_ema_static_scratch_bytes", "rvq_encode_exact", "rvq_status_string", "rvq_version", "rvq_launch_count", "rvq_ema_stats", "rvq_ema_apply", "rvq_code_bytes", "rvq_prepared_bytes",
            "rvq_prepare_codebooks", "rvq_workspace_bytes", "rvq_encode", "rvq_decode",
            "rvq_ema_update")
@@ -106,20 +122,6 @@ EXPORTS = ("rvq_attention_workspace_bytes", "rvq_attention_decode", "rvq_selftes
 def make_config(dim=128, group_dim=32, layout=CONTIGUOUS, depth=8, codebook_size=2048,
                 code_bits=16, x_dtype=BF16, std_ddof=0) -> rvq_config:
     return rvq_config(dim, group_dim, layout, depth, codebook_size, code_bits, x_dtype, std_ddof)
-
-
-def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
-
-
-def _stream(stream):
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(rc: int, what: str):
@@ -148,28 +150,28 @@ def rvq_workspace_bytes(cfg: rvq_config, n: int) -> int:
 
 
 def rvq_prepare_codebooks(cfg, codebooks, prepared, stream=None, check=True) -> int:
-    rc = lib.rvq_prepare_codebooks(ctypes.byref(cfg), _ptr(codebooks), _ptr(prepared), _stream(stream))
-    if check:
+    rc = _native.rvq_prepare_codebooks(cfg, codebooks, prepared, stream)
+    if rc and check:
         _check(rc, "rvq_prepare_codebooks")
     return rc
 
 
 def rvq_encode(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, workspace=None,
                workspace_bytes=0, status=None, stream=None, check=True, stage_energy=None) -> int:
-    rc = lib.rvq_encode(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codebooks), _ptr(prepared),
-                        _ptr(codes), _ptr(std_f16), _ptr(stage_energy), _ptr(workspace), workspace_bytes,
-                        _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_encode(cfg, x, n, x_row_stride, codebooks, prepared,
+                        codes, std_f16, stage_energy, workspace, workspace_bytes,
+                        status, stream)
+    if rc and check:
         _check(rc, "rvq_encode")
     return rc
 
 
 def rvq_encode_stats(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, batch_count, batch_sum,
                      workspace, workspace_bytes, status=None, stream=None, check=True, stage_energy=None) -> int:
-    rc = lib.rvq_encode_stats(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codebooks), _ptr(prepared),
-                              _ptr(codes), _ptr(std_f16), _ptr(stage_energy), _ptr(batch_count), _ptr(batch_sum),
-                              _ptr(workspace), workspace_bytes, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_encode_stats(cfg, x, n, x_row_stride, codebooks, prepared,
+                              codes, std_f16, stage_energy, batch_count, batch_sum,
+                              workspace, workspace_bytes, status, stream)
+    if rc and check:
         _check(rc, "rvq_encode_stats")
     return rc
 
@@ -177,56 +179,56 @@ def rvq_encode_stats(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f1
 def rvq_selftest_encode_timeout(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, wait_polls, status,
                                 stream=None, check=True) -> int:
     """rvq_encode with one MMA chain left out per CTA: its wait gives up (include/rvq_selftest.h)."""
-    rc = lib.rvq_selftest_encode_timeout(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codebooks), _ptr(prepared),
-                                         _ptr(codes), _ptr(std_f16), wait_polls, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_selftest_encode_timeout(cfg, x, n, x_row_stride, codebooks, prepared,
+                                         codes, std_f16, wait_polls, status, stream)
+    if rc and check:
         _check(rc, "rvq_selftest_encode_timeout")
     return rc
 
 
 def rvq_encode_exact(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, status=None,
                      stream=None, check=True, stage_energy=None) -> int:
-    rc = lib.rvq_encode_exact(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codebooks), _ptr(prepared),
-                              _ptr(codes), _ptr(std_f16), _ptr(stage_energy), _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_encode_exact(cfg, x, n, x_row_stride, codebooks, prepared,
+                              codes, std_f16, stage_energy, status, stream)
+    if rc and check:
         _check(rc, "rvq_encode_exact")
     return rc
 
 
 def rvq_decode(cfg, codes, std_f16, n, codebooks, prepared, x_out, out_row_stride, status=None,
                stream=None, check=True) -> int:
-    rc = lib.rvq_decode(ctypes.byref(cfg), _ptr(codes), _ptr(std_f16), n, _ptr(codebooks),
-                        _ptr(prepared), _ptr(x_out), out_row_stride, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_decode(cfg, codes, std_f16, n, codebooks,
+                        prepared, x_out, out_row_stride, status, stream)
+    if rc and check:
         _check(rc, "rvq_decode")
     return rc
 
 
 def rvq_ema_update(cfg, x, n, x_row_stride, codes, codebooks, ema_count, ema_sum, batch_count,
                    decay, eps, workspace, workspace_bytes, status=None, stream=None, check=True) -> int:
-    rc = lib.rvq_ema_update(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codes), _ptr(codebooks),
-                            _ptr(ema_count), _ptr(ema_sum), _ptr(batch_count), decay, eps,
-                            _ptr(workspace), workspace_bytes, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_ema_update(cfg, x, n, x_row_stride, codes, codebooks,
+                            ema_count, ema_sum, batch_count, decay, eps,
+                            workspace, workspace_bytes, status, stream)
+    if rc and check:
         _check(rc, "rvq_ema_update")
     return rc
 
 
 def rvq_ema_stats(cfg, x, n, x_row_stride, codes, codebooks, batch_count, batch_sum, workspace,
                   workspace_bytes, status=None, stream=None, check=True) -> int:
-    rc = lib.rvq_ema_stats(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codes), _ptr(codebooks),
-                           _ptr(batch_count), _ptr(batch_sum), _ptr(workspace), workspace_bytes,
-                           _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_ema_stats(cfg, x, n, x_row_stride, codes, codebooks,
+                           batch_count, batch_sum, workspace, workspace_bytes,
+                           status, stream)
+    if rc and check:
         _check(rc, "rvq_ema_stats")
     return rc
 
 
 def rvq_ema_apply(cfg, batch_count, batch_sum, codebooks, ema_count, ema_sum, decay, eps,
                   stream=None, check=True) -> int:
-    rc = lib.rvq_ema_apply(ctypes.byref(cfg), _ptr(batch_count), _ptr(batch_sum), _ptr(codebooks),
-                           _ptr(ema_count), _ptr(ema_sum), decay, eps, _stream(stream))
-    if check:
+    rc = _native.rvq_ema_apply(cfg, batch_count, batch_sum, codebooks,
+                           ema_count, ema_sum, decay, eps, stream)
+    if rc and check:
         _check(rc, "rvq_ema_apply")
     return rc
 
@@ -236,10 +238,10 @@ def rvq_ema_update_static(cfg, x, n, x_row_stride, codes, codebooks, ema_count, 
     """rvq_ema_update with the library's own fixed scratch: no workspace to pass, nothing
     allocated.  For callers that cannot obtain device memory themselves; see include/rvq.h
     for the size limit and for why overlapping calls must be ordered."""
-    rc = lib.rvq_ema_update_static(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codes), _ptr(codebooks),
-                                   _ptr(ema_count), _ptr(ema_sum), _ptr(batch_count), decay, eps,
-                                   _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_ema_update_static(cfg, x, n, x_row_stride, codes, codebooks,
+                                   ema_count, ema_sum, batch_count, decay, eps,
+                                   status, stream)
+    if rc and check:
         _check(rc, "rvq_ema_update_static")
     return rc
 
@@ -249,8 +251,8 @@ ROPE_HALVES, ROPE_ADJACENT = 0, 1
 
 def rvq_rope_table(dim, base, positions, cos_sin, stream=None, check=True) -> int:
     """Fill cos_sin (float32 [positions][dim/2][2]) with the rotary embedding's cosines and sines."""
-    rc = lib.rvq_rope_table(dim, float(base), positions, _ptr(cos_sin), _stream(stream))
-    if check:
+    rc = _native.rvq_rope_table(dim, float(base), positions, cos_sin, stream)
+    if rc and check:
         _check(rc, "rvq_rope_table")
     return rc
 
@@ -258,11 +260,11 @@ def rvq_rope_table(dim, base, positions, cos_sin, stream=None, check=True) -> in
 def rvq_decode_rope(cfg, codes, std_f16, n, codebooks, prepared, position, vectors_per_position, cos_sin,
                     positions, pairing, x_out, out_row_stride, status=None, stream=None, check=True) -> int:
     """Decode and rotate: x_out = RoPE(decode(codes)) at the given positions (prepared may be None)."""
-    rc = lib.rvq_decode_rope(ctypes.byref(cfg), _ptr(codes), _ptr(std_f16), n, _ptr(codebooks), _ptr(prepared),
-                             _ptr(position),
-                             vectors_per_position, _ptr(cos_sin), positions, pairing, _ptr(x_out), out_row_stride,
-                             _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_decode_rope(cfg, codes, std_f16, n, codebooks, prepared,
+                             position,
+                             vectors_per_position, cos_sin, positions, pairing, x_out, out_row_stride,
+                             status, stream)
+    if rc and check:
         _check(rc, "rvq_decode_rope")
     return rc
 
@@ -275,11 +277,11 @@ def rvq_attention_decode(cfg_k, cfg_v, q, q_heads, codes_k, std_k, codes_v, std_
                          codebooks_v, position, cos_sin, positions, pairing, scale, out, workspace, workspace_bytes,
                          status=None, stream=None, check=True) -> int:
     """out = attention of the query heads q over the compressed cache (keys rotated as they are read)."""
-    rc = lib.rvq_attention_decode(ctypes.byref(cfg_k), ctypes.byref(cfg_v), _ptr(q), q_heads, _ptr(codes_k), _ptr(std_k),
-                                  _ptr(codes_v), _ptr(std_v), tokens, kv_heads, _ptr(codebooks_k), _ptr(codebooks_v),
-                                  _ptr(position), _ptr(cos_sin), positions, pairing, scale, _ptr(out), _ptr(workspace),
-                                  workspace_bytes, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_attention_decode(cfg_k, cfg_v, q, q_heads, codes_k, std_k,
+                                  codes_v, std_v, tokens, kv_heads, codebooks_k, codebooks_v,
+                                  position, cos_sin, positions, pairing, scale, out, workspace,
+                                  workspace_bytes, status, stream)
+    if rc and check:
         _check(rc, "rvq_attention_decode")
     return rc
 
@@ -288,10 +290,10 @@ def rvq_learn_step(cfg, x, n, x_row_stride, codebooks, prepared, ema_count, ema_
                    decay, eps, workspace, workspace_bytes, status=None, stream=None, check=True,
                    stage_energy=None) -> int:
     """Encode the batch, update N, M and the codebooks from its assignments, rebuild the prepared block."""
-    rc = lib.rvq_learn_step(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(codebooks), _ptr(prepared),
-                            _ptr(ema_count), _ptr(ema_sum), _ptr(codes), _ptr(std_f16), _ptr(stage_energy), decay, eps,
-                            _ptr(workspace), workspace_bytes, _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_learn_step(cfg, x, n, x_row_stride, codebooks, prepared,
+                            ema_count, ema_sum, codes, std_f16, stage_energy, decay, eps,
+                            workspace, workspace_bytes, status, stream)
+    if rc and check:
         _check(rc, "rvq_learn_step")
     return rc
 
@@ -303,10 +305,10 @@ def rvq_kmeans_workspace_bytes(cfg: rvq_config, n: int) -> int:
 def rvq_kmeans_init(cfg, x, n, x_row_stride, seed_rows, iterations, codebooks, prepared, workspace,
                     workspace_bytes, status=None, stream=None, check=True) -> int:
     """Stage-wise k-means initialisation of the codebooks from the int64 [R][K] seed rows."""
-    rc = lib.rvq_kmeans_init(ctypes.byref(cfg), _ptr(x), n, x_row_stride, _ptr(seed_rows), iterations,
-                             _ptr(codebooks), _ptr(prepared), _ptr(workspace), workspace_bytes,
-                             _ptr(status), _stream(stream))
-    if check:
+    rc = _native.rvq_kmeans_init(cfg, x, n, x_row_stride, seed_rows, iterations,
+                             codebooks, prepared, workspace, workspace_bytes,
+                             status, stream)
+    if rc and check:
         _check(rc, "rvq_kmeans_init")
     return rc
 

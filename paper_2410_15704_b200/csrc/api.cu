@@ -1,7 +1,8 @@
 // extern "C" boundary of the RVQ library: argument checks on the host, then
 // dispatch to the kernels.  No allocation, no synchronisation.  Process-wide
-// state: the launch counter below, and (in ema.cu) the per-device address of
-// the built-in scratch array of rvq_ema_update_static.
+// state: the launch counter below, what is remembered about each device (its SM
+// count, the shared memory granted to each kernel), and (in ema.cu) the per-device
+// address of the built-in scratch array of rvq_ema_update_static.
 #include "prepared.cuh"
 #include "rvq_selftest.h"
 
@@ -11,6 +12,54 @@ namespace rvq {
 
 static std::atomic<uint64_t> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+
+namespace {
+
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_sms[kMaxDevices];
+
+// Largest dynamic shared memory granted to a kernel so far, per device: open addressing by the
+// kernel's address; entries are only ever added.  Threads may race to grant the same amount twice.
+struct Grant {
+    std::atomic<const void *> kernel{nullptr};
+    std::atomic<int> bytes{0};
+};
+constexpr int kGrantSlots = 512;                          // (a few times the library's number of kernels)
+Grant g_grants[8][kGrantSlots];
+
+}  // namespace
+
+int sm_count()
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    int sms = dev < kMaxDevices ? g_sms[dev].load(std::memory_order_relaxed) : 0;
+    if (sms > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev < kMaxDevices) g_sms[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
+bool allow_shared_memory(const void *kernel, int bytes)
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
+    auto grant = [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
+    if (dev >= 8) return grant();
+    const uint32_t h = (uint32_t)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) >> 7;
+    for (uint32_t k = 0; k < (uint32_t)kGrantSlots; ++k) {
+        Grant &g = g_grants[dev][(h + k) % kGrantSlots];
+        const void *have = g.kernel.load(std::memory_order_acquire);
+        if (have == nullptr && g.kernel.compare_exchange_strong(have, kernel)) have = kernel;
+        if (have != kernel) continue;
+        if (g.bytes.load(std::memory_order_acquire) >= bytes) return true;
+        if (!grant()) return false;
+        int old = g.bytes.load(std::memory_order_relaxed);
+        while (old < bytes && !g.bytes.compare_exchange_weak(old, bytes, std::memory_order_release)) {}
+        return true;
+    }
+    return grant();
+}
 
 static int ceil_log2(int k)
 {

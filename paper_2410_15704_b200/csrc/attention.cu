@@ -396,10 +396,8 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
                             cudaStream_t stream)
 {
     const int J = q_heads / 8;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return RVQ_ERR_DEVICE;
+    const int sms = sm_count();
+    if (sms <= 0) return RVQ_ERR_DEVICE;
     uint8_t *ws = reinterpret_cast<uint8_t *>(workspace);
     const size_t score_bytes = ((size_t)tokens * q_heads * 4 + 255) / 256 * 256;
     float *scores = reinterpret_cast<float *>(ws);
@@ -416,7 +414,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
     int rc = RVQ_OK;
     auto scores_launch = [&](auto kernel) -> int {
         const size_t smem = (size_t)sk.K * 128;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<parts * kAttSlices, kAttThreads, smem, stream>>>(sk, codes_k, std_k, tokens, cb_k, q, position,
                                                                    reinterpret_cast<const float2 *>(cos_sin), positions,
@@ -427,7 +425,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
         size_t smem = (size_t)sv.K * 128;
         const size_t red = (size_t)5 * J * 32 * 32 * 4;
         if (smem < red) smem = red;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<parts * kAttSlices, kAttThreads, smem, stream>>>(sv, codes_v, std_v, tokens, cb_v, scores, m_ord, scale,
                                                                    out_acc, weight_sum, st);

@@ -1063,20 +1063,16 @@ int launch_decode_rope(const Shape &s, const void *codes, const uint16_t *std16,
         int vpb = 256 / per_vec;
         if (vpb < 1) vpb = 1;
         int64_t blocks = (n + vpb - 1) / vpb;
-        int dev_g = 0, sms_g = 0;
-        if (cudaGetDevice(&dev_g) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms_g, cudaDevAttrMultiProcessorCount, dev_g) != cudaSuccess)
-            return RVQ_ERR_DEVICE;
+        const int sms_g = sm_count();
+        if (sms_g <= 0) return RVQ_ERR_DEVICE;
         if (blocks > (int64_t)sms_g * 16) blocks = (int64_t)sms_g * 16;
         const size_t smem = (size_t)vpb * s.dim * sizeof(float);
         decode_rope_gather_kernel<<<(unsigned)blocks, 256, smem, stream>>>(s, codes, std16, n, cb, out, stride, st, ra,
                                                                            style == 0 ? 1 : 2, vpb);
         return check_launch();
     }
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return RVQ_ERR_DEVICE;
+    const int sms = sm_count();
+    if (sms <= 0) return RVQ_ERR_DEVICE;
     const uint8_t *dsec = nullptr;
     if (levels)
         dsec = reinterpret_cast<const uint8_t *>(prepared) + (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
@@ -1089,7 +1085,7 @@ int launch_decode_rope(const Shape &s, const void *codes, const uint16_t *std16,
         auto quoted = [&](auto kernel) -> int {
             const size_t smem = (size_t)s.K * 128;               // 8 channels of levels or 4 of float32 per code
             const int grid = sms < 8 ? 8 : sms;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
                 return RVQ_ERR_LAUNCH;
             kernel<<<grid, kDecThreads, smem, stream>>>(s, codes, std16, n, d, cb, out, stride, st, ra);
             return check_launch();
@@ -1111,7 +1107,7 @@ int launch_decode_rope(const Shape &s, const void *codes, const uint16_t *std16,
         int parts = sms / ns;
         if (parts > tiles) parts = (int)tiles;
         if (parts < 1) parts = 1;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<parts * ns, kDecThreads, smem, stream>>>(s, codes, std16, n, dsec, cb, out, stride, st, ra);
         return check_launch();
@@ -1152,10 +1148,8 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
     if (n == 0) return RVQ_OK;
     const uint8_t *p = reinterpret_cast<const uint8_t *>(prepared);
     const size_t off = (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return RVQ_ERR_DEVICE;
+    const int sms = sm_count();
+    if (sms <= 0) return RVQ_ERR_DEVICE;
     // which tables: see prepared.cuh
     const bool both = decode_levels_supported(s);                  // then the deviations decide on the device
     const int lch = decode_slice_channels(s.K), fch = decode_exact_channels(s.K);
@@ -1166,7 +1160,7 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
         int parts = sms / ns;
         if (parts > tiles) parts = (int)tiles;
         if (parts < 1) parts = 1;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<parts * ns, kDecThreads, smem, stream>>>(s, codes, std16, n, p + off, cb, out, stride, st);
         return check_launch();
@@ -1177,7 +1171,7 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
         auto quoted = [&](auto kernel) -> int {
             const size_t smem = (size_t)s.K * 16 * lch > (size_t)s.K * 32 * fch ? (size_t)s.K * 16 * lch : (size_t)s.K * 32 * fch;
             int grid = sms < 8 ? 8 : sms;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
                 return RVQ_ERR_LAUNCH;
             kernel<<<grid, kDecThreads, smem, stream>>>(s, codes, std16, n, p + off, cb, out, stride, st);
             return check_launch();

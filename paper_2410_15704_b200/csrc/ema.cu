@@ -270,10 +270,8 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         return RVQ_ERR_LAUNCH;
     int rc = RVQ_OK;
     if (n > 0 && s.gd == 32 && s.G <= 8 && s.per_vector <= 32 && (size_t)bins * sizeof(uint32_t) <= 160 * 1024) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return RVQ_ERR_DEVICE;
+        const int sms = sm_count();
+        if (sms <= 0) return RVQ_ERR_DEVICE;
         const size_t smem = (size_t)bins * sizeof(uint32_t);
         // as many CTAs per SM as the histograms leave room for (up to 8 of 256 threads)
         int per_sm = (int)((200 * 1024) / (smem + 1024));
@@ -281,7 +279,7 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         int64_t want = (n + kWarpStatsThreads / 32 - 1) / (kWarpStatsThreads / 32);
         int grid = (int)(want < (int64_t)sms * per_sm ? want : (int64_t)sms * per_sm);
         auto kernel = s.G == 4 ? ema_stats_quad_kernel : ema_stats_warp_kernel;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<grid, kWarpStatsThreads, smem, stream>>>(s, x, n, stride, codes, cb, cnt, batch_sum, st);
         rc = check_launch();

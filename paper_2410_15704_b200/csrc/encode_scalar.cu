@@ -122,8 +122,8 @@ static int launch_gd(const Shape &s, const void *x, int64_t n, int64_t stride, c
                         sizeof(uint16_t) * (size_t)threads * s.R + 16;
     const int64_t blocks = (n + vpb - 1) / vpb;
     if (blocks > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(encode_scalar_kernel<GD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024 && !allow_shared_memory(reinterpret_cast<const void *>(encode_scalar_kernel<GD>), (int)smem))
+        return RVQ_ERR_LAUNCH;
     encode_scalar_kernel<GD><<<(unsigned)blocks, threads, smem, stream>>>(s, x, n, stride, cb, codes, std16, st, vpb, energy);
     return check_launch();
 }

@@ -852,11 +852,9 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     const int64_t rows = n * s.G;
     const int64_t tiles = (rows + 127) / 128;
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return RVQ_ERR_DEVICE;
-    if (cudaFuncSetAttribute(encode_tensor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
+    const int sms = sm_count();
+    if (sms <= 0) return RVQ_ERR_DEVICE;
+    if (!allow_shared_memory(reinterpret_cast<const void *>(encode_tensor_kernel), kSmemBytes))
         return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,

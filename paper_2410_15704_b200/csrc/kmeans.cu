@@ -138,7 +138,7 @@ int launch_kmeans(const Shape &s, const void *x, int64_t n, int64_t stride, cons
     {
         const size_t smem = ((size_t)vpb * s.dim + 128) * sizeof(float);
         const int64_t blocks = (n + vpb - 1) / vpb;
-        if (cudaFuncSetAttribute(kmeans_scale_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (!allow_shared_memory(reinterpret_cast<const void *>(kmeans_scale_kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kmeans_scale_kernel<<<(unsigned)blocks, 128, smem, stream>>>(s, x, n, stride, c.z, vpb);
         int rc = check_launch();
