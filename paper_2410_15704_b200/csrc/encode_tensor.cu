@@ -52,22 +52,19 @@ constexpr int kTiles = 3;
 constexpr int kRowsPerPass = 128 * kTiles;
 constexpr int kEpiThreads = kRowsPerPass;
 constexpr int kThreads = kEpiThreads + 32 * (kTiles + 1);  // + one MMA issuer warp per tile + loader warp
-constexpr int kRing = 6;                                  // operand slots in flight
+constexpr int kRing = 9;                                  // operand slots in flight
 constexpr int kTileCols = 160;                            // TMEM columns per tile: 128 scores + 32 of A operand
 constexpr int kOnesBytes = 2 * 128 * 16;                  // the constant A cells (1 1 1 0 ...) and (0 ...)
-constexpr int kListCap = 8;
 constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
 
 constexpr int kOffB = 0;
 constexpr int kOffA = kOffB + kRing * kSlotBytes;                    
 constexpr int kOffZ = kOffA + kOnesBytes;                             // parked residuals, float [32][rows]
-constexpr int kOffListV = kOffZ + 32 * kRowsPerPass * 4;              
-constexpr int kOffListI = kOffListV + (kListCap + 1) * kRowsPerPass * 4;   
-constexpr int kOffCodes = kOffListI + (kListCap + 1) * kRowsPerPass * 2;   
+constexpr int kOffCodes = kOffZ + 32 * kRowsPerPass * 4;
 constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;          
 constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: bit 0 valid, bit 1 degenerate
 constexpr int kSmemBytes = kOffFlags + 512;
-constexpr int kDeferMinSlots = 5;                                     // chunks a stage needs for its issuers to take the statistics
+constexpr int kDeferMinSlots = 6;                                     // chunks a stage needs for its issuers to take the statistics
 
 // barrier slots
 constexpr int kBarFull = 0, kBarEmpty = kRing, kBarAReady = 2 * kRing, kBarAccFull = 2 * kRing + kTiles,
@@ -139,6 +136,17 @@ __device__ __forceinline__ void mma_commit(uint32_t bar)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// One lane of a converged warp, chosen by the hardware.  The compiler knows of this predicate that a
+// single lane passes it, and lets the MMA instructions behind it read uniform registers as they are;
+// behind `lane == 0` it wraps each of them in a loop over lanes (77 against 39-67 cycles per
+// instruction, measured).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0u;
+}
+
 __device__ __forceinline__ float min3(float a, float b, float c)
 {
     float d;
@@ -190,9 +198,10 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32
 
 // Per-row state of one stage's sweep over the scores.
 struct Sweep {
-    float m1, thr, win;      // running minimum of the block minima, threshold(m1), error window
+    float win;               // error window
     float zz;                // squared norm of the scaled residual: m1 + zz is the best squared distance
-    int cnt;                 // listed chunks (kListCap + 1: the list overflowed)
+    float m1, m2, m3;        // the three lowest chunk minima ...
+    int c1, c2;              // ... and the chunks of the first two
     float bb[4];             // minimum per 32-column block position inside its 128-column chunk
     float h[2];              // minimum per half (columns 0-15, 16-31) of a block
     float d[16];             // minimum per column position inside its half
@@ -237,26 +246,39 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1)
     return m1 + w.win + 5.4e-6f * (fmaxf(m1 + w.zz, 0.0f) + w.win);
 }
 
-__device__ __forceinline__ void list_block(Sweep &w, float cb_min, int block, float *list_v, uint16_t *list_i,
-                                           int stride)
-{
-    const bool app = cb_min <= w.thr;
-    w.m1 = fminf(w.m1, cb_min);
-    w.thr = threshold(w, w.m1);
-    if (app && w.cnt == kListCap) {
-        // full: drop entries that left the window as the minimum came down
-        int keep = 0;
-        for (int e = 0; e < kListCap; ++e) {
-            const float fv = list_v[e * stride];
-            const uint16_t fi = list_i[e * stride];
-            if (fv <= w.thr) { list_v[keep * stride] = fv; list_i[keep * stride] = fi; ++keep; }
-        }
-        w.cnt = keep;
+// Members of the three partitions whose minimum is at most `limit` (bit k: member k).  The comparisons are
+// subtractions, on the floating-point pipe; one funnel shift each collects their signs.
+struct Listed {
+    uint32_t places, halves, blocks;
+    __device__ __forceinline__ bool single() const
+    {
+        return ((places & (places - 1u)) | (halves & (halves - 1u)) | (blocks & (blocks - 1u))) == 0u;
     }
-    const int slot = min(w.cnt, kListCap);
-    list_v[slot * stride] = cb_min;
-    list_i[slot * stride] = (uint16_t)block;
-    w.cnt += app ? 1 : 0;
+    // column inside the chunk of the lowest members
+    __device__ __forceinline__ int column() const { return (__ffs(blocks) - 1) * 32 + (__ffs(halves) - 1) * 16 + __ffs(places) - 1; }
+};
+__device__ __forceinline__ Listed listed(const Sweep &w, float limit)
+{
+    uint32_t q = 0u, h = 0u, b = 0u;
+#pragma unroll
+    for (int i = 15; i >= 0; --i) q = __funnelshift_l(__float_as_uint(limit - w.d[i]), q, 1);
+#pragma unroll
+    for (int i = 1; i >= 0; --i) h = __funnelshift_l(__float_as_uint(limit - w.h[i]), h, 1);
+#pragma unroll
+    for (int i = 3; i >= 0; --i) b = __funnelshift_l(__float_as_uint(limit - w.bb[i]), b, 1);
+    return {~q & 0xFFFFu, ~h & 3u, ~b & 15u};
+}
+
+// The minimum `v` of chunk c joins the three lowest chunk minima (a tie stays behind the earlier chunk,
+// and so among those that the exact re-scoring compares).
+__device__ __forceinline__ void rank_chunk(Sweep &w, float v, int c)
+{
+    const bool first = v < w.m1, second = v < w.m2;
+    w.m3 = fminf(w.m3, fmaxf(w.m2, v));
+    w.c2 = second ? (first ? w.c1 : c) : w.c2;
+    w.m2 = fminf(w.m2, fmaxf(w.m1, v));
+    w.c1 = first ? c : w.c1;
+    w.m1 = fminf(w.m1, v);
 }
 
 // 32-byte read-only global load: a codeword row costs four of these, and for
@@ -336,7 +358,7 @@ encode_tensor_kernel(const Params p)
     if (tid == 0) {
         for (int i = 0; i < kRing; ++i) { mbar_init(BAR(kBarFull + i), 1); mbar_init(BAR(kBarEmpty + i), kTiles); }
         for (int t = 0; t < kTiles; ++t) {
-            mbar_init(BAR(kBarAReady + t), 128); mbar_init(BAR(kBarAccFull + t), 1); mbar_init(BAR(kBarAccFree + t), 128);
+            mbar_init(BAR(kBarAReady + t), 4); mbar_init(BAR(kBarAccFull + t), 1); mbar_init(BAR(kBarAccFree + t), 4);
         }
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -435,14 +457,14 @@ encode_tensor_kernel(const Params p)
                 // (self-test of the give-up path: the chain that nothing comes after is left out, so that the
                 // epilogue's wait for it runs out with no copy or MMA of this CTA still in flight)
                 if (p.drop_last_chain && t == 0 && q == total - 1) break;
-                if (lane == 0) {
-                    mma_f16_ts(acc, a0, bd, idesc, 0);                      // hi[0:16]  . hi cells 0-1
-                    mma_f16_ts(acc, a0 + 8, bd + 2 * 128, idesc, 1);        // hi[16:32] . hi cells 2-3
-                    mma_f16_ts(acc, a0, bd + 4 * 128, idesc, 1);            // hi[0:16]  . lo cells 4-5
-                    mma_f16_ts(acc, a0 + 8, bd + 6 * 128, idesc, 1);        // hi[16:32] . lo cells 6-7
-                    mma_f16_ts(acc, a0 + 16, bd, idesc, 1);                 // lo[0:16]  . hi cells 0-1
-                    mma_f16_ts(acc, a0 + 24, bd + 2 * 128, idesc, 1);       // lo[16:32] . hi cells 2-3
-                    mma_f16_ss(acc, ones_desc, bd + 8 * 128, idesc, 1);     // (1 1 1 0..) . norm cells 8-9
+                if (elect_one()) {
+                    mma_f16_ts(acc, a0, bd + 1 * 128, idesc, 0);            // hi[0:16]  . hi cells 1-2
+                    mma_f16_ts(acc, a0 + 8, bd + 3 * 128, idesc, 1);        // hi[16:32] . hi cells 3-4
+                    mma_f16_ts(acc, a0, bd + 5 * 128, idesc, 1);            // hi[0:16]  . lo cells 5-6
+                    mma_f16_ts(acc, a0 + 8, bd + 7 * 128, idesc, 1);        // hi[16:32] . lo cells 7-8
+                    mma_f16_ts(acc, a0 + 16, bd + 1 * 128, idesc, 1);       // lo[0:16]  . hi cells 1-2
+                    mma_f16_ts(acc, a0 + 24, bd + 3 * 128, idesc, 1);       // lo[16:32] . hi cells 3-4
+                    mma_f16_ss(acc, ones_desc, bd, idesc, 1);               // (1 1 1 0 .. 0) . norm cell 0 (and cell 1 . 0)
                     mma_commit(bar_acc);
                     mma_commit(BAR(kBarEmpty + slot));
                 }
@@ -475,8 +497,6 @@ encode_tensor_kernel(const Params p)
         const int rloc = tile * 128 + q4 * 32 + lane;
         const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(tile * kTileCols);
         float *z_park = reinterpret_cast<float *>(smem + kOffZ) + rloc;                    // [i][row]
-        float *list_v = reinterpret_cast<float *>(smem + kOffListV) + rloc;              // [e][row]
-        uint16_t *list_i = reinterpret_cast<uint16_t *>(smem + kOffListI) + rloc;         // [e][row]
         uint16_t *codes_s = reinterpret_cast<uint16_t *>(smem + kOffCodes);                // [row][R]
         const int G = s.G;
         uint32_t chunk_use = 0;
@@ -571,14 +591,13 @@ encode_tensor_kernel(const Params p)
                 const StageParams prm = sp[r];
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
                 // scaled half-precision copy of the residual -> A operand row; error window of this row
-                float zz = 0.0f, zmax = 0.0f;
+                float zz = 0.0f;
                 {
                     uint32_t ab[32];                       // 16 words of head, 16 of remainder
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const float z0 = z[2 * i] * prm.scale, z1 = z[2 * i + 1] * prm.scale;
                         zz = fmaf(z0, z0, zz); zz = fmaf(z1, z1, zz);
-                        zmax = fmaxf(zmax, fmaxf(fabsf(z0), fabsf(z1)));
                         const __half2 h2 = __floats2half2_rn(z0, z1);
                         const float2 hf = __half22float2(h2);
                         const __half2 l2 = __floats2half2_rn(z0 - hf.x, z1 - hf.y);
@@ -588,37 +607,28 @@ encode_tensor_kernel(const Params p)
                     tmem_st32(taddr + 128, ab);
                 }
                 tc_fence_before();
-                mbar_arrive(BAR(kBarAReady + tile));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(BAR(kBarAReady + tile));
                 // park the float32 residual in shared memory for the sweep
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kRowsPerPass] = z[i];
                 Sweep w;
                 w.win = 2.125f * (prm.a * sqrtf(zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
                 w.zz = zz;
-                w.m1 = INFINITY; w.thr = INFINITY; w.cnt = 0;
+                w.m1 = w.m2 = w.m3 = INFINITY;
+                w.c1 = w.c2 = 0;
 #pragma unroll
                 for (int q = 0; q < 16; ++q) w.d[q] = INFINITY;
                 w.h[0] = w.h[1] = INFINITY;
                 w.bb[0] = w.bb[1] = w.bb[2] = w.bb[3] = INFINITY;
-                const bool force_scan = !(zmax < 60000.0f) || !(w.win < INFINITY);
+                const bool force_scan = !(zz < 3.6e9f) || !(w.win < INFINITY);      // (no entry reaches 60000 in half precision)
 
 #pragma unroll 1
                 for (int c = 0; c < S && ok; ++c) {
-                    if (c == S - 1 && w.cnt > 0) {
+                    if (c == S - 1 && c > 0) {
                         // Before the last chunk the running winner is the final one most of the time:
                         // start fetching its codeword while the MMA chain runs.
-                        int pb = 0, pq = 0, ph = 0, pbb = 0;
-#pragma unroll
-                        for (int e = kListCap - 1; e >= 0; --e)
-                            if (e < w.cnt && list_v[e * kRowsPerPass] == w.m1) pb = list_i[e * kRowsPerPass];
-#pragma unroll
-                        for (int q = 15; q >= 0; --q)
-                            if (w.d[q] == w.m1) pq = q;
-                        if (w.h[1] == w.m1 && w.h[0] != w.m1) ph = 1;
-#pragma unroll
-                        for (int i = 3; i > 0; --i)
-                            if (w.bb[i] == w.m1) pbb = i;
-                        const int pj = min(pb * 128 + pbb * 32 + 16 * ph + pq, s.K - 1);
+                        const int pj = min(max(w.c1 * 128 + listed(w, w.m1).column(), 0), s.K - 1);
                         asm volatile("prefetch.global.L1 [%0];" ::"l"(cbr + (size_t)pj * 32));
                     }
                     ok = mbar_wait(BAR(kBarAccFull + tile), chunk_use & 1u, abort_flag, p.wait_limit);
@@ -636,61 +646,33 @@ encode_tensor_kernel(const Params p)
                     tmem_ld32_issue(taddr + 96, ud);
                     tmem_ld_wait4(ua, ub, uc, ud);
                     tc_fence_before();
-                    mbar_arrive(BAR(kBarAccFree + tile));        // the accumulator may be overwritten
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(BAR(kBarAccFree + tile));        // the accumulator may be overwritten
                     const float c0 = fold_block(w, ua, 0);
                     const float c1 = fold_block(w, ub, 1);
                     const float c2 = fold_block(w, uc, 2);
                     const float c3 = fold_block(w, ud, 3);
-                    list_block(w, fminf(min3(c0, c1, c2), c3), c, list_v, list_i, kRowsPerPass);
+                    rank_chunk(w, fminf(min3(c0, c1, c2), c3), c);
                 }
                 if (!ok) break;
                 // take the residual back
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z[i] = z_park[i * kRowsPerPass];
                 const float m1 = w.m1;
-                const int cnt = w.cnt;
 
                 // ---- stage end: the columns that can still be the exact argmin are those of a listed
                 // chunk, in a listed block of the chunk, in a listed half, at a listed place.  When each of
                 // the four lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
                 const float lim = threshold(w, m1);
-                int b1 = 0, nlisted = 0;
-                {
-                    bool found = false;
-#pragma unroll
-                    for (int e = 0; e < kListCap; ++e) {
-                        const float fv = list_v[e * kRowsPerPass];
-                        const int fi = list_i[e * kRowsPerPass];
-                        const bool live = e < cnt;
-                        if (live && fv <= lim) ++nlisted;
-                        if (live && !found && fv == m1) { found = true; b1 = fi; }
-                    }
-                }
-                uint32_t qmask = 0u, hmask = 0u, bmask = 0u;
-                int q1 = 0, h1 = 0, bb1 = 0;
-#pragma unroll
-                for (int i = 3; i >= 0; --i) {
-                    if (w.bb[i] <= lim) bmask |= 1u << i;
-                    if (w.bb[i] == m1) bb1 = i;
-                }
-#pragma unroll
-                for (int q = 15; q >= 0; --q) {
-                    if (w.d[q] <= lim) qmask |= 1u << q;
-                    if (w.d[q] == m1) q1 = q;
-                }
-#pragma unroll
-                for (int c = 1; c >= 0; --c) {
-                    if (w.h[c] <= lim) hmask |= 1u << c;
-                    if (w.h[c] == m1) h1 = c;
-                }
-                const int j1 = b1 * 128 + bb1 * 32 + 16 * h1 + q1;
+                const Listed in = listed(w, lim);
+                const uint32_t qmask = in.places, hmask = in.halves, bmask = in.blocks;
+                const int j1 = w.c1 * 128 + in.column();
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
-                const bool scan_all = force_scan || cnt == 0 || cnt > kListCap || !(m1 < 59000.0f);
-                const bool unique = nlisted == 1 && (qmask & (qmask - 1u)) == 0u && (hmask & (hmask - 1u)) == 0u &&
-                                    (bmask & (bmask - 1u)) == 0u && j1 < s.K;
+                const bool scan_all = force_scan || w.m3 <= lim || !(m1 < 59000.0f);
+                const bool unique = w.m2 > lim && in.single() && (uint32_t)j1 < (uint32_t)s.K;
                 const bool flagged = !deg && (scan_all || !unique);
-                int bj = j1 < s.K ? j1 : 0;
+                int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
                 // Rows with more than one candidate: the whole warp re-scores the candidate columns of
                 // every listed block of one such row at a time (lane = place in the block; all columns
                 // when the list overflowed) exactly in float32, direct form, then reduces to the
@@ -702,13 +684,12 @@ encode_tensor_kernel(const Params p)
                     float zs[32];
 #pragma unroll
                     for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kRowsPerPass + (src - lane)];
-                    const float lim_s = __shfl_sync(0xFFFFFFFFu, lim, src);
-                    const int cnt_s = __shfl_sync(0xFFFFFFFFu, cnt, src);
+                    const int chunk1 = __shfl_sync(0xFFFFFFFFu, w.c1, src);
+                    const int chunk2 = __shfl_sync(0xFFFFFFFFu, w.m2 <= lim ? w.c2 : -1, src);
                     const uint32_t qmask_s = __shfl_sync(0xFFFFFFFFu, qmask, src);
                     const uint32_t hmask_s = __shfl_sync(0xFFFFFFFFu, hmask, src);
                     const uint32_t bmask_s = __shfl_sync(0xFFFFFFFFu, bmask, src);
                     const bool all_s = __shfl_sync(0xFFFFFFFFu, (int)scan_all, src) != 0;
-                    const int row_s = rloc - lane + src;
                     const bool mine = ((qmask_s >> (lane & 15)) & 1u) && ((hmask_s >> (lane >> 4)) & 1u);
                     float bv = INFINITY;
                     int bi = 0x7FFFFFFF;
@@ -718,15 +699,14 @@ encode_tensor_kernel(const Params p)
                             if (dj < bv) { bv = dj; bi = j; }
                         }
                     } else {
-                        for (int e = 0; e < cnt_s; ++e) {
-                            const float fv = reinterpret_cast<const float *>(smem + kOffListV)[e * kRowsPerPass + row_s];
-                            if (!(fv <= lim_s)) continue;                              // warp-uniform
-                            const int j0 = (int)reinterpret_cast<const uint16_t *>(smem + kOffListI)[e * kRowsPerPass + row_s] * 128 + lane;
+                        for (int e = 0; e < 2; ++e) {
+                            const int chunk = e == 0 ? chunk1 : chunk2;                 // warp-uniform
+                            if (chunk < 0) continue;
                             for (int i = 0; i < 4; ++i) {
-                                const int j = j0 + 32 * i;
+                                const int j = chunk * 128 + 32 * i + lane;
                                 if (((bmask_s >> i) & 1u) && mine && j < s.K) {     // (the block test is warp-uniform)
                                     const float dj = exact_distance(zs, cbr + (size_t)j * 32);
-                                    if (dj < bv) { bv = dj; bi = j; }
+                                    if (dj < bv || (dj == bv && j < bi)) { bv = dj; bi = j; }
                                 }
                             }
                         }

@@ -12,12 +12,13 @@
 // Per stage r the block holds
 //   - a power-of-two scale 2^k chosen so that the largest scaled squared norm
 //     is about 2^13 (keeps the operands out of the half-precision subnormals);
-//   - the B operand image of tcgen05.mma: for every slot of 128 codewords ten
+//   - the B operand image of tcgen05.mma: for every slot of 128 codewords nine
 //     "cells" (8 halves = 16 bytes per codeword per cell, K-major, no swizzle):
-//     cells 0-3 hold -2 e_hi, cells 4-7 hold -2 e_lo, cell 8 holds the scaled
-//     squared norm split into three halves (hi, lo, lo2) then zeros, cell 9 is
-//     zero.  The A operand carries (Z_hi, Z_lo, 1 1 1 0...), and seven K=16
-//     steps pair the cells so that the accumulator is the score;
+//     cell 0 holds the scaled squared norm split into three halves (hi, lo, lo2)
+//     then zeros, cells 1-4 hold -2 e_hi, cells 5-8 hold -2 e_lo.  The A operand
+//     carries (Z_hi, Z_lo, 1 1 1 0 ... 0), and seven K=16 steps pair the cells so
+//     that the accumulator is the score (the norm's step takes cells 0 and 1, and
+//     A is zero where cell 1 stands);
 //   - two numbers (a, b) such that |score error| <= a * ||Z|| + b, from the
 //     actual rounding errors of this codebook (see prepare_finish_kernel).
 #include "prepared.cuh"
@@ -240,20 +241,20 @@ prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *_
             const double hv = (double)__half2float(hi);
             const __half lo = __double2half(es - hv);
             const double lv = (double)__half2float(lo);
-            cell[i >> 3][i & 7] = __float2half_rn(-2.0f * __half2float(hi));          // exact doubling
-            cell[4 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(lo));
+            cell[1 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(hi));      // exact doubling
+            cell[5 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(lo));
             n2 += es * es; l2 += lv * lv; d2 += (es - hv - lv) * (es - hv - lv);
         }
         const __half n_hi = __double2half(n2);
         const double r1 = n2 - (double)__half2float(n_hi);
         const __half n_lo = __double2half(r1);
         const double r2 = r1 - (double)__half2float(n_lo);
-        cell[8][0] = n_hi; cell[8][1] = n_lo; cell[8][2] = __double2half(r2);
+        cell[0][0] = n_hi; cell[0][1] = n_lo; cell[0][2] = __double2half(r2);
         // round the maxima up so that the bound stays a bound in float32
         emax = __double2float_ru(sqrt(n2)); eerr = __double2float_ru(sqrt(d2));
         nmax = __double2float_ru(n2); elomax = __double2float_ru(sqrt(l2));
     } else {
-        cell[8][0] = __float2half_rn(60000.0f);           // padding never wins
+        cell[0][0] = __float2half_rn(60000.0f);           // padding never wins
     }
     for (int c = 0; c < kSlotCells; ++c)
         *reinterpret_cast<uint4 *>(base + ((size_t)c * kSlotCodewords + jj) * 16) = *reinterpret_cast<const uint4 *>(cell[c]);

@@ -8,8 +8,8 @@ namespace rvq {
 
 constexpr uint32_t kPreparedMagic = 0x52565133u;
 constexpr int kSlotCodewords = 128;                       // codewords per operand slot
-constexpr int kSlotCells = 10;                            // hi (4), lo (4), norm (1), zero (1) cells of 8 halves
-constexpr int kSlotBytes = kSlotCells * kSlotCodewords * 16;   // 20480
+constexpr int kSlotCells = 9;                             // norm (1), hi (4), lo (4) cells of 8 halves
+constexpr int kSlotBytes = kSlotCells * kSlotCodewords * 16;   // 18432
 constexpr size_t kPreparedParamsOffset = 256;             // StageParams[16]
 constexpr size_t kPreparedMaximaOffset = 512;             // StageMaxima[16]
 constexpr size_t kPreparedPartialsOffset = 768;           // StagePartial[16 stages][kPrepareParts], scratch of the prepare step
@@ -80,7 +80,7 @@ __host__ __device__ inline bool decode_sliced_supported(const Shape &s)
 }
 __host__ __device__ inline size_t encode_image_bytes(const Shape &s)
 {
-    return s.gd == 32 ? (size_t)s.R * ((s.K + 127) / 128) * 20480 : 0;
+    return s.gd == 32 ? (size_t)s.R * ((s.K + kSlotCodewords - 1) / kSlotCodewords) * kSlotBytes : 0;
 }
 
 struct StageParams {
