@@ -166,6 +166,8 @@ static int encode_common(const rvq_config *cfg, const void *x, int64_t n, int64_
     if (!aligned16(codebooks) || !aligned16(codes) || !aligned256(prepared)) return RVQ_ERR_ALIGN;
     if (stage_energy && cudaMemsetAsync(stage_energy, 0, (size_t)s.R * sizeof(float), (cudaStream_t)stream) != cudaSuccess)
         return RVQ_ERR_LAUNCH;
+    if (allow_tensor && !stat_sum && encode_small_wanted(s, n))
+        return launch_encode_small(s, x, n, x_row_stride, prepared, codes, std_f16, status, (cudaStream_t)stream, stage_energy);
     if (allow_tensor && encode_tensor_supported(s))
         return launch_encode_tensor(s, x, n, x_row_stride, codebooks, prepared, codes, std_f16, status,
                                     (cudaStream_t)stream, stat_cnt, stat_sum, stage_energy);

@@ -30,6 +30,10 @@ inline bool aligned256(const void *p) { return (reinterpret_cast<uintptr_t>(p) &
 int launch_encode_scalar(const Shape &s, const void *x, int64_t n, int64_t stride, const float *cb,
                          void *codes, uint16_t *std16, rvq_status *st, cudaStream_t stream,
                          float *energy = nullptr);
+// a few head vectors: the codebook split over the CTAs of a cluster, exact float32 distances
+bool encode_small_wanted(const Shape &s, int64_t n);
+int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride, const void *prepared, void *codes,
+                        uint16_t *std16, rvq_status *st, cudaStream_t stream, float *energy);
 bool encode_tensor_supported(const Shape &s);
 int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t stride, const float *cb,
                          const void *prepared, void *codes, uint16_t *std16, rvq_status *st,

@@ -1075,13 +1075,13 @@ int launch_decode_rope(const Shape &s, const void *codes, const uint16_t *std16,
     if (sms <= 0) return RVQ_ERR_DEVICE;
     const uint8_t *dsec = nullptr;
     if (levels)
-        dsec = reinterpret_cast<const uint8_t *>(prepared) + (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
+        dsec = reinterpret_cast<const uint8_t *>(prepared) + decode_section_offset(s);
     const int64_t tiles = (n * s.G + kDecThreads - 1) / kDecThreads;
     // the quoted shapes with a prepared block: one launch, tables chosen on the device
     if (prepared != nullptr && decode_levels_supported(s) && s.dim == 128 && s.G == 4 && s.R == 8 && s.K <= kDecodeWideK &&
         n * 4 < 0x7FFFFFFFLL && (s.bits == 16 || s.bits == 10 || s.bits == 11)) {
         const uint8_t *d = reinterpret_cast<const uint8_t *>(prepared) +
-                           (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
+                           decode_section_offset(s);
         auto quoted = [&](auto kernel) -> int {
             const size_t smem = (size_t)s.K * 128;               // 8 channels of levels or 4 of float32 per code
             const int grid = sms < 8 ? 8 : sms;
@@ -1147,7 +1147,7 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
 {
     if (n == 0) return RVQ_OK;
     const uint8_t *p = reinterpret_cast<const uint8_t *>(prepared);
-    const size_t off = (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
+    const size_t off = decode_section_offset(s);
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
     // which tables: see prepared.cuh

@@ -1,0 +1,383 @@
+// What the tensor-core encoders share: mbarriers and bounded waits, tcgen05 operands, chains and
+// TMEM reads, the fold of the scores into running minima, the error window, exact distances, and the
+// ends of the path (rows in, deviation, operand, codes out).
+#pragma once
+
+#include "prepared.cuh"
+
+namespace rvq {
+
+constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
+constexpr int kOnesBytes = 2 * 128 * 16;                  // the constant A cells (1 1 1 0 ...) and (0 ...)
+constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 -> f32, M = N = 128
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Bounded wait; returns false (and raises the CTA's abort flag) when it gives up.  A phase that has
+// completed already is recognised by the non-blocking test (a plain shared-memory read); only a
+// phase still pending goes through the suspending form.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag,
+                                          uint32_t limit = kWaitLimit)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+#pragma unroll 1
+    for (uint32_t it = 0; it < limit; ++it) {
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if ((it & 1023u) == 1023u && *abort_flag) return false;
+    }
+    *abort_flag = 1u;
+    return false;
+}
+
+__device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes)
+{
+    // K-major, no swizzle: 8x16-byte core matrices; LBO steps along the
+    // contraction, SBO along rows; descriptor version 1.
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16) |
+           ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// One lane of a converged warp, chosen by the hardware.  The compiler knows of this predicate that a
+// single lane passes it, and lets the MMA instructions behind it read uniform registers as they are;
+// behind `lane == 0` it wraps each of them in a loop over lanes (77 against 39-67 cycles per
+// instruction, measured).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0u;
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+#define RVQ_R32(u) u[0], u[1], u[2], u[3], u[4], u[5], u[6], u[7], u[8], u[9], u[10], u[11], u[12], u[13], u[14], u[15], \
+    u[16], u[17], u[18], u[19], u[20], u[21], u[22], u[23], u[24], u[25], u[26], u[27], u[28], u[29], u[30], u[31]
+#define RVQ_OUT32(u) "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), \
+    "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), \
+    "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), \
+    "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+#define RVQ_INOUT32(u) "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]), \
+    "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15]), \
+    "+r"(u[16]), "+r"(u[17]), "+r"(u[18]), "+r"(u[19]), "+r"(u[20]), "+r"(u[21]), "+r"(u[22]), "+r"(u[23]), \
+    "+r"(u[24]), "+r"(u[25]), "+r"(u[26]), "+r"(u[27]), "+r"(u[28]), "+r"(u[29]), "+r"(u[30]), "+r"(u[31])
+#define RVQ_IN32(u) "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]), "r"(u[7]), \
+    "r"(u[8]), "r"(u[9]), "r"(u[10]), "r"(u[11]), "r"(u[12]), "r"(u[13]), "r"(u[14]), "r"(u[15]), \
+    "r"(u[16]), "r"(u[17]), "r"(u[18]), "r"(u[19]), "r"(u[20]), "r"(u[21]), "r"(u[22]), "r"(u[23]), \
+    "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]), "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
+
+// Start loading 32 consecutive TMEM columns of this thread's lane.  The
+// registers are not valid until tmem_ld_wait() has been given the same array.
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : RVQ_OUT32(u) : "r"(taddr));
+}
+// Waits for every tcgen05.ld of this thread; the arrays pass through so that no
+// use of them can be scheduled ahead of the wait.
+__device__ __forceinline__ void tmem_ld_wait4(uint32_t (&u)[32], uint32_t (&v)[32], uint32_t (&w)[32], uint32_t (&x)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
+    asm volatile("" : RVQ_INOUT32(v) : : "memory");
+    asm volatile("" : RVQ_INOUT32(w) : : "memory");
+    asm volatile("" : RVQ_INOUT32(x) : : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+                 "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+                 : : "r"(taddr), RVQ_IN32(u) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// Per-row state of one stage's sweep over the scores.
+struct Sweep {
+    float win;               // error window
+    float zz;                // squared norm of the scaled residual: m1 + zz is the best squared distance
+    float m1, m2, m3;        // the three lowest chunk minima ...
+    int c1, c2;              // ... and the chunks of the first two
+    float bb[4];             // minimum per 32-column block position inside its 128-column chunk
+    float h[2];              // minimum per half (columns 0-15, 16-31) of a block
+    float d[16];             // minimum per column position inside its half
+};
+
+// One 32-column block of scores (block `b` of its chunk) folded into the running minima of three
+// partitions of its columns: the 16 places inside a half (one three-input minimum takes in the two
+// columns of a place), the two halves, and the block itself; returns the block minimum.  Together
+// with the chunk list a column that could be the argmin is pinned to (listed chunk) x (block of the
+// chunk) x (half) x (place): when every one of the four lists has a single entry, to one column.
+// 36 minimum operations per 32 scores: they run on the narrow integer/compare pipe, which this sweep
+// keeps about as busy as the tensor pipe, so their number per score is what the sweep's speed
+// hangs on.
+__device__ __forceinline__ float fold_block(Sweep &w, const uint32_t (&u)[32], int b)
+{
+#pragma unroll
+    for (int c = 0; c < 16; ++c) w.d[c] = min3(w.d[c], __uint_as_float(u[c]), __uint_as_float(u[c + 16]));
+    float hm[2];
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+        const uint32_t *v = u + 16 * hf;
+        const float a0 = min3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
+        const float a1 = min3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
+        const float a2 = min3(__uint_as_float(v[6]), __uint_as_float(v[7]), __uint_as_float(v[8]));
+        const float a3 = min3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
+        const float a4 = min3(__uint_as_float(v[12]), __uint_as_float(v[13]), __uint_as_float(v[14]));
+        hm[hf] = fminf(min3(a0, a1, a2), min3(a3, a4, __uint_as_float(v[15])));
+    }
+    w.h[0] = fminf(w.h[0], hm[0]);
+    w.h[1] = fminf(w.h[1], hm[1]);
+    const float m = fminf(hm[0], hm[1]);
+    w.bb[b] = fminf(w.bb[b], m);
+    return m;
+}
+
+// A column can only be the exact-L2 choice (in real arithmetic, and in the float32 direct-form
+// arithmetic of the all-float32 kernel, whose relative error on a distance is below 34 * 2^-24) if its
+// approximate score is at most threshold(m1): the window covers the approximation error of both
+// scores, the last term the float32 evaluation error of both distances (2 * 34 * 2^-24 < 2^-17.5).
+__device__ __forceinline__ float threshold(const Sweep &w, float m1)
+{
+    return m1 + w.win + 5.4e-6f * (fmaxf(m1 + w.zz, 0.0f) + w.win);
+}
+
+// Members of the three partitions whose minimum is at most `limit` (bit k: member k).  The comparisons are
+// subtractions, on the floating-point pipe; one funnel shift each collects their signs.
+struct Listed {
+    uint32_t places, halves, blocks;
+    __device__ __forceinline__ bool single() const
+    {
+        return ((places & (places - 1u)) | (halves & (halves - 1u)) | (blocks & (blocks - 1u))) == 0u;
+    }
+    // column inside the chunk of the lowest members
+    __device__ __forceinline__ int column() const { return (__ffs(blocks) - 1) * 32 + (__ffs(halves) - 1) * 16 + __ffs(places) - 1; }
+};
+__device__ __forceinline__ Listed listed(const Sweep &w, float limit)
+{
+    uint32_t q = 0u, h = 0u, b = 0u;
+#pragma unroll
+    for (int i = 15; i >= 0; --i) q = __funnelshift_l(__float_as_uint(limit - w.d[i]), q, 1);
+#pragma unroll
+    for (int i = 1; i >= 0; --i) h = __funnelshift_l(__float_as_uint(limit - w.h[i]), h, 1);
+#pragma unroll
+    for (int i = 3; i >= 0; --i) b = __funnelshift_l(__float_as_uint(limit - w.bb[i]), b, 1);
+    return {~q & 0xFFFFu, ~h & 3u, ~b & 15u};
+}
+
+// The minimum `v` of chunk c joins the three lowest chunk minima (a tie stays behind the earlier chunk,
+// and so among those that the exact re-scoring compares).
+__device__ __forceinline__ void rank_chunk(Sweep &w, float v, int c)
+{
+    const bool first = v < w.m1, second = v < w.m2;
+    w.m3 = fminf(w.m3, fmaxf(w.m2, v));
+    w.c2 = second ? (first ? w.c1 : c) : w.c2;
+    w.m2 = fminf(w.m2, fmaxf(w.m1, v));
+    w.c1 = first ? c : w.c1;
+    w.m1 = fminf(w.m1, v);
+}
+
+// 32-byte read-only global load: a codeword row costs four of these, and for
+// row-per-lane gathers it is the number of load instructions that the L1 pays for.
+__device__ __forceinline__ void ldg256(const float *p, float (&v)[8])
+{
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+
+// Exact squared distance, direct form, same operation order as the scalar kernel.
+__device__ __forceinline__ float exact_distance(const float (&z)[32], const float *__restrict__ e)
+{
+    float acc = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float ev[8];
+        ldg256(e + 8 * q, ev);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { const float t = z[8 * q + k] - ev[k]; acc = fmaf(t, t, acc); }
+    }
+    return acc;
+}
+
+// The seven K = 16 steps of one chain: 128 rows (A: TMEM columns a0 ..: 16 of head, 16 of remainder)
+// against the 128 codewords of the slot that `bd` describes, scores to the 128 columns from `acc`.  A
+// B cell is 128 codewords x 16 bytes = 128 descriptor address units.
+__device__ __forceinline__ void issue_chain(uint32_t acc, uint32_t a0, uint64_t bd, uint64_t ones_desc)
+{
+    mma_f16_ts(acc, a0, bd + 1 * 128, kChainDesc, 0);            // hi[0:16]  . hi cells 1-2
+    mma_f16_ts(acc, a0 + 8, bd + 3 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 3-4
+    mma_f16_ts(acc, a0, bd + 5 * 128, kChainDesc, 1);            // hi[0:16]  . lo cells 5-6
+    mma_f16_ts(acc, a0 + 8, bd + 7 * 128, kChainDesc, 1);        // hi[16:32] . lo cells 7-8
+    mma_f16_ts(acc, a0 + 16, bd + 1 * 128, kChainDesc, 1);       // lo[0:16]  . hi cells 1-2
+    mma_f16_ts(acc, a0 + 24, bd + 3 * 128, kChainDesc, 1);       // lo[16:32] . hi cells 3-4
+    mma_f16_ss(acc, ones_desc, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 0 (and cell 1 . 0)
+}
+
+// The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces through
+// a scratch area of shared memory in which word k sits at scr[(k / 32) * PITCH + k % 32]; piece c of
+// vector vl is at position c ^ (vl mod 8) of its vector so that the reads by row spread over the banks.
+// Lane l gets the 32 elements of group l % G of vector l / G, zeros past the last vector.
+template <int PITCH>
+__device__ __forceinline__ void load_group_rows(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride,
+                                                int64_t v_first, int lane, float *scr, float (&z)[32])
+{
+    const int G = s.G, eb = s.elem_bytes, ppv = s.dim * eb / 16;          // pieces per vector (>= 4)
+    // (four loads in flight per lane: a 16-bit head vector of 128 channels is 16 pieces, so the
+    // 8 vectors of a warp are 4 pieces per lane)
+    const int npieces = (32 / G) * ppv;
+    for (int c0 = 0; c0 < npieces; c0 += 128) {
+        uint4 val[4];
+        int kk[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + 32 * u + lane;
+            const int vl = c / ppv, off = c - vl * ppv;
+            const int64_t vv = v_first + vl;
+            val[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (c < npieces && vv < n)
+                val[u] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(x) + vv * stride * eb) + off);
+            kk[u] = (vl * ppv + (off ^ (vl & 7 & (ppv - 1)))) * 4;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (c0 + 32 * u + lane < npieces)
+                *reinterpret_cast<uint4 *>(scr + (kk[u] >> 5) * PITCH + (kk[u] & 31)) = val[u];
+    }
+    __syncwarp();
+    const int vl = lane / G, g = lane - vl * G, sw = vl & 7 & (ppv - 1);
+    const bool valid = v_first + vl < n;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const int b = channel_of(s.layout, G, 32, g, i) * eb;      // byte within the vector
+        const int k = (vl * ppv + ((b >> 4) ^ sw)) * 4 + ((b & 15) >> 2);
+        const uint32_t word = __float_as_uint(scr[(k >> 5) * PITCH + (k & 31)]);
+        float val;
+        if (s.dtype == RVQ_F32) val = __uint_as_float(word);
+        else {
+            const uint16_t h = (b & 2) ? (uint16_t)(word >> 16) : (uint16_t)(word & 0xFFFFu);
+            val = s.dtype == RVQ_BF16 ? __uint_as_float((uint32_t)h << 16) : __half2float(__ushort_as_half(h));
+        }
+        z[i] = valid ? val : 0.0f;
+    }
+    __syncwarp();
+}
+
+// Deviation over the G lanes of this lane's head vector, same summation order as the scalar kernel.
+__device__ __forceinline__ float group_deviation(const Shape &s, const float (&z)[32], int lane)
+{
+    const int base = lane & ~(s.G - 1);                      // (G is a power of two)
+    float a = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) a += z[i];
+    float mu = 0.0f;
+    for (int k = 0; k < s.G; ++k) mu += __shfl_sync(0xFFFFFFFFu, a, base + k);
+    mu /= (float)s.dim;
+    float b = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) b += (z[i] - mu) * (z[i] - mu);
+    float ss = 0.0f;
+    for (int k = 0; k < s.G; ++k) ss += __shfl_sync(0xFFFFFFFFu, b, base + k);
+    return sqrtf(ss / (float)(s.dim - s.ddof));
+}
+
+// A operand row of the residual z: 16 words of half-precision head, 16 of remainder; returns the squared
+// norm of the scaled residual.
+__device__ __forceinline__ float split_operand(const float (&z)[32], float scale, uint32_t (&ab)[32])
+{
+    float zz = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const float z0 = z[2 * i] * scale, z1 = z[2 * i + 1] * scale;
+        zz = fmaf(z0, z0, zz); zz = fmaf(z1, z1, zz);
+        const __half2 h2 = __floats2half2_rn(z0, z1);
+        const float2 hf = __half22float2(h2);
+        const __half2 l2 = __floats2half2_rn(z0 - hf.x, z1 - hf.y);
+        ab[i] = *reinterpret_cast<const uint32_t *>(&h2);
+        ab[16 + i] = *reinterpret_cast<const uint32_t *>(&l2);
+    }
+    return zz;
+}
+
+// Codes of the warp's 32 rows (first vector v_first), from codes_s[row of the warp][16], to global memory in
+// the configured storage form (Section 3.2).
+__device__ __forceinline__ void emit_codes(const Shape &s, const uint16_t *codes_s, int64_t v_first, int64_t n, int lane,
+                                           void *__restrict__ codes)
+{
+    const int G = s.G;
+    if (s.bits == 16) {
+        const int64_t v = v_first + lane / G;
+        if (v < n) {
+            uint16_t *o = reinterpret_cast<uint16_t *>(codes) + (v * G + (lane & (G - 1))) * s.R;
+            if (s.R == 8) {
+                *reinterpret_cast<uint4 *>(o) = *reinterpret_cast<const uint4 *>(codes_s + lane * 16);
+            } else {
+                for (int r = 0; r < s.R; ++r) o[r] = codes_s[lane * 16 + r];
+            }
+        }
+    } else {
+        // the warp holds 32 / G whole head vectors; one 32-bit word per lane and step
+        const int words = s.code_bytes / 4, vec_per_warp = 32 / G;
+        for (int t = lane; t < vec_per_warp * words; t += 32) {
+            const int vl = t / words, w = t - vl * words;
+            const int64_t vv = v_first + vl;
+            if (vv >= n) continue;
+            uint32_t word = 0;
+            const int k_lo = (32 * w) / s.bits, k_hi = min(s.per_vector - 1, (32 * w + 31) / s.bits);
+            for (int k = k_lo; k <= k_hi; ++k) {
+                const int gg = k / s.R, rr = k - gg * s.R;
+                const uint32_t val = codes_s[(vl * G + gg) * 16 + rr];
+                const int sh = k * s.bits - 32 * w;
+                word |= sh >= 0 ? (val << sh) : (val >> (-sh));
+            }
+            reinterpret_cast<uint32_t *>(codes)[vv * words + w] = word;
+        }
+    }
+}
+
+}  // namespace rvq

@@ -19,22 +19,16 @@
 //     carries (Z_hi, Z_lo, 1 1 1 0 ... 0), and seven K=16 steps pair the cells so
 //     that the accumulator is the score (the norm's step takes cells 0 and 1, and
 //     A is zero where cell 1 stands);
+//   - the float32 codewords again, in blocks of 128 (prepared.cuh), for the encoder of a few vectors;
 //   - two numbers (a, b) such that |score error| <= a * ||Z|| + b, from the
 //     actual rounding errors of this codebook (see prepare_finish_kernel).
 #include "prepared.cuh"
 
 namespace rvq {
 
-static size_t decode_section_offset(const Shape &s)
-{
-    return (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
-}
-
 size_t prepared_bytes(const Shape &s)
 {
-    size_t b = decode_section_offset(s);
-    if (decode_levels_prepared(s)) b += 256 + 2 * decode_table_bytes(s.K);
-    return (b + 255) / 256 * 256;
+    return (float_blocks_offset(s) + float_blocks_bytes(s) + 255) / 256 * 256;
 }
 
 // One thread per (channel octet, code, stage): 8 channels of levels, stored as one 16-byte
@@ -170,7 +164,7 @@ prepare_params_kernel(Shape s, const StagePartial *__restrict__ part, PreparedHe
         hdr->magic = kPreparedMagic; hdr->R = s.R; hdr->K = s.K; hdr->gd = s.gd;
         hdr->slots = slots_per_stage(s.K);
         hdr->decode_offset = decode_levels_prepared(s)
-            ? (uint32_t)((kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256) : 0u;
+            ? (uint32_t)(decode_section_offset(s)) : 0u;
         if (dp) {
             // a common base and integer scales 1..255: the unit of a stage becomes scale * base >= its finest
             float umax = 0.0f;
@@ -221,7 +215,7 @@ prepare_params_kernel(Shape s, const StagePartial *__restrict__ part, PreparedHe
 // bound needs.  grid = (slots * 128 / 128, R).
 __global__ void __launch_bounds__(128)
 prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *__restrict__ sp,
-                     StageMaxima *mx, uint8_t *__restrict__ image)
+                     StageMaxima *mx, uint8_t *__restrict__ image, float4 *__restrict__ blocks)
 {
     const int r = blockIdx.y;
     const int slot = blockIdx.x, jj = threadIdx.x;
@@ -258,6 +252,13 @@ prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *_
     }
     for (int c = 0; c < kSlotCells; ++c)
         *reinterpret_cast<uint4 *>(base + ((size_t)c * kSlotCodewords + jj) * 16) = *reinterpret_cast<const uint4 *>(cell[c]);
+    if (blocks) {
+        // the float32 block of this slot, piece by piece
+        float4 *o = blocks + ((size_t)r * slots_per_stage(s.K) + slot) * (kFloatBlockBytes / 16) + jj;
+        const float4 *e = reinterpret_cast<const float4 *>(cb + ((size_t)r * s.K + j) * 32);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) o[q * kSlotCodewords] = j < s.K ? e[q] : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+    }
     // non-negative floats order like their bit patterns
     atomicMax(&mx[r].emax, __float_as_uint(emax));
     atomicMax(&mx[r].eerr, __float_as_uint(eerr));
@@ -307,7 +308,8 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
     if ((rc = check_launch()) != RVQ_OK) return rc;
     if (s.gd == 32) {
         dim3 grid(slots_per_stage(s.K), s.R);
-        prepare_image_kernel<<<grid, kSlotCodewords, 0, stream>>>(s, cb, sp, mx, p + kPreparedImageOffset);
+        prepare_image_kernel<<<grid, kSlotCodewords, 0, stream>>>(s, cb, sp, mx, p + kPreparedImageOffset,
+            float_blocks_prepared(s) ? reinterpret_cast<float4 *>(p + float_blocks_offset(s)) : nullptr);
         if ((rc = check_launch()) != RVQ_OK) return rc;
         prepare_finish_kernel<<<1, 32, 0, stream>>>(s, sp, mx);
         if ((rc = check_launch()) != RVQ_OK) return rc;

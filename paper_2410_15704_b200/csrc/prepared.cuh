@@ -78,9 +78,33 @@ __host__ __device__ inline bool decode_sliced_supported(const Shape &s)
 {
     return decode_exact_tables(s) || decode_levels_supported(s);
 }
+// Float32 section (group_dim 32, R <= kFloatMaxStages, K <= kFloatMaxK), after the decoder section: the
+// codebooks as float32 with the pieces of a codeword apart, [R][blocks of 128 codewords][8 pieces][128][4], so
+// that a block is one copy and neighbouring threads read neighbouring 16 bytes of it.  Padding codewords are
+// infinite (never the nearest).
+constexpr int kFloatMaxStages = 8;
+constexpr int kFloatMaxK = 2048;
+constexpr int kFloatBlockBytes = 128 * 128;
+__host__ __device__ inline bool float_blocks_prepared(const Shape &s)
+{
+    return s.gd == 32 && s.R <= kFloatMaxStages && s.K <= kFloatMaxK;
+}
 __host__ __device__ inline size_t encode_image_bytes(const Shape &s)
 {
     return s.gd == 32 ? (size_t)s.R * ((s.K + kSlotCodewords - 1) / kSlotCodewords) * kSlotBytes : 0;
+}
+
+__host__ __device__ inline size_t decode_section_offset(const Shape &s)
+{
+    return (kPreparedImageOffset + encode_image_bytes(s) + 255) / 256 * 256;
+}
+__host__ __device__ inline size_t float_blocks_offset(const Shape &s)
+{
+    return decode_section_offset(s) + (decode_levels_prepared(s) ? 256 + 2 * decode_table_bytes(s.K) : 0);
+}
+__host__ __device__ inline size_t float_blocks_bytes(const Shape &s)
+{
+    return float_blocks_prepared(s) ? (size_t)s.R * ((s.K + 127) / 128) * kFloatBlockBytes : 0;
 }
 
 struct StageParams {

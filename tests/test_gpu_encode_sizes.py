@@ -1,0 +1,65 @@
+"""The encoders that split a row's codebook over several CTAs (few head vectors), at the sizes where a
+dispatch or a split can go wrong: codes, deviations and stage energies against the all-float32 kernel."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2410_15704_b200 as rvq
+from helpers import DT, assert_codes_match
+
+pytestmark = pytest.mark.gpu
+
+
+def batch(n, dim, K, R, dtype, seed):
+    g = np.random.default_rng(seed)
+    scale = np.where(g.random(dim) < 0.06, 20.0, 1.0)
+    x = torch.from_numpy((g.normal(size=(n, dim)) * scale).astype(np.float32)).to(rvq.TORCH_DTYPE[DT[dtype]])
+    if n % 2 == 1 and n > 3:
+        x[2] = 0.0                                          # degenerate
+    cb = np.stack([g.normal(scale=0.8 ** r, size=(K, 32)) for r in range(R)]).astype(np.float32)
+    if K > 40:
+        cb[0, 40] = cb[0, 3]                                # duplicates: the lower index wins
+    return x, cb
+
+
+def check(n, dim, K, R, layout, bits, dtype, seed, stride=None):
+    x, cb = batch(n, dim, K, R, dtype, seed)
+    cfg = rvq.make_config(dim, 32, layout, R, K, (K - 1).bit_length() if bits == "packed" else 16, DT[dtype], seed % 2)
+    stride = stride or dim
+    xd = torch.zeros(n, stride, dtype=x.dtype, device="cuda")
+    xd[:, :dim] = x.cuda()
+    b, e = rvq.alloc_buffers(cfg, n, cb), rvq.alloc_buffers(cfg, n, cb)
+    energy, energy_e = torch.full((R,), 7.0, device="cuda"), torch.empty(R, device="cuda")
+    for out in (None, energy):                              # with and without the stage energies
+        b.codes.fill_(0xAA)
+        rvq.rvq_encode(cfg, xd, n, stride, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes,
+                       b.status, stage_energy=out)
+        rvq.rvq_encode_exact(cfg, xd, n, stride, e.codebooks, e.prepared, e.codes, e.std, e.status, stage_energy=energy_e)
+        torch.cuda.synchronize()
+        assert torch.equal(b.codes, e.codes) and torch.equal(b.std, e.std)
+    if not (n % 2 == 1 and n > 3):                          # (the float32 kernel counts degenerate rows' codewords)
+        assert torch.allclose(energy, energy_e, rtol=1e-4)
+    st, ste = rvq.read_status(b.status), rvq.read_status(e.status)
+    assert st["wait_timeouts"] == 0 and st["degenerate_vectors"] == ste["degenerate_vectors"]
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 7, 8, 9, 17, 31, 32, 33, 63, 64, 65, 127, 129, 257, 600, 1111, 2049])
+@pytest.mark.parametrize("K,R,layout,bits,dtype", [(2048, 8, 1, "packed", "bf16"), (1024, 8, 0, 16, "f32"),
+                                                   (1000, 5, 1, "packed", "f16"), (256, 8, 0, 16, "f32"), (77, 3, 0, "packed", "bf16")])
+def test_few_vectors(n, K, R, layout, bits, dtype):
+    check(n, 128, K, R, layout, bits, dtype, n + K)
+
+
+@pytest.mark.parametrize("n,dim,K", [(5, 256, 2048), (70, 256, 1024), (301, 64, 512), (9, 32, 2048), (40, 96, 300), (3, 512, 129),
+                                     (13000, 128, 512), (150, 128, 5000), (4, 1024, 2049)])
+def test_other_head_sizes_and_row_strides(n, dim, K):
+    check(n, dim, K, 8 if K != 129 else 9, 1, "packed", "bf16", n, stride=dim + 16)
+
+
+def test_against_the_oracle():
+    x, cb = batch(24, 128, 1024, 8, "f32", 5)
+    cfg = rvq.make_config(128, 32, 0, 8, 1024, 16, rvq.F32, 0)
+    b = rvq.alloc_buffers(cfg, 24, cb)
+    rvq.rvq_encode(cfg, x.cuda(), 24, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    codes = b.codes.view(torch.int16).cpu().numpy().view(np.uint16).reshape(24, 4, 8).astype(np.int32)
+    assert_codes_match(x.numpy(), codes, cb, 0)
