@@ -18,14 +18,29 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::atomic<int> g_sms[kMaxDevices];
 
-// Largest dynamic shared memory granted to a kernel so far, per device: open addressing by the
-// kernel's address; entries are only ever added.  Threads may race to grant the same amount twice.
+// What has been asked of the runtime about a kernel so far, per device: the largest dynamic shared memory
+// granted to it, and how many clusters of 1 .. 8 CTAs run at a time (0: not asked, -1: none).  Open addressing
+// by the kernel's address; entries are only ever added.  Threads may race to ask the same thing twice.
 struct Grant {
     std::atomic<const void *> kernel{nullptr};
     std::atomic<int> bytes{0};
+    std::atomic<int> clusters[9] = {};
 };
 constexpr int kGrantSlots = 512;                          // (a few times the library's number of kernels)
 Grant g_grants[8][kGrantSlots];
+
+Grant *grant_of(const void *kernel, int dev)
+{
+    if (dev >= 8) return nullptr;
+    const uint32_t h = (uint32_t)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) >> 7;
+    for (uint32_t k = 0; k < (uint32_t)kGrantSlots; ++k) {
+        Grant &g = g_grants[dev][(h + k) % kGrantSlots];
+        const void *have = g.kernel.load(std::memory_order_acquire);
+        if (have == nullptr && g.kernel.compare_exchange_strong(have, kernel)) have = kernel;
+        if (have == kernel) return &g;
+    }
+    return nullptr;
+}
 
 }  // namespace
 
@@ -44,21 +59,55 @@ bool allow_shared_memory(const void *kernel, int bytes)
 {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
-    auto grant = [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
-    if (dev >= 8) return grant();
-    const uint32_t h = (uint32_t)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) >> 7;
-    for (uint32_t k = 0; k < (uint32_t)kGrantSlots; ++k) {
-        Grant &g = g_grants[dev][(h + k) % kGrantSlots];
-        const void *have = g.kernel.load(std::memory_order_acquire);
-        if (have == nullptr && g.kernel.compare_exchange_strong(have, kernel)) have = kernel;
-        if (have != kernel) continue;
-        if (g.bytes.load(std::memory_order_acquire) >= bytes) return true;
-        if (!grant()) return false;
-        int old = g.bytes.load(std::memory_order_relaxed);
-        while (old < bytes && !g.bytes.compare_exchange_weak(old, bytes, std::memory_order_release)) {}
-        return true;
+    Grant *g = grant_of(kernel, dev);
+    if (g && g->bytes.load(std::memory_order_acquire) >= bytes) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    if (g) {
+        int old = g->bytes.load(std::memory_order_relaxed);
+        while (old < bytes && !g->bytes.compare_exchange_weak(old, bytes, std::memory_order_release)) {}
     }
-    return grant();
+    return true;
+}
+
+static cudaLaunchConfig_t cluster_config(int clusters, int ctas, int threads, int smem, cudaStream_t stream, cudaLaunchAttribute *attr)
+{
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = 1; attr->val.clusterDim.y = (unsigned)ctas; attr->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)clusters, (unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = stream;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cfg;
+}
+
+int resident_clusters(const void *kernel, int ctas, int threads, int smem)
+{
+    int dev = -1;
+    if (ctas < 1 || ctas > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    Grant *g = grant_of(kernel, dev);
+    int have = g ? g->clusters[ctas].load(std::memory_order_acquire) : 0;
+    if (have == 0) {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = cluster_config(1, ctas, threads, smem, nullptr, &attr);
+        if (!allow_shared_memory(kernel, smem) || cudaOccupancyMaxActiveClusters(&have, kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            have = 0;
+        }
+        if (have <= 0) have = -1;
+        if (g) g->clusters[ctas].store(have, std::memory_order_release);
+    }
+    return have < 0 ? 0 : have;
+}
+
+int launch_clusters(const void *kernel, int clusters, int ctas, int threads, int smem, cudaStream_t stream, void **args)
+{
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = cluster_config(clusters, ctas, threads, smem, stream, &attr);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
+    const int rc = check_launch();
+    return e == cudaSuccess ? rc : RVQ_ERR_LAUNCH;
 }
 
 static int ceil_log2(int k)
@@ -168,6 +217,8 @@ static int encode_common(const rvq_config *cfg, const void *x, int64_t n, int64_
         return RVQ_ERR_LAUNCH;
     if (allow_tensor && !stat_sum && encode_small_wanted(s, n))
         return launch_encode_small(s, x, n, x_row_stride, prepared, codes, std_f16, status, (cudaStream_t)stream, stage_energy);
+    if (allow_tensor && !stat_sum && encode_split_wanted(s, n))
+        return launch_encode_split(s, x, n, x_row_stride, codebooks, prepared, codes, std_f16, status, (cudaStream_t)stream, stage_energy);
     if (allow_tensor && encode_tensor_supported(s))
         return launch_encode_tensor(s, x, n, x_row_stride, codebooks, prepared, codes, std_f16, status,
                                     (cudaStream_t)stream, stat_cnt, stat_sum, stage_energy);

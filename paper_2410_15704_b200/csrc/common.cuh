@@ -34,6 +34,10 @@ int launch_encode_scalar(const Shape &s, const void *x, int64_t n, int64_t strid
 bool encode_small_wanted(const Shape &s, int64_t n);
 int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride, const void *prepared, void *codes,
                         uint16_t *std16, rvq_status *st, cudaStream_t stream, float *energy);
+// few row tiles: each tile's sweep split over accumulators and CTAs
+bool encode_split_wanted(const Shape &s, int64_t n);
+int launch_encode_split(const Shape &s, const void *x, int64_t n, int64_t stride, const float *cb, const void *prepared,
+                        void *codes, uint16_t *std16, rvq_status *st, cudaStream_t stream, float *energy);
 bool encode_tensor_supported(const Shape &s);
 int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t stride, const float *cb,
                          const void *prepared, void *codes, uint16_t *std16, rvq_status *st,
@@ -79,6 +83,11 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
 // remembered: the three runtime queries they replace were a third of the host's time in a call.
 int sm_count();                                            // 0: no device
 bool allow_shared_memory(const void *kernel, int bytes);   // dynamic shared memory of up to `bytes` for this kernel
+
+// Clusters of `ctas` CTAs of this kernel that the current device runs at a time (0: none), and their launch:
+// `clusters` of them along x, the CTAs of a cluster along y.
+int resident_clusters(const void *kernel, int ctas, int threads, int smem);
+int launch_clusters(const void *kernel, int clusters, int ctas, int threads, int smem, cudaStream_t stream, void **args);
 
 void count_launch();
 inline int check_launch()

@@ -11,6 +11,19 @@ constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
 constexpr int kOnesBytes = 2 * 128 * 16;                  // the constant A cells (1 1 1 0 ...) and (0 ...)
 constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 -> f32, M = N = 128
 
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The address, in CTA `rank` of the cluster, of what is at `addr` in this one.
+__device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+    return a;
+}
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
@@ -121,6 +134,11 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32
 }
 // Waits for every tcgen05.ld of this thread; the arrays pass through so that no
 // use of them can be scheduled ahead of the wait.
+__device__ __forceinline__ void tmem_ld_wait2(uint32_t (&u)[32], uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
+    asm volatile("" : RVQ_INOUT32(v) : : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait4(uint32_t (&u)[32], uint32_t (&v)[32], uint32_t (&w)[32], uint32_t (&x)[32])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
@@ -195,6 +213,8 @@ struct Listed {
     {
         return ((places & (places - 1u)) | (halves & (halves - 1u)) | (blocks & (blocks - 1u))) == 0u;
     }
+    // the three in one word: places, halves << 16, blocks << 18
+    __device__ __forceinline__ uint32_t word() const { return places | (halves << 16) | (blocks << 18); }
     // column inside the chunk of the lowest members
     __device__ __forceinline__ int column() const { return (__ffs(blocks) - 1) * 32 + (__ffs(halves) - 1) * 16 + __ffs(places) - 1; }
 };
@@ -243,6 +263,52 @@ __device__ __forceinline__ float exact_distance(const float (&z)[32], const floa
         for (int k = 0; k < 8; ++k) { const float t = z[8 * q + k] - ev[k]; acc = fmaf(t, t, acc); }
     }
     return acc;
+}
+
+// Position of set bit number `k` of `bits` (which has that many).
+__device__ __forceinline__ int bit_at(uint32_t bits, int k)
+{
+    for (; k > 0; --k) bits &= bits - 1u;
+    return __ffs(bits) - 1;
+}
+
+// Exact comparison of the columns listed by `sets` (Listed::word) in chunk1 and, unless negative, chunk2, by a
+// whole warp for one row z: lane l takes the l-th column, so that their codewords arrive together (one after
+// the other they cost a trip to L2 each: 4400 cycles a row, measured).  The lane's best joins (bv, bi).
+__device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
+                                               uint32_t sets, int chunk1, int chunk2, float &bv, int &bi)
+{
+    const uint32_t places = sets & 0xFFFFu, blocks = (sets >> 18) & 15u;
+    const uint32_t columns = ((sets >> 16) & 1u ? places : 0u) | ((sets >> 17) & 1u ? places << 16 : 0u);
+    const int nc = __popc(columns), nb = __popc(blocks), total = nc * nb * (chunk2 >= 0 ? 2 : 1);
+    for (int l = lane; l < total; l += 32) {
+        const int b = l / nc, second = b >= nb ? 1 : 0;
+        const int j = (second ? chunk2 : chunk1) * 128 + bit_at(blocks, b - second * nb) * 32 + bit_at(columns, l - b * nc);
+        if (j < K) {
+            const float d = exact_distance(z, cbr + (size_t)j * 32);
+            if (d < bv || (d == bv && j < bi)) { bv = d; bi = j; }
+        }
+    }
+}
+
+// Exact comparison of all columns.
+__device__ __forceinline__ void compare_all(const float (&z)[32], const float *__restrict__ cbr, int K, int lane, float &bv, int &bi)
+{
+    for (int j = lane; j < K; j += 32) {
+        const float d = exact_distance(z, cbr + (size_t)j * 32);
+        if (d < bv) { bv = d; bi = j; }
+    }
+}
+
+// The warp's best: smallest distance, lowest index on ties.
+__device__ __forceinline__ void best_of_warp(float &bv, int &bi)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float ov = __shfl_xor_sync(0xFFFFFFFFu, bv, off);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
+        if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+    }
 }
 
 // The seven K = 16 steps of one chain: 128 rows (A: TMEM columns a0 ..: 16 of head, 16 of remainder)

@@ -13,8 +13,6 @@
 // stage's table 300.
 #include "encode_mma.cuh"
 
-#include <atomic>
-
 namespace rvq {
 
 namespace {
@@ -38,19 +36,6 @@ struct SmallParams {
     int rows;           // their group rows
     int blocks_per_stage;
 };
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_to(uint32_t addr, uint32_t rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-    return a;
-}
 
 struct SmallWork {
     // (distance bits, code) of the best of every warp's 32 codewords, from every CTA of the cluster
@@ -260,41 +245,13 @@ struct SmallPlan {
     int per_cta, ctas, at_once;
 };
 
-cudaLaunchConfig_t small_config(const SmallPlan &plan, int64_t clusters, int threads, cudaStream_t stream, cudaLaunchAttribute *attr)
-{
-    attr->id = cudaLaunchAttributeClusterDimension;
-    attr->val.clusterDim.x = 1; attr->val.clusterDim.y = (unsigned)plan.ctas; attr->val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)clusters, (unsigned)plan.ctas);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = kSmallSharedBytes;
-    cfg.stream = stream;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cfg;
-}
-
 // How a shape is split, and how many clusters of that split the current device runs at a time (0: none).
 SmallPlan small_plan(const Shape &s)
 {
-    static std::atomic<int> known[8][2][kSmallMaxCluster + 1];    // per device, split and cluster size; -1: none
     const int blocks = slots_per_stage(s.K), per = blocks <= kSmallMaxCluster ? 1 : 2;
     SmallPlan plan{per == 1 ? reinterpret_cast<const void *>(encode_small_kernel<1>) : reinterpret_cast<const void *>(encode_small_kernel<2>),
                    per, (blocks + per - 1) / per, 0};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return plan;
-    std::atomic<int> *slot = dev < 8 ? &known[dev][per - 1][plan.ctas] : nullptr;
-    int have = slot ? slot->load(std::memory_order_acquire) : 0;
-    if (have == 0) {
-        cudaLaunchAttribute attr;
-        const cudaLaunchConfig_t cfg = small_config(plan, 1, kSmallThreads, nullptr, &attr);
-        if (!allow_shared_memory(plan.kernel, kSmallSharedBytes) || cudaOccupancyMaxActiveClusters(&have, plan.kernel, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            have = 0;
-        }
-        if (have <= 0) have = -1;
-        if (slot) slot->store(have, std::memory_order_release);
-    }
-    plan.at_once = have < 0 ? 0 : have;
+    plan.at_once = resident_clusters(plan.kernel, plan.ctas, kSmallThreads, kSmallSharedBytes);
     return plan;
 }
 
@@ -323,12 +280,8 @@ int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride
                   vectors, vectors * s.G, slots_per_stage(s.K)};
     int threads = plan.per_cta * 128 * ((p.rows + kSmallAtOnce - 1) / kSmallAtOnce);
     if (threads > kSmallThreads) threads = kSmallThreads;
-    cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = small_config(plan, (n + vectors - 1) / vectors, threads, stream, &attr);
     void *args[] = {&p};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, plan.kernel, args);
-    const int rc = check_launch();
-    return e == cudaSuccess ? rc : RVQ_ERR_LAUNCH;
+    return launch_clusters(plan.kernel, (int)((n + vectors - 1) / vectors), plan.ctas, threads, kSmallSharedBytes, stream, args);
 }
 
 }  // namespace rvq

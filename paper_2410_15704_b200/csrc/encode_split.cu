@@ -1,0 +1,440 @@
+// Tensor-core encode of few row tiles (up to two per SM): one tile's codebook sweep split.
+//
+// The throughput kernel (encode_tensor.cu) gives an SM three tiles of 128 rows and lets them share the
+// operand stream; with fewer tiles than three per SM most of the chip is idle and the tiles that run
+// wait, chunk after chunk, for one accumulator each (154 tiles: 145 us at 2048 codes, as long as one).
+// Here a tile belongs to a cluster of C CTAs (1, 2, 4 or 8: as many as keep every SM busy), each of
+// which sweeps its share of the stage's chunks with up to three accumulators in flight over one A operand.
+// An epilogue group of four warps per accumulator folds its chunks into running minima of the tile's
+// 128 rows (encode_mma.cuh), as the throughput kernel does for all chunks.  At the stage end every
+// group sends, per row, its two best chunks and the sets of columns inside the error window to every CTA
+// of the cluster (st.async, counted by an mbarrier); the owner group of each CTA merges the parts of its
+// rows -- one part with one column inside the window: the choice is certified; otherwise the listed
+// columns are compared exactly in float32 -- and takes the residual to the next stage.  All CTAs of a
+// cluster make the same choice from the same parts.
+// What bounds it: the chain of the stages (MMA chain 470 cycles and its latency, fold 300-900, exchange
+// 300-500, choice, codeword and operand 2000).
+#include "encode_mma.cuh"
+
+namespace rvq {
+
+namespace {
+
+constexpr int kGroups = 3;                                // accumulators, and epilogue groups of 128 threads
+constexpr int kSplitThreads = 448;                        // 12 epilogue warps, issuer, loader
+constexpr int kSplitRing = 7;
+constexpr int kMaxParts = 16;                             // groups of a cluster that have chunks
+constexpr int kATmem = kGroups * 128;                     // TMEM column of the A operand (32 columns)
+
+struct Part {                                             // what a group knows of a row at the stage end
+    float m1, m2;                                         // its two lowest chunk minima
+    uint32_t sets;                                        // columns inside its window: places, halves << 16, blocks << 18; bit 22: a third chunk
+    uint32_t chunks;                                      // chunk of m1, chunk of m2 << 16
+};
+
+constexpr int kSOffB = 0;
+constexpr int kSOffOnes = kSOffB + kSplitRing * kSlotBytes;
+constexpr int kSOffZ = kSOffOnes + kOnesBytes;            // residuals, float [32][kZPitch]
+constexpr int kZPitch = 129;                              // (odd: neither rows nor elements of a row share banks)
+constexpr int kSOffParts = kSOffZ + 32 * kZPitch * 4;     // Part [2][kMaxParts][128]
+constexpr int kSOffCodes = kSOffParts + 2 * kMaxParts * 128 * 16;
+constexpr int kSOffNorm = kSOffCodes + 128 * 16 * 2;      // squared norms of the scaled residuals
+constexpr int kSOffBars = kSOffNorm + 128 * 4;
+constexpr int kSplitSmem = kSOffBars + 256;
+
+constexpr int kSFull = 0, kSEmpty = kSplitRing, kSReady = 2 * kSplitRing, kSAccFull = kSReady + 1, kSAccFree = kSAccFull + kGroups,
+              kSArrived = kSAccFree + kGroups, kSBars = kSArrived + 2;
+
+struct SplitParams {
+    Shape s;
+    const void *x;
+    int64_t n, stride;
+    const float *cb;
+    const uint8_t *prepared;
+    void *codes;
+    uint16_t *std16;
+    rvq_status *st;
+    float *energy;
+    int tiles;
+    int groups;         // accumulators in use: min(kGroups, chunks of a CTA)
+};
+
+__global__ void __launch_bounds__(kSplitThreads, 1)
+encode_split_kernel(const SplitParams p)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kSOffBars);
+    uint32_t *tmem_word = reinterpret_cast<uint32_t *>(smem + kSOffBars + kSBars * 8);
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + kSOffBars + kSBars * 8 + 4);
+    const Shape &s = p.s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int S = slots_per_stage(s.K), R = s.R, P = p.groups;
+    const int rank = (int)cluster_rank(), ctas = (int)gridDim.y;
+    // this CTA's chunks of every stage
+    const int per = S / ctas, rem = S - per * ctas;
+    const int base = rank * per + min(rank, rem), cnt = per + (rank < rem ? 1 : 0);
+    const int my_tiles = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const uint32_t bar0 = smem_u32(bars);
+    auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+
+    if (tid == 0) {
+        for (int i = 0; i < kSplitRing; ++i) { mbar_init(BAR(kSFull + i), 1); mbar_init(BAR(kSEmpty + i), 1); }
+        mbar_init(BAR(kSReady), 4);
+        for (int g = 0; g < kGroups; ++g) { mbar_init(BAR(kSAccFull + g), 1); mbar_init(BAR(kSAccFree + g), 4); }
+        mbar_init(BAR(kSArrived), 1);
+        mbar_init(BAR(kSArrived + 1), 1);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 12) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_word)), "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid < 128) {
+        uint8_t *a = smem + kSOffOnes + tid * 16;
+        *reinterpret_cast<uint4 *>(a) = make_uint4(0x3C003C00u, 0x00003C00u, 0u, 0u);
+        *reinterpret_cast<uint4 *>(a + 2048) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (ctas > 1) asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    const uint32_t tmem = *tmem_word;
+
+    if (warp == 13) {
+        // ------------------------------------------------------------ operand loader
+        if (lane == 0) {
+            const uint8_t *image = p.prepared + kPreparedImageOffset + (size_t)base * kSlotBytes;
+            uint32_t slot = 0, par = 1, issued = 0;
+            bool ok = true;
+            for (int t = 0; t < my_tiles && ok; ++t)
+                for (int r = 0; r < R && ok; ++r)
+                    for (int c = 0; c < cnt && ok; ++c) {
+                        if (issued >= (uint32_t)kSplitRing) ok = mbar_wait(BAR(kSEmpty + slot), par, abort_flag);
+                        if (!ok) break;
+                        mbar_expect_tx(BAR(kSFull + slot), kSlotBytes);
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                     ::"r"(smem_u32(smem + kSOffB) + slot * (uint32_t)kSlotBytes), "l"(image + ((size_t)r * S + c) * kSlotBytes),
+                                       "r"((uint32_t)kSlotBytes), "r"(BAR(kSFull + slot)) : "memory");
+                        ++issued;
+                        if (++slot == (uint32_t)kSplitRing) { slot = 0; par ^= 1u; }
+                    }
+            // (giving up: the copies in flight have to land before the CTA ends)
+            if (!ok)
+                for (uint32_t k = issued > (uint32_t)kSplitRing ? issued - kSplitRing : 0u; k < issued; ++k) {
+                    volatile uint32_t never = 0u;
+                    mbar_wait(BAR(kSFull + (int)(k % kSplitRing)), (k / kSplitRing) & 1u, &never, 100000u);
+                }
+        }
+    } else if (warp == 12) {
+        // ------------------------------------------------------------ MMA issuer
+        const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kSOffB), kSlotCodewords * 16, 128);
+        const uint64_t ones_desc = make_smem_desc(smem_u32(smem + kSOffOnes), 2048, 128);
+        uint32_t slot = 0, full_par = 0, ready_par = 0;
+        uint32_t used = 0;                                                // accumulators used at least once (bit per accumulator)
+        uint32_t free_pars = 0;                                           // next parity to wait for, bit per accumulator
+        bool ok = true;
+        const int stages = my_tiles * R;
+        for (int st = 0; st < stages && ok; ++st) {
+            ok = mbar_wait(BAR(kSReady), ready_par, abort_flag);
+            ready_par ^= 1u;
+            int a = 0;
+            for (int c = 0; c < cnt && ok; ++c) {
+                ok = mbar_wait(BAR(kSFull + slot), full_par, abort_flag);
+                if (ok && ((used >> a) & 1u)) {
+                    ok = mbar_wait(BAR(kSAccFree + a), (free_pars >> a) & 1u, abort_flag);
+                    free_pars ^= 1u << a;
+                }
+                used |= 1u << a;
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    issue_chain(tmem + 128u * (uint32_t)a, tmem + kATmem, bdesc0 + (uint64_t)(slot * (uint32_t)(kSlotBytes >> 4)), ones_desc);
+                    mma_commit(BAR(kSAccFull + a));
+                    mma_commit(BAR(kSEmpty + slot));
+                }
+                __syncwarp();
+                if (++slot == (uint32_t)kSplitRing) { slot = 0; full_par ^= 1u; }
+                if (++a == P) a = 0;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue groups
+        const int grp = warp >> 2, q4 = warp & 3;
+        const int row = q4 * 32 + lane;
+        const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
+        float *z_park = reinterpret_cast<float *>(smem + kSOffZ) + row;                 // [i][row]
+        float *norm = reinterpret_cast<float *>(smem + kSOffNorm);
+        uint16_t *codes_s = reinterpret_cast<uint16_t *>(smem + kSOffCodes);            // [row][16]
+        const Part *parts = reinterpret_cast<const Part *>(smem + kSOffParts);          // [2][kMaxParts][128]
+        const StageParams *sp = reinterpret_cast<const StageParams *>(p.prepared + kPreparedParamsOffset);
+        const int nparts = ctas * P;
+        const uint32_t mine = smem_u32(smem + kSOffParts) + (uint32_t)((rank * P + grp) * 128 + row) * 16u;
+        const int G = s.G;
+        uint32_t acc_par = 0, stage_no = 0;
+        uint32_t n_rescored = 0, n_exhaustive = 0, n_degenerate = 0, n_stdrange = 0;
+        bool ok = true;
+        const int todo_tiles = grp < P ? my_tiles : 0;                                    // (groups without an accumulator sit by)
+        // (every warp of the groups meets both barriers of every tile, given up or not)
+        for (int t = 0; t < todo_tiles; ++t) {
+            const int64_t row0 = ((int64_t)blockIdx.x + (int64_t)t * gridDim.x) * 128;
+            const int64_t v_tile = row0 / G, v_first = v_tile + q4 * 32 / G;
+            const int64_t v = v_first + lane / G;
+            const bool valid = v < p.n;
+            bool deg = true;
+            // the tile's head vectors, widened, by all groups: element i of row at [i][row]
+            if (t > 0) asm volatile("bar.sync 1, %0;" ::"r"(128 * P) : "memory");     // (the owners are through with the last tile's)
+            if (ok) {
+                const int eb = s.elem_bytes, ppv = s.dim * eb / 16, per_piece = 16 / eb, lg = __ffs(G) - 1;
+                float *zs = reinterpret_cast<float *>(smem + kSOffZ);
+                for (int k = tid; k < (128 >> lg) * ppv; k += 128 * P) {
+                    const int vl = k / ppv, off = k - vl * ppv;
+                    uint4 raw = make_uint4(0u, 0u, 0u, 0u);
+                    if (v_tile + vl < p.n)
+                        raw = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(p.x) + (v_tile + vl) * p.stride * eb) + off);
+                    const uint32_t words[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        if (u >= per_piece) break;
+                        const uint32_t word = eb == 4 ? words[u & 3] : words[u >> 1];
+                        const uint16_t h = (u & 1) ? (uint16_t)(word >> 16) : (uint16_t)(word & 0xFFFFu);
+                        const float val = eb == 4 ? __uint_as_float(word)
+                                        : s.dtype == RVQ_BF16 ? __uint_as_float((uint32_t)h << 16) : __half2float(__ushort_as_half(h));
+                        const int ch = off * per_piece + u;
+                        const int g = s.layout == RVQ_GROUP_STRIDED ? ch & (G - 1) : ch >> 5, i = s.layout == RVQ_GROUP_STRIDED ? ch >> lg : ch & 31;
+                        zs[i * kZPitch + (vl << lg) + g] = val;
+                    }
+                }
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(128 * P) : "memory");
+            if (ok && grp == 0) {
+                // (the residual lives in shared memory between its uses: in registers it would be live across the sweep)
+                float z[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kZPitch];
+                const float dev = group_deviation(s, z, lane);
+                deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) z_park[i * kZPitch] = deg ? 0.0f : (s.raw ? z[i] : z[i] / dev);
+                if (valid && (lane & (G - 1)) == 0 && !s.raw && rank == 0) {
+                    const uint16_t hb = deviation_is_degenerate(dev) ? (uint16_t)0 : __half_as_ushort(__float2half_rn(dev));
+                    p.std16[v] = hb;
+                    if (deviation_is_degenerate(dev)) ++n_degenerate;
+                    else if ((hb & 0x7FFFu) == 0 || (hb & 0x7FFFu) >= 0x7C00u) ++n_stdrange;
+                }
+            }
+#pragma unroll 1
+            for (int r = 0; r < R && ok; ++r, ++stage_no) {
+                const StageParams prm = sp[r];
+                const float *cbr = p.cb + (size_t)r * s.K * 32;
+                const uint32_t par = stage_no & 1u;
+                Sweep w;
+                w.m1 = w.m2 = w.m3 = INFINITY;
+                w.c1 = w.c2 = 0;
+#pragma unroll
+                for (int q = 0; q < 16; ++q) w.d[q] = INFINITY;
+                w.h[0] = w.h[1] = INFINITY;
+                w.bb[0] = w.bb[1] = w.bb[2] = w.bb[3] = INFINITY;
+                w.zz = 0.0f;
+                if (grp == 0) {
+                    float z[32];
+                    uint32_t ab[32];
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) z[i] = z_park[i * kZPitch];
+                    w.zz = split_operand(z, prm.scale, ab);
+                    norm[row] = w.zz;
+                    tmem_st32(tmem + lanes + kATmem, ab);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(BAR(kSReady));
+                    if (warp == 0 && lane == 0) mbar_expect_tx(BAR(kSArrived + par), (uint32_t)nparts * 128u * 16u);
+                }
+#pragma unroll 1
+                for (int c = grp; c < cnt && ok; c += P) {
+                    ok = mbar_wait(BAR(kSAccFull + grp), acc_par, abort_flag);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    acc_par ^= 1u;
+                    if (!ok) break;
+                    tc_fence_after();
+                    uint32_t ua[32], ub[32];
+                    const uint32_t acc = tmem + lanes + 128u * (uint32_t)grp;
+                    tmem_ld32_issue(acc, ua);
+                    tmem_ld32_issue(acc + 32, ub);
+                    tmem_ld_wait2(ua, ub);
+                    const float c0 = fold_block(w, ua, 0);
+                    const float c1 = fold_block(w, ub, 1);
+                    tmem_ld32_issue(acc + 64, ua);
+                    tmem_ld32_issue(acc + 96, ub);
+                    tmem_ld_wait2(ua, ub);
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(BAR(kSAccFree + grp));
+                    const float c2 = fold_block(w, ua, 2);
+                    const float c3 = fold_block(w, ub, 3);
+                    rank_chunk(w, fminf(min3(c0, c1, c2), c3), base + c);
+                }
+                if (!ok) break;
+                // this group's part of the row, to every CTA of the cluster
+                if (grp != 0 && grp < cnt) w.zz = norm[row];              // (a group without chunks has nothing inside any window)
+                w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
+                {
+                    const float lim = threshold(w, w.m1);
+                    const Listed in = listed(w, lim);
+                    const uint32_t sets = in.word() | (w.m3 <= lim ? 1u << 22 : 0u);
+                    for (int to = 0; to < ctas; ++to)
+                        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                                     ::"r"(map_to(mine + par * (uint32_t)(kMaxParts * 128 * 16), (uint32_t)to)), "r"(__float_as_uint(w.m1)),
+                                       "r"(__float_as_uint(w.m2)), "r"(sets), "r"((uint32_t)w.c1 | ((uint32_t)w.c2 << 16)),
+                                       "r"(map_to(BAR(kSArrived + par), (uint32_t)to)) : "memory");
+                }
+                ok = mbar_wait(BAR(kSArrived + par), (stage_no >> 1) & 1u, abort_flag);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok || grp != 0) continue;
+
+                // ---- the owners: merge the parts
+                const Part *mp = parts + par * (kMaxParts * 128) + row;
+                float m1 = INFINITY, next = INFINITY;                     // the two lowest minima of the parts
+                int k1 = 0;
+#pragma unroll 4
+                for (int k = 0; k < nparts; ++k) {
+                    const float m = mp[k * 128].m1;
+                    next = fminf(next, fmaxf(m1, m));
+                    k1 = m < m1 ? k : k1;
+                    m1 = fminf(m1, m);
+                }
+                const float lim = threshold(w, m1);
+                const Part best = mp[k1 * 128];
+                const Listed in{best.sets & 0xFFFFu, (best.sets >> 16) & 3u, (best.sets >> 18) & 15u};
+                const int j1 = (int)(best.chunks & 0xFFFFu) * 128 + in.column();
+                // (a padded column scores 60000: if nothing real scored less, scan everything)
+                const bool scan_all = !(w.zz < 3.6e9f) || !(w.win < INFINITY) || !(m1 < 59000.0f);
+                const bool unique = next > lim && best.m2 > lim && in.single() && (uint32_t)j1 < (uint32_t)s.K;
+                int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
+                uint32_t todo = __ballot_sync(0xFFFFFFFFu, !deg && (scan_all || !unique));
+                while (todo) {
+                    // rows with more than one candidate: the warp compares the listed columns of one row at a
+                    // time exactly (lane = column of a block), lowest index on ties
+                    const int src = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    float zs[32];
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kZPitch + (src - lane)];
+                    const float lim_s = __shfl_sync(0xFFFFFFFFu, lim, src);
+                    bool all_s = __shfl_sync(0xFFFFFFFFu, (int)scan_all, src) != 0;
+                    // lane k looks at part k of that row
+                    Part q{INFINITY, INFINITY, 0u, 0u};
+                    if (lane < nparts) q = mp[lane * 128 + (src - lane)];
+                    uint32_t inside = __ballot_sync(0xFFFFFFFFu, lane < nparts && q.m1 <= lim_s);
+                    all_s = all_s || __any_sync(0xFFFFFFFFu, ((inside >> lane) & 1u) && ((q.sets >> 22) & 1u));    // a third chunk somewhere
+                    float bv = INFINITY;
+                    int bi = 0x7FFFFFFF;
+                    if (all_s) {
+                        compare_all(zs, cbr, s.K, lane, bv, bi);
+                    } else {
+                        const int second = q.m2 <= lim_s ? (int)(q.chunks >> 16) : -1;
+                        for (; inside; inside &= inside - 1u) {
+                            const int k = __ffs(inside) - 1;
+                            compare_listed(zs, cbr, s.K, lane, __shfl_sync(0xFFFFFFFFu, q.sets, k),
+                                           (int)(__shfl_sync(0xFFFFFFFFu, q.chunks, k) & 0xFFFFu), __shfl_sync(0xFFFFFFFFu, second, k), bv, bi);
+                        }
+                    }
+                    best_of_warp(bv, bi);
+                    if (lane == src) {
+                        bj = bi < s.K ? bi : 0;
+                        if (rank == 0) { if (all_s) ++n_exhaustive; else ++n_rescored; }
+                    }
+                }
+                if (deg) bj = 0;
+                float e2 = 0.0f;
+                __syncwarp();                                             // (the comparison above reads other lanes' rows)
+                if (!deg) {
+                    const float *ew = cbr + (size_t)bj * 32;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float ev[8];
+                        ldg256(ew + 8 * q, ev);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float nz = z_park[(8 * q + k) * kZPitch] - ev[k];
+                            z_park[(8 * q + k) * kZPitch] = nz;
+                            e2 = fmaf(nz, nz, e2);
+                        }
+                    }
+                }
+                if (p.energy && rank == 0) {
+                    if (!valid) e2 = 0.0f;
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xFFFFFFFFu, e2, off);
+                    if (lane == 0) atomicAdd(p.energy + r, e2);
+                }
+                codes_s[row * 16 + r] = (uint16_t)bj;
+            }
+            if (ok && grp == 0) {
+                __syncwarp();
+                if (rank == 0) emit_codes(s, codes_s + q4 * 32 * 16, v_first, p.n, lane, p.codes);
+                __syncwarp();
+            }
+        }
+        if (p.st) {
+            if (n_rescored) atomicAdd(&p.st->rescored_rows, n_rescored);
+            if (n_exhaustive) atomicAdd(&p.st->exhaustive_rows, n_exhaustive);
+            if (n_degenerate) atomicAdd(&p.st->degenerate_vectors, n_degenerate);
+            if (n_stdrange) atomicAdd(&p.st->std_out_of_half, n_stdrange);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    // (no CTA ends while another may still send to it)
+    if (ctas > 1) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    if (warp == 12) {
+        tc_fence_after();
+        if (lane == 0 && *abort_flag && p.st) atomicAdd(&p.st->wait_timeouts, 1u);
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+}
+
+// Tiles per SM up to which one CTA per tile, its sweep split over three accumulators, is the faster way.
+#ifndef RVQ_SPLIT_TILES
+#define RVQ_SPLIT_TILES 2
+#endif
+constexpr int kSplitTilesPerSm = RVQ_SPLIT_TILES;
+
+// CTAs per tile: the most that leave every tile of the call on the chip at once (0: more tiles than that).
+int split_ctas(const Shape &s, int64_t tiles, int sms)
+{
+    const int S = slots_per_stage(s.K);
+    for (int c = 8; c >= 2; c /= 2) {
+        const int groups = (S + c - 1) / c < kGroups ? (S + c - 1) / c : kGroups;
+        if (c > S || c * groups > kMaxParts || tiles * c > sms) continue;
+        if (tiles <= resident_clusters(reinterpret_cast<const void *>(encode_split_kernel), c, kSplitThreads, kSplitSmem)) return c;
+    }
+    return tiles <= kSplitTilesPerSm * (int64_t)sms ? 1 : 0;
+}
+
+}  // namespace
+
+bool encode_split_wanted(const Shape &s, int64_t n)
+{
+    if (!encode_tensor_supported(s) || n < 1 || n > (1 << 24)) return false;
+    const int sms = sm_count();
+    return sms > 0 && split_ctas(s, (n * s.G + 127) / 128, sms) > 0;
+}
+
+int launch_encode_split(const Shape &s, const void *x, int64_t n, int64_t stride, const float *cb, const void *prepared,
+                        void *codes, uint16_t *std16, rvq_status *st, cudaStream_t stream, float *energy)
+{
+    const int sms = sm_count();
+    const int tiles = (int)((n * s.G + 127) / 128), ctas = split_ctas(s, tiles, sms);
+    const void *kernel = reinterpret_cast<const void *>(encode_split_kernel);
+    if (ctas <= 0 || !allow_shared_memory(kernel, kSplitSmem)) return RVQ_ERR_LAUNCH;
+    const int per = (slots_per_stage(s.K) + ctas - 1) / ctas;
+    SplitParams p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, energy, tiles,
+                  per < kGroups ? per : kGroups};
+    void *args[] = {&p};
+    return launch_clusters(kernel, tiles < sms ? tiles : sms, ctas, kSplitThreads, kSplitSmem, stream, args);
+}
+
+}  // namespace rvq

@@ -17,8 +17,7 @@
 //     columns issued together, hand the accumulator back to the issuer as soon
 //     as they have landed, and fold them afterwards while the next chain runs.
 //     The fold keeps running minima over four partitions of the stage's
-//     columns: by 128-column chunk (a short list of the chunks that come within
-//     the error window of the running minimum), by 32-column block of a chunk,
+//     columns: by 128-column chunk (the two lowest chunks and the value of the third), by 32-column block of a chunk,
 //     by half of a block, and by place within a half (16 places): 36 minimum
 //     operations per 32 scores.  At the stage end the sets of chunks, blocks,
 //     halves and places whose minimum lies inside the window bound where the
@@ -26,7 +25,7 @@
 //     and only that codeword is fetched; otherwise the warp re-scores every
 //     column in the product of the sets exactly in float32 against the float32
 //     codebook (direct form, lowest index on ties), and a full exact scan
-//     covers list overflow.  The emitted code is the exact-L2 choice.
+//     covers a third chunk inside the window.  The emitted code is the exact-L2 choice.
 //   - The A operand (the residual split into half-precision head and remainder)
 //     lives in TMEM next to its tile's scores, so the tensor core fetches only B
 //     from shared memory; the constant (1 1 1 0 ...) rows that pick up the
@@ -350,17 +349,15 @@ encode_tensor_kernel(const Params p)
                 // column is farther than the approximation and float32 evaluation errors can bridge.
                 const float lim = threshold(w, m1);
                 const Listed in = listed(w, lim);
-                const uint32_t qmask = in.places, hmask = in.halves, bmask = in.blocks;
                 const int j1 = w.c1 * 128 + in.column();
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
                 const bool scan_all = force_scan || w.m3 <= lim || !(m1 < 59000.0f);
                 const bool unique = w.m2 > lim && in.single() && (uint32_t)j1 < (uint32_t)s.K;
                 const bool flagged = !deg && (scan_all || !unique);
                 int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
-                // Rows with more than one candidate: the whole warp re-scores the candidate columns of
-                // every listed block of one such row at a time (lane = place in the block; all columns
-                // when the list overflowed) exactly in float32, direct form, then reduces to the
-                // smallest distance, lowest index on ties.
+                // Rows with more than one candidate: the whole warp compares the candidate columns of one such
+                // row at a time exactly in float32, direct form (all columns when a third chunk came inside the
+                // window): smallest distance, lowest index on ties.
                 uint32_t todo = __ballot_sync(0xFFFFFFFFu, flagged);
                 while (todo) {
                     const int src = __ffs(todo) - 1;
@@ -370,37 +367,13 @@ encode_tensor_kernel(const Params p)
                     for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kRowsPerPass + (src - lane)];
                     const int chunk1 = __shfl_sync(0xFFFFFFFFu, w.c1, src);
                     const int chunk2 = __shfl_sync(0xFFFFFFFFu, w.m2 <= lim ? w.c2 : -1, src);
-                    const uint32_t qmask_s = __shfl_sync(0xFFFFFFFFu, qmask, src);
-                    const uint32_t hmask_s = __shfl_sync(0xFFFFFFFFu, hmask, src);
-                    const uint32_t bmask_s = __shfl_sync(0xFFFFFFFFu, bmask, src);
+                    const uint32_t sets = __shfl_sync(0xFFFFFFFFu, in.word(), src);
                     const bool all_s = __shfl_sync(0xFFFFFFFFu, (int)scan_all, src) != 0;
-                    const bool mine = ((qmask_s >> (lane & 15)) & 1u) && ((hmask_s >> (lane >> 4)) & 1u);
                     float bv = INFINITY;
                     int bi = 0x7FFFFFFF;
-                    if (all_s) {
-                        for (int j = lane; j < s.K; j += 32) {
-                            const float dj = exact_distance(zs, cbr + (size_t)j * 32);
-                            if (dj < bv) { bv = dj; bi = j; }
-                        }
-                    } else {
-                        for (int e = 0; e < 2; ++e) {
-                            const int chunk = e == 0 ? chunk1 : chunk2;                 // warp-uniform
-                            if (chunk < 0) continue;
-                            for (int i = 0; i < 4; ++i) {
-                                const int j = chunk * 128 + 32 * i + lane;
-                                if (((bmask_s >> i) & 1u) && mine && j < s.K) {     // (the block test is warp-uniform)
-                                    const float dj = exact_distance(zs, cbr + (size_t)j * 32);
-                                    if (dj < bv || (dj == bv && j < bi)) { bv = dj; bi = j; }
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        const float ov = __shfl_xor_sync(0xFFFFFFFFu, bv, off);
-                        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
-                        if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-                    }
+                    if (all_s) compare_all(zs, cbr, s.K, lane, bv, bi);
+                    else compare_listed(zs, cbr, s.K, lane, sets, chunk1, chunk2, bv, bi);
+                    best_of_warp(bv, bi);
                     if (lane == src) {
                         bj = bi < s.K ? bi : 0;
                         if (all_s) ++n_exhaustive; else ++n_rescored;
