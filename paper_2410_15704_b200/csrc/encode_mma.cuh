@@ -196,13 +196,33 @@ __device__ __forceinline__ float fold_block(Sweep &w, const uint32_t (&u)[32], i
     return m;
 }
 
+// The stage's maxima over its codewords (prepare.cu), for the window below.
+struct StageBounds {
+    float emax, eerr, elo;                  // norms: codeword, what its two halves miss, its remainder half
+};
+__device__ __forceinline__ StageBounds stage_bounds(const uint8_t *prepared, int r)
+{
+    const uint4 m = __ldg(reinterpret_cast<const uint4 *>(prepared + kPreparedMaximaOffset) + r);     // StageMaxima
+    return {__uint_as_float(m.x), __uint_as_float(m.y), __uint_as_float(m.w)};
+}
+
 // A column can only be the exact-L2 choice (in real arithmetic, and in the float32 direct-form
 // arithmetic of the all-float32 kernel, whose relative error on a distance is below 34 * 2^-24) if its
 // approximate score is at most threshold(m1): the window covers the approximation error of both
 // scores, the last term the float32 evaluation error of both distances (2 * 34 * 2^-24 < 2^-17.5).
-__device__ __forceinline__ float threshold(const Sweep &w, float m1)
+// Both columns concerned, the approximate and the exact winner, lie within rho of the row, rho^2 being the
+// approximate winner's squared distance, at most m1 + zz + win; so their norms are at most E = ||Z|| + rho,
+// and the error bound of prepare.cu, which allows every codeword the largest norm of the stage, is taken
+// with E where that is smaller.
+__device__ __forceinline__ float threshold(const Sweep &w, float m1, const StageBounds &sb)
 {
-    return m1 + w.win + 5.4e-6f * (fmaxf(m1 + w.zz, 0.0f) + w.win);
+    const float nz = sqrtf(w.zz) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
+    const float e = fminf(sb.emax, (nz + sqrtf(d2 + w.win)) * 1.0001f);
+    const float elo = fminf(sb.elo, 4.8828125e-4f * e + 1.7e-7f), eerr = fminf(sb.eerr, 2.384185791015625e-7f * e + 1.7e-7f);
+    const float a = 2.0f * (4.8828125e-4f * elo + 2.384185791015625e-7f * e + eerr) + 3.814697265625e-6f * e;
+    const float b = e * (1.9073486328125e-6f * e + 4.76837158203125e-7f);
+    const float win = fminf(w.win, 2.125f * (a * nz + b));
+    return m1 + win + 5.4e-6f * (d2 + win);
 }
 
 // Members of the three partitions whose minimum is at most `limit` (bit k: member k).  The comparisons are
@@ -390,6 +410,43 @@ __device__ __forceinline__ float group_deviation(const Shape &s, const float (&z
     float ss = 0.0f;
     for (int k = 0; k < s.G; ++k) ss += __shfl_sync(0xFFFFFFFFu, b, base + k);
     return sqrtf(ss / (float)(s.dim - s.ddof));
+}
+
+// z[i] / dev, correctly rounded like the scalar kernel's division; zeros for a degenerate row.  Called by a whole
+// warp.  With y = RN(1 / dev), a quotient within a few ulps is made exact by q + y (a - q dev), the residual
+// being exact in a fused multiply-add (P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", 1990), done twice.  That needs every intermediate value to be a normal number;
+// rows outside a wide range of exponents are divided one by one, which as a chain of 32 divisions with
+// their checks took 3100 cycles.
+__device__ __forceinline__ void divide_row(float (&z)[32], float dev, bool deg)
+{
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const uint32_t twice = __float_as_uint(z[i]) << 1;               // (the sign gone)
+        lo = min(lo, twice - 1u);                                         // (zeros count as large)
+        hi = max(hi, twice);
+    }
+    const bool ordinary = lo >= 2u * 0x21800000u - 1u && hi <= 2u * 0x5D800000u && dev >= 9.094947e-13f && dev <= 1.0995116e12f;
+    if (__all_sync(0xFFFFFFFFu, ordinary || deg)) {                       // 2^-60 .. 2^60 over 2^-40 .. 2^40
+        const float b = deg ? 1.0f : dev, y = __frcp_rn(b);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            float q = z[i] * y;
+            q = fmaf(fmaf(-q, b, z[i]), y, q);
+            q = fmaf(fmaf(-q, b, z[i]), y, q);
+            z[i] = deg ? 0.0f : q;
+        }
+    } else {
+#pragma unroll 1
+        for (int i = 0; i < 32; ++i) {
+            // (rolled: the array is rotated so that its indices stay constants)
+            const float q = deg ? 0.0f : z[0] / dev;
+#pragma unroll
+            for (int k = 0; k < 31; ++k) z[k] = z[k + 1];
+            z[31] = q;
+        }
+    }
 }
 
 // A operand row of the residual z: 16 words of half-precision head, 16 of remainder; returns the squared

@@ -216,8 +216,9 @@ encode_split_kernel(const SplitParams p)
                 for (int i = 0; i < 32; ++i) z[i] = z_park[i * kZPitch];
                 const float dev = group_deviation(s, z, lane);
                 deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
+                if (!s.raw) divide_row(z, dev, deg);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) z_park[i * kZPitch] = deg ? 0.0f : (s.raw ? z[i] : z[i] / dev);
+                for (int i = 0; i < 32; ++i) z_park[i * kZPitch] = deg ? 0.0f : z[i];
                 if (valid && (lane & (G - 1)) == 0 && !s.raw && rank == 0) {
                     const uint16_t hb = deviation_is_degenerate(dev) ? (uint16_t)0 : __half_as_ushort(__float2half_rn(dev));
                     p.std16[v] = hb;
@@ -278,9 +279,10 @@ encode_split_kernel(const SplitParams p)
                 if (!ok) break;
                 // this group's part of the row, to every CTA of the cluster
                 if (grp != 0 && grp < cnt) w.zz = norm[row];              // (a group without chunks has nothing inside any window)
+                const StageBounds sb = stage_bounds(p.prepared, r);
                 w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
                 {
-                    const float lim = threshold(w, w.m1);
+                    const float lim = threshold(w, w.m1, sb);
                     const Listed in = listed(w, lim);
                     const uint32_t sets = in.word() | (w.m3 <= lim ? 1u << 22 : 0u);
                     for (int to = 0; to < ctas; ++to)
@@ -304,7 +306,7 @@ encode_split_kernel(const SplitParams p)
                     k1 = m < m1 ? k : k1;
                     m1 = fminf(m1, m);
                 }
-                const float lim = threshold(w, m1);
+                const float lim = threshold(w, m1, sb);
                 const Part best = mp[k1 * 128];
                 const Listed in{best.sets & 0xFFFFu, (best.sets >> 16) & 3u, (best.sets >> 18) & 15u};
                 const int j1 = (int)(best.chunks & 0xFFFFu) * 128 + in.column();

@@ -272,8 +272,12 @@ encode_tensor_kernel(const Params p)
             // (raw rows are stage inputs already: taken as they are, no deviation stored)
             const bool deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
             if (p.defer_stats) smem[kOffFlags + rloc] = (uint8_t)((valid ? 1 : 0) | (deg ? 2 : 0));
+            if (!s.raw) {
+                divide_row(z, dev, deg);
+            } else if (deg) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) z[i] = deg ? 0.0f : (s.raw ? z[i] : z[i] / dev);
+                for (int i = 0; i < 32; ++i) z[i] = 0.0f;
+            }
             if (valid && g == 0 && !s.raw) {
                 const uint16_t hb = deviation_is_degenerate(dev) ? (uint16_t)0 : __half_as_ushort(__float2half_rn(dev));
                 p.std16[v] = hb;
@@ -347,7 +351,8 @@ encode_tensor_kernel(const Params p)
                 // chunk, in a listed block of the chunk, in a listed half, at a listed place.  When each of
                 // the four lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
-                const float lim = threshold(w, m1);
+                const StageBounds sb = stage_bounds(p.prepared, r);
+                const float lim = threshold(w, m1, sb);
                 const Listed in = listed(w, lim);
                 const int j1 = w.c1 * 128 + in.column();
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
