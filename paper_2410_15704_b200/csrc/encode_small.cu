@@ -257,17 +257,14 @@ SmallPlan small_plan(const Shape &s)
 
 }  // namespace
 
-// Up to one head vector per cluster that the device runs at a time (18 clusters of eight CTAs on a B200), and
-// up to kSmallBestRows group rows per cluster where that is still faster than a tile of 128 rows split over
-// CTAs.
-constexpr int kSmallBestRows = 32;
-
+// Group rows per cluster up to which this encoder is faster than a tile of 128 rows split over CTAs: a row costs
+// about 1.6 us at two blocks per CTA and 0.8 us at one, a split tile 36-40 us.
 bool encode_small_wanted(const Shape &s, int64_t n)
 {
-    if (!float_blocks_prepared(s) || s.raw || s.G > kSmallBestRows || n < 1 || n > 4096) return false;
+    if (!float_blocks_prepared(s) || s.raw || s.G > kSmallRows || n < 1 || n > 4096) return false;
     const SmallPlan plan = small_plan(s);
     const int64_t vectors = plan.at_once > 0 ? (n + plan.at_once - 1) / plan.at_once : 0;
-    return vectors > 0 && vectors * s.G <= kSmallBestRows;
+    return vectors == 1 || (vectors > 0 && vectors * s.G <= (plan.per_cta == 2 ? 16 : 24));
 }
 
 int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride, const void *prepared, void *codes,

@@ -474,8 +474,7 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,
              stat_sum != nullptr && encode_tensor_deferred_stages(s) > 0 ? 1 : 0};
-    const int64_t groups = (tiles + kTiles - 1) / kTiles;
-    const int grid = (int)(groups < sms ? groups : sms);
+    const int grid = (int)(tiles < sms ? tiles : sms);        // (fewer tiles than three per SM: one or two in each, not three in some)
     encode_tensor_kernel<<<grid, kThreads, kSmemBytes, stream>>>(p);
     return check_launch();
 }
