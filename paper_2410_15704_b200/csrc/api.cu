@@ -299,7 +299,7 @@ int rvq_decode(const rvq_config *cfg, const void *codes, const uint16_t *std_f16
     if ((rc = check_rows(s, x_out, n, out_row_stride)) != RVQ_OK) return rc;
     if (!codebooks || !prepared || (n > 0 && (!codes || !std_f16))) return RVQ_ERR_BADARG;
     if (!aligned16(codebooks) || !aligned16(codes) || !aligned256(prepared)) return RVQ_ERR_ALIGN;
-    if (decode_direct_wanted(s, n, false))
+    if (decode_direct_wanted(s, n, false, true))
         return launch_decode_direct(s, codes, std_f16, n, codebooks, x_out, out_row_stride, status, (cudaStream_t)stream);
     if (decode_sliced_supported(s))
         return launch_decode_sliced(s, codes, std_f16, n, codebooks, prepared, x_out, out_row_stride, status, (cudaStream_t)stream);
@@ -329,7 +329,7 @@ int rvq_decode_rope(const rvq_config *cfg, const void *codes, const uint16_t *st
         return RVQ_ERR_BADARG;
     if (s.dim & 1) return RVQ_ERR_UNSUPPORTED;
     if (!aligned16(codebooks) || !aligned16(codes) || !aligned16(cos_sin) || !aligned256(prepared)) return RVQ_ERR_ALIGN;
-    if (decode_direct_wanted(s, n, true))
+    if (decode_direct_wanted(s, n, true, prepared != nullptr))
         return launch_decode_direct(s, codes, std_f16, n, codebooks, x_out, out_row_stride, status, (cudaStream_t)stream, position,
                                     vectors_per_position, cos_sin, positions, pairing);
     return launch_decode_rope(s, codes, std_f16, n, codebooks, prepared, position, vectors_per_position, cos_sin, positions,

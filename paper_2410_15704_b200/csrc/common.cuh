@@ -55,7 +55,7 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
                          const float *cb, const void *prepared, void *out, int64_t stride, rvq_status *st,
                          cudaStream_t stream);
 // few head vectors: codewords straight from the float32 codebooks (position null: no rotary embedding)
-bool decode_direct_wanted(const Shape &s, int64_t n, bool rope);
+bool decode_direct_wanted(const Shape &s, int64_t n, bool rope, bool prepared);
 int launch_decode_direct(const Shape &s, const void *codes, const uint16_t *std16, int64_t n, const float *cb, void *out,
                          int64_t stride, rvq_status *st, cudaStream_t stream, const int32_t *position = nullptr,
                          int per_position = 1, const float *table = nullptr, int positions = 0, int pairing = 0);

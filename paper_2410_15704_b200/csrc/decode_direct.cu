@@ -14,61 +14,107 @@ namespace rvq {
 
 namespace {
 
-constexpr int kDirectThreads = 128;
+constexpr int kDirectThreads = 128, kDirectBlocks = 6;        // (72-80 registers; eight blocks spill and are slower)
 
 struct DirectRope {
     const int32_t *position;
-    int per_position;
+    uint32_t per_position, heads;     // head vectors of a position; the same where they divide the call's, else 1
     const float2 *table;          // (cos, sin) [positions][dim / 2]
     int positions;
 };
 
-// ROPE 0: none; 1: pairs (k, k + dim/2); 2: pairs (2k, 2k + 1).
-template <int ROPE>
-__global__ void __launch_bounds__(kDirectThreads)
-decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t n,
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)           // two float32 additions
+{
+    uint64_t c;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
+    return c;
+}
+
+// ROPE 0: none; 1: pairs (k, k + dim/2); 2: pairs (2k, 2k + 1).  DEPTH: the depth, or 0 for any up to 8.
+template <int ROPE, int DEPTH>
+__global__ void __launch_bounds__(kDirectThreads, kDirectBlocks)
+decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, uint32_t n,
                      const float *__restrict__ cb, void *__restrict__ out, int64_t stride, rvq_status *st, DirectRope rope)
 {
-    const int lane = threadIdx.x & 31, rho = lane >> 3, q = lane & 7;
-    const int G = s.G, R = s.R, lg = __ffs(G) - 1;
+    const uint32_t lane = threadIdx.x & 31, rho = lane >> 3, q = lane & 7;
+    const uint32_t G = s.G, R = DEPTH ? DEPTH : s.R, lg = __ffs(G) - 1, lgk = lg - 2, K = s.K;
     const bool strided = s.layout == RVQ_GROUP_STRIDED;
-    const int64_t sets = n << (lg - 2);                       // of four group rows
-    const uint32_t K = (uint32_t)s.K;
     uint32_t bad = 0;
-    for (int64_t set = (int64_t)blockIdx.x * (kDirectThreads / 32) + (threadIdx.x >> 5); set < sets;
-         set += (int64_t)gridDim.x * (kDirectThreads / 32)) {
-        const int64_t v = set >> (lg - 2);
-        const int k = (int)(set & ((G >> 2) - 1));
-        // rows of the set: groups 2k, 2k + 1 and the same G / 2 further on, so that the channels of a rotary pair
-        // are in one warp whatever the pairing
-        const int g = 2 * k + (rho & 1) + (rho >> 1) * (G >> 1);
-        // lane: stage q of its row
-        uint32_t code = 0;
-        if (q < R) {
-            code = read_code(reinterpret_cast<const uint8_t *>(codes) + v * s.code_bytes, g * R + q, s.bits, s.code_bytes);
-            if (code >= K) { code = 0; ++bad; }
-        }
-        const float sd = __half2float(__ushort_as_half(__ldg(std16 + v)));
-        float4 e[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const uint32_t j = __shfl_sync(0xFFFFFFFFu, code, (lane & 24) | r);
-            e[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r < R) e[r] = __ldg(reinterpret_cast<const float4 *>(cb + ((size_t)r * K + j) * 32) + q);
-        }
-        float2 cs[4];
-        if (ROPE != 0) {
-            const int pos = min(max(__ldg(rope.position + v / rope.per_position), 0), rope.positions - 1);
-            const float2 *row = rope.table + (size_t)pos * (16 * G);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int el = 4 * q + i, c = strided ? (el << lg) + g : g * 32 + el;
-                cs[i] = __ldg(row + (ROPE == 1 ? c & (16 * G - 1) : c >> 1));
+    // every warp takes a run of consecutive sets of four group rows; code and deviation of the next set are asked
+    // for before the codewords of this one are added up.  Set number -> (head vector, part k of its groups): the
+    // parts of a vector one after the other, or with rotary pairs the heads of a token first (they share the
+    // part's cosines and sines).
+    const uint32_t sets = n << lgk, warps = gridDim.x * (kDirectThreads / 32), warp = blockIdx.x * (kDirectThreads / 32) + (threadIdx.x >> 5);
+    const uint32_t per = sets / warps, extra = sets - per * warps;
+    uint32_t set = warp * per + min(warp, extra);
+    const uint32_t end = set + per + (warp < extra ? 1u : 0u);
+    // rows of set (v, k): groups 2k, 2k + 1 and the same G / 2 further on, so that the channels of a rotary pair
+    // are in one warp whatever the pairing; lane: stage q of its row
+    const uint32_t g0 = (rho & 1) + (rho >> 1) * (G >> 1);
+    const uint32_t bits = s.bits, mask = (1u << bits) - 1u;
+    const uint32_t stage_off = q * K * 128u;                  // bytes of the codebooks before stage q
+    const bool has = q < R;
+    const uint32_t parts = G >> 2, heads = ROPE != 0 ? rope.heads : 1u;
+    struct Place { uint32_t v, k; };
+    auto place = [&](uint32_t at) -> Place {
+        if (ROPE == 0 || lgk == 0) return {at >> lgk, at & (parts - 1u)};
+        const uint32_t unit = at / heads, head = at - unit * heads;          // (token, part), head
+        return {(unit >> lgk) * heads + head, unit & (parts - 1u)};
+    };
+    auto fetch = [&](Place at, uint32_t &code, uint16_t &sd) {
+        const uint32_t v = at.v, g = g0 + 2u * at.k;
+        const uint8_t *vec = reinterpret_cast<const uint8_t *>(codes) + (size_t)v * (uint32_t)s.code_bytes;
+        const uint32_t k = g * R + q;
+        code = 0;
+        if (has) {
+            if (bits == 16) {
+                code = __ldg(reinterpret_cast<const uint16_t *>(vec) + k);
+            } else {
+                const uint32_t o = k * bits, w = o >> 5, sh = o & 31u;
+                const uint32_t *p = reinterpret_cast<const uint32_t *>(vec) + w;
+                code = __funnelshift_r(__ldg(p), sh + bits > 32u ? __ldg(p + 1) : 0u, sh) & mask;
             }
         }
-        float o[4] = {0.f, 0.f, 0.f, 0.f};
+        sd = __ldg(std16 + v);
+    };
+    uint32_t next_code = 0, pairs_of = 0xFFFFFFFFu;
+    Place next = place(min(set, sets - 1u));
+    uint16_t next_sd = 0;
+    float2 cs[4];
+    const uint8_t *piece = reinterpret_cast<const uint8_t *>(cb) + q * 16u;
+    if (set < end) fetch(next, next_code, next_sd);
+    for (; set < end; ++set) {
+        const uint32_t v = next.v, k = next.k, g = g0 + 2u * k;
+        const float sd = __half2float(__ushort_as_half(next_sd));
+        if (next_code >= K) { next_code = 0; ++bad; }
+        const uint32_t off = stage_off + next_code * 128u;    // of this lane's codeword (8 * 65536 * 128 bytes fit 32 bits)
+        uint64_t lo[8], hi[8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) { o[0] += e[r].x; o[1] += e[r].y; o[2] += e[r].z; o[3] += e[r].w; }
+        for (int r = 0; r < 8; ++r) {
+            const uint32_t at = __shfl_sync(0xFFFFFFFFu, off, (lane & 24) | r);
+            lo[r] = hi[r] = 0ull;
+            if (r < (DEPTH ? DEPTH : (int)R))
+                asm("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(lo[r]), "=l"(hi[r]) : "l"(piece + at));
+        }
+        if (set + 1 < end) { next = place(set + 1); fetch(next, next_code, next_sd); }
+        if (ROPE != 0) {
+            const uint32_t t = v / rope.per_position;
+            if (t * parts + k != pairs_of) {                  // (warp-uniform)
+                pairs_of = t * parts + k;
+                const int pos = min(max(__ldg(rope.position + t), 0), rope.positions - 1);
+                const float2 *row = rope.table + (size_t)pos * (16 * G);
+#pragma unroll
+                for (uint32_t i = 0; i < 4; ++i) {
+                    const uint32_t el = 4 * q + i, c = strided ? (el << lg) + g : g * 32 + el;
+                    cs[i] = __ldg(row + (ROPE == 1 ? c & (16 * G - 1) : c >> 1));
+                }
+            }
+        }
+        uint64_t s0 = lo[0], s1 = hi[0];
+#pragma unroll
+        for (int r = 1; r < (DEPTH ? DEPTH : 8); ++r) { s0 = add2(s0, lo[r]); s1 = add2(s1, hi[r]); }
+        float o[4] = {__uint_as_float((uint32_t)s0), __uint_as_float((uint32_t)(s0 >> 32)),
+                      __uint_as_float((uint32_t)s1), __uint_as_float((uint32_t)(s1 >> 32))};
 #pragma unroll
         for (int i = 0; i < 4; ++i) o[i] *= sd;
         if (ROPE == 2 && !strided) {
@@ -80,7 +126,7 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
             }
         } else if (ROPE != 0) {
             // the other channel of the pair: group g ^ G/2, group g ^ 1, or (half-split pairs, strided groups) 16 elements on
-            const int other = ROPE == 2 ? 8 : strided ? 4 : 16;
+            const uint32_t other = ROPE == 2 ? 8 : strided ? 4 : 16;
             const bool first = (lane & other) == 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -89,7 +135,7 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
             }
         }
         if (!strided) {
-            const int64_t at = v * stride + g * 32 + 4 * q;
+            const size_t at = (size_t)v * stride + g * 32 + 4 * q;
             if (s.dtype == RVQ_F32) {
                 *reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + at) = make_float4(o[0], o[1], o[2], o[3]);
             } else {
@@ -107,15 +153,15 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
             // lane rho of the four holds elements 4q .. 4q+3 of its group and wants element 4q + rho of all four
             float t[4];
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
+            for (uint32_t x = 0; x < 4; ++x) {
                 // round x: exchange with lane rho ^ x; both send the element that the other wants
                 const float send = (rho ^ x) == 0 ? o[0] : (rho ^ x) == 1 ? o[1] : (rho ^ x) == 2 ? o[2] : o[3];
                 const float got = x == 0 ? send : __shfl_xor_sync(0xFFFFFFFFu, send, 8 * x);
 #pragma unroll
-                for (int y = 0; y < 4; ++y) t[y] = (rho ^ x) == y ? got : t[y];
+                for (uint32_t y = 0; y < 4; ++y) t[y] = (rho ^ x) == y ? got : t[y];
             }
             // t[y]: group of row y; rows 0, 1 and rows 2, 3 are neighbouring channels
-            const int64_t at = v * stride + ((int64_t)(4 * q + rho) << lg) + 2 * k;
+            const size_t at = (size_t)v * stride + ((4 * q + rho) << lg) + 2 * k;
             if (s.dtype == RVQ_F32) {
                 float *f = reinterpret_cast<float *>(out) + at;
                 *reinterpret_cast<float2 *>(f) = make_float2(t[0], t[1]);
@@ -140,13 +186,19 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
 
 }  // namespace
 
-#ifndef RVQ_DIRECT
-#define RVQ_DIRECT 1
-#endif
-bool decode_direct_wanted(const Shape &s, int64_t n, bool rope)
+// Where the table decoders are the faster ones: 16-bit outputs at depth 8 with up to 1536 codes (8-channel level
+// tables, or 4-channel float32 ones for large deviations), from a number of group rows on that pays for filling
+// them.  Measured (us, tables / direct, K = 1024, dim 128): moderate deviations 32768 vectors 9.7 / 10.2, 65536
+// 13.5 / 18.1, 262144 37 / 63; keys 65536 23 / 20, 262144 61 / 75; rotary keys 131072 47 / 46, 262144 80 / 95; dim
+// 256: 65536 27 / 33.  Direct wins at every size for 2048 codes (262144 vectors 74 / 61; keys 117 / 75, rotary
+// 232 / 93), float32 outputs (110 / 68) and smaller depths (depth 4: 57 / 41, float32 103 / 46).
+bool decode_direct_wanted(const Shape &s, int64_t n, bool rope, bool prepared)
 {
-    if (s.gd != 32 || s.G < 4 || (s.G & (s.G - 1)) != 0 || s.R > 8) return false;
-    return n * (s.G / 4) <= (RVQ_DIRECT ? RVQ_DIRECT * 1024 : (rope ? 8192 : 4096));
+    const int64_t sets = n * (s.G / 4);
+    if (s.gd != 32 || s.G < 4 || (s.G & (s.G - 1)) != 0 || s.R > 8 || sets > 0x7FFFFFFF) return false;
+    const bool tables = prepared && s.dtype != RVQ_F32 && s.K <= kDecodeWideK && s.R == 8 && s.bits >= 10 && s.G <= 32;
+    if (!tables || (rope && s.G != 4)) return true;
+    return sets <= (rope ? 131072 : s.G == 4 ? 28672 : 65536);
 }
 
 int launch_decode_direct(const Shape &s, const void *codes, const uint16_t *std16, int64_t n, const float *cb, void *out,
@@ -157,11 +209,13 @@ int launch_decode_direct(const Shape &s, const void *codes, const uint16_t *std1
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
     const int64_t warps = n * (s.G / 4), want = (warps + kDirectThreads / 32 - 1) / (kDirectThreads / 32);
-    const unsigned grid = (unsigned)(want < (int64_t)sms * 16 ? want : (int64_t)sms * 16);
-    const DirectRope rope{position, per_position, reinterpret_cast<const float2 *>(table), positions};
-    if (!position) decode_direct_kernel<0><<<grid, kDirectThreads, 0, stream>>>(s, codes, std16, n, cb, out, stride, st, rope);
-    else if (pairing == RVQ_ROPE_HALVES) decode_direct_kernel<1><<<grid, kDirectThreads, 0, stream>>>(s, codes, std16, n, cb, out, stride, st, rope);
-    else decode_direct_kernel<2><<<grid, kDirectThreads, 0, stream>>>(s, codes, std16, n, cb, out, stride, st, rope);
+    const unsigned grid = (unsigned)(want < (int64_t)sms * kDirectBlocks ? want : (int64_t)sms * kDirectBlocks);
+    const DirectRope rope{position, (uint32_t)per_position, n % per_position == 0 ? (uint32_t)per_position : 1u, reinterpret_cast<const float2 *>(table), positions};
+    const int kind = !position ? 0 : pairing == RVQ_ROPE_HALVES ? 1 : 2;
+#define RVQ_DIRECT_KINDS(D) (kind == 0 ? decode_direct_kernel<0, D> : kind == 1 ? decode_direct_kernel<1, D> : decode_direct_kernel<2, D>)
+    auto kernel = s.R == 8 ? RVQ_DIRECT_KINDS(8) : s.R == 6 ? RVQ_DIRECT_KINDS(6) : s.R == 4 ? RVQ_DIRECT_KINDS(4) : RVQ_DIRECT_KINDS(0);
+#undef RVQ_DIRECT_KINDS
+    kernel<<<grid, kDirectThreads, 0, stream>>>(s, codes, std16, (uint32_t)n, cb, out, stride, st, rope);
     return check_launch();
 }
 
