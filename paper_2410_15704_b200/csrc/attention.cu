@@ -369,6 +369,234 @@ __global__ void att_finish_kernel(const float *__restrict__ out_acc, const float
     if (idx < heads * 128) out[idx] = out_acc[idx] / weight_sum[idx >> 7];
 }
 
+// Short caches: one pass over the tokens, codewords straight from L2 (as in decode_direct.cu), the softmax carried
+// along, instead of tables that take longer to fill than the few tokens to read (two tables, five launches:
+// 35 us for 1000 tokens).  A CTA takes one kv head and a chunk of tokens, a warp one token at a time: lane =
+// (group, four-element piece), the key's and the value's sixteen 16-byte loads in flight together; the J
+// dot products are reduced so that lanes of row group `rho` end with query head j(rho), which keeps its running
+// maximum and weight sum.  The warps' partial outputs meet in shared memory, the chunks' in att_combine_kernel.
+// What bounds it: the chain codes -> codewords -> score -> weight of a warp's few tokens, then L2 (8 KB per token
+// and kv head), which is why long caches keep the tables.
+constexpr int kShortThreads = 256, kShortWarps = kShortThreads / 32;
+constexpr int kShortMaxChunks = 64;
+
+__device__ __forceinline__ uint64_t att_add2(uint64_t a, uint64_t b)
+{
+    uint64_t c;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
+    return c;
+}
+
+// Byte offset (into the codebooks) of the codeword of stage q of group row g of vector v; bad codes read as 0.
+__device__ __forceinline__ uint32_t att_code_offset(const Shape &s, const void *__restrict__ codes, uint32_t v, uint32_t g, uint32_t q,
+                                                    uint32_t &bad)
+{
+    if (q >= (uint32_t)s.R) return 0u;
+    uint32_t code = read_code(reinterpret_cast<const uint8_t *>(codes) + (size_t)v * (uint32_t)s.code_bytes, g * s.R + q, s.bits, s.code_bytes);
+    if (code >= (uint32_t)s.K) { code = 0; ++bad; }
+    return (q * (uint32_t)s.K + code) * 128u;
+}
+
+__device__ __forceinline__ void att_load_codewords(const Shape &s, const float *__restrict__ cb, uint32_t off, uint32_t lane,
+                                                   uint64_t (&lo)[8], uint64_t (&hi)[8])
+{
+    const uint8_t *piece = reinterpret_cast<const uint8_t *>(cb) + (lane & 7u) * 16u;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const uint32_t at = __shfl_sync(0xFFFFFFFFu, off, (lane & 24u) | r);
+        lo[r] = hi[r] = 0ull;
+        if (r < s.R) asm("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(lo[r]), "=l"(hi[r]) : "l"(piece + at));
+    }
+}
+
+__device__ __forceinline__ void att_sum_codewords(const uint64_t (&lo)[8], const uint64_t (&hi)[8], float sd, float (&o)[4])
+{
+    uint64_t a = lo[0], b = hi[0];
+#pragma unroll
+    for (int r = 1; r < 8; ++r) { a = att_add2(a, lo[r]); b = att_add2(b, hi[r]); }
+    o[0] = __uint_as_float((uint32_t)a) * sd; o[1] = __uint_as_float((uint32_t)(a >> 32)) * sd;
+    o[2] = __uint_as_float((uint32_t)b) * sd; o[3] = __uint_as_float((uint32_t)(b >> 32)) * sd;
+}
+
+template <int ROPE, int J>
+__global__ void __launch_bounds__(kShortThreads, 2)
+att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__restrict__ codes_k, const uint16_t *__restrict__ std_k,
+                 const void *__restrict__ codes_v, const uint16_t *__restrict__ std_v, uint32_t tokens, const float *__restrict__ cb_k,
+                 const float *__restrict__ cb_v, const int32_t *__restrict__ position, const float2 *__restrict__ cos_sin, int positions,
+                 float scale_log2e, float *__restrict__ part, float2 *__restrict__ part_ml, rvq_status *st)
+{
+    __shared__ __align__(16) float acc_s[kShortWarps][J][128];         // [group * 32 + element]
+    __shared__ float2 ml_s[kShortWarps][J];
+    asm volatile("griddepcontrol.launch_dependents;");
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 3, piece = lane & 7;
+    const uint32_t h = blockIdx.y, chunks = gridDim.x, chunk = blockIdx.x;
+    const bool strided = sk.layout == RVQ_GROUP_STRIDED;
+    const uint32_t per = (tokens + chunks - 1) / chunks, first = chunk * per, last = min(tokens, first + per);
+    float qr[J][4];
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t e = 4 * piece + i;
+            qr[j][i] = __ldg(q + (size_t)(h * J + j) * 128 + (strided ? 4 * e + g : 32 * g + e));
+        }
+    const uint32_t my_j = J == 4 ? g : J == 2 ? g >> 1 : 0;
+    float m = -INFINITY, l = 0.0f, acc[J][4] = {};
+    uint32_t bad = 0;
+    uint32_t t = first + warp;
+    uint32_t off_k = 0, off_v = 0;
+    uint16_t sdk = 0, sdv = 0;
+    int pos = 0;
+    auto fetch = [&](uint32_t at) {
+        const uint32_t v = at * 8u + h;
+        off_k = att_code_offset(sk, codes_k, v, g, piece, bad);
+        off_v = att_code_offset(sv, codes_v, v, g, piece, bad);
+        sdk = __ldg(std_k + v);
+        sdv = __ldg(std_v + v);
+        if (ROPE != 0) pos = position ? __ldg(position + at) : (int)at;
+    };
+    if (t < last) fetch(t);
+    for (; t < last; t += kShortWarps) {
+        uint64_t klo[8], khi[8], vlo[8], vhi[8];
+        att_load_codewords(sk, cb_k, off_k, lane, klo, khi);
+        float2 cs[4];
+        if (ROPE != 0) {
+            const float2 *row = cos_sin + (size_t)min(max(pos, 0), positions - 1) * 64;
+#pragma unroll
+            for (uint32_t i = 0; i < 4; ++i) {
+                const uint32_t e = 4 * piece + i, c = strided ? 4 * e + g : 32 * g + e;
+                cs[i] = __ldg(row + (ROPE == 1 ? c & 63u : c >> 1));
+            }
+        }
+        att_load_codewords(sv, cb_v, off_v, lane, vlo, vhi);
+        const float fk = __half2float(__ushort_as_half(sdk)), fv = __half2float(__ushort_as_half(sdv));
+        if (t + kShortWarps < last) fetch(t + kShortWarps);
+        float o[4];
+        att_sum_codewords(klo, khi, fk, o);
+        if (ROPE == 2 && !strided) {
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+                const float a = o[i], b = o[i + 1];
+                o[i] = a * cs[i].x - b * cs[i].y;
+                o[i + 1] = b * cs[i].x + a * cs[i].y;
+            }
+        } else if (ROPE != 0) {
+            // the other channel of the pair: group g ^ 2, group g ^ 1, or (half-split pairs, strided groups) 16 elements on
+            const uint32_t other = ROPE == 2 ? 8 : strided ? 4 : 16;
+            const bool low = (lane & other) == 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float p = __shfl_xor_sync(0xFFFFFFFFu, o[i], other);
+                o[i] = low ? o[i] * cs[i].x - p * cs[i].y : o[i] * cs[i].x + p * cs[i].y;
+            }
+        }
+        float p[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            p[j] = o[0] * qr[j][0];
+#pragma unroll
+            for (int i = 1; i < 4; ++i) p[j] = fmaf(o[i], qr[j][i], p[j]);
+        }
+        // sums over the warp, half of the query heads going to each half of the lanes, then to each quarter
+        float sc;
+        if (J == 4) {
+            const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
+            float a = up ? p[J - 2] : p[0], b = up ? p[J - 1] : p[J > 1 ? 1 : 0];
+            a += __shfl_xor_sync(0xFFFFFFFFu, up ? p[0] : p[J - 2], 16);
+            b += __shfl_xor_sync(0xFFFFFFFFu, up ? p[J > 1 ? 1 : 0] : p[J - 1], 16);
+            sc = up2 ? b : a;
+            sc += __shfl_xor_sync(0xFFFFFFFFu, up2 ? a : b, 8);
+        } else if (J == 2) {
+            const bool up = (lane & 16) != 0;
+            sc = up ? p[J - 1] : p[0];
+            sc += __shfl_xor_sync(0xFFFFFFFFu, up ? p[0] : p[J - 1], 16);
+            sc += __shfl_xor_sync(0xFFFFFFFFu, sc, 8);
+        } else {
+            sc = p[0] + __shfl_xor_sync(0xFFFFFFFFu, p[0], 16);
+            sc += __shfl_xor_sync(0xFFFFFFFFu, sc, 8);
+        }
+#pragma unroll
+        for (int x = 4; x > 0; x >>= 1) sc += __shfl_xor_sync(0xFFFFFFFFu, sc, x);
+        sc *= scale_log2e;
+        const float m2 = fmaxf(m, sc), corr = exp2f(m - m2), w = exp2f(sc - m2);    // (the first token: exp2(-inf) = 0)
+        const bool moved = m2 != m;
+        l = fmaf(l, corr, w);
+        m = m2;
+        att_sum_codewords(vlo, vhi, fv, o);
+        if (__any_sync(0xFFFFFFFFu, moved)) {
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const float c = __shfl_sync(0xFFFFFFFFu, corr, J == 4 ? 8 * j : J == 2 ? 16 * j : 0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[j][i] *= c;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const float wj = __shfl_sync(0xFFFFFFFFu, w, J == 4 ? 8 * j : J == 2 ? 16 * j : 0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(wj, o[i], acc[j][i]);
+        }
+    }
+    // the warps' parts
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+        *reinterpret_cast<float4 *>(&acc_s[warp][j][4 * lane]) = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+    if ((lane & (J == 4 ? 7u : J == 2 ? 15u : 31u)) == 0) ml_s[warp][my_j] = make_float2(m, l);
+    __syncthreads();
+    for (uint32_t idx = threadIdx.x; idx < J * 128; idx += kShortThreads) {
+        const uint32_t j = idx >> 7, c = idx & 127;
+        float top = -INFINITY, sum = 0.0f, a = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kShortWarps; ++w) top = fmaxf(top, ml_s[w][j].x);
+#pragma unroll
+        for (int w = 0; w < kShortWarps; ++w) {
+            const float f = ml_s[w][j].x == -INFINITY ? 0.0f : exp2f(ml_s[w][j].x - top);
+            sum = fmaf(f, ml_s[w][j].y, sum);
+            a = fmaf(f, acc_s[w][j][c], a);
+        }
+        part[((size_t)(h * J + j) * chunks + chunk) * 128 + c] = a;
+        if (c == 0) part_ml[(size_t)(h * J + j) * chunks + chunk] = make_float2(top, sum);
+    }
+    if (bad && st) atomicAdd(&st->bad_codes, bad);
+}
+
+// One CTA per query head: the chunks' parts, weighted to their common maximum, over the sum of all weights.
+__global__ void __launch_bounds__(128)
+att_combine_kernel(const float *__restrict__ part, const float2 *__restrict__ part_ml, int chunks, int layout_v, float *__restrict__ out)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int head = blockIdx.x, c = threadIdx.x;
+    float top = -INFINITY, sum = 0.0f, a = 0.0f;
+    for (int k = 0; k < chunks; ++k) top = fmaxf(top, part_ml[head * chunks + k].x);
+#pragma unroll 8
+    for (int k = 0; k < chunks; ++k) {
+        const float2 ml = part_ml[head * chunks + k];
+        const float f = ml.x == -INFINITY ? 0.0f : exp2f(ml.x - top);
+        sum = fmaf(f, ml.y, sum);
+        a = fmaf(f, part[((size_t)head * chunks + k) * 128 + c], a);
+    }
+    const int g = c >> 5, e = c & 31;
+    out[head * 128 + (layout_v == RVQ_GROUP_STRIDED ? 4 * e + g : c)] = a / sum;
+}
+
+#ifndef RVQ_SHORT
+#define RVQ_SHORT 4096
+#endif
+constexpr int64_t kShortTokens = RVQ_SHORT;
+
+// Chunks of a short cache: two CTAs per SM (over the 8 kv heads), no more than the tokens feed.
+int short_chunks(int64_t tokens)
+{
+    const int64_t fed = (tokens + kShortWarps - 1) / kShortWarps;
+    return (int)(fed < 37 ? fed : 37);
+}
+
+size_t short_workspace(int64_t tokens, int q_heads)
+{
+    return (size_t)short_chunks(tokens) * q_heads * (128 * 4 + 8) + 256;
+}
+
 }  // namespace
 
 // (token counts: the kernels index group rows, 32 per token, with 32-bit integers, and step past the end
@@ -386,7 +614,9 @@ bool attention_supported(const Shape &sk, const Shape &sv, int kv_heads, int q_h
 size_t attention_workspace_bytes(int64_t tokens, int q_heads)
 {
     const size_t scores = ((size_t)tokens * q_heads * 4 + 255) / 256 * 256;
-    return scores + 256 /* maxima */ + 256 /* weight sums */ + (size_t)q_heads * 128 * 4;
+    const size_t tables = scores + 256 /* maxima */ + 256 /* weight sums */ + (size_t)q_heads * 128 * 4;
+    const size_t shorter = tokens <= kShortTokens ? short_workspace(tokens, q_heads) : 0;
+    return tables > shorter ? tables : shorter;
 }
 
 int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, int q_heads, const void *codes_k,
@@ -399,6 +629,32 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
     uint8_t *ws = reinterpret_cast<uint8_t *>(workspace);
+    if (tokens <= kShortTokens) {
+        const int chunks = short_chunks(tokens), rope = cos_sin ? (pairing == RVQ_ROPE_HALVES ? 1 : 2) : 0;
+        float *part = reinterpret_cast<float *>(ws);
+        float2 *part_ml = reinterpret_cast<float2 *>(ws + (size_t)chunks * q_heads * 128 * 4);
+        const float2 *cs = reinterpret_cast<const float2 *>(cos_sin);
+        const float sl = scale * 1.4426950408889634f;
+        auto launch = [&](auto kernel) {
+            kernel<<<dim3((unsigned)chunks, 8), kShortThreads, 0, stream>>>(sk, sv, q, codes_k, std_k, codes_v, std_v, (uint32_t)tokens, cb_k,
+                                                                           cb_v, position, cs, positions, sl, part, part_ml, st);
+        };
+#define RVQ_SHORT_J(ROPE) (J == 4 ? launch(att_short_kernel<ROPE, 4>) : J == 2 ? launch(att_short_kernel<ROPE, 2>) : launch(att_short_kernel<ROPE, 1>))
+        if (rope == 0) RVQ_SHORT_J(0); else if (rope == 1) RVQ_SHORT_J(1); else RVQ_SHORT_J(2);
+#undef RVQ_SHORT_J
+        int rc = check_launch();
+        if (rc != RVQ_OK) return rc;
+        // (its launch overlaps the first kernel; it waits for that one's results on the device)
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)q_heads); cfg.blockDim = dim3(128); cfg.stream = stream;
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, att_combine_kernel, (const float *)part, (const float2 *)part_ml, chunks, sv.layout, out);
+        rc = check_launch();
+        return e == cudaSuccess ? rc : RVQ_ERR_LAUNCH;
+    }
     const size_t score_bytes = ((size_t)tokens * q_heads * 4 + 255) / 256 * 256;
     float *scores = reinterpret_cast<float *>(ws);
     uint32_t *m_ord = reinterpret_cast<uint32_t *>(ws + score_bytes);
