@@ -378,47 +378,45 @@ __global__ void att_finish_kernel(const float *__restrict__ out_acc, const float
 // What bounds it: the chain codes -> codewords -> score -> weight of a warp's few tokens, then L2 (8 KB per token
 // and kv head), which is why long caches keep the tables.
 constexpr int kShortThreads = 256, kShortWarps = kShortThreads / 32;
-constexpr int kShortMaxChunks = 64;
+constexpr int kShortMaxChunks = 37;      // two CTAs per SM, over the 8 kv heads
 
-__device__ __forceinline__ uint64_t att_add2(uint64_t a, uint64_t b)
+// Code number k of vector v as it is stored; nothing here waits for it.
+__device__ __forceinline__ uint32_t att_raw_code(const Shape &s, const void *__restrict__ codes, uint32_t v, uint32_t k)
 {
-    uint64_t c;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
-    return c;
+    const uint8_t *vec = reinterpret_cast<const uint8_t *>(codes) + (size_t)v * (uint32_t)s.code_bytes;
+    if (s.bits == 16) return __ldg(reinterpret_cast<const uint16_t *>(vec) + k);
+    const uint32_t o = k * (uint32_t)s.bits, sh = o & 31u;
+    const uint32_t *p = reinterpret_cast<const uint32_t *>(vec) + (o >> 5);
+    return __funnelshift_r(__ldg(p), sh + s.bits > 32u ? __ldg(p + 1) : 0u, sh) & ((1u << s.bits) - 1u);
 }
 
-// Byte offset (into the codebooks) of the codeword of stage q of group row g of vector v; bad codes read as 0.
-__device__ __forceinline__ uint32_t att_code_offset(const Shape &s, const void *__restrict__ codes, uint32_t v, uint32_t g, uint32_t q,
-                                                    uint32_t &bad)
+// The codewords of four group rows: lane (row, stage = piece) has the row's code of that stage.
+template <int DEPTH>
+__device__ __forceinline__ void att_load_codewords(const Shape &s, const float *__restrict__ cb, uint32_t code, uint32_t lane,
+                                                   uint64_t (&lo)[8], uint64_t (&hi)[8], uint32_t &bad)
 {
-    if (q >= (uint32_t)s.R) return 0u;
-    uint32_t code = read_code(reinterpret_cast<const uint8_t *>(codes) + (size_t)v * (uint32_t)s.code_bytes, g * s.R + q, s.bits, s.code_bytes);
     if (code >= (uint32_t)s.K) { code = 0; ++bad; }
-    return (q * (uint32_t)s.K + code) * 128u;
-}
-
-__device__ __forceinline__ void att_load_codewords(const Shape &s, const float *__restrict__ cb, uint32_t off, uint32_t lane,
-                                                   uint64_t (&lo)[8], uint64_t (&hi)[8])
-{
+    const uint32_t off = ((lane & 7u) * (uint32_t)s.K + code) * 128u;
     const uint8_t *piece = reinterpret_cast<const uint8_t *>(cb) + (lane & 7u) * 16u;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const uint32_t at = __shfl_sync(0xFFFFFFFFu, off, (lane & 24u) | r);
-        lo[r] = hi[r] = 0ull;
-        if (r < s.R) asm("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(lo[r]), "=l"(hi[r]) : "l"(piece + at));
+        if (DEPTH == 0) lo[r] = hi[r] = 0ull;
+        if (DEPTH ? r < DEPTH : r < s.R) asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(lo[r]), "=l"(hi[r]) : "l"(piece + at));
     }
 }
 
+template <int DEPTH>
 __device__ __forceinline__ void att_sum_codewords(const uint64_t (&lo)[8], const uint64_t (&hi)[8], float sd, float (&o)[4])
 {
     uint64_t a = lo[0], b = hi[0];
 #pragma unroll
-    for (int r = 1; r < 8; ++r) { a = att_add2(a, lo[r]); b = att_add2(b, hi[r]); }
+    for (int r = 1; r < (DEPTH ? DEPTH : 8); ++r) { a = add_f32x2(a, lo[r]); b = add_f32x2(b, hi[r]); }
     o[0] = __uint_as_float((uint32_t)a) * sd; o[1] = __uint_as_float((uint32_t)(a >> 32)) * sd;
     o[2] = __uint_as_float((uint32_t)b) * sd; o[3] = __uint_as_float((uint32_t)(b >> 32)) * sd;
 }
 
-template <int ROPE, int J>
+template <int ROPE, int J, int DEPTH>                                 // DEPTH: of both, or 0 for any
 __global__ void __launch_bounds__(kShortThreads, 2)
 att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__restrict__ codes_k, const uint16_t *__restrict__ std_k,
                  const void *__restrict__ codes_v, const uint16_t *__restrict__ std_v, uint32_t tokens, const float *__restrict__ cb_k,
@@ -444,13 +442,13 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
     float m = -INFINITY, l = 0.0f, acc[J][4] = {};
     uint32_t bad = 0;
     uint32_t t = first + warp;
-    uint32_t off_k = 0, off_v = 0;
+    uint32_t code_k = 0, code_v = 0;
     uint16_t sdk = 0, sdv = 0;
     int pos = 0;
     auto fetch = [&](uint32_t at) {
         const uint32_t v = at * 8u + h;
-        off_k = att_code_offset(sk, codes_k, v, g, piece, bad);
-        off_v = att_code_offset(sv, codes_v, v, g, piece, bad);
+        if ((int)piece < (DEPTH ? DEPTH : sk.R)) code_k = att_raw_code(sk, codes_k, v, g * sk.R + piece);
+        if ((int)piece < (DEPTH ? DEPTH : sv.R)) code_v = att_raw_code(sv, codes_v, v, g * sv.R + piece);
         sdk = __ldg(std_k + v);
         sdv = __ldg(std_v + v);
         if (ROPE != 0) pos = position ? __ldg(position + at) : (int)at;
@@ -458,7 +456,7 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
     if (t < last) fetch(t);
     for (; t < last; t += kShortWarps) {
         uint64_t klo[8], khi[8], vlo[8], vhi[8];
-        att_load_codewords(sk, cb_k, off_k, lane, klo, khi);
+        att_load_codewords<DEPTH>(sk, cb_k, code_k, lane, klo, khi, bad);
         float2 cs[4];
         if (ROPE != 0) {
             const float2 *row = cos_sin + (size_t)min(max(pos, 0), positions - 1) * 64;
@@ -468,11 +466,11 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
                 cs[i] = __ldg(row + (ROPE == 1 ? c & 63u : c >> 1));
             }
         }
-        att_load_codewords(sv, cb_v, off_v, lane, vlo, vhi);
+        att_load_codewords<DEPTH>(sv, cb_v, code_v, lane, vlo, vhi, bad);
         const float fk = __half2float(__ushort_as_half(sdk)), fv = __half2float(__ushort_as_half(sdv));
         if (t + kShortWarps < last) fetch(t + kShortWarps);
         float o[4];
-        att_sum_codewords(klo, khi, fk, o);
+        att_sum_codewords<DEPTH>(klo, khi, fk, o);
         if (ROPE == 2 && !strided) {
 #pragma unroll
             for (int i = 0; i < 4; i += 2) {
@@ -522,7 +520,7 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
         const bool moved = m2 != m;
         l = fmaf(l, corr, w);
         m = m2;
-        att_sum_codewords(vlo, vhi, fv, o);
+        att_sum_codewords<DEPTH>(vlo, vhi, fv, o);
         if (__any_sync(0xFFFFFFFFu, moved)) {
 #pragma unroll
             for (int j = 0; j < J; ++j) {
@@ -565,31 +563,39 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
 __global__ void __launch_bounds__(128)
 att_combine_kernel(const float *__restrict__ part, const float2 *__restrict__ part_ml, int chunks, int layout_v, float *__restrict__ out)
 {
+    __shared__ float2 ml_s[kShortMaxChunks];
+    __shared__ float f_s[kShortMaxChunks];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int head = blockIdx.x, c = threadIdx.x;
+    if (c < chunks) ml_s[c] = part_ml[head * chunks + c];
+    __syncthreads();
     float top = -INFINITY, sum = 0.0f, a = 0.0f;
-    for (int k = 0; k < chunks; ++k) top = fmaxf(top, part_ml[head * chunks + k].x);
-#pragma unroll 8
-    for (int k = 0; k < chunks; ++k) {
-        const float2 ml = part_ml[head * chunks + k];
-        const float f = ml.x == -INFINITY ? 0.0f : exp2f(ml.x - top);
-        sum = fmaf(f, ml.y, sum);
-        a = fmaf(f, part[((size_t)head * chunks + k) * 128 + c], a);
-    }
+    for (int k = 0; k < chunks; ++k) top = fmaxf(top, ml_s[k].x);
+    if (c < chunks) f_s[c] = ml_s[c].x == -INFINITY ? 0.0f : exp2f(ml_s[c].x - top);
+    __syncthreads();
+    // (all parts asked for together)
+    float v[kShortMaxChunks];
+#pragma unroll
+    for (int k = 0; k < kShortMaxChunks; ++k) v[k] = k < chunks ? __ldcg(part + ((size_t)head * chunks + k) * 128 + c) : 0.0f;
+#pragma unroll
+    for (int k = 0; k < kShortMaxChunks; ++k)
+        if (k < chunks) {
+            sum = fmaf(f_s[k], ml_s[k].y, sum);
+            a = fmaf(f_s[k], v[k], a);
+        }
     const int g = c >> 5, e = c & 31;
     out[head * 128 + (layout_v == RVQ_GROUP_STRIDED ? 4 * e + g : c)] = a / sum;
 }
 
-#ifndef RVQ_SHORT
-#define RVQ_SHORT 4096
-#endif
-constexpr int64_t kShortTokens = RVQ_SHORT;
+// Tokens up to which the one-pass kernel is the faster one.  Measured (us, tables / one pass, 32 query heads, K =
+// 1024): 1000 tokens 35 / 13, 8000 61 / 43, 16000 90 / 77, 131072 505 / 578.
+constexpr int64_t kShortTokens = 32768;
 
-// Chunks of a short cache: two CTAs per SM (over the 8 kv heads), no more than the tokens feed.
+// Chunks of a short cache: no more than its tokens feed.
 int short_chunks(int64_t tokens)
 {
     const int64_t fed = (tokens + kShortWarps - 1) / kShortWarps;
-    return (int)(fed < 37 ? fed : 37);
+    return (int)(fed < kShortMaxChunks ? fed : kShortMaxChunks);
 }
 
 size_t short_workspace(int64_t tokens, int q_heads)
@@ -639,9 +645,14 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
             kernel<<<dim3((unsigned)chunks, 8), kShortThreads, 0, stream>>>(sk, sv, q, codes_k, std_k, codes_v, std_v, (uint32_t)tokens, cb_k,
                                                                            cb_v, position, cs, positions, sl, part, part_ml, st);
         };
-#define RVQ_SHORT_J(ROPE) (J == 4 ? launch(att_short_kernel<ROPE, 4>) : J == 2 ? launch(att_short_kernel<ROPE, 2>) : launch(att_short_kernel<ROPE, 1>))
+        const int depth = sk.R != sv.R ? 0 : sk.R;
+#define RVQ_SHORT_F(ROPE, JJ)                                                                                        \
+        (depth == 8 ? launch(att_short_kernel<ROPE, JJ, 8>) : depth == 6 ? launch(att_short_kernel<ROPE, JJ, 6>)     \
+         : depth == 4 ? launch(att_short_kernel<ROPE, JJ, 4>) : launch(att_short_kernel<ROPE, JJ, 0>))
+#define RVQ_SHORT_J(ROPE) (J == 4 ? RVQ_SHORT_F(ROPE, 4) : J == 2 ? RVQ_SHORT_F(ROPE, 2) : RVQ_SHORT_F(ROPE, 1))
         if (rope == 0) RVQ_SHORT_J(0); else if (rope == 1) RVQ_SHORT_J(1); else RVQ_SHORT_J(2);
 #undef RVQ_SHORT_J
+#undef RVQ_SHORT_F
         int rc = check_launch();
         if (rc != RVQ_OK) return rc;
         // (its launch overlaps the first kernel; it waits for that one's results on the device)

@@ -135,6 +135,14 @@ __device__ __forceinline__ uint32_t read_code(const void *vec, int k, int bits, 
     return __funnelshift_r(lo, hi, sh) & ((1u << bits) - 1u);
 }
 
+// Two float32 additions in one instruction.
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t c;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
+    return c;
+}
+
 __device__ __forceinline__ bool deviation_is_degenerate(float s) { return !(s > 0.0f) || !isfinite(s); }
 
 // Load a tile of `vpb` head vectors (first vector v0) into shared memory as

@@ -23,13 +23,6 @@ struct DirectRope {
     int positions;
 };
 
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)           // two float32 additions
-{
-    uint64_t c;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
-    return c;
-}
-
 // ROPE 0: none; 1: pairs (k, k + dim/2); 2: pairs (2k, 2k + 1).  DEPTH: the depth, or 0 for any up to 8.
 template <int ROPE, int DEPTH>
 __global__ void __launch_bounds__(kDirectThreads, kDirectBlocks)
@@ -112,7 +105,7 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
         }
         uint64_t s0 = lo[0], s1 = hi[0];
 #pragma unroll
-        for (int r = 1; r < (DEPTH ? DEPTH : 8); ++r) { s0 = add2(s0, lo[r]); s1 = add2(s1, hi[r]); }
+        for (int r = 1; r < (DEPTH ? DEPTH : 8); ++r) { s0 = add_f32x2(s0, lo[r]); s1 = add_f32x2(s1, hi[r]); }
         float o[4] = {__uint_as_float((uint32_t)s0), __uint_as_float((uint32_t)(s0 >> 32)),
                       __uint_as_float((uint32_t)s1), __uint_as_float((uint32_t)(s1 >> 32))};
 #pragma unroll

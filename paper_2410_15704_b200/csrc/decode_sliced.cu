@@ -665,7 +665,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
         // integer sums of level * scale: one 16-bit x 8-bit dot-product instruction per channel and stage,
         // or (summed levels) plain additions of the table words and two such instructions per channel
         uint32_t acc[CH], even[CH / 2], odd[CH / 2];
-        float facc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        uint64_t fa = 0ull, fb = 0ull;                          // float32 sums, two channels to a register pair
 #pragma unroll
         for (int i = 0; i < CH; ++i) acc[i] = 0u;
 #pragma unroll
@@ -679,9 +679,9 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             const uint32_t a = smem_table + (line | unit[k]);
             uint32_t e[CH / 2];
             if (F32) {
-                float f0, f1, f2, f3;
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f0), "=f"(f1), "=f"(f2), "=f"(f3) : "r"(a));
-                facc[0] += f0; facc[1] += f1; facc[2] += f2; facc[3] += f3;
+                uint64_t f01, f23;
+                asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(f01), "=l"(f23) : "r"(a));
+                fa = add_f32x2(fa, f01); fb = add_f32x2(fb, f23);
                 continue;
             }
             if (CH == 8)
@@ -710,6 +710,8 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
         float o8[CH];
         {
             const float bs = base * sd, cs = bias * sd;
+            const float facc[4] = {__uint_as_float((uint32_t)fa), __uint_as_float((uint32_t)(fa >> 32)),
+                                   __uint_as_float((uint32_t)fb), __uint_as_float((uint32_t)(fb >> 32))};
 #pragma unroll
             for (int i = 0; i < CH; ++i) o8[i] = F32 ? facc[i & 3] * sd : fmaf((float)acc[i], bs, cs);
         }
