@@ -9,7 +9,7 @@ namespace rvq {
 
 constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
 constexpr int kOnesBytes = 2 * 128 * 16;                  // the constant A cells (1 1 1 0 ...) and (0 ...)
-constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 -> f32, M = N = 128
+constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 or e4m3 x e4m3 -> f32, M = N = 128
 
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -81,6 +81,13 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uin
 {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_e4m3_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar)
@@ -158,7 +165,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32
 // Per-row state of one stage's sweep over the scores.
 struct Sweep {
     float win;               // error window
-    float zz;                // squared norm of the scaled residual: m1 + zz is the best squared distance
+    float zz, ll;            // squared norms of the scaled residual (m1 + zz is the best squared distance) and of its remainder
     float m1, m2, m3;        // the three lowest chunk minima ...
     int c1, c2;              // ... and the chunks of the first two
     float bb[4];             // minimum per 32-column block position inside its 128-column chunk
@@ -222,6 +229,29 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1, const Stage
     const float a = 2.0f * (4.8828125e-4f * elo + 2.384185791015625e-7f * e + eerr) + 3.814697265625e-6f * e;
     const float b = e * (1.9073486328125e-6f * e + 4.76837158203125e-7f);
     const float win = fminf(w.win, 2.125f * (a * nz + b));
+    return m1 + win + 5.4e-6f * (d2 + win);
+}
+
+// The same for the chain with 8-bit corrections.  With e4m3's rounding error of at most c = 0.0595 of a value (its
+// half unit in the last place, and the rounding of the remainder to a half before it) or 2^-10 near zero, and E as
+// above, the dot product is off by at most
+//   |z_lo.e - [64 z_lo][e/64]|        <= ||z_lo|| (cE + (1 + c)(cE + 64 sqrt(32) 2^-10)) + sqrt(32) 2^-16 (1 + c) E
+//   |z_hi.e_lo - [z_hi/64][64 e_lo]|  <= (cN + 0.354) L + ((1 + c) N + 0.354)(cL + sqrt(32) 2^-16)
+// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (the worst of 330000
+// chains on operands of this shape, x20 outlier channels among them, was 9.4e-5 |z||e|).
+__device__ __forceinline__ float window8(float nz, float nl, float e, const StageBounds &sb)
+{
+    constexpr float c = 0.0595f;
+    const float elo = fminf(sb.elo + sb.eerr, 4.8828125e-4f * e + 1.7e-7f);
+    const float t1 = nl * (c * e + (1.0f + c) * (c * e + 0.354f)) + 8.7e-5f * 1.06f * e;
+    const float t2 = (c * nz + 0.354f) * elo + ((1.0f + c) * nz + 0.354f) * (c * elo + 8.7e-5f);
+    return 2.125f * (2.0f * (t1 + t2) + 1.9073486328125e-6f * e * (e + 2.0f * nz) + 4.76837158203125e-7f * e);
+}
+__device__ __forceinline__ float threshold8(const Sweep &w, float m1, const StageBounds &sb)
+{
+    const float nz = sqrtf(w.zz) * 1.0001f, nl = sqrtf(w.ll) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
+    const float full = window8(nz, nl, sb.emax, sb);
+    const float win = fminf(full, window8(nz, nl, fminf(sb.emax, (nz + sqrtf(d2 + full)) * 1.0001f), sb));
     return m1 + win + 5.4e-6f * (d2 + win);
 }
 
@@ -336,13 +366,25 @@ __device__ __forceinline__ void best_of_warp(float &bv, int &bi)
 // B cell is 128 codewords x 16 bytes = 128 descriptor address units.
 __device__ __forceinline__ void issue_chain(uint32_t acc, uint32_t a0, uint64_t bd, uint64_t ones_desc)
 {
-    mma_f16_ts(acc, a0, bd + 1 * 128, kChainDesc, 0);            // hi[0:16]  . hi cells 1-2
-    mma_f16_ts(acc, a0 + 8, bd + 3 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 3-4
-    mma_f16_ts(acc, a0, bd + 5 * 128, kChainDesc, 1);            // hi[0:16]  . lo cells 5-6
-    mma_f16_ts(acc, a0 + 8, bd + 7 * 128, kChainDesc, 1);        // hi[16:32] . lo cells 7-8
-    mma_f16_ts(acc, a0 + 16, bd + 1 * 128, kChainDesc, 1);       // lo[0:16]  . hi cells 1-2
-    mma_f16_ts(acc, a0 + 24, bd + 3 * 128, kChainDesc, 1);       // lo[16:32] . hi cells 3-4
-    mma_f16_ss(acc, ones_desc, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 0 (and cell 1 . 0)
+    mma_f16_ts(acc, a0, bd + 5 * 128, kChainDesc, 0);            // hi[0:16]  . hi cells 5-6
+    mma_f16_ts(acc, a0 + 8, bd + 7 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 7-8
+    mma_f16_ts(acc, a0, bd, kChainDesc, 1);                      // hi[0:16]  . lo cells 0-1
+    mma_f16_ts(acc, a0 + 8, bd + 2 * 128, kChainDesc, 1);        // hi[16:32] . lo cells 2-3
+    mma_f16_ts(acc, a0 + 16, bd + 5 * 128, kChainDesc, 1);       // lo[0:16]  . hi cells 5-6
+    mma_f16_ts(acc, a0 + 24, bd + 7 * 128, kChainDesc, 1);       // lo[16:32] . hi cells 7-8
+    mma_f16_ss(acc, ones_desc, bd + 4 * 128, kChainDesc, 1);     // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
+}
+
+// The chain with 8-bit corrections, on the last nine cells of a slot: two K = 32 steps of e4m3 (TMEM columns a0 +
+// 16 ..: 8 of 64 times the remainder, 8 of a 64th of the head), then heads and norm in half precision.  Five
+// steps instead of seven: 327 against 455 cycles (measured).
+__device__ __forceinline__ void issue_chain8(uint32_t acc, uint32_t a0, uint64_t bd, uint64_t ones_desc)
+{
+    mma_e4m3_ts(acc, a0 + 16, bd + 5 * 128, kChainDesc, 0);      // [64 lo]_8    . [e / 64]_8 (cells 9-10 of the slot)
+    mma_e4m3_ts(acc, a0 + 24, bd + 7 * 128, kChainDesc, 1);      // [hi / 64]_8  . [64 e_lo]_8 (cells 11-12)
+    mma_f16_ts(acc, a0, bd + 1 * 128, kChainDesc, 1);            // hi[0:16]  . hi cells 5-6
+    mma_f16_ts(acc, a0 + 8, bd + 3 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 7-8
+    mma_f16_ss(acc, ones_desc, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
 }
 
 // The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces through
@@ -465,6 +507,38 @@ __device__ __forceinline__ float split_operand(const float (&z)[32], float scale
         ab[16 + i] = *reinterpret_cast<const uint32_t *>(&l2);
     }
     return zz;
+}
+
+// The same for the chain with 8-bit corrections: 16 words of head, 8 of 64 times the remainder, 8 of a 64th of the
+// head; zz, ll: squared norms of the scaled residual and of the remainder.
+__device__ __forceinline__ uint32_t e4m3x2(__half2 v)
+{
+    uint16_t d;
+    asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(d) : "r"(*reinterpret_cast<const uint32_t *>(&v)));
+    return d;
+}
+__device__ __forceinline__ void split_operand8(const float (&z)[32], float scale, uint32_t (&ab)[32], float &zz, float &ll)
+{
+    zz = ll = 0.0f;
+    const __half2 up = __floats2half2_rn(64.0f, 64.0f), down = __floats2half2_rn(0.015625f, 0.015625f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        uint32_t lo8[2], hi8[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float z0 = z[4 * i + 2 * h] * scale, z1 = z[4 * i + 2 * h + 1] * scale;
+            zz = fmaf(z0, z0, zz); zz = fmaf(z1, z1, zz);
+            const __half2 h2 = __floats2half2_rn(z0, z1);
+            const float2 hf = __half22float2(h2);
+            const float l0 = z0 - hf.x, l1 = z1 - hf.y;
+            ll = fmaf(l0, l0, ll); ll = fmaf(l1, l1, ll);
+            ab[2 * i + h] = *reinterpret_cast<const uint32_t *>(&h2);
+            lo8[h] = e4m3x2(__hmul2(__floats2half2_rn(l0, l1), up));
+            hi8[h] = e4m3x2(__hmul2(h2, down));
+        }
+        ab[16 + i] = __byte_perm(lo8[0], lo8[1], 0x5410);
+        ab[24 + i] = __byte_perm(hi8[0], hi8[1], 0x5410);
+    }
 }
 
 // Codes of the warp's 32 rows (first vector v_first), from codes_s[row of the warp][16], to global memory in

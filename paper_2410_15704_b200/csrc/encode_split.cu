@@ -105,7 +105,7 @@ encode_split_kernel(const SplitParams p)
     if (warp == 13) {
         // ------------------------------------------------------------ operand loader
         if (lane == 0) {
-            const uint8_t *image = p.prepared + kPreparedImageOffset + (size_t)base * kSlotBytes;
+            const uint8_t *image = p.prepared + kPreparedImageOffset + (size_t)base * kSlotStride;
             uint32_t slot = 0, par = 1, issued = 0;
             bool ok = true;
             for (int t = 0; t < my_tiles && ok; ++t)
@@ -115,7 +115,7 @@ encode_split_kernel(const SplitParams p)
                         if (!ok) break;
                         mbar_expect_tx(BAR(kSFull + slot), kSlotBytes);
                         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(smem_u32(smem + kSOffB) + slot * (uint32_t)kSlotBytes), "l"(image + ((size_t)r * S + c) * kSlotBytes),
+                                     ::"r"(smem_u32(smem + kSOffB) + slot * (uint32_t)kSlotBytes), "l"(image + ((size_t)r * S + c) * kSlotStride),
                                        "r"((uint32_t)kSlotBytes), "r"(BAR(kSFull + slot)) : "memory");
                         ++issued;
                         if (++slot == (uint32_t)kSplitRing) { slot = 0; par ^= 1u; }

@@ -63,6 +63,13 @@ constexpr int kOffFlags = kOffBars + 256;                             // per row
 constexpr int kSmemBytes = kOffFlags + 512;
 constexpr int kDeferMinSlots = 6;                                     // chunks a stage needs for its issuers to take the statistics
 
+// Chunks a stage needs for the chain with 8-bit corrections, which is for contiguous groups: it is a tenth faster on
+// values (262144 vectors, 2048 codes: 2520 -> 2270 us; 524288, 1024 codes: 3140 -> 2840; 512 codes: 1950 -> 2020), but
+// on keys, which strided groups are for, outlier channels leave 2.1 % of the rows and stages with more than one
+// candidate instead of 0.1 %, and their exact comparison costs more than the steps saved (1M vectors, 1024
+// codes: 6300 -> 6690).
+constexpr int kEightMinSlots = 8;
+
 // barrier slots
 constexpr int kBarFull = 0, kBarEmpty = kRing, kBarAReady = 2 * kRing, kBarAccFull = 2 * kRing + kTiles,
               kBarAccFree = 2 * kRing + 2 * kTiles, kNumBars = 2 * kRing + 3 * kTiles;
@@ -94,6 +101,8 @@ struct Work {
 
 // 16 warps, launched with 128 registers per thread; the four role warps then keep 40 each and the
 // twelve epilogue warps take 152 (4 x 40 + 12 x 152 = 1984 of the 2048 per lane).
+// EIGHT: the small products in 8 bits (issue_chain8).
+template <bool EIGHT>
 __global__ void __launch_bounds__(kThreads, 1)
 encode_tensor_kernel(const Params p)
 {
@@ -114,7 +123,7 @@ encode_tensor_kernel(const Params p)
     }
     const int my_passes = work.rounds;
     const StageParams *sp = reinterpret_cast<const StageParams *>(p.prepared + kPreparedParamsOffset);
-    const uint8_t *image = p.prepared + kPreparedImageOffset;
+    const uint8_t *image = p.prepared + kPreparedImageOffset + (EIGHT ? kSlotTail : 0);
     const uint32_t bar0 = smem_u32(bars);
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
@@ -162,7 +171,7 @@ encode_tensor_kernel(const Params p)
                 if (!ok) break;
                 mbar_expect_tx(BAR(kBarFull + slot), kSlotBytes);
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(smem_u32(smem + kOffB) + slot * (uint32_t)kSlotBytes), "l"(image + (size_t)rs * kSlotBytes),
+                             ::"r"(smem_u32(smem + kOffB) + slot * (uint32_t)kSlotBytes), "l"(image + (size_t)rs * kSlotStride),
                                "r"((uint32_t)kSlotBytes), "r"(BAR(kBarFull + slot)) : "memory");
                 if (++rs == per_pass) rs = 0;
                 if (++slot == (uint32_t)kRing) { slot = 0; empty_par ^= 1u; }
@@ -217,7 +226,8 @@ encode_tensor_kernel(const Params p)
                 // epilogue's wait for it runs out with no copy or MMA of this CTA still in flight)
                 if (p.drop_last_chain && t == 0 && q == total - 1) break;
                 if (elect_one()) {
-                    issue_chain(acc, a0, bd, ones_desc);
+                    if (EIGHT) issue_chain8(acc, a0, bd, ones_desc);
+                    else issue_chain(acc, a0, bd, ones_desc);
                     mma_commit(bar_acc);
                     mma_commit(BAR(kBarEmpty + slot));
                 }
@@ -291,7 +301,9 @@ encode_tensor_kernel(const Params p)
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
                 // scaled half-precision copy of the residual -> A operand row; error window of this row
                 uint32_t ab[32];
-                const float zz = split_operand(z, prm.scale, ab);
+                Sweep w;
+                if (EIGHT) split_operand8(z, prm.scale, ab, w.zz, w.ll);
+                else w.zz = split_operand(z, prm.scale, ab);
                 tmem_st32(taddr + 128, ab);
                 tc_fence_before();
                 __syncwarp();
@@ -299,16 +311,15 @@ encode_tensor_kernel(const Params p)
                 // park the float32 residual in shared memory for the sweep
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kRowsPerPass] = z[i];
-                Sweep w;
-                w.win = 2.125f * (prm.a * sqrtf(zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
-                w.zz = zz;
+                if (!EIGHT) w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
                 w.m1 = w.m2 = w.m3 = INFINITY;
                 w.c1 = w.c2 = 0;
 #pragma unroll
                 for (int q = 0; q < 16; ++q) w.d[q] = INFINITY;
                 w.h[0] = w.h[1] = INFINITY;
                 w.bb[0] = w.bb[1] = w.bb[2] = w.bb[3] = INFINITY;
-                const bool force_scan = !(zz < 3.6e9f) || !(w.win < INFINITY);      // (no entry reaches 60000 in half precision)
+                // (no entry reaches 60000 in half precision; none is above 2^14, where 64 times its remainder leaves the 8-bit range)
+                const bool force_scan = EIGHT ? !(w.zz < 2.68e8f) || !(prm.a < INFINITY) : !(w.zz < 3.6e9f) || !(w.win < INFINITY);
 
 #pragma unroll 1
                 for (int c = 0; c < S && ok; ++c) {
@@ -352,7 +363,7 @@ encode_tensor_kernel(const Params p)
                 // the four lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
                 const StageBounds sb = stage_bounds(p.prepared, r);
-                const float lim = threshold(w, m1, sb);
+                const float lim = EIGHT ? threshold8(w, m1, sb) : threshold(w, m1, sb);
                 const Listed in = listed(w, lim);
                 const int j1 = w.c1 * 128 + in.column();
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
@@ -469,13 +480,13 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
-    if (!allow_shared_memory(reinterpret_cast<const void *>(encode_tensor_kernel), kSmemBytes))
-        return RVQ_ERR_LAUNCH;
+    auto kernel = slots_per_stage(s.K) >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw ? encode_tensor_kernel<true> : encode_tensor_kernel<false>;
+    if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,
              stat_sum != nullptr && encode_tensor_deferred_stages(s) > 0 ? 1 : 0};
     const int grid = (int)(tiles < sms ? tiles : sms);        // (fewer tiles than three per SM: one or two in each, not three in some)
-    encode_tensor_kernel<<<grid, kThreads, kSmemBytes, stream>>>(p);
+    kernel<<<grid, kThreads, kSmemBytes, stream>>>(p);
     return check_launch();
 }
 

@@ -8,21 +8,27 @@
 // product then rivals the gap between the best codewords), so both operands
 // are split into a half-precision head and a half-precision remainder and the
 // contraction keeps the three leading products:
-//     z.e  ~  z_hi.e_hi + z_hi.e_lo + z_lo.e_hi        (error ~ 2^-22 |z||e|).
+//     z.e  ~  z_hi.e_hi + z_hi.e_lo + z_lo.e_hi        (error ~ 2^-22 |z||e|),
+// or, where a sweep is long enough to make up for more rows with several candidates, the two small products in
+// 8 bits (e4m3, twice the depth per step; error ~ 2^-15 |z||e|):
+//     z.e  ~  z_hi.e_hi + [64 z_lo]_8.[e / 64]_8 + [z_hi / 64]_8.[64 e_lo]_8.
 // Per stage r the block holds
 //   - a power-of-two scale 2^k chosen so that the largest scaled squared norm
 //     is about 2^13 (keeps the operands out of the half-precision subnormals);
-//   - the B operand image of tcgen05.mma: for every slot of 128 codewords nine
-//     "cells" (8 halves = 16 bytes per codeword per cell, K-major, no swizzle):
-//     cell 0 holds the scaled squared norm split into three halves (hi, lo, lo2)
-//     then zeros, cells 1-4 hold -2 e_hi, cells 5-8 hold -2 e_lo.  The A operand
-//     carries (Z_hi, Z_lo, 1 1 1 0 ... 0), and seven K=16 steps pair the cells so
-//     that the accumulator is the score (the norm's step takes cells 0 and 1, and
-//     A is zero where cell 1 stands);
+//   - the B operand image of tcgen05.mma: for every slot of 128 codewords thirteen
+//     "cells" (16 bytes per codeword per cell, K-major, no swizzle): cells 0-3
+//     hold -2 e_lo (8 halves each), cell 4 the scaled squared norm split into
+//     three halves (hi, lo, lo2) then zeros, cells 5-8 hold -2 e_hi, cells 9-10
+//     -2 e / 64 and cells 11-12 -2 * 64 e_lo (16 e4m3 each).  The A operand
+//     carries Z_hi and Z_lo, or Z_hi and the 8-bit 64 Z_lo and Z_hi / 64, and (1 1
+//     1 0 ... 0) for the norm, whose K = 16 step takes cells 4 and 5 (A is zero
+//     where cell 5 stands): seven or five steps make the accumulator the score;
 //   - the float32 codewords again, in blocks of 128 (prepared.cuh), for the encoder of a few vectors;
 //   - two numbers (a, b) such that |score error| <= a * ||Z|| + b, from the
 //     actual rounding errors of this codebook (see prepare_finish_kernel).
 #include "prepared.cuh"
+
+#include <cuda_fp8.h>
 
 namespace rvq {
 
@@ -221,9 +227,10 @@ prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *_
     const int slot = blockIdx.x, jj = threadIdx.x;
     const int j = slot * kSlotCodewords + jj;            // padded codeword index
     const float scale = sp[r].scale;
-    uint8_t *base = image + ((size_t)r * slots_per_stage(s.K) + slot) * kSlotBytes;
-    __half cell[kSlotCells][8];
-    for (int c = 0; c < kSlotCells; ++c)
+    uint8_t *base = image + ((size_t)r * slots_per_stage(s.K) + slot) * kSlotStride;
+    __half cell[9][8];                                    // cells 0-8
+    __align__(16) uint8_t cell8[4][16] = {};              // cells 9-12
+    for (int c = 0; c < 9; ++c)
         for (int i = 0; i < 8; ++i) cell[c][i] = __float2half_rn(0.0f);
     float emax = 0.f, eerr = 0.f, nmax = 0.f, elomax = 0.f;
     if (j < s.K) {
@@ -235,23 +242,25 @@ prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *_
             const double hv = (double)__half2float(hi);
             const __half lo = __double2half(es - hv);
             const double lv = (double)__half2float(lo);
-            cell[1 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(hi));      // exact doubling
-            cell[5 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(lo));
+            cell[5 + (i >> 3)][i & 7] = __float2half_rn(-2.0f * __half2float(hi));      // exact doubling
+            cell[i >> 3][i & 7] = __float2half_rn(-2.0f * __half2float(lo));
+            cell8[i >> 4][i & 15] = __nv_cvt_float_to_fp8((float)(es * (-2.0 / 64.0)), __NV_SATFINITE, __NV_E4M3);
+            cell8[2 + (i >> 4)][i & 15] = __nv_cvt_float_to_fp8((float)((es - hv) * (-2.0 * 64.0)), __NV_SATFINITE, __NV_E4M3);
             n2 += es * es; l2 += lv * lv; d2 += (es - hv - lv) * (es - hv - lv);
         }
         const __half n_hi = __double2half(n2);
         const double r1 = n2 - (double)__half2float(n_hi);
         const __half n_lo = __double2half(r1);
         const double r2 = r1 - (double)__half2float(n_lo);
-        cell[0][0] = n_hi; cell[0][1] = n_lo; cell[0][2] = __double2half(r2);
+        cell[4][0] = n_hi; cell[4][1] = n_lo; cell[4][2] = __double2half(r2);
         // round the maxima up so that the bound stays a bound in float32
         emax = __double2float_ru(sqrt(n2)); eerr = __double2float_ru(sqrt(d2));
         nmax = __double2float_ru(n2); elomax = __double2float_ru(sqrt(l2));
     } else {
-        cell[0][0] = __float2half_rn(60000.0f);           // padding never wins
+        cell[4][0] = __float2half_rn(60000.0f);           // padding never wins
     }
-    for (int c = 0; c < kSlotCells; ++c)
-        *reinterpret_cast<uint4 *>(base + ((size_t)c * kSlotCodewords + jj) * 16) = *reinterpret_cast<const uint4 *>(cell[c]);
+    for (int c = 0; c < 13; ++c)
+        *reinterpret_cast<uint4 *>(base + ((size_t)c * kSlotCodewords + jj) * 16) = c < 9 ? *reinterpret_cast<const uint4 *>(cell[c]) : *reinterpret_cast<const uint4 *>(cell8[c - 9]);
     if (blocks) {
         // the float32 block of this slot, piece by piece
         float4 *o = blocks + ((size_t)r * slots_per_stage(s.K) + slot) * (kFloatBlockBytes / 16) + jj;

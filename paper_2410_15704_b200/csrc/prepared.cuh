@@ -8,8 +8,13 @@ namespace rvq {
 
 constexpr uint32_t kPreparedMagic = 0x52565133u;
 constexpr int kSlotCodewords = 128;                       // codewords per operand slot
-constexpr int kSlotCells = 9;                             // norm (1), hi (4), lo (4) cells of 8 halves
-constexpr int kSlotBytes = kSlotCells * kSlotCodewords * 16;   // 18432
+// Operand slot of 128 codewords: thirteen cells of 16 bytes per codeword -- remainders as halves (4 cells), norm (1),
+// heads (4), corrections in 8 bits (4).  An encoder copies nine of them: the first nine (remainders, norm, heads) or
+// the last nine (norm, heads, corrections).
+constexpr int kCellBytes = kSlotCodewords * 16;           // 2048
+constexpr int kSlotStride = 13 * kCellBytes;              // 26624
+constexpr int kSlotBytes = 9 * kCellBytes;                // 18432, as copied
+constexpr int kSlotTail = 4 * kCellBytes;                 // where the last nine cells begin
 constexpr size_t kPreparedParamsOffset = 256;             // StageParams[16]
 constexpr size_t kPreparedMaximaOffset = 512;             // StageMaxima[16]
 constexpr size_t kPreparedPartialsOffset = 768;           // StagePartial[16 stages][kPrepareParts], scratch of the prepare step
@@ -91,7 +96,7 @@ __host__ __device__ inline bool float_blocks_prepared(const Shape &s)
 }
 __host__ __device__ inline size_t encode_image_bytes(const Shape &s)
 {
-    return s.gd == 32 ? (size_t)s.R * ((s.K + kSlotCodewords - 1) / kSlotCodewords) * kSlotBytes : 0;
+    return s.gd == 32 ? (size_t)s.R * ((s.K + kSlotCodewords - 1) / kSlotCodewords) * kSlotStride : 0;
 }
 
 __host__ __device__ inline size_t decode_section_offset(const Shape &s)

@@ -63,3 +63,19 @@ def test_against_the_oracle():
     rvq.rvq_encode(cfg, x.cuda(), 24, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
     codes = b.codes.view(torch.int16).cpu().numpy().view(np.uint16).reshape(24, 4, 8).astype(np.int32)
     assert_codes_match(x.numpy(), codes, cb, 0)
+
+
+@pytest.mark.parametrize("n,K,R,scale", [(9477, 1024, 8, 1.0), (10007, 2048, 4, 1.0), (9480, 1030, 2, 1e-3), (9500, 1024, 2, 3e4)])
+def test_eight_bit_corrections(n, K, R, scale):
+    """Contiguous groups, eight or more chunks, more than one tile per SM: ordinary codebooks, and ones whose
+    stages' scales lie far apart (rows beyond the 8-bit range take the full scan)."""
+    x, cb = batch(n, 128, K, R, "f32", n)
+    cb[0, ::7] *= 8.0
+    cb[-1] *= scale
+    cfg = rvq.make_config(128, 32, 0, R, K, 16, rvq.F32, 0)
+    b = rvq.alloc_buffers(cfg, n, cb)
+    exact = torch.empty_like(b.codes)
+    rvq.rvq_encode(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
+    torch.cuda.synchronize()
+    assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
