@@ -4,10 +4,11 @@
 // times its deviation).  The decoded keys and values never reach global memory:
 //   1. scores   s[t][h][j] = sum_c q[h J + j][c] * rot(k^[t][h])[c]        (att_scores_kernel)
 //   2. maxima   m[h][j] = max_t scale * s[t][h][j]                          (att_max_kernel)
-//   3. values   acc[h][j][c] = sum_t exp(scale s - m) v^[t][h][c], and the sum of the weights
-//                                                                          (att_values_kernel)
-//   4. out[h J + j][c] = acc / weights                                      (att_finish_kernel)
-// Steps 1 and 3 are the table decoder's gather: a CTA keeps the float32 channels of one slice of
+//   3. weights  w[t][h][j] = exp(scale s - m) times the value's deviation, and the sums of the weights
+//                                                                          (att_weights_kernel)
+//   4. values   acc[h][j][c] = sum_t w[t][h][j] * (codewords of v^[t][h])[c] (att_values_kernel)
+//   5. out[h J + j][c] = acc / weights                                      (att_finish_kernel)
+// Steps 1 and 4 are the table decoder's gather: a CTA keeps the float32 channels of one slice of
 // four codeword elements for all codes and stages in shared memory (16 bytes per code and stage,
 // stage order rotated by lane so that a quarter warp's reads never collide), a warp takes one
 // token (its 32 lanes are the 8 kv heads x 4 groups, so a thread keeps one (head, group) for the
@@ -38,12 +39,13 @@ __device__ __forceinline__ int att_channel(int g, int e)
     return LAYOUT == RVQ_GROUP_STRIDED ? 4 * e + g : 32 * g + e;
 }
 
-// table[code][stage] = the four float32 channels of this slice; absent stages are zero
-template <int LAYOUT, int ROPE>
+// table[code][8 slots] = the four float32 channels of this slice: stage r in slot r, and with up to four stages (STEPS
+// 4) once more in slot r + 4, so that eight lanes still read eight bank groups in half the steps; absent stages are zero
+template <int LAYOUT, int ROPE, int STEPS>
 __device__ __forceinline__ void att_fill_table(const Shape &s, const float *__restrict__ cb, int sl, float4 *table)
 {
     for (int t = threadIdx.x; t < s.K * 8; t += kAttThreads) {
-        const int r = t & 7, j = t >> 3;
+        const int r = t & (STEPS - 1), j = t >> 3;
         float4 e = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (r < s.R) {
             const float *src = cb + ((size_t)r * s.K + j) * 32;
@@ -59,8 +61,20 @@ __device__ __forceinline__ void att_fill_table(const Shape &s, const float *__re
     }
 }
 
-// The codes of group row `row` (= 4 * head vector + group) as four words, stage r in half r; the
-// deviation of its head vector.
+// Where the codes of this lane's group are in a head vector's words, and how they are cut out.
+struct AttCodes {
+    int form;                     // 0: eight 16-bit codes; 1: fewer of them; 2: packed codes
+    uint32_t first, shift;        // word and bit of the group's first code
+};
+__device__ __forceinline__ AttCodes att_codes(const Shape &s, int g)
+{
+    AttCodes a;
+    a.form = s.bits == 16 ? (s.R == 8 ? 0 : 1) : 2;           // (codes of 1792 values: at most 88 bits, and 31 before them)
+    a.first = (uint32_t)(g * s.R * s.bits) >> 5;
+    a.shift = (uint32_t)(g * s.R * s.bits) & 31u;
+    return a;
+}
+// The words of a group row with its codes, as they are stored, and the deviation of its head vector.
 struct AttRow {
     uint32_t c0, c1, c2, c3;
     uint16_t sd;
@@ -71,7 +85,7 @@ __device__ __forceinline__ int att_position(const int32_t *__restrict__ position
     if (token >= tokens) return 0;
     return position ? __ldg(position + token) : (int)token;
 }
-__device__ __forceinline__ void att_fetch(const Shape &s, const void *__restrict__ codes,
+__device__ __forceinline__ void att_fetch(const Shape &s, const AttCodes &ac, const void *__restrict__ codes,
                                           const uint16_t *__restrict__ std16, uint32_t token, uint32_t tokens, int lane,
                                           AttRow &a)
 {
@@ -81,21 +95,47 @@ __device__ __forceinline__ void att_fetch(const Shape &s, const void *__restrict
     const uint32_t v = token * 8u + (uint32_t)(lane >> 2);    // (the launcher keeps tokens * 32 below 2^31)
     const int g = lane & 3;
     a.sd = __ldg(std16 + v);
-    if (s.bits == 16 && s.R == 8) {
+    if (ac.form == 0) {
         const uint4 c = __ldg(reinterpret_cast<const uint4 *>(codes) + (v * 4u + (uint32_t)g));
         a.c0 = c.x; a.c1 = c.y; a.c2 = c.z; a.c3 = c.w;
-    } else {
-        const uint8_t *vec = reinterpret_cast<const uint8_t *>(codes) + (size_t)v * s.code_bytes;
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-            if (r < s.R) w[r >> 1] |= read_code(vec, g * s.R + r, s.bits, s.code_bytes) << (16 * (r & 1));
-        a.c0 = w[0]; a.c1 = w[1]; a.c2 = w[2]; a.c3 = w[3];
+        return;
     }
+    const uint8_t *vec = reinterpret_cast<const uint8_t *>(codes) + (size_t)v * s.code_bytes;
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(vec) + ac.first;
+    const uint32_t left = (uint32_t)s.code_bytes / 4u - ac.first;
+    a.c0 = __ldg(words);
+    if (left > 1) a.c1 = __ldg(words + 1);
+    if (left > 2) a.c2 = __ldg(words + 2);
+    if (left > 3) a.c3 = __ldg(words + 3);
 }
 
-// Sum over the stages of the four channels of this thread's row: eight 16-byte reads, stage
-// (rot + k) & 7 at step k.  Codes past the codebook are read as code 0 and counted.
+// The codes of a row as four words, stage r in half r, absent stages 0.
+__device__ __forceinline__ void att_cut(const Shape &s, const AttCodes &ac, AttRow &a)
+{
+    if (ac.form == 0) return;
+    uint32_t w0 = __funnelshift_r(a.c0, a.c1, ac.shift), w1 = __funnelshift_r(a.c1, a.c2, ac.shift);
+    uint32_t w2 = __funnelshift_r(a.c2, a.c3, ac.shift), w3 = a.c3 >> ac.shift;
+    if (ac.form == 2) {
+        // two codes from the low end at a time, then the window moves on by two codes
+        const uint32_t mask = (1u << s.bits) - 1u, up = 16u - (uint32_t)s.bits, two = 2u * (uint32_t)s.bits;
+        auto halves = [&](uint32_t w) { return (w & mask) | ((w << up) & (mask << 16)); };
+        a.c0 = halves(w0);
+        w0 = __funnelshift_r(w0, w1, two); w1 = __funnelshift_r(w1, w2, two); w2 = __funnelshift_r(w2, w3, two);
+        a.c1 = halves(w0);
+        w0 = __funnelshift_r(w0, w1, two); w1 = __funnelshift_r(w1, w2, two);
+        a.c2 = halves(w0);
+        w0 = __funnelshift_r(w0, w1, two);
+        a.c3 = halves(w0);
+    } else {
+        a.c0 = w0; a.c1 = w1; a.c2 = w2; a.c3 = w3;
+    }
+    auto keep = [&](uint32_t &w, int r) { w = s.R > r + 1 ? w : s.R > r ? w & 0xFFFFu : 0u; };
+    keep(a.c0, 0); keep(a.c1, 2); keep(a.c2, 4); keep(a.c3, 6);
+}
+
+// Sum over the stages of the four channels of this thread's row: STEPS 16-byte reads, stage
+// (rot + k) mod STEPS at step k.  Codes past the codebook are read as code 0 and counted.
+template <int STEPS>
 __device__ __forceinline__ void att_gather(const AttRow &a, uint32_t K, uint32_t rot, uint32_t smem_table,
                                            float (&acc)[4], uint32_t &bad)
 {
@@ -113,10 +153,14 @@ __device__ __forceinline__ void att_gather(const AttRow &a, uint32_t K, uint32_t
             }
         }
     }
-    // rotate the 8 halves left by `rot` so that step k finds its code at a fixed place
-    if (rot & 4u) { const uint32_t t0 = c0, t1 = c1; c0 = c2; c1 = c3; c2 = t0; c3 = t1; }
-    if (rot & 2u) { const uint32_t t0 = c0; c0 = c1; c1 = c2; c2 = c3; c3 = t0; }
-    if (rot & 1u) {
+    // rotate the halves left by `rot` so that step k finds its code at a fixed place
+    if (STEPS == 4) {
+        if (rot & 2u) { const uint32_t t0 = c0; c0 = c1; c1 = t0; }
+        if (rot & 1u) { const uint32_t b0 = __funnelshift_r(c0, c1, 16); c1 = __funnelshift_r(c1, c0, 16); c0 = b0; }
+    }
+    if (STEPS == 8 && (rot & 4u)) { const uint32_t t0 = c0, t1 = c1; c0 = c2; c1 = c3; c2 = t0; c3 = t1; }
+    if (STEPS == 8 && (rot & 2u)) { const uint32_t t0 = c0; c0 = c1; c1 = c2; c2 = c3; c3 = t0; }
+    if (STEPS == 8 && (rot & 1u)) {
         const uint32_t b0 = __funnelshift_r(c0, c1, 16), b1 = __funnelshift_r(c1, c2, 16);
         const uint32_t b2 = __funnelshift_r(c2, c3, 16), b3 = __funnelshift_r(c3, c0, 16);
         c0 = b0; c1 = b1; c2 = b2; c3 = b3;
@@ -124,10 +168,11 @@ __device__ __forceinline__ void att_gather(const AttRow &a, uint32_t K, uint32_t
     const uint32_t cw[4] = {c0, c1, c2, c3};
     acc[0] = acc[1] = acc[2] = acc[3] = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < STEPS; ++k) {
         const uint32_t w = cw[k >> 1];
         const uint32_t line = (k & 1) ? ((w >> 9) & (0xFFFFu << 7)) : ((w << 7) & (0xFFFFu << 7));
-        const uint32_t addr = smem_table + (line | (((rot + k) & 7u) * 16u));
+        const uint32_t slot = STEPS == 8 ? (rot + k) & 7u : ((rot + k) & 3u) | (rot & 4u);
+        const uint32_t addr = smem_table + (line | (slot * 16u));
         float f0, f1, f2, f3;
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f0), "=f"(f1), "=f"(f2), "=f"(f3) : "r"(addr));
         acc[0] += f0; acc[1] += f1; acc[2] += f2; acc[3] += f3;
@@ -166,7 +211,7 @@ __device__ __forceinline__ void att_cos_sin(const float2 *__restrict__ cos_sin, 
 }
 
 // Step 1.  ROPE 0: keys as stored; 1: pairs (k, k + 64); 2: pairs (2k, 2k + 1).
-template <int LAYOUT, int ROPE, int J>
+template <int LAYOUT, int ROPE, int J, int STEPS>
 __global__ void __launch_bounds__(kAttThreads, 1)
 att_scores_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t tokens,
                   const float *__restrict__ cb, const float *__restrict__ q, const int32_t *__restrict__ position,
@@ -177,7 +222,7 @@ att_scores_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
     if ((int)blockIdx.x >= parts * kAttSlices) return;
     const int sl = blockIdx.x % kAttSlices, part = blockIdx.x / kAttSlices;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = lane >> 2, g = lane & 3;
-    att_fill_table<LAYOUT, ROPE>(s, cb, sl, reinterpret_cast<float4 *>(smem));
+    att_fill_table<LAYOUT, ROPE, STEPS>(s, cb, sl, reinterpret_cast<float4 *>(smem));
     // the query values that meet this thread's four channels, for the J query heads of its kv head
     float qr[J][4];
 #pragma unroll
@@ -192,21 +237,23 @@ att_scores_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
     // are asked for while this one is gathered, and the position of the token after that (the address
     // of the (cos, sin) values hangs on it).
     const uint32_t T = (uint32_t)tokens, step = (uint32_t)parts * 32u, t0 = (uint32_t)part * 32u + (uint32_t)warp;
+    const AttCodes ac = att_codes(s, lane & 3);
     AttRow next;
     float cn[4], sn[4];
-    att_fetch(s, codes, std16, t0, T, lane, next);
+    att_fetch(s, ac, codes, std16, t0, T, lane, next);
     att_cos_sin<LAYOUT, ROPE>(cos_sin, positions, att_position(position, t0, T), sl, g, cn, sn);
     int pos_next = ROPE != 0 ? att_position(position, t0 + step, T) : 0;
     for (uint32_t t = t0; t < T; t += step) {
-        const AttRow cur = next;
+        AttRow cur = next;
         float cc[4], ss[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) { cc[i] = cn[i]; ss[i] = sn[i]; }
         att_cos_sin<LAYOUT, ROPE>(cos_sin, positions, pos_next, sl, g, cn, sn);
         if (ROPE != 0) pos_next = att_position(position, t + 2 * step, T);
-        att_fetch(s, codes, std16, t + step, T, lane, next);
+        att_fetch(s, ac, codes, std16, t + step, T, lane, next);
         float v[4];
-        att_gather(cur, (uint32_t)s.K, (uint32_t)lane & 7u, smem_table, v, bad);
+        att_cut(s, ac, cur);
+        att_gather<STEPS>(cur, (uint32_t)s.K, (uint32_t)lane & 7u, smem_table, v, bad);
         const float sd = __half2float(__ushort_as_half(cur.sd));
 #pragma unroll
         for (int i = 0; i < 4; ++i) v[i] *= sd;
@@ -243,16 +290,22 @@ att_scores_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
             a = fmaf(v[1], qr[j][1], a);
             a = fmaf(v[2], qr[j][2], a);
             a = fmaf(v[3], qr[j][3], a);
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, 1);
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, 2);
             part_s[j] = a;
         }
-        if (g == 0) {
-            float *dst = scores + (size_t)(t * 8u + (uint32_t)h) * J;
-            if (J == 4) atomicAdd(reinterpret_cast<float4 *>(dst), make_float4(part_s[0], part_s[1], part_s[J - 2], part_s[J - 1]));
-            else if (J == 2) atomicAdd(reinterpret_cast<float2 *>(dst), make_float2(part_s[0], part_s[J - 1]));
-            else atomicAdd(dst, part_s[0]);
+        // the sums over the four groups are shared out: lane g ends with query head g (with two heads: g & 1), so that a
+        // warp's reductions are consecutive floats
+        float total;
+        if (J == 4) {
+            const float keep0 = (g & 1) ? part_s[1 % J] : part_s[0], keep1 = (g & 1) ? part_s[3 % J] : part_s[2 % J];
+            const float send0 = (g & 1) ? part_s[0] : part_s[1 % J], send1 = (g & 1) ? part_s[2 % J] : part_s[3 % J];
+            const float pair0 = keep0 + __shfl_xor_sync(0xFFFFFFFFu, send0, 1), pair1 = keep1 + __shfl_xor_sync(0xFFFFFFFFu, send1, 1);
+            total = ((g & 2) ? pair1 : pair0) + __shfl_xor_sync(0xFFFFFFFFu, (g & 2) ? pair0 : pair1, 2);
+        } else {
+            total = J == 2 && (g & 1) ? part_s[J - 1] : part_s[0];
+            total += __shfl_xor_sync(0xFFFFFFFFu, J == 2 && !(g & 1) ? part_s[J - 1] : part_s[0], 1);
+            total += __shfl_xor_sync(0xFFFFFFFFu, total, 2);
         }
+        if (g < J) atomicAdd(scores + (size_t)(t * 8u + (uint32_t)h) * J + g, total);
     }
     if (bad && st && sl == 0) atomicAdd(&st->bad_codes, bad);
 }
@@ -286,82 +339,92 @@ att_max_kernel(const float *__restrict__ scores, int64_t tokens, int columns, fl
     }
 }
 
-// Step 3.
-template <int LAYOUT, int J>
+// Step 3: every score becomes its weight times its token's deviation, exp(scale s - m) = 2^(s * scale log2(e) -
+// m log2(e)), and the weights are summed; once per token here instead of in each of the 32 rows and slices of step 4.
+__global__ void __launch_bounds__(kAttThreads)
+att_weights_kernel(float *__restrict__ scores, const uint16_t *__restrict__ std16, uint32_t tokens, int columns, int per_head_log,
+                   float scale, const uint32_t *__restrict__ m_ord, float *__restrict__ weight_sum)
+{
+    __shared__ float part[kAttThreads];
+    constexpr float kLog2e = 1.4426950408889634f;
+    const int col = threadIdx.x % columns, rows_per_block = kAttThreads / columns;
+    const float sl2 = scale * kLog2e, mneg = -att_unordered(m_ord[col]) * kLog2e;
+    float sum = 0.0f;
+    for (uint32_t t = blockIdx.x * rows_per_block + threadIdx.x / columns; t < tokens; t += gridDim.x * rows_per_block) {
+        const float w = exp2f(fmaf(scores[(size_t)t * columns + col], sl2, mneg));
+        sum += w;
+        scores[(size_t)t * columns + col] = w * __half2float(__ushort_as_half(__ldg(std16 + (size_t)t * 8 + (col >> per_head_log))));
+    }
+    part[threadIdx.x] = sum;
+    __syncthreads();
+    if ((int)threadIdx.x < columns) {
+        for (int r = 1; r < rows_per_block; ++r) sum += part[r * columns + threadIdx.x];
+        atomicAdd(weight_sum + col, sum);
+    }
+}
+
+// Step 4.
+template <int LAYOUT, int J, int STEPS>
 __global__ void __launch_bounds__(kAttThreads, 1)
 att_values_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t tokens,
-                  const float *__restrict__ cb, const float *__restrict__ scores, const uint32_t *__restrict__ m_ord,
-                  float scale, float *__restrict__ out_acc, float *__restrict__ weight_sum, rvq_status *st)
+                  const float *__restrict__ cb, const float *__restrict__ weights, float *__restrict__ out_acc, rvq_status *st)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     const int parts = gridDim.x / kAttSlices;
     if ((int)blockIdx.x >= parts * kAttSlices) return;
     const int sl = blockIdx.x % kAttSlices, part = blockIdx.x / kAttSlices;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = lane >> 2;
-    att_fill_table<LAYOUT, 0>(s, cb, sl, reinterpret_cast<float4 *>(smem));
-    // exp(scale s - m) = 2^(s * scale log2(e) - m log2(e))
-    constexpr float kLog2e = 1.4426950408889634f;
-    const float sl2 = scale * kLog2e;
-    __shared__ float mneg_s[32];                             // -m log2(e) per query head (read back per token: registers are short)
-    if (threadIdx.x < 8 * J) mneg_s[threadIdx.x] = -att_unordered(m_ord[threadIdx.x]) * kLog2e;
+    att_fill_table<LAYOUT, 0, STEPS>(s, cb, sl, reinterpret_cast<float4 *>(smem));
     __syncthreads();
     const uint32_t smem_table = (uint32_t)__cvta_generic_to_shared(smem);
     uint32_t bad = 0;
-    float acc[J][4], wsum[J];
+    float acc[J][4];
 #pragma unroll
-    for (int j = 0; j < J; ++j) { wsum[j] = 0.0f; acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f; }
+    for (int j = 0; j < J; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
     const uint32_t T = (uint32_t)tokens, step = (uint32_t)parts * 32u;
+    const AttCodes ac = att_codes(s, lane & 3);
     AttRow next;
-    att_fetch(s, codes, std16, (uint32_t)part * 32u + (uint32_t)warp, T, lane, next);
+    att_fetch(s, ac, codes, std16, (uint32_t)part * 32u + (uint32_t)warp, T, lane, next);
     for (uint32_t t = (uint32_t)part * 32u + (uint32_t)warp; t < T; t += step) {
-        const AttRow cur = next;
-        // this token's scores, asked for before the gather
+        AttRow cur = next;
+        // this token's weights, asked for before the gather
         float sc[J];
         {
-            const float *src = scores + (size_t)(t * 8u + (uint32_t)h) * J;
+            const float *src = weights + (size_t)(t * 8u + (uint32_t)h) * J;
             if (J == 4) { const float4 f = __ldg(reinterpret_cast<const float4 *>(src)); sc[0] = f.x; sc[1] = f.y; sc[J - 2] = f.z; sc[J - 1] = f.w; }
             else if (J == 2) { const float2 f = __ldg(reinterpret_cast<const float2 *>(src)); sc[0] = f.x; sc[J - 1] = f.y; }
             else sc[0] = __ldg(src);
         }
-        att_fetch(s, codes, std16, t + step, T, lane, next);
+        att_fetch(s, ac, codes, std16, t + step, T, lane, next);
         float v[4];
-        att_gather(cur, (uint32_t)s.K, (uint32_t)lane & 7u, smem_table, v, bad);
-        const float sd = __half2float(__ushort_as_half(cur.sd));
+        att_cut(s, ac, cur);
+        att_gather<STEPS>(cur, (uint32_t)s.K, (uint32_t)lane & 7u, smem_table, v, bad);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] *= sd;
+        for (int j = 0; j < J; ++j)
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const float w = exp2f(fmaf(sc[j], sl2, mneg_s[h * J + j]));
-            wsum[j] += w;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(w, v[i], acc[j][i]);
-        }
+            for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(sc[j], v[i], acc[j][i]);
     }
     // sums over the CTA's warps (a lane is the same (head, group) in all of them), then one
     // reduction per value into global memory; the table's memory is free now
     __syncthreads();
-    float *red = reinterpret_cast<float *>(smem);            // [5 J][32 warps][32 lanes]
+    float *red = reinterpret_cast<float *>(smem);            // [4 J][32 warps][32 lanes]
 #pragma unroll
     for (int j = 0; j < J; ++j) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) red[((j * 5 + i) * 32 + warp) * 32 + lane] = acc[j][i];
-        red[((j * 5 + 4) * 32 + warp) * 32 + lane] = wsum[j];
+        for (int i = 0; i < 4; ++i) red[((j * 4 + i) * 32 + warp) * 32 + lane] = acc[j][i];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < 5 * J * 32; idx += kAttThreads) {
-        const int ln = idx & 31, what = idx >> 5, j = what / 5, i = what % 5;
+    for (int idx = threadIdx.x; idx < 4 * J * 32; idx += kAttThreads) {
+        const int ln = idx & 31, what = idx >> 5, j = what / 4, i = what % 4;
         float a = 0.0f;
         for (int w = 0; w < 32; ++w) a += red[(what * 32 + w) * 32 + ln];
         const int hh = ln >> 2, gg = ln & 3;
-        if (i < 4)
-            atomicAdd(out_acc + (size_t)(hh * J + j) * 128 + att_channel<LAYOUT>(gg, 4 * sl + i), a);
-        else if (sl == 0 && gg == 0)
-            atomicAdd(weight_sum + hh * J + j, a);
+        atomicAdd(out_acc + (size_t)(hh * J + j) * 128 + att_channel<LAYOUT>(gg, 4 * sl + i), a);
     }
     if (bad && st && sl == 0) atomicAdd(&st->bad_codes, bad);
 }
 
-// Step 4.
+// Step 5.
 __global__ void att_finish_kernel(const float *__restrict__ out_acc, const float *__restrict__ weight_sum, int heads,
                                   float *__restrict__ out)
 {
@@ -690,21 +753,20 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
     };
     auto values_launch = [&](auto kernel) -> int {
         size_t smem = (size_t)sv.K * 128;
-        const size_t red = (size_t)5 * J * 32 * 32 * 4;
+        const size_t red = (size_t)4 * J * 32 * 32 * 4;
         if (smem < red) smem = red;
         if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
-        kernel<<<parts * kAttSlices, kAttThreads, smem, stream>>>(sv, codes_v, std_v, tokens, cb_v, scores, m_ord, scale,
-                                                                   out_acc, weight_sum, st);
+        kernel<<<parts * kAttSlices, kAttThreads, smem, stream>>>(sv, codes_v, std_v, tokens, cb_v, scores, out_acc, st);
         return check_launch();
     };
-#define RVQ_ATT_S3(LAY, ROPE) (J == 4 ? scores_launch(att_scores_kernel<LAY, ROPE, 4>)                               \
-                               : J == 2 ? scores_launch(att_scores_kernel<LAY, ROPE, 2>)                             \
-                                        : scores_launch(att_scores_kernel<LAY, ROPE, 1>))
+#define RVQ_ATT_S4(LAY, ROPE, JJ) (sk.R <= 4 ? scores_launch(att_scores_kernel<LAY, ROPE, JJ, 4>) : scores_launch(att_scores_kernel<LAY, ROPE, JJ, 8>))
+#define RVQ_ATT_S3(LAY, ROPE) (J == 4 ? RVQ_ATT_S4(LAY, ROPE, 4) : J == 2 ? RVQ_ATT_S4(LAY, ROPE, 2) : RVQ_ATT_S4(LAY, ROPE, 1))
 #define RVQ_ATT_S2(LAY) (rope == 0 ? RVQ_ATT_S3(LAY, 0) : rope == 1 ? RVQ_ATT_S3(LAY, 1) : RVQ_ATT_S3(LAY, 2))
     rc = sk.layout == RVQ_GROUP_CONTIGUOUS ? RVQ_ATT_S2(RVQ_GROUP_CONTIGUOUS) : RVQ_ATT_S2(RVQ_GROUP_STRIDED);
 #undef RVQ_ATT_S2
 #undef RVQ_ATT_S3
+#undef RVQ_ATT_S4
     if (rc != RVQ_OK) return rc;
     {
         int blocks = (int)((tokens * q_heads + kAttThreads - 1) / kAttThreads);
@@ -712,11 +774,14 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
         if (blocks < 1) blocks = 1;
         att_max_kernel<<<blocks, kAttThreads, 0, stream>>>(scores, tokens, q_heads, scale, m_ord);
         if ((rc = check_launch()) != RVQ_OK) return rc;
+        att_weights_kernel<<<blocks, kAttThreads, 0, stream>>>(scores, std_v, (uint32_t)tokens, q_heads, J == 4 ? 2 : J == 2 ? 1 : 0, scale, m_ord, weight_sum);
+        if ((rc = check_launch()) != RVQ_OK) return rc;
     }
-#define RVQ_ATT_V2(LAY) (J == 4 ? values_launch(att_values_kernel<LAY, 4>)                                           \
-                         : J == 2 ? values_launch(att_values_kernel<LAY, 2>) : values_launch(att_values_kernel<LAY, 1>))
+#define RVQ_ATT_V3(LAY, JJ) (sv.R <= 4 ? values_launch(att_values_kernel<LAY, JJ, 4>) : values_launch(att_values_kernel<LAY, JJ, 8>))
+#define RVQ_ATT_V2(LAY) (J == 4 ? RVQ_ATT_V3(LAY, 4) : J == 2 ? RVQ_ATT_V3(LAY, 2) : RVQ_ATT_V3(LAY, 1))
     rc = sv.layout == RVQ_GROUP_CONTIGUOUS ? RVQ_ATT_V2(RVQ_GROUP_CONTIGUOUS) : RVQ_ATT_V2(RVQ_GROUP_STRIDED);
 #undef RVQ_ATT_V2
+#undef RVQ_ATT_V3
     if (rc != RVQ_OK) return rc;
     att_finish_kernel<<<(q_heads * 128 + 255) / 256, 256, 0, stream>>>(out_acc, weight_sum, q_heads, out);
     return check_launch();
