@@ -19,7 +19,7 @@ constexpr size_t kPreparedParamsOffset = 256;             // StageParams[16]
 constexpr size_t kPreparedMaximaOffset = 512;             // StageMaxima[16]
 constexpr size_t kPreparedPartialsOffset = 768;           // StagePartial[16 stages][kPrepareParts], scratch of the prepare step
 constexpr int kPrepareParts = 16;
-constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 16;   // operand image, [R][slots][kSlotBytes]
+constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 16;   // operand image, [R][slots][kSlotStride]
 
 struct PreparedHeader {
     uint32_t magic, R, K, gd, slots;
