@@ -245,8 +245,9 @@ int rvq_encode_stats(const rvq_config *cfg, const void *x, int64_t n, int64_t x_
     if (!batch_count || !batch_sum || !workspace) return RVQ_ERR_BADARG;
     if (!aligned16(batch_sum) || !aligned256(workspace)) return RVQ_ERR_ALIGN;
     if (workspace_bytes < ema_stats_scratch_bytes(s)) return RVQ_ERR_WORKSPACE;
-    if (!encode_tensor_supported(s)) {
-        // shapes without the fused kernel: encode, then the separate statistics pass
+    if (!encode_tensor_supported(s) || encode_small_wanted(s, n) || encode_split_wanted(s, n)) {
+        // shapes without the fused kernel, and batches that the encoders for few tiles take: encode, then the
+        // separate statistics pass
         rc = encode_common(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, stage_energy, status, stream, true);
         if (rc != RVQ_OK) return rc;
         return launch_ema_stats(s, x, n, x_row_stride, codes, codebooks, batch_count, batch_sum, workspace,
@@ -451,9 +452,10 @@ int rvq_learn_step(const rvq_config *cfg, const void *x, int64_t n, int64_t x_ro
     rc = rvq_encode_stats(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, stage_energy, bc, bs,
                           workspace, workspace_bytes, status, stream);
     if (rc != RVQ_OK) return rc;
-    rc = launch_ema_apply(s, bc, bs, codebooks, ema_count, ema_sum, decay, eps, (cudaStream_t)stream);
+    // (this call's kernels follow one another: their launches overlap)
+    rc = launch_ema_apply(s, bc, bs, codebooks, ema_count, ema_sum, decay, eps, (cudaStream_t)stream, true);
     if (rc != RVQ_OK) return rc;
-    return launch_prepare(s, codebooks, prepared, (cudaStream_t)stream);
+    return launch_prepare(s, codebooks, prepared, (cudaStream_t)stream, true);
 }
 
 size_t rvq_kmeans_workspace_bytes(const rvq_config *cfg, int64_t n)

@@ -67,7 +67,7 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
                      const float *cb, float *batch_count, float *batch_sum, void *workspace,
                      rvq_status *st, cudaStream_t stream);
 int launch_ema_apply(const Shape &s, const float *batch_count, const float *batch_sum, float *cb,
-                     float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream);
+                     float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream, bool chained = false);
 size_t ema_workspace_bytes(const Shape &s);     // all of rvq_ema_update's scratch
 size_t ema_stats_scratch_bytes(const Shape &s); // the part rvq_ema_stats itself needs
 size_t kmeans_workspace_bytes(const Shape &s, int64_t n);
@@ -82,7 +82,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
                             int positions, int pairing, float scale, float *out, void *workspace, rvq_status *st,
                             cudaStream_t stream);
 size_t prepared_bytes(const Shape &s);
-int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream);
+int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream, bool chained = false);
 
 // Facts about the current device that a launch needs, looked up once per device (and kernel) and
 // remembered: the three runtime queries they replace were a third of the host's time in a call.
@@ -102,6 +102,31 @@ inline int check_launch()
 }
 
 #ifdef __CUDACC__
+
+// A kernel of a chain: its blocks may be on the chip before the kernel before it in the stream has ended, wait here for
+// that one's end and results, and let the next of the chain come up meanwhile.  Stands first in the kernel, whose inputs
+// are not `__restrict__`: they change while it is on the chip, and its loads must not go through the read-only path.
+__device__ __forceinline__ void follow_previous()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launch of such a kernel; chained: behind another kernel of the same call (a call's first kernel is launched as usual,
+// since what the caller has before it in the stream need not wait for its own predecessors).
+template <typename... P, typename... A>
+inline int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, int threads, cudaStream_t stream, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.stream = stream;
+    cfg.attrs = &attr; cfg.numAttrs = chained ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    const int rc = check_launch();
+    return e == cudaSuccess ? rc : RVQ_ERR_LAUNCH;
+}
 
 // Section 3.1: element i of group g is channel g*gd+i (contiguous groups) or
 // channel i*G+g (channels G = d/d^ apart).

@@ -517,15 +517,14 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
                    const uint8_t *__restrict__ dsec, const float *__restrict__ cb, void *__restrict__ out,
                    int64_t stride, rvq_status *st, uint8_t *table, RopeArgs ra = RopeArgs())
 {
-    static_assert(ROPE == 0 || CH == 8 || F32, "the rotary variant uses 8-channel level slices or 4-channel float32 slices");
-    static_assert(!F32 || (CH == 4 && !SUMMED), "float32 tables: 4-channel slices");
+    static_assert(F32 ? CH == 4 && !SUMMED : CH == 8, "8-channel level slices or 4-channel float32 slices");
     // half-split pairs on strided groups: a slice is two runs of elements 16 apart (CH / 2 each), so that
     // both channels of a pair are in the thread
     constexpr bool SPLIT = ROPE == 1 && LAYOUT == RVQ_GROUP_STRIDED;
     constexpr int NS = 32 / CH;                                  // slices
     if ((int)blockIdx.x >= ((int)gridDim.x / NS) * NS) return;
-    constexpr uint32_t kEntry = F32 ? 16 : 2 * CH;               // bytes per (code, stage); a code's line is 8 entries
-    constexpr int kShift = (F32 || CH == 8) ? 7 : 6;             // log2 of the line's bytes
+    constexpr uint32_t kEntry = 16;                              // bytes per (code, stage); a code's line is 8 entries
+    constexpr int kShift = 7;                                    // log2 of the line's bytes
     const DecodeParams *dp = reinterpret_cast<const DecodeParams *>(dsec);
     const uint32_t slice = blockIdx.x % NS, part = blockIdx.x / NS, parts = gridDim.x / NS;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, rot = lane & 7u;
@@ -666,6 +665,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
         // or (summed levels) plain additions of the table words and two such instructions per channel
         uint32_t acc[CH], even[CH / 2], odd[CH / 2];
         uint64_t fa = 0ull, fb = 0ull;                          // float32 sums, two channels to a register pair
+        float fs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int i = 0; i < CH; ++i) acc[i] = 0u;
 #pragma unroll
@@ -681,13 +681,15 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             if (F32) {
                 uint64_t f01, f23;
                 asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(f01), "=l"(f23) : "r"(a));
-                fa = add_f32x2(fa, f01); fb = add_f32x2(fb, f23);
+                if (ROPE == 0) {
+                    fa = add_f32x2(fa, f01); fb = add_f32x2(fb, f23);
+                } else {                                        // (with the rotation, packed additions are slower)
+                    fs[0] += __uint_as_float((uint32_t)f01); fs[1] += __uint_as_float((uint32_t)(f01 >> 32));
+                    fs[2] += __uint_as_float((uint32_t)f23); fs[3] += __uint_as_float((uint32_t)(f23 >> 32));
+                }
                 continue;
             }
-            if (CH == 8)
-                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[CH / 2 - 2]), "=r"(e[CH / 2 - 1]) : "r"(a));
-            else
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(e[0]), "=r"(e[1]) : "r"(a));
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[CH / 2 - 2]), "=r"(e[CH / 2 - 1]) : "r"(a));
 #pragma unroll
             for (int i = 0; i < CH / 2; ++i) {
                 if (SUMMED) {
@@ -713,7 +715,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             const float facc[4] = {__uint_as_float((uint32_t)fa), __uint_as_float((uint32_t)(fa >> 32)),
                                    __uint_as_float((uint32_t)fb), __uint_as_float((uint32_t)(fb >> 32))};
 #pragma unroll
-            for (int i = 0; i < CH; ++i) o8[i] = F32 ? facc[i & 3] * sd : fmaf((float)acc[i], bs, cs);
+            for (int i = 0; i < CH; ++i) o8[i] = F32 ? (ROPE == 0 ? facc[i & 3] : fs[i & 3]) * sd : fmaf((float)acc[i], bs, cs);
         }
         if (!F32 && fabsf(sd) > exact_above && fabsf(sd) < INFINITY) {
             // too coarse for this deviation: the float32 codewords themselves, summed in stage order
@@ -928,10 +930,10 @@ __device__ __forceinline__ int sample_table_kind(const uint16_t *__restrict__ st
     return (int64_t)far_l * 64 <= samples ? 1 : 2;
 }
 
-// One launch for the quoted shapes (dim 128, depth 8, 16-bit outputs, up to 3072 codes): every CTA
+// One launch for the quoted shapes (dim 128, depth 8, 16-bit outputs, up to 1536 codes): every CTA
 // reads the same sample of deviations and takes the level tables (fast body) or, when the deviations
 // are beyond their reach, the float32 tables; both carve their slices out of whatever grid they get.
-template <int DT, int LCH, int FCH, int LAYOUT, int BITS>
+template <int DT, int LAYOUT, int BITS>
 __global__ void __launch_bounds__(kDecThreads, 1)
 decode_quoted_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t n,
                      const uint8_t *__restrict__ dsec, const float *__restrict__ cb, void *__restrict__ out,
@@ -939,14 +941,12 @@ decode_quoted_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
 {
     extern __shared__ __align__(128) uint8_t table[];
     const int kind = sample_table_kind(std16, n, dsec);
-    if (kind == 2 && FCH == 4)
+    if (kind == 2)
         decode_levels_fast<DT, 4, LAYOUT, BITS, false, 0, true>(s, codes, std16, n, dsec, cb, out, stride, st, table);
-    else if (kind == 2)
-        decode_sliced_body<DT, FCH, true>(s, codes, std16, n, dsec, cb, out, stride, st, table);
     else if (kind == 1)
-        decode_levels_fast<DT, LCH, LAYOUT, BITS, false>(s, codes, std16, n, dsec, cb, out, stride, st, table);
+        decode_levels_fast<DT, 8, LAYOUT, BITS, false>(s, codes, std16, n, dsec, cb, out, stride, st, table);
     else
-        decode_levels_fast<DT, LCH, LAYOUT, BITS, true>(s, codes, std16, n, dsec, cb, out, stride, st, table);
+        decode_levels_fast<DT, 8, LAYOUT, BITS, true>(s, codes, std16, n, dsec, cb, out, stride, st, table);
 }
 
 // The rotary decode of the quoted shapes (dim 128, depth 8, 16-bit outputs, up to 1536 codes, a prepared
@@ -1167,28 +1167,24 @@ int launch_decode_sliced(const Shape &s, const void *codes, const uint16_t *std1
         kernel<<<parts * ns, kDecThreads, smem, stream>>>(s, codes, std16, n, p + off, cb, out, stride, st);
         return check_launch();
     };
-    // the quoted shapes: one launch, tables chosen on the device
-    if (both && s.G == 4 && s.R == 8 && n * 4 < 0x7FFFFFFFLL && (s.bits == 16 || (s.bits >= 10 && s.bits <= 12)) &&
-        !(lch == 4 && fch == 4)) {
+    // the quoted shapes: one launch, tables chosen on the device (more codes, or other depths and outputs, of four
+    // groups go through decode_direct.cu)
+    if (both && s.G == 4 && s.R == 8 && n * 4 < 0x7FFFFFFFLL && s.K <= kDecodeWideK && (s.bits == 16 || s.bits == 10 || s.bits == 11)) {
         auto quoted = [&](auto kernel) -> int {
-            const size_t smem = (size_t)s.K * 16 * lch > (size_t)s.K * 32 * fch ? (size_t)s.K * 16 * lch : (size_t)s.K * 32 * fch;
+            const size_t smem = (size_t)s.K * 128;               // 8 channels of levels or 4 of float32 per code
             int grid = sms < 8 ? 8 : sms;
             if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
                 return RVQ_ERR_LAUNCH;
             kernel<<<grid, kDecThreads, smem, stream>>>(s, codes, std16, n, p + off, cb, out, stride, st);
             return check_launch();
         };
-#define RVQ_Q4(DT, LCH, FCH, LAY)                                                                                   \
-        (s.bits == 16 ? quoted(decode_quoted_kernel<DT, LCH, FCH, LAY, 16>)                                          \
-         : s.bits == 10 ? quoted(decode_quoted_kernel<DT, LCH, FCH, LAY, 10>)                                        \
-         : s.bits == 11 ? quoted(decode_quoted_kernel<DT, LCH, FCH, LAY, 11>)                                        \
-                        : quoted(decode_quoted_kernel<DT, LCH, FCH, LAY, 12>))
-#define RVQ_Q3(DT, LAY) (lch == 8 ? RVQ_Q4(DT, 8, 4, LAY) : RVQ_Q4(DT, 4, 2, LAY))
+#define RVQ_Q3(DT, LAY)                                                                                             \
+        (s.bits == 16 ? quoted(decode_quoted_kernel<DT, LAY, 16>)                                                    \
+         : s.bits == 10 ? quoted(decode_quoted_kernel<DT, LAY, 10>) : quoted(decode_quoted_kernel<DT, LAY, 11>))
 #define RVQ_Q2(DT) (s.layout == RVQ_GROUP_CONTIGUOUS ? RVQ_Q3(DT, RVQ_GROUP_CONTIGUOUS) : RVQ_Q3(DT, RVQ_GROUP_STRIDED))
         return s.dtype == RVQ_BF16 ? RVQ_Q2(RVQ_BF16) : RVQ_Q2(RVQ_F16);
 #undef RVQ_Q2
 #undef RVQ_Q3
-#undef RVQ_Q4
     }
 #define RVQ_DEC_F32(DT, PICK)                                                                                       \
     (fch == 4 ? launch(decode_sliced_kernel<DT, 4, true, PICK>, 4, true)                                           \

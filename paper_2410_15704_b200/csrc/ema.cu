@@ -203,16 +203,18 @@ ema_stats_quad_kernel(Shape s, const void *__restrict__ x, int64_t n, int64_t st
 }
 
 __global__ void __launch_bounds__(256)
-counts_to_float_kernel(const uint32_t *__restrict__ cnt, float *__restrict__ out, int total)
+counts_to_float_kernel(const uint32_t *cnt, float *out, int total)
 {
+    follow_previous();
     int t = blockIdx.x * 256 + threadIdx.x;
     if (t < total) out[t] = (float)cnt[t];
 }
 
 // N <- decay N + (1-decay) n, element-wise.
 __global__ void __launch_bounds__(256)
-ema_count_kernel(const float *__restrict__ cnt, float *__restrict__ ema_count, int total, float decay)
+ema_count_kernel(const float *cnt, float *ema_count, int total, float decay)
 {
+    follow_previous();
     const int t = blockIdx.x * 256 + threadIdx.x;
     if (t < total) ema_count[t] = decay * ema_count[t] + (1.0f - decay) * cnt[t];
 }
@@ -221,9 +223,10 @@ ema_count_kernel(const float *__restrict__ cnt, float *__restrict__ ema_count, i
 // every block, so all blocks of a stage get the same total), then updates its
 // share of M <- decay M + (1-decay) m and C = M / ((N + eps) total / (total + K eps)).
 __global__ void __launch_bounds__(256)
-ema_apply_kernel(Shape s, const float *__restrict__ sum, float *__restrict__ cb,
-                 const float *__restrict__ ema_count, float *__restrict__ ema_sum, float decay, float eps)
+ema_apply_kernel(Shape s, const float *sum, float *cb,
+                 const float *ema_count, float *ema_sum, float decay, float eps)
 {
+    follow_previous();
     __shared__ float red[256];
     const int r = blockIdx.y, tid = threadIdx.x;
     float local = 0.0f;
@@ -293,16 +296,16 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         }
     }
     if (rc != RVQ_OK) return rc;
-    counts_to_float_kernel<<<(bins + 255) / 256, 256, 0, stream>>>(cnt, batch_count, bins);
-    return check_launch();
+    return launch_chained(n > 0, counts_to_float_kernel, dim3((bins + 255) / 256), 256, stream, cnt, batch_count, bins);
 }
 
 // One thread per (bin, channel): the float32 count of the bin, and for the stages whose fused sums
 // were taken after the subtraction of the codeword, the codeword's share back: sum += count * C.
 __global__ void __launch_bounds__(256)
-stats_finish_kernel(const uint32_t *__restrict__ cnt, const float *__restrict__ cb, float *__restrict__ sum,
-                    float *__restrict__ out_count, int bins, int gd, int deferred_bins)
+stats_finish_kernel(const uint32_t *cnt, const float *cb, float *sum,
+                    float *out_count, int bins, int gd, int deferred_bins)
 {
+    follow_previous();
     const int t = blockIdx.x * 256 + threadIdx.x;
     if (t >= bins * gd) return;
     const int bin = t / gd, ch = t - bin * gd;
@@ -315,27 +318,23 @@ int launch_stats_finish(const Shape &s, const uint32_t *cnt, const float *cb, fl
                         int deferred, cudaStream_t stream)
 {
     const int bins = s.R * s.K, total = bins * s.gd;
-    stats_finish_kernel<<<(total + 255) / 256, 256, 0, stream>>>(cnt, cb, batch_sum, batch_count, bins, s.gd, deferred * s.K);
-    return check_launch();
+    return launch_chained(true, stats_finish_kernel, dim3((total + 255) / 256), 256, stream, cnt, cb, batch_sum, batch_count, bins, s.gd, deferred * s.K);
 }
 
 int launch_counts_to_float(const uint32_t *cnt, float *out, int bins, cudaStream_t stream)
 {
-    counts_to_float_kernel<<<(bins + 255) / 256, 256, 0, stream>>>(cnt, out, bins);
-    return check_launch();
+    return launch_chained(false, counts_to_float_kernel, dim3((bins + 255) / 256), 256, stream, cnt, out, bins);
 }
 
 int launch_ema_apply(const Shape &s, const float *batch_count, const float *batch_sum, float *cb,
-                     float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream)
+                     float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream, bool chained)
 {
     const int bins = s.R * s.K;
-    ema_count_kernel<<<(bins + 255) / 256, 256, 0, stream>>>(batch_count, ema_count, bins, decay);
-    int rc = check_launch();
+    int rc = launch_chained(chained, ema_count_kernel, dim3((bins + 255) / 256), 256, stream, batch_count, ema_count, bins, decay);
     if (rc != RVQ_OK) return rc;
     int parts = (s.K * s.gd + 256 * 8 - 1) / (256 * 8);
     if (parts > 32) parts = 32;
-    ema_apply_kernel<<<dim3(parts, s.R), 256, 0, stream>>>(s, batch_sum, cb, ema_count, ema_sum, decay, eps);
-    return check_launch();
+    return launch_chained(true, ema_apply_kernel, dim3(parts, s.R), 256, stream, s, batch_sum, cb, ema_count, ema_sum, decay, eps);
 }
 
 }  // namespace rvq

@@ -71,7 +71,15 @@ constexpr int kDeferMinSlots = 6;                                     // chunks 
 // on keys, which strided groups are for, outlier channels leave 2.1 % of the rows and stages with more than one
 // candidate instead of 0.1 %, and their exact comparison costs more than the steps saved (1M vectors, 1024
 // codes: 6300 -> 6690).
+// It also needs rounds of three tiles, whose chains queue up at the tensor core: with fewer tiles per SM a chain's length is
+// not what a stage waits for, and the added work at the stage end is (values, us, half precision / 8 bits, tiles per SM at
+// most: 1024 codes 64 / 75 at two, 122 / 137 at four, 145 / 138 at five; 2048 codes 147 / 156 at three, 207 / 191 at four).
 constexpr int kEightMinSlots = 8;
+inline bool eight_wanted(const Shape &s, int64_t tiles, int sms)
+{
+    const int slots = slots_per_stage(s.K);
+    return slots >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw && tiles > (int64_t)sms * (slots >= 16 ? 3 : 4);
+}
 
 // barrier slots
 constexpr int kBarFull = 0, kBarEmpty = kRing, kBarAReady = 2 * kRing, kBarAccFull = 2 * kRing + kTiles,
@@ -483,7 +491,7 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
-    auto kernel = slots_per_stage(s.K) >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw ? encode_tensor_kernel<true> : encode_tensor_kernel<false>;
+    auto kernel = eight_wanted(s, tiles, sms) ? encode_tensor_kernel<true> : encode_tensor_kernel<false>;
     if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,

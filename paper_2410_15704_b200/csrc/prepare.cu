@@ -40,9 +40,10 @@ size_t prepared_bytes(const Shape &s)
 // One thread per (channel octet, code, stage): 8 channels of levels, stored as one 16-byte
 // entry of a wide slice or as the 8-byte entries of two narrow slices.
 __global__ void __launch_bounds__(256)
-decode_table_kernel(Shape s, const float *__restrict__ cb, const DecodeParams *__restrict__ dp,
-                    const float *__restrict__ lo, uint4 *__restrict__ table)
+decode_table_kernel(Shape s, const float *cb, const DecodeParams *dp,
+                    const float *lo, uint4 *table)
 {
+    follow_previous();
     const int t = blockIdx.x * 256 + threadIdx.x, octet = blockIdx.y;
     const int j = t >> 3, r = t & 7;
     if (j >= s.K) return;
@@ -51,7 +52,7 @@ decode_table_kernel(Shape s, const float *__restrict__ cb, const DecodeParams *_
     float v[8];
     if (used) {
         const float4 *src = reinterpret_cast<const float4 *>(cb + ((size_t)r * s.K + j) * 32 + octet * 8);
-        const float4 a = __ldg(src), b = __ldg(src + 1);
+        const float4 a = src[0], b = src[1];
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
     }
     uint32_t w[4];
@@ -102,8 +103,9 @@ decode_table_kernel(Shape s, const float *__restrict__ cb, const DecodeParams *_
 
 // grid (kPrepareParts, R): largest squared norm and entry range of a share of one stage's codewords.
 __global__ void __launch_bounds__(256)
-prepare_reduce_kernel(Shape s, const float *__restrict__ cb, StagePartial *part)
+prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
 {
+    follow_previous();
     __shared__ double rn[256];
     __shared__ float rlo[256], rhi[256];
     const int r = blockIdx.y, tid = threadIdx.x;
@@ -139,9 +141,10 @@ prepare_reduce_kernel(Shape s, const float *__restrict__ cb, StagePartial *part)
 // One block, thread r per stage: scale exponent from the largest squared norm, the decoder's
 // affine map from the entry range; clears the maxima the image kernel accumulates into.
 __global__ void __launch_bounds__(32)
-prepare_params_kernel(Shape s, const StagePartial *__restrict__ part, PreparedHeader *hdr, StageParams *sp,
+prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, StageParams *sp,
                       StageMaxima *mx, DecodeParams *dp, float *dec_lo)
 {
+    follow_previous();
     __shared__ float s_lo[8], s_step[8];
     const int r = threadIdx.x;
     if (r < 8) { s_lo[r] = 0.0f; s_step[r] = 0.0f; }
@@ -220,9 +223,10 @@ prepare_params_kernel(Shape s, const StagePartial *__restrict__ part, PreparedHe
 // One thread per (padded) codeword: operand image and the maxima the error
 // bound needs.  grid = (slots * 128 / 128, R).
 __global__ void __launch_bounds__(128)
-prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *__restrict__ sp,
-                     StageMaxima *mx, uint8_t *__restrict__ image, float4 *__restrict__ blocks)
+prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
+                     StageMaxima *mx, uint8_t *image, float4 *blocks)
 {
+    follow_previous();
     const int r = blockIdx.y;
     const int slot = blockIdx.x, jj = threadIdx.x;
     const int j = slot * kSlotCodewords + jj;            // padded codeword index
@@ -290,6 +294,7 @@ prepare_image_kernel(Shape s, const float *__restrict__ cb, const StageParams *_
 //   compare tens of millions of choices with the all-float32 kernel's.
 __global__ void prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxima *mx)
 {
+    follow_previous();
     const int r = threadIdx.x;
     if (r >= s.R) return;
     const float emax = __uint_as_float(mx[r].emax), eerr = __uint_as_float(mx[r].eerr);
@@ -299,7 +304,7 @@ __global__ void prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxim
     sp[r].b = 1.9073486328125e-6f * nmax + 4.76837158203125e-7f * emax;
 }
 
-int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream)
+int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream, bool chained)
 {
     uint8_t *p = reinterpret_cast<uint8_t *>(prepared);
     PreparedHeader *hdr = reinterpret_cast<PreparedHeader *>(p);
@@ -310,24 +315,18 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
     const size_t off = decode_section_offset(s);
     DecodeParams *dp = dec ? reinterpret_cast<DecodeParams *>(p + off) : nullptr;
     float *lo = dec ? reinterpret_cast<float *>(p + off + 128) : nullptr;   // per-stage minima, second half of the parameter block
-    prepare_reduce_kernel<<<dim3(kPrepareParts, s.R), 256, 0, stream>>>(s, cb, part);
-    int rc = check_launch();
+    int rc = launch_chained(chained, prepare_reduce_kernel, dim3(kPrepareParts, s.R), 256, stream, s, cb, part);
     if (rc != RVQ_OK) return rc;
-    prepare_params_kernel<<<1, 32, 0, stream>>>(s, part, hdr, sp, mx, dp, lo);
-    if ((rc = check_launch()) != RVQ_OK) return rc;
+    if ((rc = launch_chained(true, prepare_params_kernel, dim3(1), 32, stream, s, part, hdr, sp, mx, dp, lo)) != RVQ_OK) return rc;
     if (s.gd == 32) {
-        dim3 grid(slots_per_stage(s.K), s.R);
-        prepare_image_kernel<<<grid, kSlotCodewords, 0, stream>>>(s, cb, sp, mx, p + kPreparedImageOffset,
-            float_blocks_prepared(s) ? reinterpret_cast<float4 *>(p + float_blocks_offset(s)) : nullptr);
-        if ((rc = check_launch()) != RVQ_OK) return rc;
-        prepare_finish_kernel<<<1, 32, 0, stream>>>(s, sp, mx);
-        if ((rc = check_launch()) != RVQ_OK) return rc;
+        rc = launch_chained(true, prepare_image_kernel, dim3(slots_per_stage(s.K), s.R), kSlotCodewords, stream, s, cb, sp, mx, p + kPreparedImageOffset,
+                            float_blocks_prepared(s) ? reinterpret_cast<float4 *>(p + float_blocks_offset(s)) : nullptr);
+        if (rc != RVQ_OK) return rc;
+        if ((rc = launch_chained(true, prepare_finish_kernel, dim3(1), 32, stream, s, sp, mx)) != RVQ_OK) return rc;
     }
-    if (dec) {
-        dim3 grid((s.K * 8 + 255) / 256, 4);
-        decode_table_kernel<<<grid, 256, 0, stream>>>(s, cb, dp, lo, reinterpret_cast<uint4 *>(p + off + 256));
-        if ((rc = check_launch()) != RVQ_OK) return rc;
-    }
+    if (dec)
+        return launch_chained(true, decode_table_kernel, dim3((s.K * 8 + 255) / 256, 4), 256, stream, s, cb, dp, lo,
+                              reinterpret_cast<uint4 *>(p + off + 256));
     return RVQ_OK;
 }
 

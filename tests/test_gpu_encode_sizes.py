@@ -65,9 +65,9 @@ def test_against_the_oracle():
     assert_codes_match(x.numpy(), codes, cb, 0)
 
 
-@pytest.mark.parametrize("n,K,R,scale", [(9477, 1024, 8, 1.0), (10007, 2048, 4, 1.0), (9480, 1030, 2, 1e-3), (9500, 1024, 2, 3e4)])
+@pytest.mark.parametrize("n,K,R,scale", [(18945, 1024, 8, 1.0), (14219, 2048, 4, 1.0), (18960, 1030, 2, 1e-3), (19000, 1024, 2, 3e4)])
 def test_eight_bit_corrections(n, K, R, scale):
-    """Contiguous groups, eight or more chunks, more than one tile per SM: ordinary codebooks, and ones whose
+    """Contiguous groups, eight or more chunks, more than four tiles per SM (three with 2048 codes): ordinary codebooks, and ones whose
     stages' scales lie far apart (rows beyond the 8-bit range take the full scan)."""
     x, cb = batch(n, 128, K, R, "f32", n)
     cb[0, ::7] *= 8.0
@@ -79,3 +79,23 @@ def test_eight_bit_corrections(n, K, R, scale):
     rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
     torch.cuda.synchronize()
     assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
+
+
+@pytest.mark.parametrize("n,dim,K,R,layout", [(1, 128, 1024, 8, 0), (33, 128, 512, 4, 1), (2055, 128, 1000, 8, 1), (1025, 256, 2048, 6, 0),
+                                              (4737, 128, 1024, 2, 0)])
+def test_statistics_of_few_tiles(n, dim, K, R, layout):
+    """Batches whose statistics are taken by the separate pass (the last one: just beyond them), against float64."""
+    x, cb = batch(n, dim, K, R, "f32", n)
+    x[2 % n] = x[0]                                         # (no degenerate row)
+    cfg = rvq.make_config(dim, 32, layout, R, K, 16, rvq.F32, 0)
+    b, G, xd = rvq.alloc_buffers(cfg, n, cb), dim // 32, x.cuda()
+    count, total = torch.empty(R, K, device="cuda"), torch.empty(R, K, 32, device="cuda")
+    rvq.rvq_encode_stats(cfg, xd, n, dim, b.codebooks, b.prepared, b.codes, b.std, count, total, b.workspace, b.workspace_bytes, b.status)
+    codes = (b.codes.view(torch.int16).view(n, -1)[:, :G * R].reshape(n * G, R).long() & 0xFFFF)
+    z = xd.double() / xd.double().std(dim=1, unbiased=False, keepdim=True)
+    z = (z.view(n, 32, G).transpose(1, 2) if layout else z.view(n, G, 32)).reshape(n * G, 32)
+    for r in range(R):
+        assert torch.equal(count[r].long(), torch.bincount(codes[:, r], minlength=K))
+        want = torch.zeros(K, 32, dtype=torch.float64, device="cuda").index_add_(0, codes[:, r], z)
+        assert (total[r].double() - want).abs().max() <= 1e-5 * max(1.0, want.abs().max().item())
+        z = z - b.codebooks.view(R, K, 32)[r][codes[:, r]].double()
