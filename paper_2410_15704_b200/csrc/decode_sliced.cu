@@ -679,13 +679,14 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             const uint32_t a = smem_table + (line | unit[k]);
             uint32_t e[CH / 2];
             if (F32) {
-                uint64_t f01, f23;
-                asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(f01), "=l"(f23) : "r"(a));
                 if (ROPE == 0) {
+                    uint64_t f01, f23;
+                    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(f01), "=l"(f23) : "r"(a));
                     fa = add_f32x2(fa, f01); fb = add_f32x2(fb, f23);
                 } else {                                        // (with the rotation, packed additions are slower)
-                    fs[0] += __uint_as_float((uint32_t)f01); fs[1] += __uint_as_float((uint32_t)(f01 >> 32));
-                    fs[2] += __uint_as_float((uint32_t)f23); fs[3] += __uint_as_float((uint32_t)(f23 >> 32));
+                    float f0, f1, f2, f3;
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(f0), "=f"(f1), "=f"(f2), "=f"(f3) : "r"(a));
+                    fs[0] += f0; fs[1] += f1; fs[2] += f2; fs[3] += f3;
                 }
                 continue;
             }
