@@ -245,9 +245,12 @@ int rvq_encode_stats(const rvq_config *cfg, const void *x, int64_t n, int64_t x_
     if (!batch_count || !batch_sum || !workspace) return RVQ_ERR_BADARG;
     if (!aligned16(batch_sum) || !aligned256(workspace)) return RVQ_ERR_ALIGN;
     if (workspace_bytes < ema_stats_scratch_bytes(s)) return RVQ_ERR_WORKSPACE;
-    if (!encode_tensor_supported(s) || encode_small_wanted(s, n) || encode_split_wanted(s, n)) {
-        // shapes without the fused kernel, and batches that the encoders for few tiles take: encode, then the
-        // separate statistics pass
+    if (!encode_tensor_supported(s) || encode_small_wanted(s, n) || encode_split_wanted(s, n) ||
+        (encode_tensor_deferred_stages(s) == 0 && ema_stats_quad_supported(s) && (s.K > 256 || n * s.G <= (1 << 19)))) {
+        // shapes without the fused kernel, batches that the encoders for few tiles take, and codebooks too small to hide
+        // the additions behind (fused, the epilogue waits for them): encode, then the separate statistics pass.  A learning
+        // step fused / separate, us: 32000 vectors and 256 codes 193 / 175, 240000 940 / 944, 1M 4050 / 4100 (all
+        // rows meet in a few bins either way); 512 codes 80000 426 / 416, 480000 2312 / 2222.
         rc = encode_common(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, stage_energy, status, stream, true);
         if (rc != RVQ_OK) return rc;
         return launch_ema_stats(s, x, n, x_row_stride, codes, codebooks, batch_count, batch_sum, workspace,

@@ -132,9 +132,10 @@ ema_stats_warp_kernel(Shape s, const void *__restrict__ x, int64_t n, int64_t st
     if (bad && st && lane < 32) atomicAdd(&st->bad_codes, bad);
 }
 
-// The same for head vectors of exactly four groups (dim 128): the warp takes the four rows of a vector
-// at once, lane = (group, four-channel piece), so that every stage is one 16-byte reduction and one
+// The same for head vectors of four groups or eight (PARTS 1, 2; dim 128 and 256): the warp takes four rows of a
+// vector at once, lane = (group, four-channel piece), so that every stage is one 16-byte reduction and one
 // 16-byte load per lane (four cache lines per instruction) instead of eight instructions per row.
+template <int PARTS>
 __global__ void __launch_bounds__(kWarpStatsThreads)
 ema_stats_quad_kernel(Shape s, const void *__restrict__ x, int64_t n, int64_t stride,
                       const void *__restrict__ codes, const float *__restrict__ cb,
@@ -146,53 +147,60 @@ ema_stats_quad_kernel(Shape s, const void *__restrict__ x, int64_t n, int64_t st
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int warps = (kWarpStatsThreads / 32) * gridDim.x;
-    const int R = s.R, per = s.per_vector;                     // per = 4 * R <= 32
-    const int g = lane >> 3, q = lane & 7;                     // this lane: elements 4q .. 4q+3 of group g
+    const int R = s.R, per = 4 * R;                            // codes of four groups, <= 32
+    const int g = lane >> 3, q = lane & 7;                     // this lane: elements 4q .. 4q+3 of group 4 part + g
     uint32_t bad = 0;
     for (int64_t v = (int64_t)blockIdx.x * (kWarpStatsThreads / 32) + warp; v < n; v += warps) {
-        float z[4];
+        // lane l holds code l of each part's 4 R (group l / R, stage l % R)
+        uint32_t code[PARTS];
+#pragma unroll
+        for (int p = 0; p < PARTS; ++p)
+            code[p] = lane < per ? read_code(reinterpret_cast<const uint8_t *>(codes) + v * s.code_bytes, p * per + lane, s.bits, s.code_bytes) : 0u;
+        float z[PARTS][4];
         float a = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            z[k] = load_as_float(x, v * stride + channel_of(s.layout, 4, 32, g, 4 * q + k), s.dtype);
-            a += z[k];
-        }
+        for (int p = 0; p < PARTS; ++p)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                z[p][k] = load_as_float(x, v * stride + channel_of(s.layout, 4 * PARTS, 32, 4 * p + g, 4 * q + k), s.dtype);
+                a += z[p][k];
+            }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, off);
         const float mu = a / (float)s.dim;
         float b = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) b += (z[k] - mu) * (z[k] - mu);
+        for (int p = 0; p < PARTS; ++p)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) b += (z[p][k] - mu) * (z[p][k] - mu);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) b += __shfl_xor_sync(0xFFFFFFFFu, b, off);
         const float dev = sqrtf(b / (float)(s.dim - s.ddof));
         const bool deg = deviation_is_degenerate(dev);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) z[k] = deg ? 0.0f : z[k] / dev;
-        // lane l holds code l of the vector (group l / R, stage l % R) and counts it
-        uint32_t code = 0;
-        if (lane < per) {
-            code = read_code(reinterpret_cast<const uint8_t *>(codes) + v * s.code_bytes, lane, s.bits, s.code_bytes);
-            if (code >= (uint32_t)s.K) { code = 0; ++bad; }
-        }
-        const int my_bin = lane < per ? (lane % R) * s.K + (int)code : -1 - lane;   // (idle lanes: bins of their own)
-        const uint32_t same = __match_any_sync(0xFFFFFFFFu, my_bin);
-        if (lane < per && lane == __ffs(same) - 1) atomicAdd(&hist[my_bin], (uint32_t)__popc(same));
-        // the codewords of all stages are asked for first (they depend on the codes only), then the
-        // residual walks through the stages (R <= 8 here: four groups, at most 32 codes)
-        size_t at[8];
-        float4 e[8];
+        for (int p = 0; p < PARTS; ++p) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const uint32_t j = __shfl_sync(0xFFFFFFFFu, code, g * R + (r < R ? r : 0));
-            at[r] = ((size_t)(r < R ? r : 0) * s.K + j) * 32 + 4 * q;
-            e[r] = __ldg(reinterpret_cast<const float4 *>(cb + at[r]));
-        }
+            for (int k = 0; k < 4; ++k) z[p][k] = deg ? 0.0f : z[p][k] / dev;
+            if (code[p] >= (uint32_t)s.K) { code[p] = 0; ++bad; }
+            const int my_bin = lane < per ? (lane % R) * s.K + (int)code[p] : -1 - lane;   // (idle lanes: bins of their own)
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, my_bin);
+            if (lane < per && lane == __ffs(same) - 1) atomicAdd(&hist[my_bin], (uint32_t)__popc(same));
+            // the codewords of all stages are asked for first (they depend on the codes only), then the
+            // residual walks through the stages
+            size_t at[8];
+            float4 e[8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if (r < R) {
-                atomicAdd(reinterpret_cast<float4 *>(sum + at[r]), make_float4(z[0], z[1], z[2], z[3]));
-                z[0] -= e[r].x; z[1] -= e[r].y; z[2] -= e[r].z; z[3] -= e[r].w;
+            for (int r = 0; r < 8; ++r) {
+                const uint32_t j = __shfl_sync(0xFFFFFFFFu, code[p], g * R + (r < R ? r : 0));
+                at[r] = ((size_t)(r < R ? r : 0) * s.K + j) * 32 + 4 * q;
+                e[r] = __ldg(reinterpret_cast<const float4 *>(cb + at[r]));
+            }
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                if (r < R) {
+                    atomicAdd(reinterpret_cast<float4 *>(sum + at[r]), make_float4(z[p][0], z[p][1], z[p][2], z[p][3]));
+                    z[p][0] -= e[r].x; z[p][1] -= e[r].y; z[p][2] -= e[r].z; z[p][3] -= e[r].w;
+                }
             }
         }
     }
@@ -262,6 +270,11 @@ static int stats_gd(const Shape &s, const void *x, int64_t n, int64_t stride, co
     return check_launch();
 }
 
+bool ema_stats_quad_supported(const Shape &s)
+{
+    return s.gd == 32 && (s.G == 4 || s.G == 8) && s.R <= 8 && (size_t)s.R * s.K * sizeof(uint32_t) <= 160 * 1024;
+}
+
 int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, const void *codes,
                      const float *cb, float *batch_count, float *batch_sum, void *workspace,
                      rvq_status *st, cudaStream_t stream)
@@ -272,7 +285,8 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         cudaMemsetAsync(batch_sum, 0, (size_t)bins * s.gd * sizeof(float), stream) != cudaSuccess)
         return RVQ_ERR_LAUNCH;
     int rc = RVQ_OK;
-    if (n > 0 && s.gd == 32 && s.G <= 8 && s.per_vector <= 32 && (size_t)bins * sizeof(uint32_t) <= 160 * 1024) {
+    const bool quad = ema_stats_quad_supported(s);
+    if (n > 0 && (quad || (s.gd == 32 && s.G <= 8 && s.per_vector <= 32 && (size_t)bins * sizeof(uint32_t) <= 160 * 1024))) {
         const int sms = sm_count();
         if (sms <= 0) return RVQ_ERR_DEVICE;
         const size_t smem = (size_t)bins * sizeof(uint32_t);
@@ -281,7 +295,7 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         per_sm = per_sm < 1 ? 1 : (per_sm > 8 ? 8 : per_sm);
         int64_t want = (n + kWarpStatsThreads / 32 - 1) / (kWarpStatsThreads / 32);
         int grid = (int)(want < (int64_t)sms * per_sm ? want : (int64_t)sms * per_sm);
-        auto kernel = s.G == 4 ? ema_stats_quad_kernel : ema_stats_warp_kernel;
+        auto kernel = !quad ? ema_stats_warp_kernel : s.G == 4 ? ema_stats_quad_kernel<1> : ema_stats_quad_kernel<2>;
         if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<grid, kWarpStatsThreads, smem, stream>>>(s, x, n, stride, codes, cb, cnt, batch_sum, st);

@@ -81,10 +81,10 @@ def test_eight_bit_corrections(n, K, R, scale):
     assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
 
 
-@pytest.mark.parametrize("n,dim,K,R,layout", [(1, 128, 1024, 8, 0), (33, 128, 512, 4, 1), (2055, 128, 1000, 8, 1), (1025, 256, 2048, 6, 0),
+@pytest.mark.parametrize("n,dim,K,R,layout", [(1, 128, 1024, 8, 0), (33, 128, 512, 4, 1), (2055, 128, 1000, 8, 1), (1025, 256, 2048, 6, 0), (5003, 256, 512, 8, 1),
                                               (4737, 128, 1024, 2, 0)])
 def test_statistics_of_few_tiles(n, dim, K, R, layout):
-    """Batches whose statistics are taken by the separate pass (the last one: just beyond them), against float64."""
+    """Batches whose statistics are taken by the separate pass, with four groups and eight (the last one: fused), against float64."""
     x, cb = batch(n, dim, K, R, "f32", n)
     x[2 % n] = x[0]                                         # (no degenerate row)
     cfg = rvq.make_config(dim, 32, layout, R, K, 16, rvq.F32, 0)
