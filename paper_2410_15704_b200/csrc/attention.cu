@@ -217,6 +217,7 @@ att_scores_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
                   const float *__restrict__ cb, const float *__restrict__ q, const int32_t *__restrict__ position,
                   const float2 *__restrict__ cos_sin, int positions, float *__restrict__ scores, rvq_status *st)
 {
+    asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(128) uint8_t smem[];
     const int parts = gridDim.x / kAttSlices;
     if ((int)blockIdx.x >= parts * kAttSlices) return;
@@ -323,8 +324,9 @@ __device__ __forceinline__ float att_unordered(uint32_t u)
 
 // Step 2: m[column] = max over the tokens of scale * s[token][column]; columns = 8 J (divides 1024).
 __global__ void __launch_bounds__(kAttThreads)
-att_max_kernel(const float *__restrict__ scores, int64_t tokens, int columns, float scale, uint32_t *__restrict__ m_ord)
+att_max_kernel(const float *scores, int64_t tokens, int columns, float scale, uint32_t *m_ord)
 {
+    follow_previous();
     __shared__ float part[kAttThreads];
     const int col = threadIdx.x % columns, rows_per_block = kAttThreads / columns;
     float m = -INFINITY;
@@ -342,9 +344,10 @@ att_max_kernel(const float *__restrict__ scores, int64_t tokens, int columns, fl
 // Step 3: every score becomes its weight times its token's deviation, exp(scale s - m) = 2^(s * scale log2(e) -
 // m log2(e)), and the weights are summed; once per token here instead of in each of the 32 rows and slices of step 4.
 __global__ void __launch_bounds__(kAttThreads)
-att_weights_kernel(float *__restrict__ scores, const uint16_t *__restrict__ std16, uint32_t tokens, int columns, int per_head_log,
-                   float scale, const uint32_t *__restrict__ m_ord, float *__restrict__ weight_sum)
+att_weights_kernel(float *scores, const uint16_t *__restrict__ std16, uint32_t tokens, int columns, int per_head_log,
+                   float scale, const uint32_t *m_ord, float *weight_sum)
 {
+    follow_previous();
     __shared__ float part[kAttThreads];
     constexpr float kLog2e = 1.4426950408889634f;
     const int col = threadIdx.x % columns, rows_per_block = kAttThreads / columns;
@@ -367,14 +370,16 @@ att_weights_kernel(float *__restrict__ scores, const uint16_t *__restrict__ std1
 template <int LAYOUT, int J, int STEPS>
 __global__ void __launch_bounds__(kAttThreads, 1)
 att_values_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t tokens,
-                  const float *__restrict__ cb, const float *__restrict__ weights, float *__restrict__ out_acc, rvq_status *st)
+                  const float *__restrict__ cb, const float *weights, float *out_acc, rvq_status *st)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     const int parts = gridDim.x / kAttSlices;
     if ((int)blockIdx.x >= parts * kAttSlices) return;
     const int sl = blockIdx.x % kAttSlices, part = blockIdx.x / kAttSlices;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = lane >> 2;
+    // (the table does not hang on the weights: it is filled while they are made)
     att_fill_table<LAYOUT, 0, STEPS>(s, cb, sl, reinterpret_cast<float4 *>(smem));
+    follow_previous();
     __syncthreads();
     const uint32_t smem_table = (uint32_t)__cvta_generic_to_shared(smem);
     uint32_t bad = 0;
@@ -391,9 +396,9 @@ att_values_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
         float sc[J];
         {
             const float *src = weights + (size_t)(t * 8u + (uint32_t)h) * J;
-            if (J == 4) { const float4 f = __ldg(reinterpret_cast<const float4 *>(src)); sc[0] = f.x; sc[1] = f.y; sc[J - 2] = f.z; sc[J - 1] = f.w; }
-            else if (J == 2) { const float2 f = __ldg(reinterpret_cast<const float2 *>(src)); sc[0] = f.x; sc[J - 1] = f.y; }
-            else sc[0] = __ldg(src);
+            if (J == 4) { const float4 f = *reinterpret_cast<const float4 *>(src); sc[0] = f.x; sc[1] = f.y; sc[J - 2] = f.z; sc[J - 1] = f.w; }
+            else if (J == 2) { const float2 f = *reinterpret_cast<const float2 *>(src); sc[0] = f.x; sc[J - 1] = f.y; }
+            else sc[0] = *src;
         }
         att_fetch(s, ac, codes, std16, t + step, T, lane, next);
         float v[4];
@@ -425,9 +430,10 @@ att_values_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__res
 }
 
 // Step 5.
-__global__ void att_finish_kernel(const float *__restrict__ out_acc, const float *__restrict__ weight_sum, int heads,
-                                  float *__restrict__ out)
+__global__ void att_finish_kernel(const float *out_acc, const float *weight_sum, int heads,
+                                  float *out)
 {
+    follow_previous();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx < heads * 128) out[idx] = out_acc[idx] / weight_sum[idx >> 7];
 }
@@ -624,7 +630,7 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
 
 // One CTA per query head: the chunks' parts, weighted to their common maximum, over the sum of all weights.
 __global__ void __launch_bounds__(128)
-att_combine_kernel(const float *__restrict__ part, const float2 *__restrict__ part_ml, int chunks, int layout_v, float *__restrict__ out)
+att_combine_kernel(const float *part, const float2 *part_ml, int chunks, int layout_v, float *out)
 {
     __shared__ float2 ml_s[kShortMaxChunks];
     __shared__ float f_s[kShortMaxChunks];
@@ -719,15 +725,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
         int rc = check_launch();
         if (rc != RVQ_OK) return rc;
         // (its launch overlaps the first kernel; it waits for that one's results on the device)
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)q_heads); cfg.blockDim = dim3(128); cfg.stream = stream;
-        cfg.attrs = &attr; cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, att_combine_kernel, (const float *)part, (const float2 *)part_ml, chunks, sv.layout, out);
-        rc = check_launch();
-        return e == cudaSuccess ? rc : RVQ_ERR_LAUNCH;
+        return launch_chained(true, att_combine_kernel, dim3((unsigned)q_heads), 128, 0, stream, part, part_ml, chunks, sv.layout, out);
     }
     const size_t score_bytes = ((size_t)tokens * q_heads * 4 + 255) / 256 * 256;
     float *scores = reinterpret_cast<float *>(ws);
@@ -757,8 +755,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
         if (smem < red) smem = red;
         if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
-        kernel<<<parts * kAttSlices, kAttThreads, smem, stream>>>(sv, codes_v, std_v, tokens, cb_v, scores, out_acc, st);
-        return check_launch();
+        return launch_chained(true, kernel, dim3(parts * kAttSlices), kAttThreads, smem, stream, sv, codes_v, std_v, tokens, cb_v, scores, out_acc, st);
     };
 #define RVQ_ATT_S4(LAY, ROPE, JJ) (sk.R <= 4 ? scores_launch(att_scores_kernel<LAY, ROPE, JJ, 4>) : scores_launch(att_scores_kernel<LAY, ROPE, JJ, 8>))
 #define RVQ_ATT_S3(LAY, ROPE) (J == 4 ? RVQ_ATT_S4(LAY, ROPE, 4) : J == 2 ? RVQ_ATT_S4(LAY, ROPE, 2) : RVQ_ATT_S4(LAY, ROPE, 1))
@@ -772,10 +769,11 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
         int blocks = (int)((tokens * q_heads + kAttThreads - 1) / kAttThreads);
         if (blocks > sms * 2) blocks = sms * 2;
         if (blocks < 1) blocks = 1;
-        att_max_kernel<<<blocks, kAttThreads, 0, stream>>>(scores, tokens, q_heads, scale, m_ord);
-        if ((rc = check_launch()) != RVQ_OK) return rc;
-        att_weights_kernel<<<blocks, kAttThreads, 0, stream>>>(scores, std_v, (uint32_t)tokens, q_heads, J == 4 ? 2 : J == 2 ? 1 : 0, scale, m_ord, weight_sum);
-        if ((rc = check_launch()) != RVQ_OK) return rc;
+        rc = launch_chained(true, att_max_kernel, dim3(blocks), kAttThreads, 0, stream, scores, tokens, q_heads, scale, m_ord);
+        if (rc != RVQ_OK) return rc;
+        rc = launch_chained(true, att_weights_kernel, dim3(blocks), kAttThreads, 0, stream, scores, std_v, tokens, q_heads,
+                            J == 4 ? 2 : J == 2 ? 1 : 0, scale, m_ord, weight_sum);
+        if (rc != RVQ_OK) return rc;
     }
 #define RVQ_ATT_V3(LAY, JJ) (sv.R <= 4 ? values_launch(att_values_kernel<LAY, JJ, 4>) : values_launch(att_values_kernel<LAY, JJ, 8>))
 #define RVQ_ATT_V2(LAY) (J == 4 ? RVQ_ATT_V3(LAY, 4) : J == 2 ? RVQ_ATT_V3(LAY, 2) : RVQ_ATT_V3(LAY, 1))
@@ -783,8 +781,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
 #undef RVQ_ATT_V2
 #undef RVQ_ATT_V3
     if (rc != RVQ_OK) return rc;
-    att_finish_kernel<<<(q_heads * 128 + 255) / 256, 256, 0, stream>>>(out_acc, weight_sum, q_heads, out);
-    return check_launch();
+    return launch_chained(true, att_finish_kernel, dim3((q_heads * 128 + 255) / 256), 256, 0, stream, out_acc, weight_sum, q_heads, out);
 }
 
 }  // namespace rvq

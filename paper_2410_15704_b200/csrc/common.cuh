@@ -116,13 +116,13 @@ __device__ __forceinline__ void follow_previous()
 // Launch of such a kernel; chained: behind another kernel of the same call (a call's first kernel is launched as usual,
 // since what the caller has before it in the stream need not wait for its own predecessors).
 template <typename... P, typename... A>
-inline int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, int threads, cudaStream_t stream, A... args)
+inline int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.stream = stream;
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cfg.attrs = &attr; cfg.numAttrs = chained ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     const int rc = check_launch();

@@ -310,7 +310,7 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         }
     }
     if (rc != RVQ_OK) return rc;
-    return launch_chained(n > 0, counts_to_float_kernel, dim3((bins + 255) / 256), 256, stream, cnt, batch_count, bins);
+    return launch_chained(n > 0, counts_to_float_kernel, dim3((bins + 255) / 256), 256, 0, stream, cnt, batch_count, bins);
 }
 
 // One thread per (bin, channel): the float32 count of the bin, and for the stages whose fused sums
@@ -332,23 +332,23 @@ int launch_stats_finish(const Shape &s, const uint32_t *cnt, const float *cb, fl
                         int deferred, cudaStream_t stream)
 {
     const int bins = s.R * s.K, total = bins * s.gd;
-    return launch_chained(true, stats_finish_kernel, dim3((total + 255) / 256), 256, stream, cnt, cb, batch_sum, batch_count, bins, s.gd, deferred * s.K);
+    return launch_chained(true, stats_finish_kernel, dim3((total + 255) / 256), 256, 0, stream, cnt, cb, batch_sum, batch_count, bins, s.gd, deferred * s.K);
 }
 
 int launch_counts_to_float(const uint32_t *cnt, float *out, int bins, cudaStream_t stream)
 {
-    return launch_chained(false, counts_to_float_kernel, dim3((bins + 255) / 256), 256, stream, cnt, out, bins);
+    return launch_chained(false, counts_to_float_kernel, dim3((bins + 255) / 256), 256, 0, stream, cnt, out, bins);
 }
 
 int launch_ema_apply(const Shape &s, const float *batch_count, const float *batch_sum, float *cb,
                      float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream, bool chained)
 {
     const int bins = s.R * s.K;
-    int rc = launch_chained(chained, ema_count_kernel, dim3((bins + 255) / 256), 256, stream, batch_count, ema_count, bins, decay);
+    int rc = launch_chained(chained, ema_count_kernel, dim3((bins + 255) / 256), 256, 0, stream, batch_count, ema_count, bins, decay);
     if (rc != RVQ_OK) return rc;
     int parts = (s.K * s.gd + 256 * 8 - 1) / (256 * 8);
     if (parts > 32) parts = 32;
-    return launch_chained(true, ema_apply_kernel, dim3(parts, s.R), 256, stream, s, batch_sum, cb, ema_count, ema_sum, decay, eps);
+    return launch_chained(true, ema_apply_kernel, dim3(parts, s.R), 256, 0, stream, s, batch_sum, cb, ema_count, ema_sum, decay, eps);
 }
 
 }  // namespace rvq

@@ -315,17 +315,17 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
     const size_t off = decode_section_offset(s);
     DecodeParams *dp = dec ? reinterpret_cast<DecodeParams *>(p + off) : nullptr;
     float *lo = dec ? reinterpret_cast<float *>(p + off + 128) : nullptr;   // per-stage minima, second half of the parameter block
-    int rc = launch_chained(chained, prepare_reduce_kernel, dim3(kPrepareParts, s.R), 256, stream, s, cb, part);
+    int rc = launch_chained(chained, prepare_reduce_kernel, dim3(kPrepareParts, s.R), 256, 0, stream, s, cb, part);
     if (rc != RVQ_OK) return rc;
-    if ((rc = launch_chained(true, prepare_params_kernel, dim3(1), 32, stream, s, part, hdr, sp, mx, dp, lo)) != RVQ_OK) return rc;
+    if ((rc = launch_chained(true, prepare_params_kernel, dim3(1), 32, 0, stream, s, part, hdr, sp, mx, dp, lo)) != RVQ_OK) return rc;
     if (s.gd == 32) {
-        rc = launch_chained(true, prepare_image_kernel, dim3(slots_per_stage(s.K), s.R), kSlotCodewords, stream, s, cb, sp, mx, p + kPreparedImageOffset,
+        rc = launch_chained(true, prepare_image_kernel, dim3(slots_per_stage(s.K), s.R), kSlotCodewords, 0, stream, s, cb, sp, mx, p + kPreparedImageOffset,
                             float_blocks_prepared(s) ? reinterpret_cast<float4 *>(p + float_blocks_offset(s)) : nullptr);
         if (rc != RVQ_OK) return rc;
-        if ((rc = launch_chained(true, prepare_finish_kernel, dim3(1), 32, stream, s, sp, mx)) != RVQ_OK) return rc;
+        if ((rc = launch_chained(true, prepare_finish_kernel, dim3(1), 32, 0, stream, s, sp, mx)) != RVQ_OK) return rc;
     }
     if (dec)
-        return launch_chained(true, decode_table_kernel, dim3((s.K * 8 + 255) / 256, 4), 256, stream, s, cb, dp, lo,
+        return launch_chained(true, decode_table_kernel, dim3((s.K * 8 + 255) / 256, 4), 256, 0, stream, s, cb, dp, lo,
                               reinterpret_cast<uint4 *>(p + off + 256));
     return RVQ_OK;
 }
