@@ -230,30 +230,51 @@ ema_count_kernel(const float *cnt, float *ema_count, int total, float decay)
 // grid (parts, R): every block sums the stage's updated counts (same order in
 // every block, so all blocks of a stage get the same total), then updates its
 // share of M <- decay M + (1-decay) m and C = M / ((N + eps) total / (total + K eps)).
+template <int V>                                              // channels per thread: 4, or 1 for buffers that are not 16-byte aligned
 __global__ void __launch_bounds__(256)
 ema_apply_kernel(Shape s, const float *sum, float *cb,
                  const float *ema_count, float *ema_sum, float decay, float eps)
 {
     follow_previous();
-    __shared__ float red[256];
-    const int r = blockIdx.y, tid = threadIdx.x;
+    __shared__ float red[8];
+    const int r = blockIdx.y, tid = threadIdx.x, per_stage = s.K * s.gd;
+    float *const cb_r = cb + (size_t)r * per_stage, *const sum_r = ema_sum + (size_t)r * per_stage;
+    const float *const batch_r = sum + (size_t)r * per_stage, *const count_r = ema_count + (size_t)r * s.K;
+    // V channels of a codeword per thread, asked for before the stage's total is added up
+    const int first = (blockIdx.x * 256 + tid) * V;
+    float m[V], b[V];
+    float c = 0.0f;
+    auto ask = [&](int t) {
+        if (V == 4) {
+            const float4 f = *reinterpret_cast<const float4 *>(sum_r + t), h = *reinterpret_cast<const float4 *>(batch_r + t);
+            m[0] = f.x; m[1 % V] = f.y; m[2 % V] = f.z; m[3 % V] = f.w;
+            b[0] = h.x; b[1 % V] = h.y; b[2 % V] = h.z; b[3 % V] = h.w;
+        } else {
+            m[0] = sum_r[t]; b[0] = batch_r[t];
+        }
+        c = count_r[t / s.gd];
+    };
+    if (first < per_stage) ask(first);
     float local = 0.0f;
-    for (int j = tid; j < s.K; j += 256) local += ema_count[(size_t)r * s.K + j];
-    red[tid] = local;
+    for (int j = tid; j < s.K; j += 256) local += count_r[j];
+    for (int off = 16; off > 0; off >>= 1) local += __shfl_xor_sync(0xFFFFFFFFu, local, off);
+    if ((tid & 31) == 0) red[tid >> 5] = local;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (tid < w) red[tid] += red[tid + w];
-        __syncthreads();
-    }
-    const float tot = red[0];
+    float tot = 0.0f;
+    for (int w = 0; w < 8; ++w) tot += red[w];
     const float scale = tot / (tot + (float)s.K * eps);
-    const int per_stage = s.K * s.gd;
-    for (int t = blockIdx.x * 256 + tid; t < per_stage; t += gridDim.x * 256) {
-        const size_t p = (size_t)r * per_stage + t;
-        const int j = t / s.gd;
-        const float mm = decay * ema_sum[p] + (1.0f - decay) * sum[p];
-        ema_sum[p] = mm;
-        cb[p] = mm / ((ema_count[(size_t)r * s.K + j] + eps) * scale);
+    for (int t = first; t < per_stage; t += gridDim.x * 256 * V) {
+        if (t != first) ask(t);
+        const float den = (c + eps) * scale;
+#pragma unroll
+        for (int i = 0; i < V; ++i) m[i] = fmaf(decay, m[i], (1.0f - decay) * b[i]);
+        if (V == 4) {
+            *reinterpret_cast<float4 *>(sum_r + t) = make_float4(m[0], m[1 % V], m[2 % V], m[3 % V]);
+            *reinterpret_cast<float4 *>(cb_r + t) = make_float4(m[0] / den, m[1 % V] / den, m[2 % V] / den, m[3 % V] / den);
+        } else {
+            sum_r[t] = m[0];
+            cb_r[t] = m[0] / den;
+        }
     }
 }
 
@@ -346,9 +367,12 @@ int launch_ema_apply(const Shape &s, const float *batch_count, const float *batc
     const int bins = s.R * s.K;
     int rc = launch_chained(chained, ema_count_kernel, dim3((bins + 255) / 256), 256, 0, stream, batch_count, ema_count, bins, decay);
     if (rc != RVQ_OK) return rc;
-    int parts = (s.K * s.gd + 256 * 8 - 1) / (256 * 8);
-    if (parts > 32) parts = 32;
-    return launch_chained(true, ema_apply_kernel, dim3(parts, s.R), 256, 0, stream, s, batch_sum, cb, ema_count, ema_sum, decay, eps);
+    const bool aligned = ((reinterpret_cast<uintptr_t>(batch_sum) | reinterpret_cast<uintptr_t>(cb) | reinterpret_cast<uintptr_t>(ema_sum)) & 15) == 0;
+    const int per_block = aligned ? 1024 : 256;
+    int parts = (s.K * s.gd + per_block - 1) / per_block;
+    if (parts > 64) parts = 64;
+    return launch_chained(true, aligned ? ema_apply_kernel<4> : ema_apply_kernel<1>, dim3(parts, s.R), 256, 0, stream, s, batch_sum, cb, ema_count,
+                          ema_sum, decay, eps);
 }
 
 }  // namespace rvq

@@ -116,10 +116,15 @@ prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
     for (int j = j0 + tid; j < j1; j += 256) {
         const float *e = cb + ((size_t)r * s.K + j) * s.gd;
         double acc = 0.0;
-        for (int i = 0; i < s.gd; ++i) {
-            const float v = e[i];
-            acc += (double)v * (double)v;
-            lo = fminf(lo, v); hi = fmaxf(hi, v);
+        auto add = [&](float v) { acc += (double)v * (double)v; lo = fminf(lo, v); hi = fmaxf(hi, v); };
+        if (s.gd == 32) {
+            float4 f[8];                                      // (asked for together)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = reinterpret_cast<const float4 *>(e)[q];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) { add(f[q].x); add(f[q].y); add(f[q].z); add(f[q].w); }
+        } else {
+            for (int i = 0; i < s.gd; ++i) add(e[i]);
         }
         m = fmax(m, acc);
     }
@@ -152,8 +157,9 @@ prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, St
     if (r < s.R) {
         double maxn = 0.0;
         float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
         for (int q = 0; q < kPrepareParts; ++q) {
-            const StagePartial &pp = part[r * kPrepareParts + q];
+            const StagePartial pp = part[r * kPrepareParts + q];
             maxn = fmax(maxn, pp.max_norm2); lo = fminf(lo, pp.lo); hi = fmaxf(hi, pp.hi);
         }
         int k = 12;
@@ -232,14 +238,23 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
     const int j = slot * kSlotCodewords + jj;            // padded codeword index
     const float scale = sp[r].scale;
     uint8_t *base = image + ((size_t)r * slots_per_stage(s.K) + slot) * kSlotStride;
-    __half cell[9][8];                                    // cells 0-8
+    __align__(16) __half cell[9][8];                      // cells 0-8
     __align__(16) uint8_t cell8[4][16] = {};              // cells 9-12
+#pragma unroll
     for (int c = 0; c < 9; ++c)
+#pragma unroll
         for (int i = 0; i < 8; ++i) cell[c][i] = __float2half_rn(0.0f);
     float emax = 0.f, eerr = 0.f, nmax = 0.f, elomax = 0.f;
+    float e[32];
     if (j < s.K) {
-        const float *e = cb + ((size_t)r * s.K + j) * 32;
+        const float4 *src = reinterpret_cast<const float4 *>(cb + ((size_t)r * s.K + j) * 32);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 f = src[q];
+            e[4 * q] = f.x; e[4 * q + 1] = f.y; e[4 * q + 2] = f.z; e[4 * q + 3] = f.w;
+        }
         double n2 = 0.0, l2 = 0.0, d2 = 0.0;
+#pragma unroll
         for (int i = 0; i < 32; ++i) {
             const double es = (double)e[i] * (double)scale;     // exact: power-of-two scale
             const __half hi = __double2half(es);
@@ -263,20 +278,24 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
     } else {
         cell[4][0] = __float2half_rn(60000.0f);           // padding never wins
     }
+#pragma unroll
     for (int c = 0; c < 13; ++c)
         *reinterpret_cast<uint4 *>(base + ((size_t)c * kSlotCodewords + jj) * 16) = c < 9 ? *reinterpret_cast<const uint4 *>(cell[c]) : *reinterpret_cast<const uint4 *>(cell8[c - 9]);
     if (blocks) {
         // the float32 block of this slot, piece by piece
         float4 *o = blocks + ((size_t)r * slots_per_stage(s.K) + slot) * (kFloatBlockBytes / 16) + jj;
-        const float4 *e = reinterpret_cast<const float4 *>(cb + ((size_t)r * s.K + j) * 32);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) o[q * kSlotCodewords] = j < s.K ? e[q] : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        for (int q = 0; q < 8; ++q) o[q * kSlotCodewords] = j < s.K ? make_float4(e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3]) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
     }
-    // non-negative floats order like their bit patterns
-    atomicMax(&mx[r].emax, __float_as_uint(emax));
-    atomicMax(&mx[r].eerr, __float_as_uint(eerr));
-    atomicMax(&mx[r].nmax, __float_as_uint(nmax));
-    atomicMax(&mx[r].elomax, __float_as_uint(elomax));
+    // non-negative floats order like their bit patterns (a NaN's is above all); one addition to the maxima per warp
+    const uint32_t b0 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(emax)), b1 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(eerr));
+    const uint32_t b2 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(nmax)), b3 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(elomax));
+    if ((jj & 31) == 0) {
+        atomicMax(&mx[r].emax, b0);
+        atomicMax(&mx[r].eerr, b1);
+        atomicMax(&mx[r].nmax, b2);
+        atomicMax(&mx[r].elomax, b3);
+    }
 }
 
 // |approximate score - exact score| <= a * ||Z|| + b for every codeword of the

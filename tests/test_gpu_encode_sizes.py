@@ -99,3 +99,18 @@ def test_statistics_of_few_tiles(n, dim, K, R, layout):
         want = torch.zeros(K, 32, dtype=torch.float64, device="cuda").index_add_(0, codes[:, r], z)
         assert (total[r].double() - want).abs().max() <= 1e-5 * max(1.0, want.abs().max().item())
         z = z - b.codebooks.view(R, K, 32)[r][codes[:, r]].double()
+
+
+@pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
+def test_update_of_buffers_that_are_not_aligned(K, gd):
+    """rvq_ema_apply on buffers that start 4 bytes past a 16-byte boundary equals that on aligned ones."""
+    g = torch.Generator(device="cuda").manual_seed(K)
+    cfg = rvq.make_config(gd * 4, gd, 0, 3, K, 16, rvq.F32, 0)
+    count, total = torch.rand(3, K, device="cuda", generator=g), torch.randn(3, K, gd, device="cuda", generator=g)
+    state = [torch.rand(3, K, device="cuda", generator=g) + 0.1, torch.randn(3, K, gd, device="cuda", generator=g), torch.zeros(3, K, gd, device="cuda")]
+    want = [t.clone() for t in state]
+    rvq.rvq_ema_apply(cfg, count, total, want[2], want[0], want[1], 0.9, 1e-5)
+    shifted = [torch.empty(t.numel() + 1, device="cuda")[1:].view(t.shape).copy_(t) for t in state + [total]]
+    rvq.rvq_ema_apply(cfg, count, shifted[3], shifted[2], shifted[0], shifted[1], 0.9, 1e-5)
+    for a, b in zip(shifted, want):
+        assert torch.equal(a, b)
