@@ -146,8 +146,9 @@ int rvq_encode(const rvq_config *cfg /* host */, const void *x, int64_t n, int64
  * Encode and, in the same pass, the EMA statistics of this batch (Section 3:
  * the codebooks are learnt from the encoder's own assignments, batch after
  * batch).  Results are those of rvq_encode followed by rvq_ema_stats on the
- * codes it produced: the residual entering every stage is already in registers
- * when its code is chosen, so x is not read and re-scaled a second time.
+ * codes it produced: with many vectors and codes the residual entering every stage is already on the
+ * chip when its code is chosen, so x is not read and re-scaled a second time; few tiles of vectors, or up to
+ * 640 codes, take the statistics in a kernel of their own, which is faster there.
  *   stage_energy out  optional [R], as under rvq_encode
  *   batch_count  out  float32 [R][K]             (overwritten)
  *   batch_sum    out  float32 [R][K][group_dim]  (overwritten; 16-byte aligned)
@@ -174,7 +175,9 @@ int rvq_encode_exact(const rvq_config *cfg /* host */, const void *x, int64_t n,
  * Decode (Section 2.2, last sentence; Section 3.2).  For every head vector and
  * channel c = channel(g, i): x_out[c] = std * sum_r C_r[code[g][r]][i], summed
  * in float32 and rounded once to x_dtype.  For groups of 32 (a power-of-two number
- * of them) with depth <= 8 the codebook entries are read from shared-memory tables: float32
+ * of them) with depth <= 8 the codebook entries are read from the float32 codebooks in L2 (four groups or
+ * more: few vectors, float32 outputs, more than 1536 codes or other depths than 8; exact float32 sums)
+ * or from shared-memory tables: float32
  * copies (up to 3584 codes per stage) or, for 16-bit outputs and up to 3072
  * codes, 16-bit levels of each stage's value range kept in the prepared block.
  * With the levels the sum before the multiplication by std is within
@@ -210,7 +213,9 @@ int rvq_decode(const rvq_config *cfg /* host */, const void *codes, const uint16
  *   cos_sin               in  device float32 [positions][dim/2][2], 16-byte aligned, e.g. from
  *                             rvq_rope_table
  *   prepared              in  block of rvq_prepare_codebooks for these codebooks, or NULL
- * Two or more groups of 32 (a power-of-two number) with depth <= 8: up to 3584 codes per stage float32
+ * Four or more groups of 32 (a power-of-two number) with depth <= 8 read the float32 codebooks in L2 (exact
+ * sums), but for many vectors of dim 128 at depth 8 with up to 1536 codes, 16-bit outputs and a prepared block.  Those,
+ * and two groups: up to 3584 codes per stage float32
  * shared-memory tables (exact float32 sums); with 16-bit outputs and a prepared block also
  * the level tables described under rvq_decode (dim 128 at depth 8 with up to 1536 codes:
  * both kinds of level table, 8-channel slices, one launch; 1537..3072 codes: the per-stage
@@ -254,7 +259,7 @@ int rvq_rope_table(int32_t dim, double base, int32_t positions, float *cos_sin /
  *                       the keys are used as stored
  *   out            out  device float32 [q_heads][128]
  *   workspace           rvq_attention_workspace_bytes(tokens, q_heads) bytes, 256-byte aligned
- * Arithmetic: float32 codeword tables in shared memory (exact float32 sums), float32
+ * Arithmetic: float32 codewords, from shared-memory tables or, up to 32768 tokens, from L2 (exact float32 sums), float32
  * dot products and weights; the order of the float32 sums over tokens and channel
  * slices is not fixed (reductions in global memory).  Codes >= K are read as code 0
  * and counted in status->bad_codes.  Other shapes: RVQ_ERR_UNSUPPORTED.
