@@ -259,7 +259,7 @@ int rvq_rope_table(int32_t dim, double base, int32_t positions, float *cos_sin /
  *                       the keys are used as stored
  *   out            out  device float32 [q_heads][128]
  *   workspace           rvq_attention_workspace_bytes(tokens, q_heads) bytes, 256-byte aligned
- * Arithmetic: float32 codewords, from shared-memory tables or, up to 32768 tokens, from L2 (exact float32 sums), float32
+ * Arithmetic: float32 codewords, from shared-memory tables or, up to 28672 tokens, from L2 (exact float32 sums), float32
  * dot products and weights; the order of the float32 sums over tokens and channel
  * slices is not fixed (reductions in global memory).  Codes >= K are read as code 0
  * and counted in status->bad_codes.  Other shapes: RVQ_ERR_UNSUPPORTED.

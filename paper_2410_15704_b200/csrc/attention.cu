@@ -656,9 +656,14 @@ att_combine_kernel(const float *part, const float2 *part_ml, int chunks, int lay
     out[head * 128 + (layout_v == RVQ_GROUP_STRIDED ? 4 * e + g : c)] = a / sum;
 }
 
-// Tokens up to which the one-pass kernel is the faster one.  Measured (us, tables / one pass, 32 query heads, K =
-// 1024): 1000 tokens 35 / 13, 8000 61 / 43, 16000 90 / 77, 131072 505 / 578.
-constexpr int64_t kShortTokens = 32768;
+// Tokens up to which the one-pass kernel is the faster one.  Measured (us, tables / one pass, K = 1024, depth 8): 32 query
+// heads 12000 tokens 75 / 62, 20000 103 / 94, 26000 123 / 119, 32768 146 / 146; 8 heads, packed 26000 126 / 125, 32768
+// 149 / 156.  With up to four stages on both sides the tables take half the reads: 12000 tokens 63 / 63, 20000 90 / 95.
+constexpr int64_t kShortTokens = 28672, kShortTokensShallow = 12288;
+bool short_wanted(const Shape &sk, const Shape &sv, int64_t tokens)
+{
+    return tokens <= (sk.R <= 4 && sv.R <= 4 ? kShortTokensShallow : kShortTokens);
+}
 
 // Chunks of a short cache: no more than its tokens feed.
 int short_chunks(int64_t tokens)
@@ -704,7 +709,7 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
     uint8_t *ws = reinterpret_cast<uint8_t *>(workspace);
-    if (tokens <= kShortTokens) {
+    if (short_wanted(sk, sv, tokens)) {
         const int chunks = short_chunks(tokens), rope = cos_sin ? (pairing == RVQ_ROPE_HALVES ? 1 : 2) : 0;
         float *part = reinterpret_cast<float *>(ws);
         float2 *part_ml = reinterpret_cast<float2 *>(ws + (size_t)chunks * q_heads * 128 * 4);

@@ -1,4 +1,4 @@
-"""GPU parity of the table kernels of rvq_attention_decode (caches of more than 32768 tokens) at the code widths,
+"""GPU parity of the table kernels of rvq_attention_decode (caches of more than 28672 tokens, 12288 with up to four stages) at the code widths,
 depths and query-head counts that take their own branch."""
 import pytest
 
@@ -11,7 +11,10 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("tokens, q_heads, depths, bits, K, layouts, pairing", [
     (32769, 32, (8, 8), (16, 16), 1024, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_HALVES),
-    (32800, 16, (4, 3), (9, 16), 300, (rvq_synth.CONTIGUOUS, rvq_synth.STRIDED), rvq.ROPE_HALVES),
+    (28672, 32, (8, 8), (16, 16), 256, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_HALVES),
+    (28673, 8, (8, 4), (16, 16), 256, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_HALVES),
+    (12288, 16, (4, 4), (8, 8), 256, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_HALVES),
+    (12289, 16, (4, 3), (9, 16), 300, (rvq_synth.CONTIGUOUS, rvq_synth.STRIDED), rvq.ROPE_HALVES),
     (33001, 8, (6, 8), (10, 16), 1000, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_ADJACENT),
     (32769, 32, (5, 4), (16, 8), 256, (rvq_synth.STRIDED, rvq_synth.STRIDED), rvq.ROPE_HALVES),
     (32769, 32, (1, 2), (1, 1), 2, (rvq_synth.STRIDED, rvq_synth.CONTIGUOUS), rvq.ROPE_HALVES),
