@@ -89,9 +89,10 @@ const char *rvq_status_string(int code);
 int rvq_version(void);
 
 /* Diagnostic: number of kernels this library has launched in this process so
- * far.  (Process-wide state of the library: this counter, and the per-device
- * address of the built-in scratch array that rvq_ema_update_static resolves on
- * its first call.) */
+ * far.  (Process-wide state of the library: this counter, what launches have
+ * asked about each device and context (SM count, shared memory granted to each
+ * kernel, resident clusters), and the per-device address of the built-in scratch
+ * array that rvq_ema_update_static resolves on its first call.) */
 uint64_t rvq_launch_count(void);
 
 /* Bytes of one head vector's codes in the configured storage form

@@ -1,10 +1,13 @@
 // extern "C" boundary of the RVQ library: argument checks on the host, then
 // dispatch to the kernels.  No allocation, no synchronisation.  Process-wide
 // state: the launch counter below, what is remembered about each device (its SM
-// count, the shared memory granted to each kernel), and (in ema.cu) the per-device
-// address of the built-in scratch array of rvq_ema_update_static.
+// count) and each context (the shared memory granted to each kernel), and (in
+// ema.cu) the per-device address of the built-in scratch array of
+// rvq_ema_update_static.
 #include "prepared.cuh"
 #include "rvq_selftest.h"
+
+#include <cuda.h>
 
 #include <atomic>
 
@@ -18,7 +21,7 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::atomic<int> g_sms[kMaxDevices];
 
-// What has been asked of the runtime about a kernel so far, per device: the largest dynamic shared memory
+// What has been asked of the runtime about a kernel so far, per context: the largest dynamic shared memory
 // granted to it, and how many clusters of 1 .. 8 CTAs run at a time (0: not asked, -1: none).  Open addressing
 // by the kernel's address; entries are only ever added.  Threads may race to ask the same thing twice.
 struct Grant {
@@ -27,14 +30,46 @@ struct Grant {
     std::atomic<int> clusters[9] = {};
 };
 constexpr int kGrantSlots = 512;                          // (a few times the library's number of kernels)
-Grant g_grants[8][kGrantSlots];
+// A grant is the context's: another context of the same device, or the primary one after a reset, starts without
+// any.  Contexts are told apart by the driver's number, which it never gives twice.  A process that has gone
+// through more contexts than there is room for asks the runtime on every launch in the further ones.
+constexpr int kContexts = 8;
+struct Context {
+    std::atomic<uint64_t> number{0};                      // the driver's, plus one
+    Grant grants[kGrantSlots];
+};
+Context g_contexts[kContexts];
 
-Grant *grant_of(const void *kernel, int dev)
+// The calling thread's context, as the driver's number for it plus one; 0 if it has none yet.
+uint64_t current_context()
 {
-    if (dev >= 8) return nullptr;
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    static const GetId get_id = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &fn, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+        if (!ok) cudaGetLastError();
+        return ok ? reinterpret_cast<GetId>(fn) : nullptr;
+    }();
+    unsigned long long number = 0;
+    return get_id && get_id(nullptr, &number) == CUDA_SUCCESS ? (uint64_t)number + 1 : 0;
+}
+
+Grant *grant_of(const void *kernel)
+{
+    const uint64_t number = current_context();
+    if (number == 0) return nullptr;
+    Grant *grants = nullptr;
+    for (int k = 0; k < kContexts && !grants; ++k) {
+        Context &c = g_contexts[k];
+        uint64_t have = c.number.load(std::memory_order_acquire);
+        if (have == 0 && c.number.compare_exchange_strong(have, number)) have = number;
+        if (have == number) grants = c.grants;
+    }
+    if (!grants) return nullptr;
     const uint32_t h = (uint32_t)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) >> 7;
     for (uint32_t k = 0; k < (uint32_t)kGrantSlots; ++k) {
-        Grant &g = g_grants[dev][(h + k) % kGrantSlots];
+        Grant &g = grants[(h + k) % kGrantSlots];
         const void *have = g.kernel.load(std::memory_order_acquire);
         if (have == nullptr && g.kernel.compare_exchange_strong(have, kernel)) have = kernel;
         if (have == kernel) return &g;
@@ -57,9 +92,7 @@ int sm_count()
 
 bool allow_shared_memory(const void *kernel, int bytes)
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return false;
-    Grant *g = grant_of(kernel, dev);
+    Grant *g = grant_of(kernel);
     if (g && g->bytes.load(std::memory_order_acquire) >= bytes) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
     if (g) {
@@ -84,9 +117,8 @@ static cudaLaunchConfig_t cluster_config(int clusters, int ctas, int threads, in
 
 int resident_clusters(const void *kernel, int ctas, int threads, int smem)
 {
-    int dev = -1;
-    if (ctas < 1 || ctas > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-    Grant *g = grant_of(kernel, dev);
+    if (ctas < 1 || ctas > 8) return 0;
+    Grant *g = grant_of(kernel);
     int have = g ? g->clusters[ctas].load(std::memory_order_acquire) : 0;
     if (have == 0) {
         cudaLaunchAttribute attr;

@@ -85,8 +85,8 @@ int launch_attention_decode(const Shape &sk, const Shape &sv, const float *q, in
 size_t prepared_bytes(const Shape &s);
 int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream, bool chained = false);
 
-// Facts about the current device that a launch needs, looked up once per device (and kernel) and
-// remembered: the three runtime queries they replace were a third of the host's time in a call.
+// Facts that a launch needs, looked up once per device or per context and kernel and remembered: the three
+// runtime queries they replace were a third of the host's time in a call.
 int sm_count();                                            // 0: no device
 bool allow_shared_memory(const void *kernel, int bytes);   // dynamic shared memory of up to `bytes` for this kernel
 
