@@ -32,7 +32,10 @@ bool from_python(PyObject *o, T *out)
         if (o == Py_None) {
             *out = nullptr;
         } else if (THPVariable_Check(o)) {
-            *out = reinterpret_cast<T>(const_cast<void *>(THPVariable_Unpack(o).const_data_ptr()));
+            // (a buffer that the call writes is asked for as such: a tensor that shares its storage until the
+            // first write gets storage of its own)
+            if constexpr (std::is_const_v<std::remove_pointer_t<T>>) *out = reinterpret_cast<T>(THPVariable_Unpack(o).const_data_ptr());
+            else *out = reinterpret_cast<T>(THPVariable_Unpack(o).mutable_data_ptr());
         } else if (PyLong_Check(o)) {
             *out = reinterpret_cast<T>(PyLong_AsVoidPtr(o));
         } else {
