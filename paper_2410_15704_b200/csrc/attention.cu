@@ -585,7 +585,8 @@ att_short_kernel(Shape sk, Shape sv, const float *__restrict__ q, const void *__
 #pragma unroll
         for (int x = 4; x > 0; x >>= 1) sc += __shfl_xor_sync(0xFFFFFFFFu, sc, x);
         sc *= scale_log2e;
-        const float m2 = fmaxf(m, sc), corr = exp2f(m - m2), w = exp2f(sc - m2);    // (the first token: exp2(-inf) = 0)
+        // (the first token: exp2(-inf) = 0; while no score is above -inf, so is every token's weight)
+        const float m2 = fmaxf(m, sc), top = m2 == -INFINITY ? 0.0f : m2, corr = exp2f(m - top), w = exp2f(sc - top);
         const bool moved = m2 != m;
         l = fmaf(l, corr, w);
         m = m2;

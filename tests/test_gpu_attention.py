@@ -103,6 +103,31 @@ def test_attention_at_cache_size_of_a_long_context_slice():
     print(f"attention over 16384 tokens: max-abs {err:.2e}")
 
 
+@pytest.mark.parametrize("tokens", [9, 700, 28673])
+@pytest.mark.parametrize("q_heads", [8, 16, 32])
+def test_attention_gives_a_score_of_minus_infinity_no_weight(tokens, q_heads):
+    """A key whose deviation is beyond binary16 is stored with an infinite one.  With codewords above zero and a
+    query below zero it scores -inf, and softmax gives it weight 0, wherever it comes in the cache."""
+    g = np.random.default_rng(tokens)
+    ck, sk, cbk = make_cache(g, tokens, 256, 8)
+    cv, sv, cbv = make_cache(g, tokens, 256, 8)
+    cbk = np.abs(cbk) + np.float32(0.01)
+    sk = sk.reshape(tokens, 8).copy()
+    sk[np.arange(tokens) % 3 != 2] = 0x7C00                              # two thirds of the tokens, the first ones among them
+    cfg = rvq.make_config(128, 32, rvq_synth.CONTIGUOUS, 8, 256, 16, rvq.BF16, 0)
+    q = -np.abs(g.normal(size=(q_heads, 128))).astype(np.float32) - np.float32(0.01)
+    ws_bytes = rvq.rvq_attention_workspace_bytes(tokens, q_heads)
+    ws, out = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda"), torch.full((q_heads, 128), 7.0, device="cuda")
+    rvq.rvq_attention_decode(cfg, cfg, torch.from_numpy(q).cuda(), q_heads, codes_to_device(cfg, ck), torch.from_numpy(sk.view(np.int16)).cuda(),
+                             codes_to_device(cfg, cv), torch.from_numpy(sv.view(np.int16)).cuda(), tokens, 8, torch.from_numpy(cbk).cuda(),
+                             torch.from_numpy(cbv).cuda(), None, None, 0, 0, 0.02, out, ws, ws_bytes)
+    torch.cuda.synchronize()
+    left = np.arange(2, tokens, 3)
+    rows = (left[:, None] * 8 + np.arange(8)).reshape(-1)                # head vectors of the tokens that count
+    ref = oracle.attention_decode(q, ck[rows], sk.reshape(-1)[rows], cv[rows], sv[rows], cbk, cbv, 8, 0.02, None)
+    assert np.abs(out.cpu().numpy() - ref).max() <= 2e-5 * max(1.0, np.abs(ref).max())
+
+
 def test_attention_counts_bad_codes_and_rejects_bad_arguments():
     g = np.random.default_rng(5)
     tokens = 64
