@@ -61,6 +61,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// Wait, when a role ends, for what it has left in flight (a phase of `bar` that a copy or a chain of MMAs will
+// complete): shared memory and TMEM stay the CTA's until then, also when its other waits have given up.  With nothing in
+// flight, as always at a regular end, this is one test of the barrier.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok = 0u;
+#pragma unroll 1
+    for (uint32_t it = 0; it < 100000u && !ok; ++it)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+}
+
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes)
 {
     // K-major, no swizzle: 8x16-byte core matrices; LBO steps along the

@@ -140,8 +140,9 @@ encode_small_kernel(const SmallParams p)
     bool ok = true;
     int buffer = 0;
     uint32_t full_par = 0;
+    int r = 0;
 #pragma unroll 1
-    for (int r = 0; r < R; ++r) {
+    for (; r < R; ++r) {
         const uint32_t par = (uint32_t)r & 1u;
         if (tid == 0) mbar_expect_tx(arrived0 + 8u * par, (uint32_t)(p.rows * slots * 8));
         ok = mbar_wait(smem_u32(&w.full[buffer]), full_par, &w.abort_flag);
@@ -215,7 +216,12 @@ encode_small_kernel(const SmallParams p)
         if (PER == 2 && tid == 0 && r >= 1 && r - 1 + kBuffers < R) copy_stage(r - 1 + kBuffers, r - 1);
         if (++buffer == kBuffers) { buffer = 0; full_par ^= 1u; }
     }
-    if (!ok && tid == 0 && p.st) atomicAdd(&p.st->wait_timeouts, 1u);
+    if (!ok && tid == 0) {
+        // (the stages from here on are still coming in)
+        for (int k = r; k < R && k < kBuffers + max(r - 1, 0); ++k)
+            mbar_drain(smem_u32(&w.full[k % kBuffers]), (uint32_t)(k / kBuffers) & 1u);
+        if (p.st) atomicAdd(&p.st->wait_timeouts, 1u);
+    }
     if (ctas > 1 && (p.energy || !ok))                            // (codewords of other CTAs were read last)
         asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     if (rank != 0) return;

@@ -120,12 +120,8 @@ encode_split_kernel(const SplitParams p)
                         ++issued;
                         if (++slot == (uint32_t)kSplitRing) { slot = 0; par ^= 1u; }
                     }
-            // (giving up: the copies in flight have to land before the CTA ends)
-            if (!ok)
-                for (uint32_t k = issued > (uint32_t)kSplitRing ? issued - kSplitRing : 0u; k < issued; ++k) {
-                    volatile uint32_t never = 0u;
-                    mbar_wait(BAR(kSFull + (int)(k % kSplitRing)), (k / kSplitRing) & 1u, &never, 100000u);
-                }
+            for (uint32_t k = issued > (uint32_t)kSplitRing ? issued - kSplitRing : 0u; k < issued; ++k)
+                mbar_drain(BAR(kSFull + (int)(k % kSplitRing)), (k / kSplitRing) & 1u);
         }
     } else if (warp == 12) {
         // ------------------------------------------------------------ MMA issuer
@@ -134,6 +130,7 @@ encode_split_kernel(const SplitParams p)
         uint32_t slot = 0, full_par = 0, ready_par = 0;
         uint32_t used = 0;                                                // accumulators used at least once (bit per accumulator)
         uint32_t free_pars = 0;                                           // next parity to wait for, bit per accumulator
+        uint32_t odd = 0;                                                 // chains issued are odd in number, bit per accumulator
         bool ok = true;
         const int stages = my_tiles * R;
         for (int st = 0; st < stages && ok; ++st) {
@@ -156,10 +153,12 @@ encode_split_kernel(const SplitParams p)
                     mma_commit(BAR(kSEmpty + slot));
                 }
                 __syncwarp();
+                odd ^= 1u << a;
                 if (++slot == (uint32_t)kSplitRing) { slot = 0; full_par ^= 1u; }
                 if (++a == P) a = 0;
             }
         }
+        for (int a = 0; a < kGroups; ++a) mbar_drain(BAR(kSAccFull + a), ~(odd >> a) & 1u);
     } else {
         // ------------------------------------------------------------ epilogue groups
         const int grp = warp >> 2, q4 = warp & 3;

@@ -42,8 +42,8 @@
 //     last stage's input is added by the epilogue warps.
 // TMEM columns of tile t: scores [160 t, 160 t + 128), A operand
 // [160 t + 128, 160 t + 160) (16 columns of head, 16 of remainder).
-// Every wait is bounded; a wait that gives up sets status->wait_timeouts and
-// the kernel drains and returns.
+// Every wait is bounded; a wait that gives up sets status->wait_timeouts, and
+// the kernel waits (bounded as well) for its copies and chains in flight and returns.
 #include "encode_mma.cuh"
 
 namespace rvq {
@@ -176,10 +176,9 @@ encode_tensor_kernel(const Params p)
             const uint32_t total = (uint32_t)my_passes * (uint32_t)s.R * (uint32_t)S;
             const uint32_t per_pass = (uint32_t)s.R * (uint32_t)S;
             uint32_t slot = 0, rs = 0, empty_par = 1;          // parity of the previous completion of empty[slot]
-            bool ok = true;
-            for (uint32_t nl = 0; nl < total && ok; ++nl) {
-                if (nl >= (uint32_t)kRing) ok = mbar_wait(BAR(kBarEmpty + slot), empty_par, abort_flag);
-                if (!ok) break;
+            uint32_t nl = 0;
+            for (; nl < total; ++nl) {
+                if (nl >= (uint32_t)kRing && !mbar_wait(BAR(kBarEmpty + slot), empty_par, abort_flag)) break;
                 mbar_expect_tx(BAR(kBarFull + slot), kSlotBytes);
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                              ::"r"(smem_u32(smem + kOffB) + slot * (uint32_t)kSlotBytes), "l"(image + (size_t)rs * kSlotStride),
@@ -187,6 +186,8 @@ encode_tensor_kernel(const Params p)
                 if (++rs == per_pass) rs = 0;
                 if (++slot == (uint32_t)kRing) { slot = 0; empty_par ^= 1u; }
             }
+            for (uint32_t k = nl > (uint32_t)kRing ? nl - kRing : 0u; k < nl; ++k)
+                mbar_drain(BAR(kBarFull + (int)(k % kRing)), (k / kRing) & 1u);
         }
     } else if (warp >= kEpiThreads / 32) {
         // ------------------------------------------------------------ MMA issuer of tile t
@@ -216,6 +217,7 @@ encode_tensor_kernel(const Params p)
             const uint16_t *codes_s = reinterpret_cast<const uint16_t *>(smem + kOffCodes);
             const uint8_t *flags_s = smem + kOffFlags;
             bool ok = true, first = true, active = t < work.round_size(0);
+            uint32_t last_par = 1;                                   // parity of this tile's last chain
             for (uint32_t q = 0; q < total && ok; ++q) {
                 ok = mbar_wait(BAR(kBarFull + slot), full_par, abort_flag);
                 ok = __all_sync(0xFFFFFFFFu, ok);
@@ -243,6 +245,7 @@ encode_tensor_kernel(const Params p)
                     mma_commit(BAR(kBarEmpty + slot));
                 }
                 __syncwarp();
+                last_par ^= 1u;
                 if (p.defer_stats && stage >= 1u && s_in >= 1u && s_in <= 4u) {
                     const int rl = t * 128 + (int)(s_in - 1u) * 32 + lane;
                     const uint32_t fl = flags_s[rl];
@@ -264,6 +267,7 @@ encode_tensor_kernel(const Params p)
                 if (++s_in == (uint32_t)S) { s_in = 0; ready_par ^= 1u; ++stage; }
                 if (++in_round == per_round) { in_round = 0; stage = 0; ++round; active = round < work.rounds && t < work.round_size(round); }
             }
+            mbar_drain(bar_acc, last_par);
         }
     } else {
         // ------------------------------------------------------------ epilogue warps
