@@ -1,9 +1,9 @@
-// Tensor-core encode of few row tiles (up to two per SM): one tile's codebook sweep split.
+// Tensor-core encode of few row tiles (up to one per SM): one tile's codebook sweep split.
 //
 // The throughput kernel (encode_tensor.cu) gives an SM three tiles of 128 rows and lets them share the
 // operand stream; with fewer tiles than three per SM most of the chip is idle and the tiles that run
 // wait, chunk after chunk, for one accumulator each (154 tiles: 145 us at 2048 codes, as long as one).
-// Here a tile belongs to a cluster of C CTAs (1, 2, 4 or 8: as many as keep every SM busy), each of
+// Here a tile belongs to a cluster of C CTAs (1 .. 8: split_ctas), each of
 // which sweeps its share of the stage's chunks with up to three accumulators in flight over one A operand.
 // An epilogue group of four warps per accumulator folds its chunks into running minima of the tile's
 // 128 rows (encode_mma.cuh), as the throughput kernel does for all chunks.  At the stage end every
@@ -55,7 +55,6 @@ struct SplitParams {
     uint16_t *std16;
     rvq_status *st;
     float *energy;
-    int tiles;
     int groups;         // accumulators in use: min(kGroups, chunks of a CTA)
 };
 
@@ -73,7 +72,6 @@ encode_split_kernel(const SplitParams p)
     // this CTA's chunks of every stage
     const int per = S / ctas, rem = S - per * ctas;
     const int base = rank * per + min(rank, rem), cnt = per + (rank < rem ? 1 : 0);
-    const int my_tiles = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const uint32_t bar0 = smem_u32(bars);
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
@@ -108,18 +106,17 @@ encode_split_kernel(const SplitParams p)
             const uint8_t *image = p.prepared + kPreparedImageOffset + (size_t)base * kSlotStride;
             uint32_t slot = 0, par = 1, issued = 0;
             bool ok = true;
-            for (int t = 0; t < my_tiles && ok; ++t)
-                for (int r = 0; r < R && ok; ++r)
-                    for (int c = 0; c < cnt && ok; ++c) {
-                        if (issued >= (uint32_t)kSplitRing) ok = mbar_wait(BAR(kSEmpty + slot), par, abort_flag);
-                        if (!ok) break;
-                        mbar_expect_tx(BAR(kSFull + slot), kSlotBytes);
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(smem_u32(smem + kSOffB) + slot * (uint32_t)kSlotBytes), "l"(image + ((size_t)r * S + c) * kSlotStride),
-                                       "r"((uint32_t)kSlotBytes), "r"(BAR(kSFull + slot)) : "memory");
-                        ++issued;
-                        if (++slot == (uint32_t)kSplitRing) { slot = 0; par ^= 1u; }
-                    }
+            for (int r = 0; r < R && ok; ++r)
+                for (int c = 0; c < cnt; ++c) {
+                    if (issued >= (uint32_t)kSplitRing) ok = mbar_wait(BAR(kSEmpty + slot), par, abort_flag);
+                    if (!ok) break;
+                    mbar_expect_tx(BAR(kSFull + slot), kSlotBytes);
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(smem_u32(smem + kSOffB) + slot * (uint32_t)kSlotBytes), "l"(image + ((size_t)r * S + c) * kSlotStride),
+                                   "r"((uint32_t)kSlotBytes), "r"(BAR(kSFull + slot)) : "memory");
+                    ++issued;
+                    if (++slot == (uint32_t)kSplitRing) { slot = 0; par ^= 1u; }
+                }
             for (uint32_t k = issued > (uint32_t)kSplitRing ? issued - kSplitRing : 0u; k < issued; ++k)
                 mbar_drain(BAR(kSFull + (int)(k % kSplitRing)), (k / kSplitRing) & 1u);
         }
@@ -132,8 +129,7 @@ encode_split_kernel(const SplitParams p)
         uint32_t free_pars = 0;                                           // next parity to wait for, bit per accumulator
         uint32_t odd = 0;                                                 // chains issued are odd in number, bit per accumulator
         bool ok = true;
-        const int stages = my_tiles * R;
-        for (int st = 0; st < stages && ok; ++st) {
+        for (int r = 0; r < R && ok; ++r) {
             ok = mbar_wait(BAR(kSReady), ready_par, abort_flag);
             ready_par ^= 1u;
             int a = 0;
@@ -172,20 +168,17 @@ encode_split_kernel(const SplitParams p)
         const int nparts = ctas * P;
         const uint32_t mine = smem_u32(smem + kSOffParts) + (uint32_t)((rank * P + grp) * 128 + row) * 16u;
         const int G = s.G;
-        uint32_t acc_par = 0, stage_no = 0;
+        uint32_t acc_par = 0;
         uint32_t n_rescored = 0, n_exhaustive = 0, n_degenerate = 0, n_stdrange = 0;
         bool ok = true;
-        const int todo_tiles = grp < P ? my_tiles : 0;                                    // (groups without an accumulator sit by)
-        // (every warp of the groups meets both barriers of every tile, given up or not)
-        for (int t = 0; t < todo_tiles; ++t) {
-            const int64_t row0 = ((int64_t)blockIdx.x + (int64_t)t * gridDim.x) * 128;
+        if (grp < P) {                                                                    // (groups without an accumulator sit by)
+            const int64_t row0 = (int64_t)blockIdx.x * 128;
             const int64_t v_tile = row0 / G, v_first = v_tile + q4 * 32 / G;
             const int64_t v = v_first + lane / G;
             const bool valid = v < p.n;
             bool deg = true;
             // the tile's head vectors, widened, by all groups: element i of row at [i][row]
-            if (t > 0) asm volatile("bar.sync 1, %0;" ::"r"(128 * P) : "memory");     // (the owners are through with the last tile's)
-            if (ok) {
+            {
                 const int eb = s.elem_bytes, ppv = s.dim * eb / 16, per_piece = 16 / eb, lg = __ffs(G) - 1;
                 float *zs = reinterpret_cast<float *>(smem + kSOffZ);
                 for (int k = tid; k < (128 >> lg) * ppv; k += 128 * P) {
@@ -208,17 +201,17 @@ encode_split_kernel(const SplitParams p)
                 }
             }
             asm volatile("bar.sync 1, %0;" ::"r"(128 * P) : "memory");
-            if (ok && grp == 0) {
+            if (grp == 0) {
                 // (the residual lives in shared memory between its uses: in registers it would be live across the sweep)
                 float z[32];
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z[i] = z_park[i * kZPitch];
                 const float dev = group_deviation(s, z, lane);
-                deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
-                if (!s.raw) divide_row(z, dev, deg);
+                deg = deviation_is_degenerate(dev) || !valid;
+                divide_row(z, dev, deg);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kZPitch] = deg ? 0.0f : z[i];
-                if (valid && (lane & (G - 1)) == 0 && !s.raw && rank == 0) {
+                if (valid && (lane & (G - 1)) == 0 && rank == 0) {
                     const uint16_t hb = deviation_is_degenerate(dev) ? (uint16_t)0 : __half_as_ushort(__float2half_rn(dev));
                     p.std16[v] = hb;
                     if (deviation_is_degenerate(dev)) ++n_degenerate;
@@ -226,10 +219,10 @@ encode_split_kernel(const SplitParams p)
                 }
             }
 #pragma unroll 1
-            for (int r = 0; r < R && ok; ++r, ++stage_no) {
+            for (int r = 0; r < R && ok; ++r) {
                 const StageParams prm = sp[r];
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
-                const uint32_t par = stage_no & 1u;
+                const uint32_t par = (uint32_t)r & 1u;
                 Sweep w;
                 w.m1 = w.m2 = w.m3 = INFINITY;
                 w.c1 = w.c2 = 0;
@@ -290,7 +283,7 @@ encode_split_kernel(const SplitParams p)
                                        "r"(__float_as_uint(w.m2)), "r"(sets), "r"((uint32_t)w.c1 | ((uint32_t)w.c2 << 16)),
                                        "r"(map_to(BAR(kSArrived + par), (uint32_t)to)) : "memory");
                 }
-                ok = mbar_wait(BAR(kSArrived + par), (stage_no >> 1) & 1u, abort_flag);
+                ok = mbar_wait(BAR(kSArrived + par), (uint32_t)(r >> 1) & 1u, abort_flag);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok || grp != 0) continue;
 
@@ -375,7 +368,6 @@ encode_split_kernel(const SplitParams p)
             if (ok && grp == 0) {
                 __syncwarp();
                 if (rank == 0) emit_codes(s, codes_s + q4 * 32 * 16, v_first, p.n, lane, p.codes);
-                __syncwarp();
             }
         }
         if (p.st) {
@@ -435,10 +427,9 @@ int launch_encode_split(const Shape &s, const void *x, int64_t n, int64_t stride
     const void *kernel = reinterpret_cast<const void *>(encode_split_kernel);
     if (ctas <= 0 || !allow_shared_memory(kernel, kSplitSmem)) return RVQ_ERR_LAUNCH;
     const int per = (slots_per_stage(s.K) + ctas - 1) / ctas;
-    SplitParams p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, energy, tiles,
-                  per < kGroups ? per : kGroups};
+    SplitParams p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, energy, per < kGroups ? per : kGroups};
     void *args[] = {&p};
-    return launch_clusters(kernel, tiles < sms ? tiles : sms, ctas, kSplitThreads, kSplitSmem, stream, args);
+    return launch_clusters(kernel, tiles, ctas, kSplitThreads, kSplitSmem, stream, args);
 }
 
 }  // namespace rvq
