@@ -356,11 +356,6 @@ int launch_stats_finish(const Shape &s, const uint32_t *cnt, const float *cb, fl
     return launch_chained(true, stats_finish_kernel, dim3((total + 255) / 256), 256, 0, stream, cnt, cb, batch_sum, batch_count, bins, s.gd, deferred * s.K);
 }
 
-int launch_counts_to_float(const uint32_t *cnt, float *out, int bins, cudaStream_t stream)
-{
-    return launch_chained(false, counts_to_float_kernel, dim3((bins + 255) / 256), 256, 0, stream, cnt, out, bins);
-}
-
 int launch_ema_apply(const Shape &s, const float *batch_count, const float *batch_sum, float *cb,
                      float *ema_count, float *ema_sum, float decay, float eps, cudaStream_t stream, bool chained)
 {
