@@ -1,19 +1,21 @@
-// Bandwidth decode for groups of 32 (a power-of-two number of them per head
-// vector; written around dim 128 = 4 groups), depth <= 8 (Section 2.2, last
-// sentence; Section 3.2).
+// Decode through tables in shared memory, for groups of 32 (a power-of-two number of them per head vector),
+// depth <= 8 (Section 2.2, last sentence; Section 3.2): the shapes and sizes for which codewords straight from L2
+// (decode_direct.cu) are slower or not built -- many vectors of 128 channels at depth 8 with 16-bit outputs and up to
+// 1536 codes (decode_quoted_kernel, decode_rope_quoted_kernel), of eight and more groups likewise, and head
+// vectors of one or two groups (decode_sliced_kernel, decode_rope_kernel).
 //
 // Every output element needs one codeword element per stage, so a head vector of
 // 128 channels (256 output bytes) gathers 1024 table entries: the gather, not HBM, is the
 // limit, and it has to come from shared memory without bank conflicts.
 //   - A CTA keeps one channel slice (CH = 8 of the 32 codeword channels, 4 when
 //     there are more than 1536 codes per stage) of all stages as 16-bit levels:
-//     16 CH bytes per code = 8 stages x 2 CH bytes.  The 32 / CH slices of a row
-//     tile are handled by as many CTAs; the codes they share come from L2.
+//     16 CH bytes per code = 8 stages x 2 CH bytes; or 4 (2) channels as float32.  The 32 / CH
+//     slices of a row tile are handled by as many CTAs; the codes they share come from L2.
 //   - One thread produces the CH channels of one (group row, slice).  It reads
 //     its codes as one 16-byte load (or cuts them out of the packed bit stream) and
-//     visits the stages in an order rotated by its lane, so with CH = 8 the 8
+//     visits the stages in an order rotated by its lane, so with 16-byte entries the 8
 //     lanes of a quarter warp always touch 8 different 16-byte bank groups
-//     whatever the codes are (with CH = 4 two lanes of a half warp can meet).
+//     whatever the codes are (with 8-byte ones two lanes of a half warp can meet).
 //   - A table entry is a 16-bit level q of its stage's value range, whose unit is
 //     an integer multiple (1..255) of a base common to all stages.  One 16-bit x
 //     8-bit dot-product instruction per channel and stage accumulates q * scale
@@ -24,8 +26,8 @@
 //     the deviation.  A row whose deviation makes that more than 0.9e-3 sums the
 //     float32 codewords instead (stage order, from global memory), so the result
 //     before the output rounding is always within 1e-3 of the exact sum.
-//   - With strided groups the 4 lanes of a head vector exchange their results so
-//     that every lane stores 16 contiguous bytes.
+//   - With four strided groups the 4 lanes of a head vector exchange their results so
+//     that every lane stores 16 (or 8) contiguous bytes; other strided shapes store element by element.
 #include "prepared.cuh"
 
 namespace rvq {
@@ -70,7 +72,7 @@ __device__ __forceinline__ void cut_codes(uint32_t u0, uint32_t u1, uint32_t u2,
 struct RopeArgs {
     const int32_t *position;      // position of head vector v: position[v / per_position]
     int per_position;
-    const float2 *table;          // (cos, sin) [positions][64]
+    const float2 *table;          // (cos, sin) [positions][dim / 2]
     int positions;
     int shift;                    // log2(per_position) when that is a power of two, else -1
 };
@@ -84,9 +86,9 @@ __device__ __forceinline__ int slice_element(int layout, int slice, int i)
     return slice * CH + i;
 }
 
-// ROPE (float32 tables with 4-channel slices only): the rotary embedding is applied to the decoded
-// head vector before it is rounded and stored (1: pairs are channels (k, k + 64), 2: (2k, 2k + 1)).
-// Both channels of a pair are in one thread, or in two lanes of the head vector's four, for every
+// ROPE (4- or 2-channel slices): the rotary embedding is applied to the decoded
+// head vector before it is rounded and stored (1: pairs are channels (k, k + dim / 2), 2: (2k, 2k + 1)).
+// Both channels of a pair are in one thread, or in two lanes of the head vector's, for every
 // combination but one: strided groups with half-split pairs, where the partner of element i of a
 // group is element i + 16 of the same group.  There a slice is the elements {2 sl, 2 sl + 1,
 // 2 sl + 16, 2 sl + 17} instead of four consecutive ones.
@@ -163,8 +165,7 @@ decode_sliced_body(const Shape &s, const void *__restrict__ codes, const uint16_
     const float exact_above = F32T ? INFINITY : (dp->err > 0.0f ? (ROPE != 0 ? 0.6e-3f : 0.9e-3f) / dp->err : INFINITY);
     __syncthreads();
 
-    // dim = 32 G with G a power of two; the stores of strided groups below are written for G = 4 (dim 128),
-    // other G store element by element
+    // dim = 32 G with G a power of two
     const int gs = __ffs(s.G) - 1;
     const int64_t rows = n << gs;
     uint32_t bad = 0;
@@ -372,112 +373,32 @@ decode_sliced_body(const Shape &s, const void *__restrict__ codes, const uint16_
                 }
             }
         }
-        if (s.G != 4 && s.layout == RVQ_GROUP_STRIDED) {
+        if (live && s.layout == RVQ_GROUP_STRIDED) {
             // channel of place i: element * G + g
-            if (live) {
 #pragma unroll
-                for (int i = 0; i < CH; ++i)
-                    store_from_float(out, v * stride + (int64_t)slice_element<CH, ROPE>(s.layout, slice, i) * s.G + g, DT, o8[i]);
-            }
-        } else if constexpr (CH == 2) {
-            // two places per thread
-            if (DT == RVQ_F32) {
-                float *o = reinterpret_cast<float *>(out) + v * stride;
-                if (s.layout == RVQ_GROUP_CONTIGUOUS) {
-                    if (live) *reinterpret_cast<float2 *>(o + g * 32 + slice * 2) = make_float2(o8[0], o8[1]);
-                } else if (live) {
-                    o[4 * slice_element<CH, ROPE>(s.layout, slice, 0) + g] = o8[0];
-                    o[4 * slice_element<CH, ROPE>(s.layout, slice, 1) + g] = o8[1];
-                }
-            } else {
-                const uint32_t w0 = Out<DT == RVQ_F32 ? RVQ_BF16 : DT>::pack(o8[0], o8[1]);
-                uint16_t *o16 = reinterpret_cast<uint16_t *>(out) + v * stride;
-                if (s.layout == RVQ_GROUP_CONTIGUOUS) {
-                    if (live) *reinterpret_cast<uint32_t *>(o16 + g * 32 + slice * 2) = w0;
-                } else {
-                    // Lane g holds places 0 and 1 of group g; the four lanes cover, per place, the four
-                    // consecutive channels 4 element .. 4 element + 3.  Lane L stores two of them: place L / 2,
-                    // groups 2 (L % 2) and 2 (L % 2) + 1, fetched from those two lanes.
-                    const int base_lane = (tid & 31) & ~3, ga = 2 * (g & 1);
-                    const uint32_t wa = __shfl_sync(0xFFFFFFFFu, w0, base_lane + ga);
-                    const uint32_t wb = __shfl_sync(0xFFFFFFFFu, w0, base_lane + ga + 1);
-                    const uint32_t both = __byte_perm(wa, wb, (g & 2) ? 0x7632 : 0x5410);
-                    if (live)
-                        *reinterpret_cast<uint32_t *>(o16 + 4 * slice_element<CH, ROPE>(s.layout, slice, g >> 1) + ga) = both;
-                }
-            }
-        } else {
-            if (DT == RVQ_F32) {
-                if (s.layout == RVQ_GROUP_CONTIGUOUS) {
-                    if (live) {
-                        float4 *o = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + v * stride + g * 32 + slice * CH);
-    #pragma unroll
-                        for (int i = 0; i < CH / 4; ++i)
-                            o[i] = make_float4(o8[4 * i], o8[4 * i + 1], o8[4 * i + 2], o8[4 * i + 3]);
-                    }
-                } else if (live) {
-                    float *o = reinterpret_cast<float *>(out) + v * stride + g;
-    #pragma unroll
-                    for (int i = 0; i < CH; ++i) o[4 * slice_element<CH, ROPE>(s.layout, slice, i)] = o8[i];   // channel 4 element + g
-                }
-            } else {
-                uint32_t w[CH / 2];
-    #pragma unroll
-                for (int c = 0; c < CH / 2; ++c) w[c] = Out<DT == RVQ_F32 ? RVQ_BF16 : DT>::pack(o8[2 * c], o8[2 * c + 1]);
-                uint16_t *o16 = reinterpret_cast<uint16_t *>(out) + v * stride;
-                if (s.layout == RVQ_GROUP_CONTIGUOUS) {
-                    if (live) {
-                        if (CH == 8)
-                            *reinterpret_cast<uint4 *>(o16 + g * 32 + slice * 8) = make_uint4(w[0], w[1], w[CH / 2 - 2], w[CH / 2 - 1]);
-                        else
-                            *reinterpret_cast<uint2 *>(o16 + g * 32 + slice * 4) = make_uint2(w[0], w[1]);
-                    }
-                } else if (CH == 8) {
-                    // Lane g holds element pairs (2c, 2c+1) of group g, i.e. channels 32 slice + 8c + g and + 4.
-                    // Lane c' of the 4-lane set wants pairs c' of all four groups: a 4x4 transpose of words.
-                    // two butterfly steps: exchange odd/even words with lane g^1, then word pairs with lane g^2
-                    uint32_t &w0 = w[0], &w1 = w[1], &w2 = w[CH / 2 - 2], &w3 = w[CH / 2 - 1];
-                    {
-                        const bool b1 = g & 1, b2 = g & 2;
-                        const uint32_t r0 = __shfl_xor_sync(0xFFFFFFFFu, b1 ? w0 : w1, 1);
-                        const uint32_t r1 = __shfl_xor_sync(0xFFFFFFFFu, b1 ? w2 : w3, 1);
-                        if (b1) { w0 = r0; w2 = r1; } else { w1 = r0; w3 = r1; }
-                        const uint32_t r2 = __shfl_xor_sync(0xFFFFFFFFu, b2 ? w0 : w2, 2);
-                        const uint32_t r3 = __shfl_xor_sync(0xFFFFFFFFu, b2 ? w1 : w3, 2);
-                        if (b2) { w0 = r2; w1 = r3; } else { w2 = r2; w3 = r3; }
-                    }
-                    // now w[q] = pair g of group q: (element 2g of group q, element 2g+1 of group q)
-                    const uint32_t o0 = __byte_perm(w0, w1, 0x5410), o1 = __byte_perm(w2, w3, 0x5410);
-                    const uint32_t o2 = __byte_perm(w0, w1, 0x7632), o3 = __byte_perm(w2, w3, 0x7632);
-                    // channels 32 slice + 8 g + 0..7: element 2g of groups 0..3, then element 2g+1 of groups 0..3
-                    if (live) *reinterpret_cast<uint4 *>(o16 + slice * 32 + g * 8) = make_uint4(o0, o1, o2, o3);
-                } else {
-                    // Lane g holds elements 4 slice + 0..3 of group g as w[0] = (e0, e1), w[1] = (e2, e3); the
-                    // 16 channels 16 slice .. 16 slice + 15 are element-major, so lane L stores element L of
-                    // the four groups.  Exchange words with lane g^2, then halves with lane g^1.
-                    const bool b1 = g & 1, b2 = g & 2;
-                    const uint32_t r0 = __shfl_xor_sync(0xFFFFFFFFu, b2 ? w[0] : w[1], 2);
-                    // lanes 0, 1 now hold (e0, e1) of groups g and g + 2; lanes 2, 3 hold (e2, e3) of g - 2 and g
-                    const uint32_t lo_g = b2 ? r0 : w[0], hi_g = b2 ? w[1] : r0;   // lower and upper group of the pair
-                    // keep the half this lane stores (e_L), send the other one
-                    const uint32_t keep = __byte_perm(lo_g, hi_g, b1 ? 0x7632 : 0x5410);
-                    const uint32_t send = __byte_perm(lo_g, hi_g, b1 ? 0x5410 : 0x7632);
-                    const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, send, 1);
-                    // keep = element L of groups (g & 1) and (g & 1) + 2, got = element L of the other two
-                    const uint32_t even = b1 ? got : keep, odd = b1 ? keep : got;   // groups (0, 2) and (1, 3)
-                    if (live)
-                        *reinterpret_cast<uint2 *>(o16 + 4 * slice_element<CH, ROPE>(s.layout, slice, g)) =
-                            make_uint2(__byte_perm(even, odd, 0x5410), __byte_perm(even, odd, 0x7632));
-                }
-            }
-    
+            for (int i = 0; i < CH; ++i)
+                store_from_float(out, v * stride + (int64_t)slice_element<CH, ROPE>(s.layout, slice, i) * s.G + g, DT, o8[i]);
+        } else if (live && DT == RVQ_F32) {
+            float *o = reinterpret_cast<float *>(out) + v * stride + g * 32 + slice * CH;
+            if (CH == 2) *reinterpret_cast<float2 *>(o) = make_float2(o8[0], o8[1]);
+#pragma unroll
+            for (int i = 0; i < CH / 4; ++i)
+                reinterpret_cast<float4 *>(o)[i] = make_float4(o8[4 * i], o8[4 * i + 1], o8[4 * i + 2], o8[4 * i + 3]);
+        } else if (live) {
+            uint32_t w[CH / 2];
+#pragma unroll
+            for (int c = 0; c < CH / 2; ++c) w[c] = Out<DT == RVQ_F32 ? RVQ_BF16 : DT>::pack(o8[2 * c], o8[2 * c + 1]);
+            uint16_t *o16 = reinterpret_cast<uint16_t *>(out) + v * stride + g * 32 + slice * CH;
+            if (CH == 8) *reinterpret_cast<uint4 *>(o16) = make_uint4(w[0], w[1 % (CH / 2)], w[CH / 2 - 2 > 0 ? CH / 2 - 2 : 0], w[CH / 2 - 1]);
+            else if (CH == 4) *reinterpret_cast<uint2 *>(o16) = make_uint2(w[0], w[1 % (CH / 2)]);
+            else *reinterpret_cast<uint32_t *>(o16) = w[0];
         }
     }
     if (bad && st && slice == 0) atomicAdd(&st->bad_codes, bad);   // every slice sees the same codes
 }
 
 // The level-table decoder for the shapes the timings are quoted on: head vectors of four groups of 32
-// (dim 128), depth 8, 16-bit outputs; codes as uint16 or as a packed stream of 10 to 12 bits.  Same
+// (dim 128), depth 8, 16-bit outputs; codes as uint16 or as a packed stream of 10 or 11 bits.  Same
 // tables, same arithmetic and same results as decode_sliced_body<DT, CH, false>; what differs is the
 // instruction count (the loop is issue bound): 32-bit row numbers, table addresses cut out of the
 // code words with one shift and one mask-or each, one scale register per stage for both halves of
@@ -969,8 +890,9 @@ decode_rope_quoted_kernel(Shape s, const void *__restrict__ codes, const uint16_
         decode_levels_fast<DT, 8, LAYOUT, BITS, true, ROPE>(s, codes, std16, n, dsec, cb, out, stride, st, table, ra);
 }
 
-// Decode with the rotary embedding, 4-channel slices (dim 128): float32 tables up to 1792 codes per stage,
-// 16-bit level tables (16-bit outputs) up to 3072.
+// Decode with the rotary embedding of head vectors of two groups (four and more go through decode_direct.cu or the
+// quoted kernel): float32 tables up to 1792 codes per stage with 4-channel slices, up to 3584 with 2-channel ones;
+// level tables (16-bit outputs, a prepared block) from 1537 to 3072.
 template <int DT, int ROPE, int CH, bool F32T, int PICK>
 __global__ void __launch_bounds__(kDecThreads, 1)
 decode_rope_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t n,
