@@ -82,11 +82,11 @@ def test_decode_bandwidth_full_size(layout):
     (2048, 16, rvq_synth.STRIDED, "f16"), (1537, 11, rvq_synth.CONTIGUOUS, "f16"),
     (3072, 12, rvq_synth.STRIDED, "bf16"), (1536, 11, rvq_synth.STRIDED, "bf16"),
     (3073, 12, rvq_synth.CONTIGUOUS, "bf16"),
-    (2048, 11, rvq_synth.CONTIGUOUS, "f32"), (2048, 16, rvq_synth.STRIDED, "f32"),      # float32 tables, 2-channel slices
+    (2048, 11, rvq_synth.CONTIGUOUS, "f32"), (2048, 16, rvq_synth.STRIDED, "f32"),
     (3584, 12, rvq_synth.STRIDED, "f16"), (3585, 12, rvq_synth.STRIDED, "f32"),
 ])
 def test_decode_large_codebooks(K, bits, layout, dtype):
-    """More than 1536 codes per stage: narrow table slices (up to 3072 codes), gathers beyond."""
+    """More than 1536 codes per stage, any output type: codewords from L2, ragged numbers of vectors."""
     w = rvq_synth.decode_bandwidth(tokens=1111, size=K, layout=layout)      # 8888 vectors: ragged tiles
     cfg = rvq.make_config(w.dim, w.group_dim, layout, w.depth, K, bits, DT[dtype], 0)
     got, st = gpu_decode(cfg, w.codes, w.std_bits, w.codebooks, w.n)
@@ -98,8 +98,8 @@ def test_decode_large_codebooks(K, bits, layout, dtype):
 @pytest.mark.parametrize("K,layout,every", [(1024, rvq_synth.CONTIGUOUS, 3), (1024, rvq_synth.STRIDED, 20),
                                             (2048, rvq_synth.STRIDED, 3)])
 def test_decode_large_deviations_take_the_exact_route(K, layout, every):
-    """Rows whose deviation would scale the level tables' error past 1e-3 sum float32 codewords:
-    one by one when they are few, through float32 tables when they are many (K <= 1536)."""
+    """Rows whose deviation would scale a level table's error past 1e-3.  At this size the codewords come from L2 and all
+    sums are exact; test_gpu_decode_tables.py has such rows, few and many, among tables."""
     w = rvq_synth.decode_bandwidth(tokens=700, size=K, layout=layout)
     sd = oracle.f16_value(w.std_bits)
     sd[::every] *= 64.0                                 # table error would be ~1e-2 on these rows
@@ -122,7 +122,7 @@ def test_decode_large_deviations_take_the_exact_route(K, layout, every):
     (512, 300, 9, rvq_synth.CONTIGUOUS, "f16", 1.0),
 ])
 def test_decode_other_head_sizes(dim, K, bits, layout, dtype, std_scale):
-    """Head vectors of 2, 8 and 16 groups of 32 (head_dim 64, 256, 512) on the table kernels."""
+    """Head vectors of 2 (table kernels), 8 and 16 groups of 32 (codewords from L2): head_dim 64, 256, 512."""
     g = np.random.default_rng(dim + K + layout)
     n, G, R = 1531, dim // 32, 8
     codes = g.integers(0, K, size=(n, G, R)).astype(np.int32)

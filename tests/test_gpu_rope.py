@@ -65,7 +65,8 @@ def run_case(dim, gd, R, K, bits, layout, dtype, pairing, tokens=333, heads=8, m
 @pytest.mark.parametrize("pairing", [rvq.ROPE_HALVES, rvq.ROPE_ADJACENT])
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_decode_rope_table_path(layout, pairing, dtype):
-    """dim 128, 1024 codes: float32 shared-memory tables; all four pairings of layout and convention."""
+    """dim 128, 1024 codes; all four pairings of layout and convention.  (As many vectors as here take their codewords
+    from L2, exact float32 sums; test_gpu_decode_tables.py has the sizes that go through tables.)"""
     err = run_case(128, 32, 8, 1024, 16, layout, dtype, pairing)
     print(f"rope layout {layout} pairing {pairing} {dtype}: max-abs {err:.2e}")
 
@@ -91,11 +92,12 @@ def test_decode_rope_other_shapes(dim, gd, R, K, bits, layout, dtype, pairing):
 @pytest.mark.parametrize("layout", [rvq_synth.CONTIGUOUS, rvq_synth.STRIDED])
 @pytest.mark.parametrize("pairing", [rvq.ROPE_HALVES, rvq.ROPE_ADJACENT])
 def test_decode_rope_level_tables(layout, pairing):
-    """2048 and 3072 codes with 16-bit outputs: level tables; large deviations take float32 sums."""
+    """2048 codes and more, moderate and large deviations, with and without a prepared block: exact float32 sums whatever
+    the deviations.  (Level tables with that many codes: head vectors of two groups, test_gpu_decode_tables.py.)"""
     run_case(128, 32, 8, 2048, 11, layout, "bf16", pairing, tokens=211)
     run_case(128, 32, 8, 3072, 12, layout, "f16", pairing, tokens=57)
     run_case(128, 32, 8, 2048, 16, layout, "bf16", pairing, tokens=57, std_scale=40.0)
-    # float32 tables with 2-channel slices: float32 outputs, and 16-bit outputs without a prepared block
+    # float32 outputs, and 16-bit outputs without a prepared block
     run_case(128, 32, 8, 2048, 11, layout, "f32", pairing, tokens=57)
     run_case(128, 32, 8, 3584, 12, layout, "bf16", pairing, tokens=57, with_prepared=False)
 
@@ -103,9 +105,9 @@ def test_decode_rope_level_tables(layout, pairing):
 @pytest.mark.parametrize("layout", [rvq_synth.CONTIGUOUS, rvq_synth.STRIDED])
 @pytest.mark.parametrize("pairing", [rvq.ROPE_HALVES, rvq.ROPE_ADJACENT])
 def test_decode_rope_quoted_shapes_take_every_kind_of_table(layout, pairing):
-    """dim 128, depth 8, up to 1536 codes, 16-bit outputs and a prepared block: one launch that picks the
-    summed levels (small deviations), the per-stage levels (moderate), or the float32 tables (large); uint16
-    and packed codes; a mixed batch sends single rows down the exact route."""
+    """dim 128, depth 8, up to 1536 codes, 16-bit outputs and a prepared block, deviations of every kind of table, uint16
+    and packed codes, at sizes below the line from which on the tables are used (test_gpu_decode_tables.py is past it):
+    the same call has to hold the same bound on both sides."""
     for std_scale in (0.3, 1.0, 3.0, 40.0):
         run_case(128, 32, 8, 1024, 16, layout, "bf16", pairing, tokens=333, std_scale=std_scale)
     run_case(128, 32, 8, 1024, 10, layout, "f16", pairing, tokens=131, std_scale=0.3)
