@@ -148,8 +148,8 @@ int rvq_encode(const rvq_config *cfg /* host */, const void *x, int64_t n, int64
  * the codebooks are learnt from the encoder's own assignments, batch after
  * batch).  Results are those of rvq_encode followed by rvq_ema_stats on the
  * codes it produced: with many vectors and codes the residual entering every stage is already on the
- * chip when its code is chosen, so x is not read and re-scaled a second time; few tiles of vectors, or up to
- * 640 codes, take the statistics in a kernel of their own, which is faster there.
+ * chip when its code is chosen, so x is not read and re-scaled a second time; few vectors, or up to 640 codes with four or
+ * eight groups, take the statistics in a kernel of their own, which is faster there.
  *   stage_energy out  optional [R], as under rvq_encode
  *   batch_count  out  float32 [R][K]             (overwritten)
  *   batch_sum    out  float32 [R][K][group_dim]  (overwritten; 16-byte aligned)

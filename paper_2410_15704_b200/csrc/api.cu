@@ -266,6 +266,29 @@ int rvq_encode(const rvq_config *cfg, const void *x, int64_t n, int64_t x_row_st
     return encode_common(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, stage_energy, status, stream, true);
 }
 
+// Whether the batch's statistics are taken by a pass of their own after the encode, or fused into the throughput kernel
+// (us of rvq_encode_stats, fused / apart).
+//   - Batches that the encoders for few tiles take (up to one tile per SM): apart, those encoders can run, but the pass costs
+//     its time per row, while the throughput kernel takes as long for one row as for all tiles of such a batch, and
+//     longer with more codes.  So apart up to a number of group rows that grows with the codes, and with how fast the
+//     pass is (depth 8 but where said otherwise):
+//     four rows of a warp, 16 K: 512 codes 8192 rows 50 / 48, 16384 54 / 58; 700 codes 8192 60 / 54, 16384 61 / 66; 1024 codes 8192 69 / 56, 16384
+//     70 / 71, 18944 70 / 73; 2048 codes 18944 107 / 99 (depth 4, 512 codes 8192 32 / 35, 1024 codes 16384 42 / 46, 2048 codes 18944 61 / 61);
+//     one row of a warp, 8 K: 512 codes 4096 rows 51 / 50, 8192 52 / 54; 1024 codes 8192 69 / 61, 16384 70 / 77; 2048 codes 16384 107 / 105;
+//     a thread per row, 4 K from 1024 codes on: 512 codes lose at any size (256 rows 50 / 55); 1024 codes, 16 groups 4096 69 / 70, 8192 69 / 76,
+//     depth 12 4096 96 / 90, 8192 96 / 98; 2048 codes 8192 106 / 89, 16384 106 / 113.
+//   - More tiles with codebooks too small to hide the additions behind (fused, the epilogue waits for them), with four
+//     groups or eight.  A learning step: 32000 vectors and 256 codes 193 / 175, 240000 940 / 944, 1M 4050 / 4100 (all
+//     rows meet in a few bins either way); 512 codes 80000 426 / 416, 480000 2312 / 2222.
+static bool statistics_apart(const Shape &s, int64_t n)
+{
+    const StatsPass pass = ema_stats_pass(s);
+    const int64_t rows = n * s.G;
+    if (encode_small_wanted(s, n) || encode_split_wanted(s, n))
+        return rows <= (pass == StatsPass::kQuad ? 16 : pass == StatsPass::kWarp ? 8 : s.K >= 1024 ? 4 : 0) * (int64_t)s.K;
+    return encode_tensor_deferred_stages(s) == 0 && pass == StatsPass::kQuad && (s.K > 256 || rows <= (1 << 19));
+}
+
 int rvq_encode_stats(const rvq_config *cfg, const void *x, int64_t n, int64_t x_row_stride,
                      const float *codebooks, const void *prepared, void *codes, uint16_t *std_f16,
                      float *stage_energy, float *batch_count, float *batch_sum, void *workspace,
@@ -277,12 +300,7 @@ int rvq_encode_stats(const rvq_config *cfg, const void *x, int64_t n, int64_t x_
     if (!batch_count || !batch_sum || !workspace) return RVQ_ERR_BADARG;
     if (!aligned16(batch_sum) || !aligned256(workspace)) return RVQ_ERR_ALIGN;
     if (workspace_bytes < ema_stats_scratch_bytes(s)) return RVQ_ERR_WORKSPACE;
-    if (!encode_tensor_supported(s) || encode_small_wanted(s, n) || encode_split_wanted(s, n) ||
-        (encode_tensor_deferred_stages(s) == 0 && ema_stats_quad_supported(s) && (s.K > 256 || n * s.G <= (1 << 19)))) {
-        // shapes without the fused kernel, batches that the encoders for few tiles take, and codebooks too small to hide
-        // the additions behind (fused, the epilogue waits for them): encode, then the separate statistics pass.  A learning
-        // step fused / separate, us: 32000 vectors and 256 codes 193 / 175, 240000 940 / 944, 1M 4050 / 4100 (all
-        // rows meet in a few bins either way); 512 codes 80000 426 / 416, 480000 2312 / 2222.
+    if (!encode_tensor_supported(s) || statistics_apart(s, n)) {
         rc = encode_common(cfg, x, n, x_row_stride, codebooks, prepared, codes, std_f16, stage_energy, status, stream, true);
         if (rc != RVQ_OK) return rc;
         return launch_ema_stats(s, x, n, x_row_stride, codes, codebooks, batch_count, batch_sum, workspace,

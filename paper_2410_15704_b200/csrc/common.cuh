@@ -62,7 +62,9 @@ int launch_rope_table(int dim, double base, int positions, float *table, cudaStr
 int launch_decode_rope(const Shape &s, const void *codes, const uint16_t *std16, int64_t n, const float *cb,
                        const void *prepared, const int32_t *position, int per_position, const float *table,
                        int positions, int style, void *out, int64_t stride, rvq_status *st, cudaStream_t stream);
-bool ema_stats_quad_supported(const Shape &s);   // the statistics pass at its fastest: four or eight groups
+// The statistics pass of a shape: a warp per head vector, four rows at a time (four groups or eight) or one; else a thread per row.
+enum class StatsPass { kQuad, kWarp, kThread };
+StatsPass ema_stats_pass(const Shape &s);
 int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, const void *codes,
                      const float *cb, float *batch_count, float *batch_sum, void *workspace,
                      rvq_status *st, cudaStream_t stream);

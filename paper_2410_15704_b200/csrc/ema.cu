@@ -291,9 +291,11 @@ static int stats_gd(const Shape &s, const void *x, int64_t n, int64_t stride, co
     return check_launch();
 }
 
-bool ema_stats_quad_supported(const Shape &s)
+StatsPass ema_stats_pass(const Shape &s)
 {
-    return s.gd == 32 && (s.G == 4 || s.G == 8) && s.R <= 8 && (size_t)s.R * s.K * sizeof(uint32_t) <= 160 * 1024;
+    if (s.gd != 32 || s.G > 8 || (size_t)s.R * s.K * sizeof(uint32_t) > 160 * 1024) return StatsPass::kThread;
+    if ((s.G == 4 || s.G == 8) && s.R <= 8) return StatsPass::kQuad;
+    return s.per_vector <= 32 ? StatsPass::kWarp : StatsPass::kThread;
 }
 
 int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, const void *codes,
@@ -306,8 +308,8 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         cudaMemsetAsync(batch_sum, 0, (size_t)bins * s.gd * sizeof(float), stream) != cudaSuccess)
         return RVQ_ERR_LAUNCH;
     int rc = RVQ_OK;
-    const bool quad = ema_stats_quad_supported(s);
-    if (n > 0 && (quad || (s.gd == 32 && s.G <= 8 && s.per_vector <= 32 && (size_t)bins * sizeof(uint32_t) <= 160 * 1024))) {
+    const StatsPass pass = ema_stats_pass(s);
+    if (n > 0 && pass != StatsPass::kThread) {
         const int sms = sm_count();
         if (sms <= 0) return RVQ_ERR_DEVICE;
         const size_t smem = (size_t)bins * sizeof(uint32_t);
@@ -316,7 +318,7 @@ int launch_ema_stats(const Shape &s, const void *x, int64_t n, int64_t stride, c
         per_sm = per_sm < 1 ? 1 : (per_sm > 8 ? 8 : per_sm);
         int64_t want = (n + kWarpStatsThreads / 32 - 1) / (kWarpStatsThreads / 32);
         int grid = (int)(want < (int64_t)sms * per_sm ? want : (int64_t)sms * per_sm);
-        auto kernel = !quad ? ema_stats_warp_kernel : s.G == 4 ? ema_stats_quad_kernel<1> : ema_stats_quad_kernel<2>;
+        auto kernel = pass == StatsPass::kWarp ? ema_stats_warp_kernel : s.G == 4 ? ema_stats_quad_kernel<1> : ema_stats_quad_kernel<2>;
         if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), (int)smem))
             return RVQ_ERR_LAUNCH;
         kernel<<<grid, kWarpStatsThreads, smem, stream>>>(s, x, n, stride, codes, cb, cnt, batch_sum, st);

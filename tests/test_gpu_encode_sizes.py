@@ -101,6 +101,16 @@ def test_statistics_of_few_tiles(n, dim, K, R, layout):
         z = z - b.codebooks.view(R, K, 32)[r][codes[:, r]].double()
 
 
+@pytest.mark.parametrize("n,dim,K,R,layout", [(4096, 32, 512, 8, 0), (4097, 32, 512, 8, 0), (1200, 64, 300, 8, 1), (1201, 64, 300, 8, 1),
+                                              (256, 512, 1024, 8, 1), (257, 512, 1024, 8, 1), (1024, 128, 1024, 12, 0), (1025, 128, 1024, 12, 0),
+                                              (8, 1024, 512, 8, 1), (8, 1024, 1023, 4, 0), (700, 128, 6000, 8, 0), (2048, 128, 512, 4, 1), (2049, 128, 512, 4, 1),
+                                              (1100, 256, 550, 8, 0), (1101, 256, 550, 8, 0)])
+def test_statistics_by_the_other_passes(n, dim, K, R, layout):
+    """The same on both sides of the lines between fused statistics and a pass of their own, for head vectors of one, two,
+    four, eight, sixteen and thirty-two groups, more than eight stages, and more codes than a histogram in shared memory holds."""
+    test_statistics_of_few_tiles(n, dim, K, R, layout)
+
+
 @pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
 def test_update_of_buffers_that_are_not_aligned(K, gd):
     """rvq_ema_apply on buffers that start 4 bytes past a 16-byte boundary equals that on aligned ones."""
