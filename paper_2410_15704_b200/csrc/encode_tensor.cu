@@ -11,8 +11,8 @@
 //     half-precision operands described in prepare.cu), accumulated in float32
 //     in TMEM.
 //     EIGHT: the two small products of the split (remainder x head) in e4m3, as two K=32 steps beside
-//     three K=16 ones: 327 cycles per chain instead of 455, at an error of 2^-15 |z||e| that the window
-//     allows for.  For contiguous groups and eight or more chunks (kEightMinSlots says why).
+//     three K=16 ones: 327 cycles per chain instead of 455, at an error of up to 2^-13 |z||e| in the score that the
+//     window allows for (window8).  For contiguous groups, eight or more chunks and even codebooks (eight_possible says why).
 //   - The B operand (128 codewords per slot) streams from the prepared block
 //     through a ring of shared-memory slots filled by cp.async.bulk; every
 //     slot serves all three tiles.
@@ -67,15 +67,20 @@ constexpr int kSmemBytes = kOffFlags + 512;
 constexpr int kDeferMinSlots = 6;                                     // chunks a stage needs for its issuers to take the statistics
 
 // Chunks a stage needs for the chain with 8-bit corrections, which is for contiguous groups: it is a tenth faster on
-// values (262144 vectors, 2048 codes: 2520 -> 2270 us; 524288, 1024 codes: 3140 -> 2840; 512 codes: 1950 -> 2020), but
-// on keys, which strided groups are for, outlier channels leave 2.1 % of the rows and stages with more than one
-// candidate instead of 0.1 %, and their exact comparison costs more than the steps saved (1M vectors, 1024
-// codes: 6300 -> 6690).
+// values (262144 vectors, 2048 codes: 2545 -> 2315 us in a burst, 2928 -> 2625 under the power cap; 524288, 1024 codes: 2850 -> 2660, 3271 -> 3005;
+// 512 codes: 1950 -> 2020).
 // It also needs rounds of three tiles, whose chains queue up at the tensor core: with fewer tiles per SM a chain's length is
 // not what a stage waits for, and the added work at the stage end is (values, us, half precision / 8 bits, tiles per SM at
 // most: 1024 codes 64 / 75 at two, 122 / 137 at four, 145 / 138 at five; 2048 codes 147 / 156 at three, 207 / 191 at four).
+// And it needs rows whose window stays narrow.  With outlier channels 2.4-2.9 % of the rows and stages have more than one
+// candidate instead of 0.5 %, and their exact comparison costs more than the steps saved (keys on contiguous groups: 131072
+// vectors, 1024 codes 735 -> 1056, 65536, 2048 codes 653 -> 1172).  The data are not known on the host; the codebooks, which follow them, are
+// looked at when they are prepared (PreparedHeader::even), and the kernel reads there which chain to take.  131072 vectors,
+// us in a burst, by the kurtosis of the codewords' entries (1024 codes; 2048 codes): 3: 721 -> 722, 1265 -> 1165; 4.1: 721 -> 744, 1261 -> 1204;
+// 4.4: 720 -> 726, 1264 -> 1197; 7.8: 721 -> 762, 1261 -> 1230; 9.3: 718 -> 769, 1259 -> 1273; 13: 720 -> 768, 1270 -> 1314; 24: 720 -> 807,
+// 1280 -> 1343; 44: 722 -> 904, 1274 -> 1590.  (Under the power cap the shorter chain gains another 6-7 % on both.)
 constexpr int kEightMinSlots = 8;
-inline bool eight_wanted(const Shape &s, int64_t tiles, int sms)
+inline bool eight_possible(const Shape &s, int64_t tiles, int sms)
 {
     const int slots = slots_per_stage(s.K);
     return slots >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw && tiles > (int64_t)sms * (slots >= 16 ? 3 : 4);
@@ -114,8 +119,7 @@ struct Work {
 // twelve epilogue warps take 152 (4 x 40 + 12 x 152 = 1984 of the 2048 per lane).
 // EIGHT: the small products in 8 bits (issue_chain8).
 template <bool EIGHT>
-__global__ void __launch_bounds__(kThreads, 1)
-encode_tensor_kernel(const Params p)
+__device__ __forceinline__ void encode_tensor_body(const Params &p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBars);
@@ -470,6 +474,15 @@ encode_tensor_kernel(const Params p)
     }
 }
 
+__global__ void __launch_bounds__(kThreads, 1) encode_tensor_kernel(const __grid_constant__ Params p) { encode_tensor_body<false>(p); }
+
+// Where the 8-bit corrections are possible: by the codebooks.
+__global__ void __launch_bounds__(kThreads, 1) encode_tensor_either_kernel(const __grid_constant__ Params p)
+{
+    if (reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true>(p);
+    else encode_tensor_body<false>(p);
+}
+
 }  // namespace
 
 bool encode_tensor_supported(const Shape &s)
@@ -495,7 +508,7 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
-    auto kernel = eight_wanted(s, tiles, sms) ? encode_tensor_kernel<true> : encode_tensor_kernel<false>;
+    auto kernel = eight_possible(s, tiles, sms) ? encode_tensor_either_kernel : encode_tensor_kernel;
     if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,

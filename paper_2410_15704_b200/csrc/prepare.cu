@@ -9,8 +9,8 @@
 // are split into a half-precision head and a half-precision remainder and the
 // contraction keeps the three leading products:
 //     z.e  ~  z_hi.e_hi + z_hi.e_lo + z_lo.e_hi        (error ~ 2^-22 |z||e|),
-// or, where a sweep is long enough to make up for more rows with several candidates, the two small products in
-// 8 bits (e4m3, twice the depth per step; error ~ 2^-15 |z||e|):
+// or, where a sweep is long enough to make up for more rows with several candidates and the codewords' energy is
+// not in a few outliers, the two small products in 8 bits (e4m3, twice the depth per step; error up to ~ 2^-13 |z||e|):
 //     z.e  ~  z_hi.e_hi + [64 z_lo]_8.[e / 64]_8 + [z_hi / 64]_8.[64 e_lo]_8.
 // Per stage r the block holds
 //   - a power-of-two scale 2^k chosen so that the largest scaled squared norm
@@ -101,22 +101,22 @@ decode_table_kernel(Shape s, const float *cb, const DecodeParams *dp,
 }
 
 
-// grid (kPrepareParts, R): largest squared norm and entry range of a share of one stage's codewords.
+// grid (kPrepareParts, R): largest squared norm, entry range and moments of a share of one stage's codewords.
 __global__ void __launch_bounds__(256)
 prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
 {
     follow_previous();
-    __shared__ double rn[256];
+    __shared__ double rn[256], r2[256], r4[256];
     __shared__ float rlo[256], rhi[256];
     const int r = blockIdx.y, tid = threadIdx.x;
     const int per = (s.K + kPrepareParts - 1) / kPrepareParts;
     const int j0 = blockIdx.x * per, j1 = min(s.K, j0 + per);
-    double m = 0.0;
+    double m = 0.0, sum2 = 0.0, sum4 = 0.0;
     float lo = INFINITY, hi = -INFINITY;
     for (int j = j0 + tid; j < j1; j += 256) {
         const float *e = cb + ((size_t)r * s.K + j) * s.gd;
         double acc = 0.0;
-        auto add = [&](float v) { acc += (double)v * (double)v; lo = fminf(lo, v); hi = fmaxf(hi, v); };
+        auto add = [&](float v) { const double v2 = (double)v * (double)v; acc += v2; sum4 = fma(v2, v2, sum4); lo = fminf(lo, v); hi = fmaxf(hi, v); };
         if (s.gd == 32) {
             float4 f[8];                                      // (asked for together)
 #pragma unroll
@@ -127,19 +127,21 @@ prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
             for (int i = 0; i < s.gd; ++i) add(e[i]);
         }
         m = fmax(m, acc);
+        sum2 += acc;
     }
-    rn[tid] = m; rlo[tid] = lo; rhi[tid] = hi;
+    rn[tid] = m; r2[tid] = sum2; r4[tid] = sum4; rlo[tid] = lo; rhi[tid] = hi;
     __syncthreads();
     for (int w = 128; w > 0; w >>= 1) {
         if (tid < w) {
             rn[tid] = fmax(rn[tid], rn[tid + w]);
+            r2[tid] += r2[tid + w]; r4[tid] += r4[tid + w];
             rlo[tid] = fminf(rlo[tid], rlo[tid + w]); rhi[tid] = fmaxf(rhi[tid], rhi[tid + w]);
         }
         __syncthreads();
     }
     if (tid == 0) {
         StagePartial &o = part[r * kPrepareParts + blockIdx.x];
-        o.max_norm2 = rn[0]; o.lo = rlo[0]; o.hi = rhi[0];
+        o.max_norm2 = rn[0]; o.sum2 = r2[0]; o.sum4 = r4[0]; o.lo = rlo[0]; o.hi = rhi[0];
     }
 }
 
@@ -154,14 +156,16 @@ prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, St
     const int r = threadIdx.x;
     if (r < 8) { s_lo[r] = 0.0f; s_step[r] = 0.0f; }
     __syncwarp();
+    bool even = false;
     if (r < s.R) {
-        double maxn = 0.0;
+        double maxn = 0.0, sum2 = 0.0, sum4 = 0.0;
         float lo = INFINITY, hi = -INFINITY;
 #pragma unroll
         for (int q = 0; q < kPrepareParts; ++q) {
             const StagePartial pp = part[r * kPrepareParts + q];
-            maxn = fmax(maxn, pp.max_norm2); lo = fminf(lo, pp.lo); hi = fmaxf(hi, pp.hi);
+            maxn = fmax(maxn, pp.max_norm2); sum2 += pp.sum2; sum4 += pp.sum4; lo = fminf(lo, pp.lo); hi = fmaxf(hi, pp.hi);
         }
+        even = sum4 * (double)s.K * (double)s.gd <= kEvenKurtosis * sum2 * sum2;
         int k = 12;
         if (maxn > 0.0 && isfinite(maxn)) {
             k = (int)floor(0.5 * log2(8192.0 / maxn));
@@ -174,8 +178,9 @@ prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, St
         mx[r].emax = 0u; mx[r].eerr = 0u; mx[r].nmax = 0u; mx[r].elomax = 0u;
         if (r < 8) { s_lo[r] = lo; s_step[r] = hi > lo ? (hi - lo) / 65535.0f : 0.0f; }     // finest unit the range allows
     }
-    __syncwarp();
+    const int evens = __popc(__ballot_sync(0xFFFFFFFFu, even));
     if (r == 0) {
+        hdr->even = 2 * evens >= s.R ? 1u : 0u;
         hdr->magic = kPreparedMagic; hdr->R = s.R; hdr->K = s.K; hdr->gd = s.gd;
         hdr->slots = slots_per_stage(s.K);
         hdr->decode_offset = decode_levels_prepared(s)

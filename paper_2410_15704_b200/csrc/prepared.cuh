@@ -19,12 +19,17 @@ constexpr size_t kPreparedParamsOffset = 256;             // StageParams[16]
 constexpr size_t kPreparedMaximaOffset = 512;             // StageMaxima[16]
 constexpr size_t kPreparedPartialsOffset = 768;           // StagePartial[16 stages][kPrepareParts], scratch of the prepare step
 constexpr int kPrepareParts = 16;
-constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 16;   // operand image, [R][slots][kSlotStride]
+constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 32;   // operand image, [R][slots][kSlotStride]
 
 struct PreparedHeader {
     uint32_t magic, R, K, gd, slots;
     uint32_t decode_offset;   // byte offset of the decoder section, 0 if absent
+    uint32_t even;            // 1: the codewords' energy is spread over their entries (kEvenKurtosis), 0: outliers carry it
 };
+// A stage's codewords count as even when the fourth moment of their entries is at most this many times the square of the
+// second (3 for a normal distribution); the block does when at least half of its stages do.  The throughput encoder
+// takes the 8-bit corrections by it (encode_tensor.cu).
+constexpr double kEvenKurtosis = 6.0;
 
 // Decoder section (group_dim 32, R <= 8, K <= kDecodeMaxK): per stage an affine
 // map value = lo_r + q * scale_r * base with q a 16-bit level, scale_r an integer in
@@ -120,6 +125,7 @@ struct StageParams {
 
 struct StagePartial {
     double max_norm2;   // largest squared norm among this part's codewords
+    double sum2, sum4;  // sums of the entries' squares and fourth powers
     float lo, hi;       // smallest and largest entry
 };
 

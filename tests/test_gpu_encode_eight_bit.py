@@ -1,0 +1,99 @@
+"""The throughput encoder's chain with 8-bit corrections: contiguous groups, 1024 codes and more, more than four tiles of 128 group
+rows per SM (three from 1921 codes on), and codebooks without outliers.  Its error window is some fifty times that of the
+half-precision chain, so these cases aim at it: planted pairs of codewords at gaps on both sides of the window, the
+statistics taken in the same pass, and codebooks with outliers, which keep the half-precision chain at the same sizes."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2410_15704_b200 as rvq
+from helpers import assert_codes_match
+
+pytestmark = pytest.mark.gpu
+
+
+def kurtosis(cb):
+    """Fourth moment of a stage's entries over the square of the second: 3 for a normal distribution."""
+    e = cb.astype(np.float64).reshape(len(cb), -1)
+    return (e ** 4).mean(axis=1) / (e ** 2).mean(axis=1) ** 2
+
+
+def encode_both(x, cb, R, K):
+    n = len(x)
+    cfg = rvq.make_config(128, 32, rvq.CONTIGUOUS, R, K, 16, rvq.F32, 0)
+    b, xd = rvq.alloc_buffers(cfg, n, cb), torch.from_numpy(x).cuda()
+    exact = torch.empty_like(b.codes)
+    rvq.rvq_encode(cfg, xd, n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    st = rvq.read_status(b.status)
+    rvq.rvq_encode_exact(cfg, xd, n, 128, b.codebooks, b.prepared, exact, b.std, None)
+    torch.cuda.synchronize()
+    assert st["wait_timeouts"] == 0
+    return cfg, b, xd, exact, st
+
+
+@pytest.mark.parametrize("K,outliers", [(1024, False), (2048, False), (1024, True)])
+def test_pairs_at_the_edge_of_the_window(K, outliers):
+    """Every row has two codewords at nearly the same distance, relative gaps of 1e-3 ... 6e-2, either one ahead.  The
+    window is some 9e-3 of the squared distance: half of the rows are compared exactly, the others certified right
+    outside it, and all choices must be the float32 kernel's.  (outliers: some channels of the rows, not of the codewords.)"""
+    g = np.random.default_rng(K)
+    base = g.normal(size=(K // 8, 128))                                  # K / 2 group rows
+    z = (base / base.std(axis=1, keepdims=True)).reshape(-1, 32)
+    d = z[g.permutation(len(z))]
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    a = 0.2 * np.linalg.norm(z, axis=1, keepdims=True)
+    gamma = np.exp(g.uniform(np.log(1e-3), np.log(6e-2), size=(len(z), 1)))
+    pair = np.stack([z + a * d, z - a * (1.0 + 0.5 * gamma) * d], axis=1).reshape(K, 32)
+    cb = pair[g.permutation(K)][None].astype(np.float32)
+    assert kurtosis(cb).max() < 5.0
+    x = np.repeat(base, 32768 // len(base), axis=0) * (1.0 + 1e-3 * g.normal(size=(32768, 128)))
+    if outliers:
+        x[::5, :3] *= 30.0
+    x = x.astype(np.float32)
+    cfg, b, _, exact, st = encode_both(x, cb, 1, K)
+    assert torch.equal(b.codes, exact)
+    codes = b.codes.view(torch.int16).cpu().numpy().view(np.uint16).reshape(len(x), 4, 1).astype(np.int32)
+    assert_codes_match(x, codes, cb, rvq.CONTIGUOUS, sample=np.arange(0, len(x), 7))
+    assert 0.2 < st["rescored_rows"] / (len(x) * 4) < 0.8 and st["exhaustive_rows"] < 0.1 * len(x)
+
+
+@pytest.mark.parametrize("n,K", [(18945, 1024), (14219, 2048), (40000, 1030)])
+def test_statistics_in_the_same_pass(n, K):
+    """rvq_encode_stats where the chain has 8-bit corrections: the codes of rvq_encode, the counts and sums of rvq_ema_stats."""
+    g = np.random.default_rng(n)
+    R = 3
+    x = g.normal(size=(n, 128)).astype(np.float32)
+    cb = np.stack([g.normal(scale=0.8 ** r, size=(K, 32)) for r in range(R)]).astype(np.float32)
+    assert kurtosis(cb).max() < 5.0
+    cfg, b, xd, exact, _ = encode_both(x, cb, R, K)
+    assert torch.equal(b.codes, exact)
+    energy, fused_energy = torch.empty(R, device="cuda"), torch.empty(R, device="cuda")
+    rvq.rvq_encode(cfg, xd, n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status, stage_energy=energy)
+    count, total = torch.empty(R, K, device="cuda"), torch.empty(R, K, 32, device="cuda")
+    rvq.rvq_ema_stats(cfg, xd, n, 128, b.codes, b.codebooks, count, total, b.workspace, b.workspace_bytes, b.status)
+    f = rvq.alloc_buffers(cfg, n, cb)
+    fused_count, fused_total = torch.full((R, K), -1.0, device="cuda"), torch.full((R, K, 32), 9.0, device="cuda")
+    rvq.rvq_encode_stats(cfg, xd, n, 128, f.codebooks, f.prepared, f.codes, f.std, fused_count, fused_total, f.workspace, f.workspace_bytes,
+                         f.status, stage_energy=fused_energy)
+    torch.cuda.synchronize()
+    assert torch.equal(f.codes, b.codes) and torch.equal(f.std, b.std) and torch.equal(fused_count, count)
+    assert (torch.abs(fused_total - total) / count.clamp(min=1.0)[..., None]).max().item() <= 1e-4
+    # (float32 additions of some 2e5 row energies each, warp by warp, in another order)
+    assert torch.allclose(energy, fused_energy, rtol=1e-4)
+    assert rvq.read_status(f.status)["wait_timeouts"] == 0
+
+
+@pytest.mark.parametrize("n,K", [(18945, 1024), (14219, 2048)])
+def test_codebooks_with_outliers(n, K):
+    """Keys on contiguous groups: outlier channels, and codebooks that follow them."""
+    g = np.random.default_rng(n)
+    scale = 0.25 + np.abs(g.laplace(size=128))
+    scale[g.permutation(128)[:8]] *= 20.0
+    x = (g.normal(size=(n, 128)) * scale).astype(np.float32)
+    unit = (scale / np.sqrt((scale ** 2).mean())).reshape(4, 32)
+    cb = np.stack([g.normal(size=(K, 32)) * unit[g.integers(0, 4, size=K)] * 0.8 ** r for r in range(4)]).astype(np.float32)
+    assert kurtosis(cb).min() > 8.0
+    _, b, _, exact, st = encode_both(x, cb, 4, K)
+    assert torch.equal(b.codes, exact)
+    # (with 8-bit corrections 2-3 % of the rows and stages were compared exactly)
+    assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * 4
