@@ -62,7 +62,7 @@ constexpr int kOffA = kOffB + kRing * kSlotBytes;
 constexpr int kOffZ = kOffA + kOnesBytes;                             // parked residuals, float [32][rows]
 constexpr int kOffCodes = kOffZ + 32 * kRowsPerPass * 4;
 constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;          
-constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: bit 0 valid, bit 1 degenerate
+constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: 1 for a vector's, 0 past the last
 constexpr int kSmemBytes = kOffFlags + 512;
 constexpr int kDeferMinSlots = 6;                                     // chunks a stage needs for its issuers to take the statistics
 
@@ -252,17 +252,14 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 last_par ^= 1u;
                 if (p.defer_stats && stage >= 1u && s_in >= 1u && s_in <= 4u) {
                     const int rl = t * 128 + (int)(s_in - 1u) * 32 + lane;
-                    const uint32_t fl = flags_s[rl];
-                    if (fl & 1u) {
+                    if (flags_s[rl]) {
                         const size_t bin = (size_t)(stage - 1u) * s.K + codes_s[rl * 16 + (int)(stage - 1u)];
                         atomicAdd(p.stat_cnt + bin, 1u);
-                        if (!(fl & 2u)) {
-                            float4 *m = reinterpret_cast<float4 *>(p.stat_sum + bin * 32);
+                        float4 *m = reinterpret_cast<float4 *>(p.stat_sum + bin * 32);
 #pragma unroll
-                            for (int q4 = 0; q4 < 8; ++q4)
-                                atomicAdd(m + q4, make_float4(zp[(4 * q4) * kRowsPerPass + rl], zp[(4 * q4 + 1) * kRowsPerPass + rl],
-                                                              zp[(4 * q4 + 2) * kRowsPerPass + rl], zp[(4 * q4 + 3) * kRowsPerPass + rl]));
-                        }
+                        for (int q4 = 0; q4 < 8; ++q4)
+                            atomicAdd(m + q4, make_float4(zp[(4 * q4) * kRowsPerPass + rl], zp[(4 * q4 + 1) * kRowsPerPass + rl],
+                                                          zp[(4 * q4 + 2) * kRowsPerPass + rl], zp[(4 * q4 + 3) * kRowsPerPass + rl]));
                     }
                     __syncwarp();
                 }
@@ -300,7 +297,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
             const float dev = group_deviation(s, z, lane);
             // (raw rows are stage inputs already: taken as they are, no deviation stored)
             const bool deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
-            if (p.defer_stats) smem[kOffFlags + rloc] = (uint8_t)((valid ? 1 : 0) | (deg ? 2 : 0));
+            if (p.defer_stats) smem[kOffFlags + rloc] = valid ? 1 : 0;
             if (!s.raw) {
                 divide_row(z, dev, deg);
             } else if (deg) {
@@ -420,14 +417,13 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     // (all stages but the last are the issuer warps' when deferred)
                     const size_t bin = (size_t)r * s.K + bj;
                     atomicAdd(p.stat_cnt + bin, 1u);
-                    if (!deg) {
-                        float4 *m = reinterpret_cast<float4 *>(p.stat_sum + bin * 32);
+                    float4 *m = reinterpret_cast<float4 *>(p.stat_sum + bin * 32);
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            atomicAdd(m + q, make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]));
-                    }
+                    for (int q = 0; q < 8; ++q)
+                        atomicAdd(m + q, make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]));
                 }
-                if (!deg) {
+                // (a degenerate row's codes are 0 whatever its residual, which starts from zero and matters to the statistics only)
+                if (!deg || (p.stat_sum && valid)) {
                     const float *ew = cbr + (size_t)bj * 32;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -443,7 +439,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     float e2 = 0.0f;
 #pragma unroll
                     for (int i = 0; i < 32; ++i) e2 = fmaf(z[i], z[i], e2);
-                    if (!valid) e2 = 0.0f;
+                    if (deg) e2 = 0.0f;
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xFFFFFFFFu, e2, off);
                     if (lane == 0) atomicAdd(p.energy + r, e2);

@@ -4,8 +4,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2410_15704_b200 as rvq
-from helpers import DT, assert_codes_match
+from helpers import DT, assert_codes_match, codes_to_numpy
 
 pytestmark = pytest.mark.gpu
 
@@ -109,6 +110,30 @@ def test_statistics_by_the_other_passes(n, dim, K, R, layout):
     """The same on both sides of the lines between fused statistics and a pass of their own, for head vectors of one, two,
     four, eight, sixteen and thirty-two groups, more than eight stages, and more codes than a histogram in shared memory holds."""
     test_statistics_of_few_tiles(n, dim, K, R, layout)
+
+
+@pytest.mark.parametrize("n,dim,K,R,layout", [(4737, 128, 1024, 4, 1), (18945, 128, 1024, 3, 0), (8000, 64, 300, 3, 0), (20000, 128, 256, 1, 0), (600, 128, 1024, 4, 0)])
+def test_statistics_of_degenerate_vectors(n, dim, K, R, layout):
+    """Vectors of zero or non-finite deviation have codes 0 and count for them, and their stage inputs are what those codes
+    leave of zero: statistics taken in the encoder's pass (all cases but the last) are those of rvq_ema_stats, and the oracle's."""
+    x, cb = batch(n, dim, K, R, "f32", 2 * n)
+    x[::97] = 0.0
+    x[5, 3], x[n - 1, 0] = float("nan"), float("inf")
+    cfg = rvq.make_config(dim, 32, layout, R, K, 16, rvq.F32, 0)
+    b, xd = rvq.alloc_buffers(cfg, n, cb), x.cuda()
+    got, want = [[torch.empty(R, K, device="cuda"), torch.empty(R, K, 32, device="cuda")] for _ in range(2)]
+    rvq.rvq_encode_stats(cfg, xd, n, dim, b.codebooks, b.prepared, b.codes, b.std, *got, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_ema_stats(cfg, xd, n, dim, b.codes, b.codebooks, *want, b.workspace, b.workspace_bytes, b.status)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], want[0])
+    # (float32 sums of up to a bin's count of rows in another order, and a codeword subtracted and added back)
+    scale = want[0].clamp(min=1.0)[..., None]
+    assert ((got[1] - want[1]).abs() / scale).max().item() <= 1e-4
+    codes = codes_to_numpy(cfg, b.codes, n)
+    assert not codes[::97].any()
+    count, total = oracle.ema_stats(x.numpy(), codes, cb, layout)
+    assert np.array_equal(got[0].cpu().numpy(), count)
+    assert np.max(np.abs(got[1].cpu().numpy() - total) / scale.cpu().numpy()) <= 1e-4
 
 
 @pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
