@@ -130,6 +130,7 @@ size_t rvq_workspace_bytes(const rvq_config *cfg /* host */, int64_t n);
  *   stage_energy out  optional (may be NULL): float32 [R], overwritten; entry r is the sum over
  *                     all groups of all n head vectors of ||z_{r+1}||^2, the squared norm of the
  *                     residual that stage r leaves, in scaled units (after the division by s).
+ *                     Vectors of zero or non-finite deviation (they decode to zeros) add nothing.
  *                     Entry R-1 is the quantization error of the batch: the quantity Section 3
  *                     watches while the codebooks are learnt.  Float32 atomics: the order of
  *                     the additions, and so the last bits, vary from call to call.

@@ -70,7 +70,7 @@ encode_scalar_kernel(Shape s, const void *__restrict__ x, int64_t n, int64_t str
             float4 ev = __ldg(e + q);
             z[4 * q] -= ev.x; z[4 * q + 1] -= ev.y; z[4 * q + 2] -= ev.z; z[4 * q + 3] -= ev.w;
         }
-        if (energy && gv < n) {
+        if (energy && gv < n && !deg) {
             float e2 = 0.0f;
 #pragma unroll
             for (int i = 0; i < GD; ++i) e2 = fmaf(z[i], z[i], e2);

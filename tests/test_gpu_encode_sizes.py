@@ -38,8 +38,7 @@ def check(n, dim, K, R, layout, bits, dtype, seed, stride=None):
         rvq.rvq_encode_exact(cfg, xd, n, stride, e.codebooks, e.prepared, e.codes, e.std, e.status, stage_energy=energy_e)
         torch.cuda.synchronize()
         assert torch.equal(b.codes, e.codes) and torch.equal(b.std, e.std)
-    if not (n % 2 == 1 and n > 3):                          # (the float32 kernel counts degenerate rows' codewords)
-        assert torch.allclose(energy, energy_e, rtol=1e-4)
+    assert torch.allclose(energy, energy_e, rtol=1e-4)
     st, ste = rvq.read_status(b.status), rvq.read_status(e.status)
     assert st["wait_timeouts"] == 0 and st["degenerate_vectors"] == ste["degenerate_vectors"]
 
@@ -134,6 +133,27 @@ def test_statistics_of_degenerate_vectors(n, dim, K, R, layout):
     count, total = oracle.ema_stats(x.numpy(), codes, cb, layout)
     assert np.array_equal(got[0].cpu().numpy(), count)
     assert np.max(np.abs(got[1].cpu().numpy() - total) / scale.cpu().numpy()) <= 1e-4
+
+
+@pytest.mark.parametrize("n,K", [(5, 1024), (601, 1024), (4001, 256), (601, 256)])
+def test_stage_energy_leaves_degenerate_vectors_out(n, K):
+    """In every encoder: the energies of a batch with vectors of zero and non-finite deviation are those of the others."""
+    x, cb = batch(n, 128, K, 3, "f32", 2 * n)
+    x[::4] = 0.0
+    x[1, 3], x[n - 2, 0] = float("nan"), float("inf")
+    keep = torch.isfinite(x).all(dim=1) & (x != 0).any(dim=1)
+    cfg = rvq.make_config(128, 32, 0, 3, K, 16, rvq.F32, 0)
+    z = oracle.encode(x[keep].numpy(), cb, 32, 0, want_residual=True)
+    last = float((z["residual"] ** 2).sum())
+    for exact in (False, True):
+        b, energy = rvq.alloc_buffers(cfg, n, cb), torch.empty(3, device="cuda")
+        if exact:
+            rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.status, stage_energy=energy)
+        else:
+            rvq.rvq_encode(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status,
+                           stage_energy=energy)
+        torch.cuda.synchronize()
+        assert abs(energy[-1].item() - last) <= 1e-4 * last       # (float32 additions of row energies, in any order)
 
 
 @pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
