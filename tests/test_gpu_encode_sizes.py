@@ -156,6 +156,36 @@ def test_stage_energy_leaves_degenerate_vectors_out(n, K):
         assert abs(energy[-1].item() - last) <= 1e-4 * last       # (float32 additions of row energies, in any order)
 
 
+@pytest.mark.parametrize("seed", range(4))
+def test_quotients_of_the_encoder_are_those_of_a_division(seed):
+    """The throughput encoder divides a row by its deviation with corrected reciprocals, or one by one where a value is
+    outside a wide range of exponents.  Every row has a codeword of its own here, so that the sum of a bin is one row's
+    scaled values, bit for bit; rvq_ema_stats with 16 groups divides.  Half of the vectors keep to the ordinary range, the
+    others hold elements far below and above it, deviations beyond it on both sides, and zeros."""
+    g = np.random.default_rng(seed)
+    dim, K, live, n = 512, 4096, 256, 1300
+    x = g.normal(size=(live, dim))
+    x[:128] *= 2.0 ** g.integers(-38, 39, size=(128, 1))
+    wild = x[128:]
+    wild[:32] *= 2.0 ** -g.integers(62, 140, size=(32, dim)) ** (g.random((32, dim)) < 0.1)
+    wild[32:64] *= 2.0 ** g.integers(41, 60, size=(32, 1))
+    wild[64:96] *= 2.0 ** -g.integers(41, 55, size=(32, 1))
+    wild[96:][g.random((32, dim)) < 0.2] = 0.0
+    wild[112:, 0] *= 2.0 ** 10
+    x = np.concatenate([x, np.zeros((n - live, dim))]).astype(np.float32)
+    z = x[:live].astype(np.float64)
+    z = (z / z.std(axis=1, keepdims=True)).reshape(-1, 32)
+    cb = z[g.permutation(K)][None].astype(np.float32)
+    cfg = rvq.make_config(dim, 32, 0, 1, K, 16, rvq.F32, 0)
+    b, xd = rvq.alloc_buffers(cfg, n, cb), torch.from_numpy(x).cuda()
+    got, want = [[torch.empty(1, K, device="cuda"), torch.empty(1, K, 32, device="cuda")] for _ in range(2)]
+    rvq.rvq_encode_stats(cfg, xd, n, dim, b.codebooks, b.prepared, b.codes, b.std, *got, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_ema_stats(cfg, xd, n, dim, b.codes, b.codebooks, *want, b.workspace, b.workspace_bytes, b.status)
+    torch.cuda.synchronize()
+    assert len(np.unique(codes_to_numpy(cfg, b.codes, n)[:live])) == K
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
 @pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
 def test_update_of_buffers_that_are_not_aligned(K, gd):
     """rvq_ema_apply on buffers that start 4 bytes past a 16-byte boundary equals that on aligned ones."""
