@@ -96,7 +96,8 @@ int rvq_version(void);
 uint64_t rvq_launch_count(void);
 
 /* Bytes of one head vector's codes in the configured storage form
- * (Section 3.2: G*R indices of code_bits bits).  0 on a bad config. */
+ * (Section 3.2: G*R indices of code_bits bits; 2*G*R for code_bits 16, a multiple
+ * of 4 for the packed form).  0 on a bad config. */
 size_t rvq_code_bytes(const rvq_config *cfg /* host */);
 
 /* Size of the prepared-codebook block for this shape. 0 on a bad config. */

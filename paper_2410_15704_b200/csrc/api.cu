@@ -166,7 +166,7 @@ int make_shape(const rvq_config *c, Shape *s)
     s->ddof = c->std_ddof;
     if (s->G > 128 || s->dim - s->ddof <= 0) return RVQ_ERR_UNSUPPORTED;
     s->per_vector = s->G * s->R;
-    s->code_bytes = (s->per_vector * s->bits + 31) / 32 * 4;
+    s->code_bytes = s->bits == 16 ? s->per_vector * 2 : (s->per_vector * s->bits + 31) / 32 * 4;
     s->elem_bytes = c->x_dtype == RVQ_F32 ? 4 : 2;
     s->raw = 0;
     return RVQ_OK;

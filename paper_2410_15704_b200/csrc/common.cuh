@@ -15,7 +15,7 @@ namespace rvq {
 struct Shape {
     int dim, gd, G, layout, R, K, bits, dtype, ddof;
     int per_vector;       // G * R codes per head vector
-    int code_bytes;       // bytes of one head vector's codes
+    int code_bytes;       // bytes of one head vector's codes: 2 each, or a packed stream padded to a multiple of 4
     int elem_bytes;       // bytes of one x element
     int raw;              // library-internal: the rows are stage inputs already (no deviation, no scaling)
 };
@@ -151,7 +151,7 @@ __device__ __forceinline__ void store_from_float(void *base, int64_t idx, int dt
     else reinterpret_cast<__half *>(base)[idx] = __float2half_rn(v);
 }
 
-// Code number k of one head vector whose codes start at `vec` (4-byte aligned).
+// Code number k of one head vector whose codes start at `vec` (4-byte aligned where they are packed).
 __device__ __forceinline__ uint32_t read_code(const void *vec, int k, int bits, int code_bytes)
 {
     if (bits == 16) return reinterpret_cast<const uint16_t *>(vec)[k];

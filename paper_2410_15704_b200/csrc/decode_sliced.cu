@@ -216,7 +216,7 @@ decode_sliced_body(const Shape &s, const void *__restrict__ codes, const uint16_
             if (s.bits == 16 && s.R == 8) {
                 const uint4 c = __ldg(reinterpret_cast<const uint4 *>(codes) + row);
                 cw[0] = c.x; cw[1] = c.y; cw[2] = c.z; cw[3] = c.w;
-            } else if (s.R * s.bits <= 96) {
+            } else if (s.R * s.bits <= 96 && (s.code_bytes & 3) == 0) {
                 // The row's R codes are R * bits <= 96 consecutive bits of the vector's stream, starting
                 // at bit g * R * bits: fetch the (up to four) words that hold them, shift the window
                 // down to bit 0, and cut the codes out of it.

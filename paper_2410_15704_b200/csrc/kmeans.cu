@@ -22,7 +22,7 @@ Shape stage_shape(const Shape &s)
     Shape t = s;
     t.R = 1; t.dtype = RVQ_F32; t.layout = RVQ_GROUP_CONTIGUOUS; t.bits = 16; t.elem_bytes = 4;
     t.per_vector = t.G;
-    t.code_bytes = (t.G * 16 + 31) / 32 * 4;
+    t.code_bytes = t.G * 2;
     t.raw = 1;
     return t;
 }

@@ -6,7 +6,8 @@ import torch
 
 import oracle
 import paper_2410_15704_b200 as rvq
-from helpers import DT, assert_codes_match, codes_to_numpy
+from helpers import DT, RECON_TOL, assert_codes_match, codes_to_numpy
+import test_gpu_learning
 
 pytestmark = pytest.mark.gpu
 
@@ -184,6 +185,40 @@ def test_quotients_of_the_encoder_are_those_of_a_division(seed):
     torch.cuda.synchronize()
     assert len(np.unique(codes_to_numpy(cfg, b.codes, n)[:live])) == K
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("dim,gd,K,R", [(32, 32, 300, 3), (32, 32, 1024, 1), (32, 32, 600, 9), (96, 32, 129, 5), (24, 8, 50, 3), (64, 64, 70, 1)])
+@pytest.mark.parametrize("n", [1, 2, 700])
+def test_odd_numbers_of_16_bit_codes(dim, gd, K, R, n):
+    """uint16 codes are [n][G][R] without gaps also where a vector has an odd number of them, for what writes and what reads them."""
+    g = np.random.default_rng(dim + K + R + n)
+    x = g.normal(size=(n, dim)).astype(np.float32)
+    cb = np.stack([g.normal(scale=0.8 ** r, size=(K, gd)) for r in range(R)]).astype(np.float32)
+    cfg = rvq.make_config(dim, gd, 1, R, K, 16, rvq.F32, 0)
+    assert rvq.rvq_code_bytes(cfg) == dim // gd * R * 2
+    b, xd = rvq.alloc_buffers(cfg, n, cb), torch.from_numpy(x).cuda()
+    out, rotated = torch.empty_like(xd), torch.empty_like(xd)
+    count, total = torch.empty(R, K, device="cuda"), torch.empty(R, K, gd, device="cuda")
+    table, pos = torch.empty(1, dim // 2, 2, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    rvq.rvq_rope_table(dim, 10000.0, 1, table)                             # position 0: nothing is rotated
+    rvq.rvq_encode(cfg, xd, n, dim, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_decode(cfg, b.codes, b.std, n, b.codebooks, b.prepared, out, dim, b.status)
+    rvq.rvq_decode_rope(cfg, b.codes, b.std, n, b.codebooks, b.prepared, pos, 1, table, 1, rvq.ROPE_HALVES, rotated, dim, b.status)
+    rvq.rvq_ema_stats(cfg, xd, n, dim, b.codes, b.codebooks, count, total, b.workspace, b.workspace_bytes, b.status)
+    torch.cuda.synchronize()
+    codes = codes_to_numpy(cfg, b.codes, n)
+    assert_codes_match(x, codes, cb, 1)
+    want = oracle.decode(codes, b.std.cpu().numpy().view(np.uint16)[:n], cb, dim, 1)
+    assert np.abs(out.cpu().numpy() - want).max() <= RECON_TOL and np.abs(rotated.cpu().numpy() - want).max() <= RECON_TOL
+    want_count, want_total = oracle.ema_stats(x, codes, cb, 1)
+    assert np.array_equal(count.cpu().numpy(), want_count)
+    assert np.max(np.abs(total.cpu().numpy() - want_total) / np.maximum(1.0, want_count)[..., None]) <= 1e-4
+    assert rvq.read_status(b.status)["bad_codes"] == 0
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+def test_kmeans_of_one_group(layout):
+    test_gpu_learning.test_kmeans_init_on_separated_clusters(layout, 1)
 
 
 @pytest.mark.parametrize("K,gd", [(2, 8), (33, 64), (1000, 32), (2048, 32)])
