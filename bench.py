@@ -51,12 +51,14 @@ def workload_name(tokens):
 # kernels as they stand, keyed by (kernel, workload, tokens): an entry holds for that launch only, any other size
 # reports null.  An entry is taken out when its kernel changes.
 DRAM_TRAFFIC = {
-    # encode with the EMA statistics fused in: 272.2 MB read + 56.1 MB written over 1,048,576 head vectors
-    ("encode_tensor_kernel", "ema_learning", 131072): 272150528 + 56126208,
-    # decode, strided layout: 70.0 MB read + 214.3 MB written (the rest of the 268 MB output still sat in L2
+    # encode with the EMA statistics fused in: 272.9 MB read + 55.0 MB written over 1,048,576 head vectors
+    ("encode_tensor_kernel", "ema_learning", 131072): 272936192 + 54961408,
+    # decode, contiguous layout: 72.4 MB read + 213.1 MB written (the rest of the 268 MB output still sat in L2
     # when the kernel ended)
-    ("decode_quoted_kernel", "decode_bandwidth", 131072): 70008064 + 214296320,
+    ("decode_quoted_kernel", "decode_bandwidth", 131072): 72387584 + 213052160,
 }
+# share of the tensor pipe's cycles that one launch keeps busy (%), from the same captures
+TENSOR_PIPE_PCT = {("encode_tensor_kernel", "ema_learning", 131072): 61.1}
 
 
 def algorithmic_numbers(w, bits=None):
@@ -207,13 +209,12 @@ def side_workloads(torch, rvq, peaks, flush):
     out = {}
     hbm, tensor = peaks["hbm_gbs"], peaks["bf16_tflops"]
 
-    def encode_line(w, cfg, b, x):
+    def encode_line(w, cfg, b, x, steps):
+        # steps: K-steps of a score chain on this workload (five where the two small products are taken in 8 bits)
         alg = algorithmic_numbers(w)
         med, best = time_launches(torch, lambda: rvq.rvq_encode(cfg, x, w.n, w.dim, b.codebooks, b.prepared, b.codes,
                                                                 b.std, b.workspace, b.workspace_bytes, b.status), flush)
         tf = alg["encode_flops"] / med / 1e9
-        # K-steps of a score chain: many values on 1024 codes or more take the two small products in 8 bits
-        steps = 5 if w.layout == rvq.CONTIGUOUS and w.codebook_size >= 1024 and w.n * 4 > 128 * 4 * 148 else 7
         return {"ms": med, "ms_best": best, "Mvectors/s": w.n / med / 1e3, "useful_TFLOP/s": tf,
                 "frac_tensor": tf / tensor, "pipe_equivalent_TFLOP/s": steps / 2 * tf,
                 "note": f"useful = 2*32*K*R*4 flop per head vector; the MMA chains execute {steps / 2}x that ({steps} K-steps, 2 useful)"}
@@ -273,7 +274,7 @@ def side_workloads(torch, rvq, peaks, flush):
     cfg = rvq.make_config(w.dim, w.group_dim, w.layout, w.depth, w.codebook_size, w.code_bits, rvq.BF16, 0)
     b = rvq.alloc_buffers(cfg, w.n, w.codebooks)
     x = torch.from_numpy(w.x_bits.view(np.int16)).view(torch.bfloat16).cuda()
-    enc = encode_line(w, cfg, b, x)
+    enc = encode_line(w, cfg, b, x, 5)
     out_t = torch.empty(w.n, w.dim, dtype=torch.bfloat16, device="cuda")
     out["value_cache"] = {"workload": "262144 head vectors, K=2048, R=8, contiguous groups, 11-bit packed codes",
                           "encode": enc, "decode": decode_line(w, cfg, b, out_t, None)}
@@ -284,7 +285,7 @@ def side_workloads(torch, rvq, peaks, flush):
     cfg = rvq.make_config(w.dim, w.group_dim, w.layout, w.depth, w.codebook_size, w.code_bits, rvq.BF16, 0)
     b = rvq.alloc_buffers(cfg, w.n, w.codebooks)
     x = torch.from_numpy(w.x_bits.view(np.int16)).view(torch.bfloat16).cuda()
-    out["key_cache"] = {"workload": "32768 head vectors, K=1024, R=8, strided groups", "encode": encode_line(w, cfg, b, x)}
+    out["key_cache"] = {"workload": "32768 head vectors, K=1024, R=8, strided groups", "encode": encode_line(w, cfg, b, x, 7)}
     del b, x
     torch.cuda.empty_cache()
     return out
@@ -519,7 +520,7 @@ def run_ours(args):
                                         "EMA apply) on all GPUs",
                             "encode_Mvectors/s_per_gpu": n / enc_ms / 1e3,
                             "encode_useful_fraction_of_tensor_peak": enc_tflops / tensor_peak,
-                            "encode_tensor_pipe_active_pct_ncu": 52.2 if args.tokens == 131072 else None,
+                            "encode_tensor_pipe_active_pct_ncu": TENSOR_PIPE_PCT.get(("encode_tensor_kernel", "ema_learning", args.tokens)),
                             "decode_in_step_GB/s": alg["decode_bytes"] / dec_ms / 1e6}
     if world == 1:
         del x_slot, out_slot, recon, x_dev
@@ -534,7 +535,7 @@ def run_ours(args):
                                    "bound": "hbm", "achieved": d4["GB/s"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
                                    "frac": d4["frac_hbm"],
                                    "traffic": dtraffic,
-                                   "traffic_note": "dram bytes read + written by one launch under ncu, strided layout",
+                                   "traffic_note": "dram bytes read + written by one launch under ncu, contiguous layout",
                                    "peak_source": f"{peaks['source']} copy bandwidth"}
 
     if world == 1 and not args.no_cpu_baseline:

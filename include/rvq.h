@@ -178,11 +178,12 @@ int rvq_encode_exact(const rvq_config *cfg /* host */, const void *x, int64_t n,
  * Decode (Section 2.2, last sentence; Section 3.2).  For every head vector and
  * channel c = channel(g, i): x_out[c] = std * sum_r C_r[code[g][r]][i], summed
  * in float32 and rounded once to x_dtype.  For groups of 32 (a power-of-two number
- * of them) with depth <= 8 the codebook entries are read from the float32 codebooks in L2 (four groups or
- * more: few vectors, float32 outputs, more than 1536 codes or other depths than 8; exact float32 sums)
- * or from shared-memory tables: float32
- * copies (up to 3584 codes per stage) or, for 16-bit outputs and up to 3072
- * codes, 16-bit levels of each stage's value range kept in the prepared block.
+ * of them) with depth <= 8 the codebook entries come from the float32 codebooks in L2 (four groups or
+ * more: few vectors, float32 outputs, more than 1536 codes or depths below 8; exact float32 sums)
+ * or from shared-memory tables (one or two groups; four and more for 16-bit outputs at depth 8 with up to
+ * 1536 codes of 10 or more bits and, for four groups, more than 28672 vectors): float32 copies (one or two groups up to 3584 codes
+ * per stage) or, for 16-bit outputs and up to 3072 codes, 16-bit levels of each stage's value range kept in the
+ * prepared block.
  * With the levels the sum before the multiplication by std is within
  * err <= 1.04 * sum_r (max C_r - min C_r) * 2^-17 of the float32 one (levels of
  * each stage's own range), or within 4.1 * sum_r (max C_r - min C_r) * 2^-17 (levels
@@ -191,8 +192,9 @@ int rvq_encode_exact(const rvq_config *cfg /* host */, const void *x, int64_t n,
  * and takes the coarsest table that keeps std * err below 0.9e-3, or the float32
  * tables; a single head vector whose std would still make std * err exceed 0.9e-3
  * gets the float32 sum instead, so the value before the final rounding is always
- * within 1e-3 of the exact one.  Other shapes gather the float32 codebooks from
- * global memory.
+ * within 1e-3 of the exact one.  A vector may so be rounded differently in a batch of few
+ * vectors (float32 sums) and in one of many (tables), always within that bound.
+ * Other shapes gather the float32 codebooks from global memory.
  *   codes, std_f16  in   as produced by rvq_encode
  *   x_out           out  n rows of x_dtype, row v at element v * out_row_stride
  * A code >= K is read as code 0 and counted in status->bad_codes.
@@ -217,14 +219,13 @@ int rvq_decode(const rvq_config *cfg /* host */, const void *codes, const uint16
  *                             rvq_rope_table
  *   prepared              in  block of rvq_prepare_codebooks for these codebooks, or NULL
  * Four or more groups of 32 (a power-of-two number) with depth <= 8 read the float32 codebooks in L2 (exact
- * sums), but for many vectors of dim 128 at depth 8 with up to 1536 codes, 16-bit outputs and a prepared block.  Those,
- * and two groups: up to 3584 codes per stage float32
- * shared-memory tables (exact float32 sums); with 16-bit outputs and a prepared block also
- * the level tables described under rvq_decode (dim 128 at depth 8 with up to 1536 codes:
- * both kinds of level table, 8-channel slices, one launch; 1537..3072 codes: the per-stage
- * levels), chosen when the deviations are moderate (a head vector whose std would make
+ * sums), but for more than 131072 vectors of dim 128 at depth 8 with up to 1536 codes (of 10, 11 or 16 bits),
+ * 16-bit outputs and a prepared block: there one launch takes level tables of either kind described under
+ * rvq_decode, or float32 ones, by a sample of the deviations.  Two groups: float32 tables in shared memory
+ * up to 3584 codes per stage (exact float32 sums); with 16-bit outputs, a prepared block and
+ * 1537..3072 codes also the per-stage levels.  With level tables a head vector whose std would make
  * std * err exceed 0.6e-3 gets float32 sums, so the rotated value before the final
- * rounding stays within 1e-3 of the exact one).  Other shapes gather from global memory.
+ * rounding stays within 1e-3 of the exact one.  Other shapes gather from global memory.
  */
 enum { RVQ_ROPE_HALVES = 0, RVQ_ROPE_ADJACENT = 1 };
 int rvq_decode_rope(const rvq_config *cfg /* host */, const void *codes, const uint16_t *std_f16,

@@ -181,9 +181,14 @@ decode_direct_kernel(Shape s, const void *__restrict__ codes, const uint16_t *__
 
 // Where the table decoders are the faster ones: 16-bit outputs at depth 8 with up to 1536 codes (8-channel level
 // tables, or 4-channel float32 ones for large deviations), from a number of group rows on that pays for filling
-// them.  Measured (us, tables / direct, K = 1024, dim 128): moderate deviations 32768 vectors 9.7 / 10.2, 65536
-// 13.5 / 18.1, 262144 37 / 63; keys 65536 23 / 20, 262144 61 / 75; rotary keys 131072 47 / 46, 262144 80 / 95; dim
-// 256: 65536 27 / 33.  Direct wins at every size for 2048 codes (262144 vectors 74 / 61; keys 117 / 75, rotary
+// them.  Which tables a batch takes, and so where it crosses, hangs on its deviations, which the host does not know: the lines
+// stand where values cross, and for rotated vectors where keys do.  Measured (us, tables / direct, K = 1024, dim 128):
+//   values (level tables)     16384 vectors 8.3 / 8.2, 28672 10.4 / 10.3, 32768 10.4 / 10.4, 65536 14.4 / 18.6, 131072 22.6 / 33.1;
+//   keys (float32 tables)     28672 16.5 / 11.8, 65536 22.7 / 20.6, 98304 29.4 / 28.8, 131072 37.0 / 39.2, 262144 62 / 78: from 28673 to
+//                             about 100000 keys that are read back unrotated lose up to 5 us;
+//   keys, rotated             65536 30.9 / 25.6, 98304 39.1 / 37.1, 131072 47.3 / 49.7, 196608 66 / 74;
+//   moderate deviations, rotated   32768 14.4 / 13.3, 65536 18.6 / 22.6, 131072 32.9 / 43.1: these lose up to 10 us before the line.
+// dim 256: 65536 27 / 33.  Direct wins at every size for 2048 codes (262144 vectors 74 / 61; keys 117 / 75, rotary
 // 232 / 93), float32 outputs (110 / 68) and smaller depths (depth 4: 57 / 41, float32 103 / 46).
 bool decode_direct_wanted(const Shape &s, int64_t n, bool rope, bool prepared)
 {

@@ -250,8 +250,9 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1, const Stage
 // above, the dot product is off by at most
 //   |z_lo.e - [64 z_lo][e/64]|        <= ||z_lo|| (cE + (1 + c)(cE + 64 sqrt(32) 2^-10)) + sqrt(32) 2^-16 (1 + c) E
 //   |z_hi.e_lo - [z_hi/64][64 e_lo]|  <= (cN + 0.354) L + ((1 + c) N + 0.354)(cL + sqrt(32) 2^-16)
-// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (the worst of 330000
-// chains on operands of this shape, x20 outlier channels among them, was 9.4e-5 |z||e|).
+// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (prepare.cu; five instructions
+// of two kinds add up no worse than seven of one).  That comes to some 2^-13 |z||e|; the worst of 6.3 million
+// chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.
 __device__ __forceinline__ float window8(float nz, float nl, float e, const StageBounds &sb)
 {
     constexpr float c = 0.0595f;

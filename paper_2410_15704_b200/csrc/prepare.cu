@@ -312,9 +312,10 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
 //   times 2 for the factor -2 of the score; plus the accumulation of 115 terms
 //   in the tensor core, taken as 2^-19 of nmax + 2 ||Z|| emax, which bounds the
 //   sum of the terms' magnitudes.  The hardware's accumulation is not
-//   documented; measured on B200 against float64 on operands of this shape
-//   (with and without x20 outlier channels) the chain's error stayed below
-//   2^-20.6 of the sum of magnitudes, so 2^-19 leaves a factor of 3; the tests
+//   documented; measured on B200 against float64 sums of the very operands, 6.3
+//   million chains each, the error was at most 2^-20.7 of the sum of magnitudes on
+//   normal data and 2^-20.0 with x20 outlier channels, so 2^-19 leaves a factor of
+//   2 (the chain with 8-bit corrections: 2^-22.3 and 2^-20.9); the tests
 //   compare tens of millions of choices with the all-float32 kernel's.
 __global__ void prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxima *mx)
 {

@@ -62,15 +62,16 @@ __host__ __device__ inline size_t decode_table_bytes(int K) { return (size_t)K *
 // the prepared block holds two such tables: levels scaled per stage, then levels summed per stage parity
 constexpr int kDecodeExactWideK = 1792;                   // float32 tables: 128 bytes per code per 4-channel slice
 constexpr int kDecodeExactK = 3584;                       // ... 64 bytes per code per 2-channel slice
-// Which decoder serves a shape (group_dim 32, a power-of-two number of groups up to 32, depth <= 8; everything
+// Which tables a shape can be decoded through (group_dim 32, a power-of-two number of groups up to 32, depth <= 8; of
+// these, four groups and more take their codewords from L2 instead where decode_direct_wanted says so; everything
 // else gathers from global memory):
 //   - float32 table slices (exact sums, any output type) fit shared memory up to kDecodeExactK codes
 //     (4 channels per slice up to kDecodeExactWideK, 2 beyond);
 //   - 16-bit level tables (16-bit outputs only: their own rounding, 2^-9 or 2^-12 relative, dwarfs the
 //     tables') fit up to kDecodeMaxK codes and are the faster ones while the deviations are moderate;
 //   - where both fit (16-bit outputs, up to kDecodeMaxK codes) a sample of the deviations decides on the
-//     device: four groups at depth 8 in one launch that holds all three kinds of table, other shapes as
-//     two launches of which the one not called for returns at once.
+//     device: four groups at depth 8 with up to kDecodeWideK codes in one launch that holds all three kinds of table, other
+//     shapes as two launches of which the one not called for returns at once.
 __host__ __device__ inline bool decode_exact_tables(const Shape &s)
 {
     return s.gd == 32 && s.G <= 32 && (s.G & (s.G - 1)) == 0 && s.R <= 8 && s.K <= kDecodeExactK;
