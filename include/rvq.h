@@ -89,10 +89,10 @@ const char *rvq_status_string(int code);
 int rvq_version(void);
 
 /* Diagnostic: number of kernels this library has launched in this process so
- * far.  (Process-wide state of the library: this counter, what launches have
- * asked about each device and context (SM count, shared memory granted to each
- * kernel, resident clusters), and the per-device address of the built-in scratch
- * array that rvq_ema_update_static resolves on its first call.) */
+ * far.  (Process-wide state of the library: this counter, and what launches have
+ * asked about each device and context: SM count, shared memory granted to each
+ * kernel, resident clusters, and the address of the built-in scratch array that
+ * rvq_ema_update_static resolves on its first call.) */
 uint64_t rvq_launch_count(void);
 
 /* Bytes of one head vector's codes in the configured storage form
@@ -386,12 +386,10 @@ int rvq_kmeans_init(const rvq_config *cfg /* host */, const void *x, int64_t n, 
  * allocates and frees nothing.
  *
  * Arguments, results and error codes are those of rvq_ema_update.  Differences:
- *   - The first call on each device looks up the array's device address (a
- *     runtime query, not a launch) and keeps it.  Make that first call outside
- *     any stream capture.  The kept address belongs to the device's primary
- *     context: after cudaDeviceReset the array lives elsewhere, so do not call
- *     this entry point on a device that has been reset since its first call.
- *   - All calls, on every stream, share the one array, and it still holds the
+ *   - The first call in each context looks up the array's device address (a
+ *     runtime query, not a launch) and keeps it for that context.  Make that
+ *     first call outside any stream capture.
+ *   - All calls of a context, on every stream, share the one array, and it still holds the
  *     previous call's numbers when the next begins; each call clears the parts
  *     it accumulates into.  Two calls that can overlap on the GPU (different
  *     streams without an ordering between them) corrupt each other: order them.

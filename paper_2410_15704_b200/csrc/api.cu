@@ -1,9 +1,8 @@
 // extern "C" boundary of the RVQ library: argument checks on the host, then
 // dispatch to the kernels.  No allocation, no synchronisation.  Process-wide
-// state: the launch counter below, what is remembered about each device (its SM
-// count) and each context (the shared memory granted to each kernel), and (in
-// ema.cu) the per-device address of the built-in scratch array of
-// rvq_ema_update_static.
+// state: the launch counter below, and what is remembered about each device (its
+// SM count) and each context (the shared memory granted to each kernel, resident
+// clusters, the address of the built-in scratch array of rvq_ema_update_static).
 #include "prepared.cuh"
 #include "rvq_selftest.h"
 
@@ -36,6 +35,7 @@ constexpr int kGrantSlots = 512;                          // (a few times the li
 constexpr int kContexts = 8;
 struct Context {
     std::atomic<uint64_t> number{0};                      // the driver's, plus one
+    std::atomic<void *> scratch{nullptr};                 // (context_scratch)
     Grant grants[kGrantSlots];
 };
 Context g_contexts[kContexts];
@@ -55,21 +55,26 @@ uint64_t current_context()
     return get_id && get_id(nullptr, &number) == CUDA_SUCCESS ? (uint64_t)number + 1 : 0;
 }
 
-Grant *grant_of(const void *kernel)
+// What is remembered about it; null: nothing can be.
+Context *context()
 {
     const uint64_t number = current_context();
     if (number == 0) return nullptr;
-    Grant *grants = nullptr;
-    for (int k = 0; k < kContexts && !grants; ++k) {
-        Context &c = g_contexts[k];
+    for (Context &c : g_contexts) {
         uint64_t have = c.number.load(std::memory_order_acquire);
         if (have == 0 && c.number.compare_exchange_strong(have, number)) have = number;
-        if (have == number) grants = c.grants;
+        if (have == number) return &c;
     }
-    if (!grants) return nullptr;
+    return nullptr;
+}
+
+Grant *grant_of(const void *kernel)
+{
+    Context *const c = context();
+    if (!c) return nullptr;
     const uint32_t h = (uint32_t)((reinterpret_cast<uintptr_t>(kernel) >> 4) * 2654435761u) >> 7;
     for (uint32_t k = 0; k < (uint32_t)kGrantSlots; ++k) {
-        Grant &g = grants[(h + k) % kGrantSlots];
+        Grant &g = c->grants[(h + k) % kGrantSlots];
         const void *have = g.kernel.load(std::memory_order_acquire);
         if (have == nullptr && g.kernel.compare_exchange_strong(have, kernel)) have = kernel;
         if (have == kernel) return &g;
@@ -78,6 +83,12 @@ Grant *grant_of(const void *kernel)
 }
 
 }  // namespace
+
+std::atomic<void *> *context_scratch()
+{
+    Context *const c = context();
+    return c ? &c->scratch : nullptr;
+}
 
 int sm_count()
 {

@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "rvq.h"
 
 namespace rvq {
@@ -89,6 +91,7 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
 // Facts that a launch needs, looked up once per device or per context and kernel and remembered: the three
 // runtime queries they replace were a third of the host's time in a call.
 int sm_count();                                            // 0: no device
+std::atomic<void *> *context_scratch();                    // this context's place for the address of a device array; null: none
 bool allow_shared_memory(const void *kernel, int bytes);   // dynamic shared memory of up to `bytes` for this kernel
 
 // Clusters of `ctas` CTAs of this kernel that the current device runs at a time (0: none), and their launch:

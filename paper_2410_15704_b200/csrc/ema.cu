@@ -3,8 +3,6 @@
 // normalisation.
 #include "common.cuh"
 
-#include <atomic>
-
 namespace rvq {
 
 static size_t round256(size_t b) { return (b + 255) / 256 * 256; }
@@ -389,23 +387,15 @@ namespace {
 constexpr size_t kStaticScratchBytes = 65536 + 65536 + 2097152;
 static __device__ __align__(256) unsigned char g_ema_scratch[kStaticScratchBytes];
 
-constexpr int kMaxDevices = 64;
-// Device address of g_ema_scratch per device ordinal (null: not looked up yet).  Host threads may race to
-// fill an entry: they all store the same value, and the atomic keeps the store and the loads whole.  The
-// cache assumes the runtime's one primary context per device; after cudaDeviceReset the array lives at a
-// new address, so a process that resets a device must not call this entry point on it again.
-std::atomic<void *> g_scratch_addr[kMaxDevices];
-
-// The array's name is only a handle on the host; the address a kernel can use
-// has to be asked for, once per device, with that device current.
+// The array's name is only a handle on the host; the address a kernel can use has to be asked for, once in every
+// context (each has an array of its own).  Host threads may race to ask: they all store the same value.
 int static_scratch(void **out)
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return RVQ_ERR_DEVICE;
-    void *ptr = g_scratch_addr[dev].load(std::memory_order_acquire);
+    std::atomic<void *> *const slot = rvq::context_scratch();
+    void *ptr = slot ? slot->load(std::memory_order_acquire) : nullptr;
     if (!ptr) {
         if (cudaGetSymbolAddress(&ptr, g_ema_scratch) != cudaSuccess || !ptr) return RVQ_ERR_DEVICE;
-        g_scratch_addr[dev].store(ptr, std::memory_order_release);
+        if (slot) slot->store(ptr, std::memory_order_release);
     }
     *out = ptr;
     return RVQ_OK;

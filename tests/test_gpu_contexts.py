@@ -63,7 +63,15 @@ def run():
             assert rc == 0, ("decode", rc)
             ask("cuCtxSynchronize")
             out.append(download(back, n * 256))
-    return out
+    # the update whose scratch is an array of the library, one to a context (whole numbers: exact sums in any order)
+    cfg = rvq.make_config(128, 32, 0, 1, 64, 16, rvq.F32, 0)
+    x, codes = upload(np.tile(np.repeat(np.float32([1, -1]), 64), (500, 1))), upload((np.arange(2000) % 64).astype(np.uint16))
+    cb, count, total = upload(np.ones((64, 32), np.float32)), upload(np.ones(64, np.float32)), upload(np.ones((64, 32), np.float32))
+    for _ in range(2):
+        rc = rvq.lib.rvq_ema_update_static(ctypes.byref(cfg), x, 500, 128, codes, cb, count, total, None, 0.5, 0.0, None, None)
+        assert rc == 0, ("update", rc)
+    ask("cuCtxSynchronize")
+    return out + [download(cb, 64 * 32 * 4), download(count, 64 * 4), download(total, 64 * 32 * 4)]
 
 
 device, primary, second = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_void_p()
