@@ -106,17 +106,16 @@ __global__ void __launch_bounds__(256)
 prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
 {
     follow_previous();
-    __shared__ double rn[256], r2[256], r4[256];
-    __shared__ float rlo[256], rhi[256];
+    __shared__ StagePartial warps[8];
     const int r = blockIdx.y, tid = threadIdx.x;
     const int per = (s.K + kPrepareParts - 1) / kPrepareParts;
     const int j0 = blockIdx.x * per, j1 = min(s.K, j0 + per);
-    double m = 0.0, sum2 = 0.0, sum4 = 0.0;
-    float lo = INFINITY, hi = -INFINITY;
+    double m = 0.0;
+    float lo = INFINITY, hi = -INFINITY, sum2 = 0.0f, sum4 = 0.0f;
     for (int j = j0 + tid; j < j1; j += 256) {
         const float *e = cb + ((size_t)r * s.K + j) * s.gd;
         double acc = 0.0;
-        auto add = [&](float v) { const double v2 = (double)v * (double)v; acc += v2; sum4 = fma(v2, v2, sum4); lo = fminf(lo, v); hi = fmaxf(hi, v); };
+        auto add = [&](float v) { acc += (double)v * (double)v; sum4 = fmaf(v * v, v * v, sum4); lo = fminf(lo, v); hi = fmaxf(hi, v); };
         if (s.gd == 32) {
             float4 f[8];                                      // (asked for together)
 #pragma unroll
@@ -127,21 +126,26 @@ prepare_reduce_kernel(Shape s, const float *cb, StagePartial *part)
             for (int i = 0; i < s.gd; ++i) add(e[i]);
         }
         m = fmax(m, acc);
-        sum2 += acc;
+        sum2 += (float)acc;
     }
-    rn[tid] = m; r2[tid] = sum2; r4[tid] = sum4; rlo[tid] = lo; rhi[tid] = hi;
+    // (within a warp by shuffles: with the moments in a tree over 256 entries in shared memory, preparing 2048 codes took 19.5 us, in
+    // float64 20.5; this way 18.5, as without them)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
+        sum2 += __shfl_xor_sync(0xFFFFFFFFu, sum2, off); sum4 += __shfl_xor_sync(0xFFFFFFFFu, sum4, off);
+        lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, off)); hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, off));
+    }
+    if ((tid & 31) == 0) warps[tid >> 5] = StagePartial{m, sum2, sum4, lo, hi};
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (tid < w) {
-            rn[tid] = fmax(rn[tid], rn[tid + w]);
-            r2[tid] += r2[tid + w]; r4[tid] += r4[tid + w];
-            rlo[tid] = fminf(rlo[tid], rlo[tid + w]); rhi[tid] = fmaxf(rhi[tid], rhi[tid + w]);
-        }
-        __syncthreads();
-    }
     if (tid == 0) {
-        StagePartial &o = part[r * kPrepareParts + blockIdx.x];
-        o.max_norm2 = rn[0]; o.sum2 = r2[0]; o.sum4 = r4[0]; o.lo = rlo[0]; o.hi = rhi[0];
+        StagePartial o = warps[0];
+        for (int w = 1; w < 8; ++w) {
+            o.max_norm2 = fmax(o.max_norm2, warps[w].max_norm2);
+            o.sum2 += warps[w].sum2; o.sum4 += warps[w].sum4;
+            o.lo = fminf(o.lo, warps[w].lo); o.hi = fmaxf(o.hi, warps[w].hi);
+        }
+        part[r * kPrepareParts + blockIdx.x] = o;
     }
 }
 
@@ -158,14 +162,14 @@ prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, St
     __syncwarp();
     bool even = false;
     if (r < s.R) {
-        double maxn = 0.0, sum2 = 0.0, sum4 = 0.0;
-        float lo = INFINITY, hi = -INFINITY;
+        double maxn = 0.0;
+        float lo = INFINITY, hi = -INFINITY, sum2 = 0.0f, sum4 = 0.0f;
 #pragma unroll
         for (int q = 0; q < kPrepareParts; ++q) {
             const StagePartial pp = part[r * kPrepareParts + q];
             maxn = fmax(maxn, pp.max_norm2); sum2 += pp.sum2; sum4 += pp.sum4; lo = fminf(lo, pp.lo); hi = fmaxf(hi, pp.hi);
         }
-        even = sum4 * (double)s.K * (double)s.gd <= kEvenKurtosis * sum2 * sum2;
+        even = sum4 * (float)(s.K * s.gd) <= kEvenKurtosis * sum2 * sum2;
         int k = 12;
         if (maxn > 0.0 && isfinite(maxn)) {
             k = (int)floor(0.5 * log2(8192.0 / maxn));

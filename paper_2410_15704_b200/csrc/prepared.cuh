@@ -19,7 +19,7 @@ constexpr size_t kPreparedParamsOffset = 256;             // StageParams[16]
 constexpr size_t kPreparedMaximaOffset = 512;             // StageMaxima[16]
 constexpr size_t kPreparedPartialsOffset = 768;           // StagePartial[16 stages][kPrepareParts], scratch of the prepare step
 constexpr int kPrepareParts = 16;
-constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 32;   // operand image, [R][slots][kSlotStride]
+constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 24;   // operand image, [R][slots][kSlotStride]
 
 struct PreparedHeader {
     uint32_t magic, R, K, gd, slots;
@@ -29,7 +29,7 @@ struct PreparedHeader {
 // A stage's codewords count as even when the fourth moment of their entries is at most this many times the square of the
 // second (3 for a normal distribution); the block does when at least half of its stages do.  The throughput encoder
 // takes the 8-bit corrections by it (encode_tensor.cu).
-constexpr double kEvenKurtosis = 6.0;
+constexpr float kEvenKurtosis = 6.0f;
 
 // Decoder section (group_dim 32, R <= 8, K <= kDecodeMaxK): per stage an affine
 // map value = lo_r + q * scale_r * base with q a 16-bit level, scale_r an integer in
@@ -126,7 +126,7 @@ struct StageParams {
 
 struct StagePartial {
     double max_norm2;   // largest squared norm among this part's codewords
-    double sum2, sum4;  // sums of the entries' squares and fourth powers
+    float sum2, sum4;   // sums of the entries' squares and fourth powers
     float lo, hi;       // smallest and largest entry
 };
 
