@@ -8,7 +8,6 @@
 namespace rvq {
 
 constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
-constexpr int kOnesBytes = 2 * 128 * 16;                  // the constant A cells (1 1 1 0 ...) and (0 ...)
 constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 or e4m3 x e4m3 -> f32, M = N = 128
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -82,13 +81,6 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
            ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
-__device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                           uint32_t accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
 __device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
                                            uint32_t accumulate)
 {
@@ -175,6 +167,15 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// The constant A operand of the norm's step, (1 1 1 0 ... 0) in every row: eight TMEM columns, written once by the
+// four warps that reach the 128 lanes.  (From shared memory the tensor core read 4 KB for it in every chain.)
+__device__ __forceinline__ void tmem_ones(uint32_t taddr)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %3, %3, %3, %3, %3};"
+                 : : "r"(taddr), "r"(0x3C003C00u), "r"(0x00003C00u), "r"(0u) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
 // Per-row state of one stage's sweep over the scores.
 struct Sweep {
     float win;               // error window
@@ -216,14 +217,27 @@ __device__ __forceinline__ float fold_block(Sweep &w, const uint32_t (&u)[32], i
     return m;
 }
 
-// The stage's maxima over its codewords (prepare.cu), for the window below.
-struct StageBounds {
-    float emax, eerr, elo;                  // norms: codeword, what its two halves miss, its remainder half
+// What a stage's rows need to know of its codebook (prepare.cu), copied to shared memory at the start: asked for in the
+// prepared block when it was needed, every stage end waited for it.
+struct StageConst {
+    float scale, a, b;                      // operand scale; |score error| <= a ||Z|| + b
+    float emax, eerr, elo;                  // norms, the stage's largest: codeword, what its two halves miss, its remainder half
 };
-__device__ __forceinline__ StageBounds stage_bounds(const uint8_t *prepared, int r)
+__device__ __forceinline__ void load_stage_consts(const uint8_t *prepared, int R, int tid, StageConst *out)
 {
-    const uint4 m = __ldg(reinterpret_cast<const uint4 *>(prepared + kPreparedMaximaOffset) + r);     // StageMaxima
-    return {__uint_as_float(m.x), __uint_as_float(m.y), __uint_as_float(m.w)};
+    if (tid < R) {
+        const StageParams q = reinterpret_cast<const StageParams *>(prepared + kPreparedParamsOffset)[tid];
+        const uint4 m = __ldg(reinterpret_cast<const uint4 *>(prepared + kPreparedMaximaOffset) + tid);     // StageMaxima
+        out[tid] = StageConst{q.scale, q.a, q.b, __uint_as_float(m.x), __uint_as_float(m.y), __uint_as_float(m.w)};
+    }
+}
+
+// Square root for the bounds below, whose factors of 1.0001 leave room for its 2^-22; the rounded one is a subroutine.
+__device__ __forceinline__ float rough_sqrt(float v)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 // A column can only be the exact-L2 choice (in real arithmetic, and in the float32 direct-form
@@ -234,10 +248,10 @@ __device__ __forceinline__ StageBounds stage_bounds(const uint8_t *prepared, int
 // approximate winner's squared distance, at most m1 + zz + win; so their norms are at most E = ||Z|| + rho,
 // and the error bound of prepare.cu, which allows every codeword the largest norm of the stage, is taken
 // with E where that is smaller.
-__device__ __forceinline__ float threshold(const Sweep &w, float m1, const StageBounds &sb)
+__device__ __forceinline__ float threshold(const Sweep &w, float m1, const StageConst &sb)
 {
-    const float nz = sqrtf(w.zz) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
-    const float e = fminf(sb.emax, (nz + sqrtf(d2 + w.win)) * 1.0001f);
+    const float nz = rough_sqrt(w.zz) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
+    const float e = fminf(sb.emax, (nz + rough_sqrt(d2 + w.win)) * 1.0001f);
     const float elo = fminf(sb.elo, 4.8828125e-4f * e + 1.7e-7f), eerr = fminf(sb.eerr, 2.384185791015625e-7f * e + 1.7e-7f);
     const float a = 2.0f * (4.8828125e-4f * elo + 2.384185791015625e-7f * e + eerr) + 3.814697265625e-6f * e;
     const float b = e * (1.9073486328125e-6f * e + 4.76837158203125e-7f);
@@ -253,7 +267,7 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1, const Stage
 // with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (prepare.cu; five instructions
 // of two kinds add up no worse than seven of one).  That comes to some 2^-13 |z||e|; the worst of 6.3 million
 // chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.
-__device__ __forceinline__ float window8(float nz, float nl, float e, const StageBounds &sb)
+__device__ __forceinline__ float window8(float nz, float nl, float e, const StageConst &sb)
 {
     constexpr float c = 0.0595f;
     const float elo = fminf(sb.elo + sb.eerr, 4.8828125e-4f * e + 1.7e-7f);
@@ -261,11 +275,11 @@ __device__ __forceinline__ float window8(float nz, float nl, float e, const Stag
     const float t2 = (c * nz + 0.354f) * elo + ((1.0f + c) * nz + 0.354f) * (c * elo + 8.7e-5f);
     return 2.125f * (2.0f * (t1 + t2) + 1.9073486328125e-6f * e * (e + 2.0f * nz) + 4.76837158203125e-7f * e);
 }
-__device__ __forceinline__ float threshold8(const Sweep &w, float m1, const StageBounds &sb)
+__device__ __forceinline__ float threshold8(const Sweep &w, float m1, const StageConst &sb)
 {
-    const float nz = sqrtf(w.zz) * 1.0001f, nl = sqrtf(w.ll) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
+    const float nz = rough_sqrt(w.zz) * 1.0001f, nl = rough_sqrt(w.ll) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
     const float full = window8(nz, nl, sb.emax, sb);
-    const float win = fminf(full, window8(nz, nl, fminf(sb.emax, (nz + sqrtf(d2 + full)) * 1.0001f), sb));
+    const float win = fminf(full, window8(nz, nl, fminf(sb.emax, (nz + rough_sqrt(d2 + full)) * 1.0001f), sb));
     return m1 + win + 5.4e-6f * (d2 + win);
 }
 
@@ -313,6 +327,17 @@ __device__ __forceinline__ void ldg256(const float *p, float (&v)[8])
     asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "l"(p));
+}
+
+__device__ __forceinline__ void load_codeword(const float *__restrict__ e, float (&v)[32])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float part[8];
+        ldg256(e + 8 * q, part);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[8 * q + k] = part[k];
+    }
 }
 
 // Exact squared distance, direct form, same operation order as the scalar kernel.
@@ -378,7 +403,7 @@ __device__ __forceinline__ void best_of_warp(float &bv, int &bi)
 // The seven K = 16 steps of one chain: 128 rows (A: TMEM columns a0 ..: 16 of head, 16 of remainder)
 // against the 128 codewords of the slot that `bd` describes, scores to the 128 columns from `acc`.  A
 // B cell is 128 codewords x 16 bytes = 128 descriptor address units.
-__device__ __forceinline__ void issue_chain(uint32_t acc, uint32_t a0, uint64_t bd, uint64_t ones_desc)
+__device__ __forceinline__ void issue_chain(uint32_t acc, uint32_t a0, uint64_t bd, uint32_t ones)
 {
     mma_f16_ts(acc, a0, bd + 5 * 128, kChainDesc, 0);            // hi[0:16]  . hi cells 5-6
     mma_f16_ts(acc, a0 + 8, bd + 7 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 7-8
@@ -386,19 +411,19 @@ __device__ __forceinline__ void issue_chain(uint32_t acc, uint32_t a0, uint64_t 
     mma_f16_ts(acc, a0 + 8, bd + 2 * 128, kChainDesc, 1);        // hi[16:32] . lo cells 2-3
     mma_f16_ts(acc, a0 + 16, bd + 5 * 128, kChainDesc, 1);       // lo[0:16]  . hi cells 5-6
     mma_f16_ts(acc, a0 + 24, bd + 7 * 128, kChainDesc, 1);       // lo[16:32] . hi cells 7-8
-    mma_f16_ss(acc, ones_desc, bd + 4 * 128, kChainDesc, 1);     // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
+    mma_f16_ts(acc, ones, bd + 4 * 128, kChainDesc, 1);     // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
 }
 
 // The chain with 8-bit corrections, on the last nine cells of a slot: two K = 32 steps of e4m3 (TMEM columns a0 +
 // 16 ..: 8 of 64 times the remainder, 8 of a 64th of the head), then heads and norm in half precision.  Five
 // steps instead of seven: 327 against 455 cycles (measured).
-__device__ __forceinline__ void issue_chain8(uint32_t acc, uint32_t a0, uint64_t bd, uint64_t ones_desc)
+__device__ __forceinline__ void issue_chain8(uint32_t acc, uint32_t a0, uint64_t bd, uint32_t ones)
 {
     mma_e4m3_ts(acc, a0 + 16, bd + 5 * 128, kChainDesc, 0);      // [64 lo]_8    . [e / 64]_8 (cells 9-10 of the slot)
     mma_e4m3_ts(acc, a0 + 24, bd + 7 * 128, kChainDesc, 1);      // [hi / 64]_8  . [64 e_lo]_8 (cells 11-12)
     mma_f16_ts(acc, a0, bd + 1 * 128, kChainDesc, 1);            // hi[0:16]  . hi cells 5-6
     mma_f16_ts(acc, a0 + 8, bd + 3 * 128, kChainDesc, 1);        // hi[16:32] . hi cells 7-8
-    mma_f16_ss(acc, ones_desc, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
+    mma_f16_ts(acc, ones, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
 }
 
 // The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces through

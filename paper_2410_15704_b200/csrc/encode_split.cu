@@ -24,7 +24,7 @@ constexpr int kGroups = 3;                                // accumulators, and e
 constexpr int kSplitThreads = 448;                        // 12 epilogue warps, issuer, loader
 constexpr int kSplitRing = 6;
 constexpr int kMaxParts = 18;                             // groups of a cluster that have chunks
-constexpr int kATmem = kGroups * 128;                     // TMEM column of the A operand (32 columns)
+constexpr int kATmem = kGroups * 128, kOnesTmem = kATmem + 32;                     // TMEM column of the A operand (32 columns), and of the constant one (8)
 
 struct Part {                                             // what a group knows of a row at the stage end
     float m1, m2;                                         // its two lowest chunk minima
@@ -33,14 +33,14 @@ struct Part {                                             // what a group knows 
 };
 
 constexpr int kSOffB = 0;
-constexpr int kSOffOnes = kSOffB + kSplitRing * kSlotBytes;
-constexpr int kSOffZ = kSOffOnes + kOnesBytes;            // residuals, float [32][kZPitch]
+constexpr int kSOffZ = kSOffB + kSplitRing * kSlotBytes;  // residuals, float [32][kZPitch]
 constexpr int kZPitch = 129;                              // (odd: neither rows nor elements of a row share banks)
 constexpr int kSOffParts = kSOffZ + 32 * kZPitch * 4;     // Part [2][kMaxParts][128]
 constexpr int kSOffCodes = kSOffParts + 2 * kMaxParts * 128 * 16;
 constexpr int kSOffNorm = kSOffCodes + 128 * 16 * 2;      // squared norms of the scaled residuals
 constexpr int kSOffBars = kSOffNorm + 128 * 4;
-constexpr int kSplitSmem = kSOffBars + 256;
+constexpr int kSOffStages = kSOffBars + 256;              // StageConst[16]
+constexpr int kSplitSmem = kSOffStages + 16 * (int)sizeof(StageConst);
 
 constexpr int kSFull = 0, kSEmpty = kSplitRing, kSReady = 2 * kSplitRing, kSAccFull = kSReady + 1, kSAccFree = kSAccFull + kGroups,
               kSArrived = kSAccFree + kGroups, kSBars = kSArrived + 2;
@@ -88,17 +88,15 @@ encode_split_kernel(const SplitParams p)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_word)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (tid < 128) {
-        uint8_t *a = smem + kSOffOnes + tid * 16;
-        *reinterpret_cast<uint4 *>(a) = make_uint4(0x3C003C00u, 0x00003C00u, 0u, 0u);
-        *reinterpret_cast<uint4 *>(a + 2048) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    StageConst *sc = reinterpret_cast<StageConst *>(smem + kSOffStages);
+    load_stage_consts(p.prepared, R, tid, sc);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (ctas > 1) asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     const uint32_t tmem = *tmem_word;
+    // the constant A operand (the issuer hears of it with the first A operand, from the same warps)
+    if (warp < 4) tmem_ones(tmem + ((uint32_t)(warp * 32) << 16) + kOnesTmem);
 
     if (warp == 13) {
         // ------------------------------------------------------------ operand loader
@@ -123,7 +121,6 @@ encode_split_kernel(const SplitParams p)
     } else if (warp == 12) {
         // ------------------------------------------------------------ MMA issuer
         const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kSOffB), kSlotCodewords * 16, 128);
-        const uint64_t ones_desc = make_smem_desc(smem_u32(smem + kSOffOnes), 2048, 128);
         uint32_t slot = 0, full_par = 0, ready_par = 0;
         uint32_t used = 0;                                                // accumulators used at least once (bit per accumulator)
         uint32_t free_pars = 0;                                           // next parity to wait for, bit per accumulator
@@ -144,7 +141,7 @@ encode_split_kernel(const SplitParams p)
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
-                    issue_chain(tmem + 128u * (uint32_t)a, tmem + kATmem, bdesc0 + (uint64_t)(slot * (uint32_t)(kSlotBytes >> 4)), ones_desc);
+                    issue_chain(tmem + 128u * (uint32_t)a, tmem + kATmem, bdesc0 + (uint64_t)(slot * (uint32_t)(kSlotBytes >> 4)), tmem + kOnesTmem);
                     mma_commit(BAR(kSAccFull + a));
                     mma_commit(BAR(kSEmpty + slot));
                 }
@@ -164,7 +161,6 @@ encode_split_kernel(const SplitParams p)
         float *norm = reinterpret_cast<float *>(smem + kSOffNorm);
         uint16_t *codes_s = reinterpret_cast<uint16_t *>(smem + kSOffCodes);            // [row][16]
         const Part *parts = reinterpret_cast<const Part *>(smem + kSOffParts);          // [2][kMaxParts][128]
-        const StageParams *sp = reinterpret_cast<const StageParams *>(p.prepared + kPreparedParamsOffset);
         const int nparts = ctas * P;
         const uint32_t mine = smem_u32(smem + kSOffParts) + (uint32_t)((rank * P + grp) * 128 + row) * 16u;
         const int G = s.G;
@@ -220,7 +216,7 @@ encode_split_kernel(const SplitParams p)
             }
 #pragma unroll 1
             for (int r = 0; r < R && ok; ++r) {
-                const StageParams prm = sp[r];
+                const StageConst prm = sc[r];
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
                 const uint32_t par = (uint32_t)r & 1u;
                 Sweep w;
@@ -271,10 +267,9 @@ encode_split_kernel(const SplitParams p)
                 if (!ok) break;
                 // this group's part of the row, to every CTA of the cluster
                 if (grp != 0 && grp < cnt) w.zz = norm[row];              // (a group without chunks has nothing inside any window)
-                const StageBounds sb = stage_bounds(p.prepared, r);
-                w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
+                w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);
                 {
-                    const float lim = threshold(w, w.m1, sb);
+                    const float lim = threshold(w, w.m1, prm);
                     const Listed in = listed(w, lim);
                     const uint32_t sets = in.word() | (w.m3 <= lim ? 1u << 22 : 0u);
                     for (int to = 0; to < ctas; ++to)
@@ -298,7 +293,7 @@ encode_split_kernel(const SplitParams p)
                     k1 = m < m1 ? k : k1;
                     m1 = fminf(m1, m);
                 }
-                const float lim = threshold(w, m1, sb);
+                const float lim = threshold(w, m1, prm);
                 const Part best = mp[k1 * 128];
                 const Listed in{best.sets & 0xFFFFu, (best.sets >> 16) & 3u, (best.sets >> 18) & 15u};
                 const int j1 = (int)(best.chunks & 0xFFFFu) * 128 + in.column();

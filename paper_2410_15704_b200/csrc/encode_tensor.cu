@@ -32,7 +32,7 @@
 //   - The A operand (the residual split into half-precision head and remainder)
 //     lives in TMEM next to its tile's scores, so the tensor core fetches only B
 //     from shared memory; the constant (1 1 1 0 ...) rows that pick up the
-//     squared norms are one small shared-memory tile used by every MMA chain.
+//     squared norms are eight more columns, used by every MMA chain.
 //   - The float32 residual lives in registers between stages and is parked in
 //     shared memory during a stage's sweep; x is read once and only codes and
 //     the half-precision deviation are written.
@@ -41,7 +41,7 @@
 //     two chains of that sweep (count x codeword is added back by the caller's finishing kernel); the
 //     last stage's input is added by the epilogue warps.
 // TMEM columns of tile t: scores [160 t, 160 t + 128), A operand
-// [160 t + 128, 160 t + 160) (16 columns of head, 16 of remainder).
+// [160 t + 128, 160 t + 160) (16 columns of head, 16 of remainder); the constant operand [480, 488).
 // Every wait is bounded; a wait that gives up sets status->wait_timeouts, and
 // the kernel waits (bounded as well) for its copies and chains in flight and returns.
 #include "encode_mma.cuh"
@@ -55,15 +55,16 @@ constexpr int kRowsPerPass = 128 * kTiles;
 constexpr int kEpiThreads = kRowsPerPass;
 constexpr int kThreads = kEpiThreads + 32 * (kTiles + 1);  // + one MMA issuer warp per tile + loader warp
 constexpr int kRing = 9;                                  // operand slots in flight
+constexpr int kOnesCol = 480;                             // TMEM column of the constant operand (8 columns)
 constexpr int kTileCols = 160;                            // TMEM columns per tile: 128 scores + 32 of A operand
 
 constexpr int kOffB = 0;
-constexpr int kOffA = kOffB + kRing * kSlotBytes;                    
-constexpr int kOffZ = kOffA + kOnesBytes;                             // parked residuals, float [32][rows]
+constexpr int kOffZ = kOffB + kRing * kSlotBytes;                     // parked residuals, float [32][rows]
 constexpr int kOffCodes = kOffZ + 32 * kRowsPerPass * 4;
 constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;          
 constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: 1 for a vector's, 0 past the last
-constexpr int kSmemBytes = kOffFlags + 512;
+constexpr int kOffStages = kOffFlags + kRowsPerPass;                  // StageConst[16]
+constexpr int kSmemBytes = kOffStages + 16 * (int)sizeof(StageConst);
 constexpr int kDeferMinSlots = 6;                                     // chunks a stage needs for its issuers to take the statistics
 
 // Chunks a stage needs for the chain with 8-bit corrections, which is for contiguous groups: it is a tenth faster on
@@ -137,7 +138,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
         work.rounds = (work.count + kTiles - 1) / kTiles;
     }
     const int my_passes = work.rounds;
-    const StageParams *sp = reinterpret_cast<const StageParams *>(p.prepared + kPreparedParamsOffset);
+    StageConst *sc = reinterpret_cast<StageConst *>(smem + kOffStages);
     const uint8_t *image = p.prepared + kPreparedImageOffset + (EIGHT ? kSlotTail : 0);
     const uint32_t bar0 = smem_u32(bars);
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
@@ -154,17 +155,16 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_word)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    // constant A cells shared by all tiles: (1, 1, 1, 0...) per row, then zeros
-    if (tid < 128) {
-        uint8_t *a = smem + kOffA + tid * 16;
-        *reinterpret_cast<uint4 *>(a) = make_uint4(0x3C003C00u, 0x00003C00u, 0u, 0u);
-        *reinterpret_cast<uint4 *>(a + 2048) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    load_stage_consts(p.prepared, s.R, tid, sc);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_word;
+    // the constant A operand, shared by all tiles (the issuers hear of it with their first A operand)
+    if (warp < 4) tmem_ones(tmem + ((uint32_t)(warp * 32) << 16) + kOnesCol);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
 
     // The four role warps run one lane each and need few registers; their share goes to the
     // epilogue warps, which hold three 32-column blocks of scores at a time
@@ -204,7 +204,6 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
             const int t = __shfl_sync(0xFFFFFFFFu, warp, 0) - kEpiThreads / 32;
             const uint32_t total = (uint32_t)my_passes * (uint32_t)s.R * (uint32_t)S;
             const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kOffB), kSlotCodewords * 16, 128);
-            const uint64_t ones_desc = make_smem_desc(smem_u32(smem + kOffA), 2048, 128);
             const uint32_t acc = tmem + t * kTileCols, a0 = acc + 128;
             const uint32_t bar_ready = BAR(kBarAReady + t), bar_free = BAR(kBarAccFree + t), bar_acc = BAR(kBarAccFull + t);
             const uint32_t per_round = (uint32_t)s.R * (uint32_t)S;
@@ -243,8 +242,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 // epilogue's wait for it runs out with no copy or MMA of this CTA still in flight)
                 if (p.drop_last_chain && t == 0 && q == total - 1) break;
                 if (elect_one()) {
-                    if (EIGHT) issue_chain8(acc, a0, bd, ones_desc);
-                    else issue_chain(acc, a0, bd, ones_desc);
+                    if (EIGHT) issue_chain8(acc, a0, bd, tmem + kOnesCol);
+                    else issue_chain(acc, a0, bd, tmem + kOnesCol);
                     mma_commit(bar_acc);
                     mma_commit(BAR(kBarEmpty + slot));
                 }
@@ -313,7 +312,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
 #pragma unroll 1
             for (int r = 0; r < s.R && ok; ++r) {
-                const StageParams prm = sp[r];
+                const StageConst prm = sc[r];
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
                 // scaled half-precision copy of the residual -> A operand row; error window of this row
                 uint32_t ab[32];
@@ -327,7 +326,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 // park the float32 residual in shared memory for the sweep
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kRowsPerPass] = z[i];
-                if (!EIGHT) w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
+                if (!EIGHT) w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
                 w.m1 = w.m2 = w.m3 = INFINITY;
                 w.c1 = w.c2 = 0;
 #pragma unroll
@@ -339,12 +338,6 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
 #pragma unroll 1
                 for (int c = 0; c < S && ok; ++c) {
-                    if (c == S - 1 && c > 0) {
-                        // Before the last chunk the running winner is the final one most of the time:
-                        // start fetching its codeword while the MMA chain runs.
-                        const int pj = min(max(w.c1 * 128 + listed(w, w.m1).column(), 0), s.K - 1);
-                        asm volatile("prefetch.global.L1 [%0];" ::"l"(cbr + (size_t)pj * 32));
-                    }
                     ok = mbar_wait(BAR(kBarAccFull + tile), chunk_use & 1u, abort_flag, p.wait_limit);
                     ok = __all_sync(0xFFFFFFFFu, ok);          // tcgen05.ld below needs the whole warp
                     ++chunk_use;
@@ -369,17 +362,20 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     rank_chunk(w, fminf(min3(c0, c1, c2), c3), c);
                 }
                 if (!ok) break;
-                // take the residual back
-#pragma unroll
-                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kRowsPerPass];
+                // The column of the lowest score is the choice of nearly every row: its codeword is asked for before it is
+                // known to be (the trip to L2 takes as long as the rest of the stage end: asked for after it, 225 -> 217 us on
+                // 32768 keys, 30.7 -> 28.2 on 4096 float32 vectors with 256 codes; a prefetch of the running winner into L1 before the last
+                // chunk, on top of this, costs 1.2 %).
                 const float m1 = w.m1;
+                const int jm = min(max(w.c1 * 128 + listed(w, m1).column(), 0), s.K - 1);
+                float ev[32];
+                load_codeword(cbr + (size_t)jm * 32, ev);
 
                 // ---- stage end: the columns that can still be the exact argmin are those of a listed
                 // chunk, in a listed block of the chunk, in a listed half, at a listed place.  When each of
                 // the four lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
-                const StageBounds sb = stage_bounds(p.prepared, r);
-                const float lim = EIGHT ? threshold8(w, m1, sb) : threshold(w, m1, sb);
+                const float lim = EIGHT ? threshold8(w, m1, sc[r]) : threshold(w, m1, sc[r]);
                 const Listed in = listed(w, lim);
                 const int j1 = w.c1 * 128 + in.column();
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
@@ -412,6 +408,10 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     }
                 }
                 if (deg) bj = 0;
+                if (bj != jm) load_codeword(cbr + (size_t)bj * 32, ev);
+                // take the residual back
+#pragma unroll
+                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kRowsPerPass];
                 if (p.stat_sum && valid && !(p.defer_stats && r < s.R - 1)) {
                     // EMA statistics (Section 3): this row's stage input joins the bin of its code
                     // (all stages but the last are the issuer warps' when deferred)
@@ -424,14 +424,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 }
                 // (a degenerate row's codes are 0 whatever its residual, which starts from zero and matters to the statistics only)
                 if (!deg || (p.stat_sum && valid)) {
-                    const float *ew = cbr + (size_t)bj * 32;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float ev[8];
-                        ldg256(ew + 8 * q, ev);
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) z[8 * q + k] -= ev[k];
-                    }
+                    for (int i = 0; i < 32; ++i) z[i] -= ev[i];
                 }
                 if (p.energy) {
                     // squared norm of the residual leaving this stage (scaled units), summed over the
