@@ -426,53 +426,80 @@ __device__ __forceinline__ void issue_chain8(uint32_t acc, uint32_t a0, uint64_t
     mma_f16_ts(acc, ones, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
 }
 
-// The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces through
-// a scratch area of shared memory in which word k sits at scr[(k / 32) * PITCH + k % 32]; piece c of
-// vector vl is at position c ^ (vl mod 8) of its vector so that the reads by row spread over the banks.
-// Lane l gets the 32 elements of group l % G of vector l / G, zeros past the last vector.
+// The elements of 16-byte piece `off` of a head vector, widened, to where its group rows stand: element i of group g at
+// zv[i * PITCH + g].  PITCH is odd, so that neither the pieces of a vector nor its rows share banks.
+template <int PITCH, int N>
+__device__ __forceinline__ void scatter_piece(const Shape &s, const float (&val)[N], int off, float *zv)
+{
+    const int ch = off * N;
+    if (s.layout == RVQ_GROUP_CONTIGUOUS) {
+        float *p = zv + (ch & 31) * PITCH + (ch >> 5);
+#pragma unroll
+        for (int u = 0; u < N; ++u) p[u * PITCH] = val[u];
+    } else if (s.G == 4) {
+        float *p = zv + (ch >> 2) * PITCH;
+#pragma unroll
+        for (int u = 0; u < N; ++u) p[(u >> 2) * PITCH + (u & 3)] = val[u];
+    } else {
+        const int lg = __ffs(s.G) - 1;
+#pragma unroll
+        for (int u = 0; u < N; ++u) zv[((ch + u) >> lg) * PITCH + ((ch + u) & (s.G - 1))] = val[u];
+    }
+}
+template <int PITCH>
+__device__ __forceinline__ void scatter_piece(const Shape &s, uint4 raw, int off, float *zv)
+{
+    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+    if (s.dtype == RVQ_F32) {
+        const float val[4] = {__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3])};
+        scatter_piece<PITCH>(s, val, off, zv);
+    } else {
+        float val[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (s.dtype == RVQ_BF16) {
+                val[2 * k] = __uint_as_float(w[k] << 16);
+                val[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+            } else {
+                const float2 h = __half22float2(*reinterpret_cast<const __half2 *>(&w[k]));
+                val[2 * k] = h.x;
+                val[2 * k + 1] = h.y;
+            }
+        }
+        scatter_piece<PITCH>(s, val, off, zv);
+    }
+}
+// Piece `off` of head vector v; zeros past the last.
+__device__ __forceinline__ uint4 load_piece(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride, int64_t v, int off)
+{
+    if (v >= n) return make_uint4(0u, 0u, 0u, 0u);
+    return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(x) + v * stride * s.elem_bytes) + off);
+}
+
+// The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces, four loads in flight per lane;
+// lane l gets the 32 elements of group l % G of vector l / G, zeros past the last vector.  `rows`: element 0 of the
+// warp's first row in a scratch area [32][PITCH].
 template <int PITCH>
 __device__ __forceinline__ void load_group_rows(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride,
-                                                int64_t v_first, int lane, float *scr, float (&z)[32])
+                                                int64_t v_first, int lane, float *rows, float (&z)[32])
 {
-    const int G = s.G, eb = s.elem_bytes, ppv = s.dim * eb / 16;          // pieces per vector (>= 4)
-    // (four loads in flight per lane: a 16-bit head vector of 128 channels is 16 pieces, so the
-    // 8 vectors of a warp are 4 pieces per lane)
-    const int npieces = (32 / G) * ppv;
-    for (int c0 = 0; c0 < npieces; c0 += 128) {
-        uint4 val[4];
-        int kk[4];
+    const int lg = __ffs(s.G) - 1, lp = lg + (s.elem_bytes == 4 ? 3 : 2);       // log2 of the pieces of a vector
+    for (int c0 = lane; c0 < 32 << (lp - lg); c0 += 128) {
+        uint4 raw[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int c = c0 + 32 * u + lane;
-            const int vl = c / ppv, off = c - vl * ppv;
-            const int64_t vv = v_first + vl;
-            val[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (c < npieces && vv < n)
-                val[u] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(x) + vv * stride * eb) + off);
-            kk[u] = (vl * ppv + (off ^ (vl & 7 & (ppv - 1)))) * 4;
+            const int c = c0 + 32 * u;
+            raw[u] = load_piece(s, x, n, stride, v_first + (c >> lp), c & ((1 << lp) - 1));
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (c0 + 32 * u + lane < npieces)
-                *reinterpret_cast<uint4 *>(scr + (kk[u] >> 5) * PITCH + (kk[u] & 31)) = val[u];
-    }
-    __syncwarp();
-    const int vl = lane / G, g = lane - vl * G, sw = vl & 7 & (ppv - 1);
-    const bool valid = v_first + vl < n;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        const int b = channel_of(s.layout, G, 32, g, i) * eb;      // byte within the vector
-        const int k = (vl * ppv + ((b >> 4) ^ sw)) * 4 + ((b & 15) >> 2);
-        const uint32_t word = __float_as_uint(scr[(k >> 5) * PITCH + (k & 31)]);
-        float val;
-        if (s.dtype == RVQ_F32) val = __uint_as_float(word);
-        else {
-            const uint16_t h = (b & 2) ? (uint16_t)(word >> 16) : (uint16_t)(word & 0xFFFFu);
-            val = s.dtype == RVQ_BF16 ? __uint_as_float((uint32_t)h << 16) : __half2float(__ushort_as_half(h));
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + 32 * u;
+            scatter_piece<PITCH>(s, raw[u], c & ((1 << lp) - 1), rows + ((c >> lp) << lg));
         }
-        z[i] = valid ? val : 0.0f;
     }
     __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) z[i] = rows[i * PITCH + lane];
 }
 
 // Deviation over the G lanes of this lane's head vector, same summation order as the scalar kernel.
@@ -599,14 +626,17 @@ __device__ __forceinline__ void emit_codes(const Shape &s, const uint16_t *codes
     } else {
         // the warp holds 32 / G whole head vectors; one 32-bit word per lane and step
         const int words = s.code_bytes / 4, vec_per_warp = 32 / G;
+        // quotients as products with 2^20 / d, rounded up: exact while the dividend is below 2^20 / d (here 512 codes of a vector by
+        // up to 16 stages, 8192 + 31 bits by up to 16, 256 words by 256); divisions were most of this loop
+        const uint32_t by_words = (1u << 20) / (uint32_t)words + 1u, by_bits = (1u << 20) / (uint32_t)s.bits + 1u, by_R = (1u << 20) / (uint32_t)s.R + 1u;
         for (int t = lane; t < vec_per_warp * words; t += 32) {
-            const int vl = t / words, w = t - vl * words;
+            const int vl = (int)((uint32_t)t * by_words >> 20), w = t - vl * words;
             const int64_t vv = v_first + vl;
             if (vv >= n) continue;
             uint32_t word = 0;
-            const int k_lo = (32 * w) / s.bits, k_hi = min(s.per_vector - 1, (32 * w + 31) / s.bits);
+            const int k_lo = (int)((uint32_t)(32 * w) * by_bits >> 20), k_hi = min(s.per_vector - 1, (int)((uint32_t)(32 * w + 31) * by_bits >> 20));
             for (int k = k_lo; k <= k_hi; ++k) {
-                const int gg = k / s.R, rr = k - gg * s.R;
+                const int gg = (int)((uint32_t)k * by_R >> 20), rr = k - gg * s.R;
                 const uint32_t val = codes_s[(vl * G + gg) * 16 + rr];
                 const int sh = k * s.bits - 32 * w;
                 word |= sh >= 0 ? (val << sh) : (val >> (-sh));

@@ -175,26 +175,10 @@ encode_split_kernel(const SplitParams p)
             bool deg = true;
             // the tile's head vectors, widened, by all groups: element i of row at [i][row]
             {
-                const int eb = s.elem_bytes, ppv = s.dim * eb / 16, per_piece = 16 / eb, lg = __ffs(G) - 1;
-                float *zs = reinterpret_cast<float *>(smem + kSOffZ);
-                for (int k = tid; k < (128 >> lg) * ppv; k += 128 * P) {
-                    const int vl = k / ppv, off = k - vl * ppv;
-                    uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-                    if (v_tile + vl < p.n)
-                        raw = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(p.x) + (v_tile + vl) * p.stride * eb) + off);
-                    const uint32_t words[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (u >= per_piece) break;
-                        const uint32_t word = eb == 4 ? words[u & 3] : words[u >> 1];
-                        const uint16_t h = (u & 1) ? (uint16_t)(word >> 16) : (uint16_t)(word & 0xFFFFu);
-                        const float val = eb == 4 ? __uint_as_float(word)
-                                        : s.dtype == RVQ_BF16 ? __uint_as_float((uint32_t)h << 16) : __half2float(__ushort_as_half(h));
-                        const int ch = off * per_piece + u;
-                        const int g = s.layout == RVQ_GROUP_STRIDED ? ch & (G - 1) : ch >> 5, i = s.layout == RVQ_GROUP_STRIDED ? ch >> lg : ch & 31;
-                        zs[i * kZPitch + (vl << lg) + g] = val;
-                    }
-                }
+                const int lg = __ffs(G) - 1, lp = lg + (s.elem_bytes == 4 ? 3 : 2);      // log2 of the pieces of a vector
+                for (int k = tid; k < 128 << (lp - lg); k += 128 * P)
+                    scatter_piece<kZPitch>(s, load_piece(s, p.x, p.n, p.stride, v_tile + (k >> lp), k & ((1 << lp) - 1)), k & ((1 << lp) - 1),
+                                           reinterpret_cast<float *>(smem + kSOffZ) + ((k >> lp) << lg));
             }
             asm volatile("bar.sync 1, %0;" ::"r"(128 * P) : "memory");
             if (grp == 0) {

@@ -59,8 +59,9 @@ constexpr int kOnesCol = 480;                             // TMEM column of the 
 constexpr int kTileCols = 160;                            // TMEM columns per tile: 128 scores + 32 of A operand
 
 constexpr int kOffB = 0;
-constexpr int kOffZ = kOffB + kRing * kSlotBytes;                     // parked residuals, float [32][rows]
-constexpr int kOffCodes = kOffZ + 32 * kRowsPerPass * 4;
+constexpr int kOffZ = kOffB + kRing * kSlotBytes;                     // parked residuals, float [32][kPitch]
+constexpr int kPitch = kRowsPerPass + 1;                              // (odd: scatter_piece)
+constexpr int kOffCodes = kOffZ + 32 * kPitch * 4;
 constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;          
 constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: 1 for a vector's, 0 past the last
 constexpr int kOffStages = kOffFlags + kRowsPerPass;                  // StageConst[16]
@@ -181,13 +182,25 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
             const uint32_t per_pass = (uint32_t)s.R * (uint32_t)S;
             uint32_t slot = 0, rs = 0, empty_par = 1;          // parity of the previous completion of empty[slot]
             uint32_t nl = 0;
+            int pass = 0;
             for (; nl < total; ++nl) {
+                if (rs == (uint32_t)S && pass + 1 < my_passes) {
+                    // the next round's head vectors into L2, while this round's stages run
+                    const int64_t v0 = (int64_t)work.round_first(pass + 1) * 128 / s.G;
+                    int64_t left = (int64_t)work.round_size(pass + 1) * 128 / s.G;
+                    left = v0 + left <= p.n ? left : p.n - v0;
+                    const bool dense = p.stride == s.dim;
+                    const uint32_t bytes = (uint32_t)(s.dim * s.elem_bytes) * (dense ? (uint32_t)left : 1u);
+                    const uint8_t *from = reinterpret_cast<const uint8_t *>(p.x) + v0 * p.stride * s.elem_bytes;
+                    for (int64_t k = 0; k < (dense ? 1 : left); ++k, from += p.stride * s.elem_bytes)
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(from), "r"(bytes) : "memory");
+                }
                 if (nl >= (uint32_t)kRing && !mbar_wait(BAR(kBarEmpty + slot), empty_par, abort_flag)) break;
                 mbar_expect_tx(BAR(kBarFull + slot), kSlotBytes);
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                              ::"r"(smem_u32(smem + kOffB) + slot * (uint32_t)kSlotBytes), "l"(image + (size_t)rs * kSlotStride),
                                "r"((uint32_t)kSlotBytes), "r"(BAR(kBarFull + slot)) : "memory");
-                if (++rs == per_pass) rs = 0;
+                if (++rs == per_pass) { rs = 0; ++pass; }
                 if (++slot == (uint32_t)kRing) { slot = 0; empty_par ^= 1u; }
             }
             for (uint32_t k = nl > (uint32_t)kRing ? nl - kRing : 0u; k < nl; ++k)
@@ -257,8 +270,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                         float4 *m = reinterpret_cast<float4 *>(p.stat_sum + bin * 32);
 #pragma unroll
                         for (int q4 = 0; q4 < 8; ++q4)
-                            atomicAdd(m + q4, make_float4(zp[(4 * q4) * kRowsPerPass + rl], zp[(4 * q4 + 1) * kRowsPerPass + rl],
-                                                          zp[(4 * q4 + 2) * kRowsPerPass + rl], zp[(4 * q4 + 3) * kRowsPerPass + rl]));
+                            atomicAdd(m + q4, make_float4(zp[(4 * q4) * kPitch + rl], zp[(4 * q4 + 1) * kPitch + rl],
+                                                          zp[(4 * q4 + 2) * kPitch + rl], zp[(4 * q4 + 3) * kPitch + rl]));
                     }
                     __syncwarp();
                 }
@@ -291,8 +304,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
             // (through the warp's share of the parking area)
             float z[32];
-            load_group_rows<kRowsPerPass>(s, p.x, p.n, p.stride, (row0 + q4 * 32) / G, lane,
-                                          reinterpret_cast<float *>(smem + kOffZ) + (rloc - lane), z);
+            load_group_rows<kPitch>(s, p.x, p.n, p.stride, (row0 + q4 * 32) / G, lane, z_park - lane, z);
             const float dev = group_deviation(s, z, lane);
             // (raw rows are stage inputs already: taken as they are, no deviation stored)
             const bool deg = s.raw ? !valid : (deviation_is_degenerate(dev) || !valid);
@@ -325,7 +337,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 if (lane == 0) mbar_arrive(BAR(kBarAReady + tile));
                 // park the float32 residual in shared memory for the sweep
 #pragma unroll
-                for (int i = 0; i < 32; ++i) z_park[i * kRowsPerPass] = z[i];
+                for (int i = 0; i < 32; ++i) z_park[i * kPitch] = z[i];
                 if (!EIGHT) w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
                 w.m1 = w.m2 = w.m3 = INFINITY;
                 w.c1 = w.c2 = 0;
@@ -392,7 +404,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     todo &= todo - 1;
                     float zs[32];
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kRowsPerPass + (src - lane)];
+                    for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kPitch + (src - lane)];
                     const int chunk1 = __shfl_sync(0xFFFFFFFFu, w.c1, src);
                     const int chunk2 = __shfl_sync(0xFFFFFFFFu, w.m2 <= lim ? w.c2 : -1, src);
                     const uint32_t sets = __shfl_sync(0xFFFFFFFFu, in.word(), src);
@@ -411,7 +423,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 if (bj != jm) load_codeword(cbr + (size_t)bj * 32, ev);
                 // take the residual back
 #pragma unroll
-                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kRowsPerPass];
+                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kPitch];
                 if (p.stat_sum && valid && !(p.defer_stats && r < s.R - 1)) {
                     // EMA statistics (Section 3): this row's stage input joins the bin of its code
                     // (all stages but the last are the issuer warps' when deferred)
