@@ -57,6 +57,23 @@ def test_other_head_sizes_and_row_strides(n, dim, K):
     check(n, dim, K, 8 if K != 129 else 9, 1, "packed", "bf16", n, stride=dim + 16)
 
 
+@pytest.mark.parametrize("tiles", [1, 19, 37, 74, 148])
+@pytest.mark.parametrize("K", [400, 520, 770, 1024, 1400, 2048, 5000])
+def test_chunks_over_accumulators_and_ctas(tiles, K):
+    """Tiles split over one to eight CTAs of one to forty chunks each: chains that go out together and one by one, groups
+    without a chunk, slots and accumulators that come round; equal codewords in different chunks, groups and CTAs."""
+    n = 32 * tiles - tiles % 3
+    x, cb = batch(n, 128, K, 5, "bf16", tiles + K)
+    cb[:, 130], cb[:, K - 1], cb[:, K // 2] = cb[:, 2], cb[:, 5], cb[:, 9]
+    cfg = rvq.make_config(128, 32, 1, 5, K, 16, rvq.BF16, 0)
+    b = rvq.alloc_buffers(cfg, n, cb)
+    exact = torch.empty_like(b.codes)
+    rvq.rvq_encode(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
+    torch.cuda.synchronize()
+    assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
+
+
 def test_against_the_oracle():
     x, cb = batch(24, 128, 1024, 8, "f32", 5)
     cfg = rvq.make_config(128, 32, 0, 8, 1024, 16, rvq.F32, 0)
