@@ -186,7 +186,8 @@ encode_split_kernel(const SplitParams p)
         // them come from a warp per accumulator, whose waits overlap.
         // No wait may be more than one phase ahead of its barrier, or it would take an old phase for its own.  Accumulators: every
         // issuer waits for each fold in turn.  Slots: the use before, six chunks back, is the issuer's own or of an
-        // earlier stage; of that the first issuer knows by the other groups' parts, the others by the fold of this stage's first chunk.
+        // earlier stage; of that the first issuer, where it has not waited for all of a stage's slots itself, knows by the other groups' parts, the
+        // others by the fold of this stage's first chunk.
         const int mine = warp == 12 ? 0 : warp - 13;
         const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kSOffB), kSlotCodewords * 16, 128);
         const int first = min(cnt, P);
@@ -196,7 +197,7 @@ encode_split_kernel(const SplitParams p)
         for (int r = 0; r < R && ok; ++r) {
             const uint32_t use0 = (uint32_t)(r * cnt);                    // the CTA's chunks are numbered through all stages
             if (mine == 0) {
-                if (r > 0 && P > 1) ok = mbar_wait(BAR(kSLocal), (uint32_t)(r - 1) & 1u, abort_flag);
+                if (r > 0 && cnt > P) ok = mbar_wait(BAR(kSLocal), (uint32_t)(r - 1) & 1u, abort_flag);
                 for (int c = 0; c < first && ok; ++c) ok = mbar_wait(BAR(kSFull + (use0 + c) % kSplitRing), ((use0 + c) / kSplitRing) & 1u, abort_flag);
                 if (ok) ok = mbar_wait(BAR(kSReady), (uint32_t)r & 1u, abort_flag);
                 ok = __all_sync(0xFFFFFFFFu, ok);
@@ -273,6 +274,11 @@ encode_split_kernel(const SplitParams p)
 #pragma unroll 1
                 for (int r = 0; r < R; ++r) {
                     const StageConst prm = sc[r];
+                    if (grp >= cnt) {
+                        // a group without chunks, which no chain holds back: not before the owners, who have read its last part by then
+                        const bool ok = mbar_wait(BAR(kSReady), (uint32_t)r & 1u, abort_flag);
+                        if (!__all_sync(0xFFFFFFFFu, ok)) break;
+                    }
                     Sweep w;
                     if (!sweep_chunks(w, grp, P, base, cnt, acc, BAR(kSAccFull + grp), BAR(kSAccFree + grp), acc_par, BAR(kSEmpty), (uint32_t)(r * cnt), lane, abort_flag)) break;
                     w.zz = grp < cnt ? norm[row] : 0.0f;                  // (a group without chunks has nothing inside any window)
@@ -282,10 +288,6 @@ encode_split_kernel(const SplitParams p)
                                                   (uint32_t)w.c1 | ((uint32_t)w.c2 << 16)};
                     __syncwarp();
                     if (lane == 0) mbar_arrive(BAR(kSLocal));
-                    if (grp >= cnt) {                                     // (nothing holds it back: not before the owners have read this part)
-                        bool ok = mbar_wait(BAR(kSLocal), (uint32_t)r & 1u, abort_flag);
-                        if (!__all_sync(0xFFFFFFFFu, ok)) break;
-                    }
                 }
             } else {
             // (the owners hold the residual from the stage end to the next operand and park it during the sweep)
