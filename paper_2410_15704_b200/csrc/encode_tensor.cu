@@ -120,7 +120,11 @@ struct Work {
 // 16 warps, launched with 128 registers per thread; the four role warps then keep 40 each and the
 // twelve epilogue warps take 152 (4 x 40 + 12 x 152 = 1984 of the 2048 per lane).
 // EIGHT: the small products in 8 bits (issue_chain8).
-template <bool EIGHT>
+// LONE: one tile per CTA, of up to three chunks a stage, without statistics.  The other tiles' accumulators take the tile's second and third
+// chunk, whose chains go out behind the first's at once instead of after its fold; all warps take part in the way in.
+// (4096 float32 vectors at 256 codes 27.8 -> 24.9 us, at 384 34.1 -> 30.5.  The split encoder with a CTA per tile takes 30.8 and 35.7: with up to
+// three chunks the parts' join costs more than the folds that it puts side by side.)
+template <bool EIGHT, bool LONE>
 __device__ __forceinline__ void encode_tensor_body(const Params &p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -141,11 +145,22 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     const int my_passes = work.rounds;
     StageConst *sc = reinterpret_cast<StageConst *>(smem + kOffStages);
     const uint8_t *image = p.prepared + kPreparedImageOffset + (EIGHT ? kSlotTail : 0);
+    uint4 raw[3];
+    const int lg = __ffs(s.G) - 1, lp = lg + (s.elem_bytes == 4 ? 3 : 2);          // log2 of a vector's groups and pieces
+    const int pieces = 128 << (lp - lg);
+    if (LONE) {
+        const int64_t v_tile = ((int64_t)blockIdx.x * 128) >> lg;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int k = tid + kEpiThreads * u;
+            if (tid < kEpiThreads && k < pieces) raw[u] = load_piece(s, p.x, p.n, p.stride, v_tile + (k >> lp), k & ((1 << lp) - 1));
+        }
+    }
     const uint32_t bar0 = smem_u32(bars);
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
     if (tid == 0) {
-        for (int i = 0; i < kRing; ++i) { mbar_init(BAR(kBarFull + i), 1); mbar_init(BAR(kBarEmpty + i), kTiles); }
+        for (int i = 0; i < kRing; ++i) { mbar_init(BAR(kBarFull + i), 1); mbar_init(BAR(kBarEmpty + i), LONE ? 1 : kTiles); }
         for (int t = 0; t < kTiles; ++t) {
             mbar_init(BAR(kBarAReady + t), 4); mbar_init(BAR(kBarAccFull + t), 1); mbar_init(BAR(kBarAccFree + t), 4);
         }
@@ -163,6 +178,14 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     const uint32_t tmem = *tmem_word;
     // the constant A operand, shared by all tiles (the issuers hear of it with their first A operand)
     if (warp < 4) tmem_ones(tmem + ((uint32_t)(warp * 32) << 16) + kOnesCol);
+    if (LONE) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int k = tid + kEpiThreads * u;
+            if (tid < kEpiThreads && k < pieces)
+                scatter_piece<kPitch>(s, raw[u], k & ((1 << lp) - 1), reinterpret_cast<float *>(smem + kOffZ) + ((k >> lp) << lg));
+        }
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -170,9 +193,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     // The four role warps run one lane each and need few registers; their share goes to the
     // epilogue warps, which hold three 32-column blocks of scores at a time
     // (12 warps x 32 x 152 + 4 warps x 32 x 40 = 63488 of the 65536 the block was launched with).
-    if (warp >= kEpiThreads / 32) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    else asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
-
+    if (warp >= kEpiThreads / 32) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == kEpiThreads / 32 + kTiles) {
         // ------------------------------------------------------------ operand loader
         // One thread streams the B slots of every (pass, stage) through the ring; a slot is
@@ -206,14 +228,38 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
             for (uint32_t k = nl > (uint32_t)kRing ? nl - kRing : 0u; k < nl; ++k)
                 mbar_drain(BAR(kBarFull + (int)(k % kRing)), (k / kRing) & 1u);
         }
-    } else if (warp >= kEpiThreads / 32) {
+    } else {
         // ------------------------------------------------------------ MMA issuer of tile t
         // One thread per tile, each in a warp of its own so that the tiles' waits overlap.
         // Whatever it does between two tcgen05.mma chains delays its tile, so descriptors
         // are built once and all counters advance by increments.
         // (The whole warp runs the loop with warp-uniform values and one lane issues: operands that the
         // compiler knows to be uniform can stay in uniform registers, which tcgen05.mma reads directly.)
-        if (my_passes > 0) {
+        if (LONE) {
+            if (warp == kEpiThreads / 32) {
+                const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kOffB), kSlotCodewords * 16, 128);
+                int sent = 0;                                             // chains
+                bool ok = true;
+                for (int r = 0; r < s.R && ok; ++r) {
+                    const uint32_t use0 = (uint32_t)(r * S);
+                    for (int c = 0; c < S && ok; ++c) ok = mbar_wait(BAR(kBarFull + (int)((use0 + c) % kRing)), ((use0 + c) / kRing) & 1u, abort_flag);
+                    if (ok) ok = mbar_wait(BAR(kBarAReady), (uint32_t)r & 1u, abort_flag);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int k = 0; k < S; ++k, ++sent) {
+                        if (p.drop_last_chain && r == s.R - 1 && k == S - 1) break;
+                        if (elect_one()) {
+                            issue_chain(tmem + (uint32_t)(k * kTileCols), tmem + 128, bdesc0 + (uint64_t)((use0 + k) % kRing * (uint32_t)(kSlotBytes >> 4)), tmem + kOnesCol);
+                            mma_commit(BAR(kBarAccFull + k));
+                        }
+                        __syncwarp();
+                    }
+                }
+                for (int k = max(sent - S, 0); k < sent; ++k) mbar_drain(BAR(kBarAccFull + k % S), (uint32_t)(k / S) & 1u);
+            }
+        } else if (my_passes > 0) {
             const int t = __shfl_sync(0xFFFFFFFFu, warp, 0) - kEpiThreads / 32;
             const uint32_t total = (uint32_t)my_passes * (uint32_t)s.R * (uint32_t)S;
             const uint64_t bdesc0 = make_smem_desc(smem_u32(smem + kOffB), kSlotCodewords * 16, 128);
@@ -282,8 +328,10 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
             }
             mbar_drain(bar_acc, last_par);
         }
+    }
     } else {
         // ------------------------------------------------------------ epilogue warps
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
         const int tile = warp >> 2, q4 = warp & 3;
         const int rloc = tile * 128 + q4 * 32 + lane;
         const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(tile * kTileCols);
@@ -291,6 +339,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
         uint16_t *codes_s = reinterpret_cast<uint16_t *>(smem + kOffCodes);                // [row][R]
         const int G = s.G;
         uint32_t chunk_use = 0;
+        int slot = 0;
         uint32_t n_rescored = 0, n_exhaustive = 0, n_degenerate = 0, n_stdrange = 0;
         bool ok = true;
 
@@ -304,6 +353,10 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
             // (through the warp's share of the parking area)
             float z[32];
+            if (LONE) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) z[i] = z_park[i * kPitch];
+            } else
             load_group_rows<kPitch>(s, p.x, p.n, p.stride, (row0 + q4 * 32) / G, lane, z_park - lane, z);
             const float dev = group_deviation(s, z, lane);
             // (raw rows are stage inputs already: taken as they are, no deviation stored)
@@ -350,23 +403,29 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
 #pragma unroll 1
                 for (int c = 0; c < S && ok; ++c) {
-                    ok = mbar_wait(BAR(kBarAccFull + tile), chunk_use & 1u, abort_flag, p.wait_limit);
+                    ok = LONE ? mbar_wait(BAR(kBarAccFull + c), (uint32_t)r & 1u, abort_flag, p.wait_limit)
+                              : mbar_wait(BAR(kBarAccFull + tile), chunk_use & 1u, abort_flag, p.wait_limit);
                     ok = __all_sync(0xFFFFFFFFu, ok);          // tcgen05.ld below needs the whole warp
                     ++chunk_use;
                     if (!ok) break;
+                    if (LONE) {
+                        if (tid == 0) mbar_arrive(BAR(kBarEmpty + slot));       // the chain has read its slot
+                        slot = slot + 1 < kRing ? slot + 1 : 0;
+                    }
                     tc_fence_after();
                     // All four 32-column blocks are asked for at once and the accumulator goes back to
                     // the MMA issuer as soon as they have landed: the reduction below runs while the
                     // next chain computes.
+                    const uint32_t acc = LONE ? taddr + (uint32_t)(c * kTileCols) : taddr;
                     uint32_t ua[32], ub[32], uc[32], ud[32];
-                    tmem_ld32_issue(taddr, ua);
-                    tmem_ld32_issue(taddr + 32, ub);
-                    tmem_ld32_issue(taddr + 64, uc);
-                    tmem_ld32_issue(taddr + 96, ud);
+                    tmem_ld32_issue(acc, ua);
+                    tmem_ld32_issue(acc + 32, ub);
+                    tmem_ld32_issue(acc + 64, uc);
+                    tmem_ld32_issue(acc + 96, ud);
                     tmem_ld_wait4(ua, ub, uc, ud);
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(BAR(kBarAccFree + tile));        // the accumulator may be overwritten
+                    if (!LONE && lane == 0) mbar_arrive(BAR(kBarAccFree + tile));    // the accumulator may be overwritten
                     const float c0 = fold_block(w, ua, 0);
                     const float c1 = fold_block(w, ub, 1);
                     const float c2 = fold_block(w, uc, 2);
@@ -476,13 +535,14 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) encode_tensor_kernel(const __grid_constant__ Params p) { encode_tensor_body<false>(p); }
+__global__ void __launch_bounds__(kThreads, 1) encode_tensor_kernel(const __grid_constant__ Params p) { encode_tensor_body<false, false>(p); }
+__global__ void __launch_bounds__(kThreads, 1) encode_tensor_lone_kernel(const __grid_constant__ Params p) { encode_tensor_body<false, true>(p); }
 
 // Where the 8-bit corrections are possible: by the codebooks.
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_either_kernel(const __grid_constant__ Params p)
 {
-    if (reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true>(p);
-    else encode_tensor_body<false>(p);
+    if (reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true, false>(p);
+    else encode_tensor_body<false, false>(p);
 }
 
 }  // namespace
@@ -510,7 +570,8 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
-    auto kernel = eight_possible(s, tiles, sms) ? encode_tensor_either_kernel : encode_tensor_kernel;
+    const bool lone = tiles <= sms && slots_per_stage(s.K) <= kTiles && !s.raw && !stat_sum;
+    auto kernel = lone ? encode_tensor_lone_kernel : eight_possible(s, tiles, sms) ? encode_tensor_either_kernel : encode_tensor_kernel;
     if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
              energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,

@@ -58,13 +58,13 @@ def test_other_head_sizes_and_row_strides(n, dim, K):
 
 
 @pytest.mark.parametrize("tiles", [1, 19, 37, 74, 148])
-@pytest.mark.parametrize("K", [400, 520, 770, 1024, 1400, 2048, 5000])
+@pytest.mark.parametrize("K", [100, 140, 256, 384, 400, 520, 770, 1024, 1400, 2048, 5000])
 def test_chunks_over_accumulators_and_ctas(tiles, K):
-    """Tiles split over one to eight CTAs of one to forty chunks each: chains that go out together and one by one, groups
+    """Up to three chunks: one tile per CTA, an accumulator per chunk.  More: tiles split over one to eight CTAs of one to forty chunks each: chains that go out together and one by one, groups
     without a chunk, slots and accumulators that come round; equal codewords in different chunks, groups and CTAs."""
     n = 32 * tiles - tiles % 3
     x, cb = batch(n, 128, K, 5, "bf16", tiles + K)
-    cb[:, 130], cb[:, K - 1], cb[:, K // 2] = cb[:, 2], cb[:, 5], cb[:, 9]
+    cb[:, min(130, K - 2)], cb[:, K - 1], cb[:, K // 2] = cb[:, 2], cb[:, 5], cb[:, 9]
     cfg = rvq.make_config(128, 32, 1, 5, K, 16, rvq.BF16, 0)
     b = rvq.alloc_buffers(cfg, n, cb)
     exact = torch.empty_like(b.codes)
