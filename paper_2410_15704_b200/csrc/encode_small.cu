@@ -263,14 +263,17 @@ SmallPlan small_plan(const Shape &s)
 
 }  // namespace
 
-// Group rows per cluster up to which this encoder is faster than a tile of 128 rows split over CTAs: a row costs
-// about 1.6 us at two blocks per CTA and 0.8 us at one, a split tile 36-40 us.
+// Group rows per cluster up to which this encoder is faster than tiles of 128 rows: a row costs about 1.6 us at two blocks per CTA and
+// 1 us at one, a tile's stages about the same for one row as for 128.  us, this encoder / tiles: 2048 codes 16 rows 32.6 / 32.9, 20 39.1 / 33.3; 1024 codes 20 rows
+// 27.5 / 28.1, 24 29.8 / 28.1; 512 codes 20 rows 25.6 / 26.1, 24 27.7 / 26.1; at depth 4, 1024 codes, 24 rows 16.6 / 17.7.  Up to three chunks, where
+// a tile is one CTA's (encode_tensor.cu): 256 codes 16 rows 20.4 / 22.0, 20 25.0 / 22.0.
 bool encode_small_wanted(const Shape &s, int64_t n)
 {
     if (!float_blocks_prepared(s) || s.raw || s.G > kSmallRows || n < 1 || n > 4096) return false;
     const SmallPlan plan = small_plan(s);
     const int64_t vectors = plan.at_once > 0 ? (n + plan.at_once - 1) / plan.at_once : 0;
-    return vectors == 1 || (vectors > 0 && vectors * s.G <= (plan.per_cta == 2 ? 16 : 24));
+    const int most = plan.per_cta == 2 || slots_per_stage(s.K) <= 3 ? 16 : s.R <= 4 ? 24 : 20;
+    return vectors == 1 || (vectors > 0 && vectors * s.G <= most);
 }
 
 int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride, const void *prepared, void *codes,

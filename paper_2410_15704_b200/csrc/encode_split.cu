@@ -475,9 +475,8 @@ encode_split_kernel(const SplitParams p)
 
 // CTAs per tile; 0: this kernel is not the one to take.  A stage of a tile costs its CTAs about 450 cycles per
 // chunk (the chains follow one another), 350 per fold of a group, and 60 per CTA that parts go to, beside 3000
-// that do not depend on the split; all tiles have to be on the chip at once.  Measured against the throughput
-// kernel with one tile per SM: 80 us against 94 at 2048 codes and 54 against 57 at 1024 with 148 tiles, 33.6
-// against 30.4 at 256; with more tiles than SMs two tiles one after the other lose (155 against 101 us).
+// that do not depend on the split; all tiles have to be on the chip at once.  With more tiles than SMs, two tiles one after the other
+// lose to the throughput kernel (2048 codes: 130 us against 101), and so does this kernel with up to three chunks (there).
 int split_ctas(const Shape &s, int64_t tiles, int sms)
 {
     const int S = slots_per_stage(s.K);
