@@ -182,20 +182,29 @@ struct Sweep {
     float zz, ll;            // squared norms of the scaled residual (m1 + zz is the best squared distance) and of its remainder
     float m1, m2, m3;        // the three lowest chunk minima ...
     int c1, c2;              // ... and the chunks of the first two
-    float bb[4];             // minimum per 32-column block position inside its 128-column chunk
-    float h[2];              // minimum per half (columns 0-15, 16-31) of a block
-    float d[16];             // minimum per column position inside its half
+    float hb[8];             // minimum per block of 16 columns inside its 128-column chunk
+    float d[16];             // minimum per column position inside its block
+
+    __device__ __forceinline__ void clear()
+    {
+        m1 = m2 = m3 = INFINITY;
+        c1 = c2 = 0;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) d[q] = INFINITY;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) hb[q] = INFINITY;
+    }
 };
 
-// One 32-column block of scores (block `b` of its chunk) folded into the running minima of three
-// partitions of its columns: the 16 places inside a half (one three-input minimum takes in the two
-// columns of a place), the two halves, and the block itself; returns the block minimum.  Together
+// 32 columns of scores (blocks 2 b and 2 b + 1 of their chunk) folded into the running minima of two
+// partitions of a chunk's columns: the 16 places inside a block (one three-input minimum takes in the two
+// columns of a place) and the eight blocks; `chunk`, the chunk's own minimum, takes them in as well.  Together
 // with the chunk list a column that could be the argmin is pinned to (listed chunk) x (block of the
-// chunk) x (half) x (place): when every one of the four lists has a single entry, to one column.
-// 36 minimum operations per 32 scores: they run on the narrow integer/compare pipe, which this sweep
+// chunk) x (place): when every one of the three lists has a single entry, to one column.
+// 35 minimum operations per 32 scores: they run on the narrow integer/compare pipe, which this sweep
 // keeps about as busy as the tensor pipe, so their number per score is what the sweep's speed
-// hangs on.
-__device__ __forceinline__ float fold_block(Sweep &w, const uint32_t (&u)[32], int b)
+// hangs on (36.5 with blocks of 32 columns and their halves as two partitions).
+__device__ __forceinline__ void fold_block(Sweep &w, const uint32_t (&u)[32], int b, float &chunk)
 {
 #pragma unroll
     for (int c = 0; c < 16; ++c) w.d[c] = min3(w.d[c], __uint_as_float(u[c]), __uint_as_float(u[c + 16]));
@@ -209,12 +218,9 @@ __device__ __forceinline__ float fold_block(Sweep &w, const uint32_t (&u)[32], i
         const float a3 = min3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
         const float a4 = min3(__uint_as_float(v[12]), __uint_as_float(v[13]), __uint_as_float(v[14]));
         hm[hf] = fminf(min3(a0, a1, a2), min3(a3, a4, __uint_as_float(v[15])));
+        w.hb[2 * b + hf] = fminf(w.hb[2 * b + hf], hm[hf]);
     }
-    w.h[0] = fminf(w.h[0], hm[0]);
-    w.h[1] = fminf(w.h[1], hm[1]);
-    const float m = fminf(hm[0], hm[1]);
-    w.bb[b] = fminf(w.bb[b], m);
-    return m;
+    chunk = b == 0 ? fminf(hm[0], hm[1]) : min3(chunk, hm[0], hm[1]);
 }
 
 // What a stage's rows need to know of its codebook (prepare.cu), copied to shared memory at the start: asked for in the
@@ -283,29 +289,25 @@ __device__ __forceinline__ float threshold8(const Sweep &w, float m1, const Stag
     return m1 + win + 5.4e-6f * (d2 + win);
 }
 
-// Members of the three partitions whose minimum is at most `limit` (bit k: member k).  The comparisons are
+// Members of the two partitions whose minimum is at most `limit` (bit k: member k).  The comparisons are
 // subtractions, on the floating-point pipe; one funnel shift each collects their signs.
 struct Listed {
-    uint32_t places, halves, blocks;
-    __device__ __forceinline__ bool single() const
-    {
-        return ((places & (places - 1u)) | (halves & (halves - 1u)) | (blocks & (blocks - 1u))) == 0u;
-    }
-    // the three in one word: places, halves << 16, blocks << 18
-    __device__ __forceinline__ uint32_t word() const { return places | (halves << 16) | (blocks << 18); }
+    uint32_t places, blocks;
+    __device__ __forceinline__ bool single() const { return ((places & (places - 1u)) | (blocks & (blocks - 1u))) == 0u; }
+    // the two in one word: places, blocks << 16
+    __device__ __forceinline__ uint32_t word() const { return places | (blocks << 16); }
     // column inside the chunk of the lowest members
-    __device__ __forceinline__ int column() const { return (__ffs(blocks) - 1) * 32 + (__ffs(halves) - 1) * 16 + __ffs(places) - 1; }
+    __device__ __forceinline__ int column() const { return (__ffs(blocks) - 1) * 16 + __ffs(places) - 1; }
 };
+__device__ __forceinline__ Listed listed_of(uint32_t word) { return {word & 0xFFFFu, (word >> 16) & 0xFFu}; }
 __device__ __forceinline__ Listed listed(const Sweep &w, float limit)
 {
-    uint32_t q = 0u, h = 0u, b = 0u;
+    uint32_t q = 0u, b = 0u;
 #pragma unroll
     for (int i = 15; i >= 0; --i) q = __funnelshift_l(__float_as_uint(limit - w.d[i]), q, 1);
 #pragma unroll
-    for (int i = 1; i >= 0; --i) h = __funnelshift_l(__float_as_uint(limit - w.h[i]), h, 1);
-#pragma unroll
-    for (int i = 3; i >= 0; --i) b = __funnelshift_l(__float_as_uint(limit - w.bb[i]), b, 1);
-    return {~q & 0xFFFFu, ~h & 3u, ~b & 15u};
+    for (int i = 7; i >= 0; --i) b = __funnelshift_l(__float_as_uint(limit - w.hb[i]), b, 1);
+    return {~q & 0xFFFFu, ~b & 0xFFu};
 }
 
 // The minimum `v` of chunk c joins the three lowest chunk minima (a tie stays behind the earlier chunk,
@@ -367,12 +369,11 @@ __device__ __forceinline__ int bit_at(uint32_t bits, int k)
 __device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
                                                uint32_t sets, int chunk1, int chunk2, float &bv, int &bi)
 {
-    const uint32_t places = sets & 0xFFFFu, blocks = (sets >> 18) & 15u;
-    const uint32_t columns = ((sets >> 16) & 1u ? places : 0u) | ((sets >> 17) & 1u ? places << 16 : 0u);
-    const int nc = __popc(columns), nb = __popc(blocks), total = nc * nb * (chunk2 >= 0 ? 2 : 1);
+    const Listed in = listed_of(sets);
+    const int nc = __popc(in.places), nb = __popc(in.blocks), total = nc * nb * (chunk2 >= 0 ? 2 : 1);
     for (int l = lane; l < total; l += 32) {
         const int b = l / nc, second = b >= nb ? 1 : 0;
-        const int j = (second ? chunk2 : chunk1) * 128 + bit_at(blocks, b - second * nb) * 32 + bit_at(columns, l - b * nc);
+        const int j = (second ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b - second * nb) * 16 + bit_at(in.places, l - b * nc);
         if (j < K) {
             const float d = exact_distance(z, cbr + (size_t)j * 32);
             if (d < bv || (d == bv && j < bi)) { bv = d; bi = j; }

@@ -32,7 +32,7 @@ constexpr int kATmem = kGroups * 128, kOnesTmem = kATmem + 32;                  
 
 struct Part {                                             // what a group, or a CTA, knows of a row at the stage end
     float m1, m2;                                         // its two lowest chunk minima
-    uint32_t sets;                                        // columns inside its window: places, halves << 16, blocks << 18; bit 22: a third chunk
+    uint32_t sets;                                        // columns inside its window (Listed::word); bit 24: a third chunk
     uint32_t chunks;                                      // chunk of m1, chunk of m2 << 16
 };
 
@@ -67,12 +67,7 @@ struct SplitParams {
 __device__ __forceinline__ bool sweep_chunks(Sweep &w, int grp, int P, int base, int cnt, uint32_t acc, uint32_t bar_full, uint32_t bar_free,
                                              uint32_t &acc_par, uint32_t bar_empty, uint32_t first_use, int lane, volatile uint32_t *abort_flag)
 {
-    w.m1 = w.m2 = w.m3 = INFINITY;
-    w.c1 = w.c2 = 0;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) w.d[q] = INFINITY;
-    w.h[0] = w.h[1] = INFINITY;
-    w.bb[0] = w.bb[1] = w.bb[2] = w.bb[3] = INFINITY;
+    w.clear();
     const bool releases = (threadIdx.x & 127) < 32;
     uint32_t slot = (first_use + (uint32_t)grp) % (uint32_t)kSplitRing;
 #pragma unroll 1
@@ -94,11 +89,12 @@ __device__ __forceinline__ bool sweep_chunks(Sweep &w, int grp, int P, int base,
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_free);
-        const float c0 = fold_block(w, ua, 0);
-        const float c1 = fold_block(w, ub, 1);
-        const float c2 = fold_block(w, uc, 2);
-        const float c3 = fold_block(w, ud, 3);
-        rank_chunk(w, fminf(min3(c0, c1, c2), c3), base + c);
+        float lowest;
+        fold_block(w, ua, 0, lowest);
+        fold_block(w, ub, 1, lowest);
+        fold_block(w, uc, 2, lowest);
+        fold_block(w, ud, 3, lowest);
+        rank_chunk(w, lowest, base + c);
     }
     return true;
 }
@@ -284,7 +280,7 @@ encode_split_kernel(const SplitParams p)
                     w.zz = grp < cnt ? norm[row] : 0.0f;                  // (a group without chunks has nothing inside any window)
                     w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);
                     const float lim = threshold(w, w.m1, prm);
-                    local[(grp - 1) * 128] = Part{w.m1, w.m2, listed(w, lim).word() | (w.m3 <= lim ? 1u << 22 : 0u),
+                    local[(grp - 1) * 128] = Part{w.m1, w.m2, listed(w, lim).word() | (w.m3 <= lim ? 1u << 24 : 0u),
                                                   (uint32_t)w.c1 | ((uint32_t)w.c2 << 16)};
                     __syncwarp();
                     if (lane == 0) mbar_arrive(BAR(kSLocal));
@@ -326,7 +322,7 @@ encode_split_kernel(const SplitParams p)
                 uint32_t sets;
                 {
                     const float lim = threshold(w, w.m1, prm);
-                    sets = listed(w, lim).word() | (w.m3 <= lim ? 1u << 22 : 0u);
+                    sets = listed(w, lim).word() | (w.m3 <= lim ? 1u << 24 : 0u);
                 }
                 // ---- the owners: the CTA's part, to every CTA of the cluster.  A group's sets were taken against its own minimum, a
                 // limit at least as high as the CTA's: they hold every column that counts.
@@ -346,7 +342,7 @@ encode_split_kernel(const SplitParams p)
                     sets = own <= lim ? sets : 0u;
 #pragma unroll
                     for (int k = 0; k < kGroups - 1; ++k) sets |= q[k].m1 <= lim ? q[k].sets : 0u;
-                    sets |= w.m3 <= lim ? 1u << 22 : 0u;
+                    sets |= w.m3 <= lim ? 1u << 24 : 0u;
                 }
                 Part best{w.m1, w.m2, sets, (uint32_t)w.c1 | ((uint32_t)w.c2 << 16)};
                 float next = INFINITY;                                    // the second lowest minimum of the parts
@@ -379,14 +375,14 @@ encode_split_kernel(const SplitParams p)
                 }
                 // The column of the lowest score is the choice of nearly every row: its codeword is asked for before it is known to be.
                 const float m1 = best.m1;
-                const Listed in{best.sets & 0xFFFFu, (best.sets >> 16) & 3u, (best.sets >> 18) & 15u};
+                const Listed in = listed_of(best.sets);
                 const int j1 = (int)(best.chunks & 0xFFFFu) * 128 + in.column(), jm = min(max(j1, 0), s.K - 1);
                 float ev[32];
                 load_codeword(cbr + (size_t)jm * 32, ev);
                 const float lim = threshold(w, m1, prm);
                 // (a padded column scores 60000: if nothing real scored less, scan everything)
                 const bool scan_all = !(w.zz < 3.6e9f) || !(w.win < INFINITY) || !(m1 < 59000.0f);
-                const bool unique = next > lim && best.m2 > lim && ((best.sets >> 22) & 1u) == 0u && in.single() && (uint32_t)j1 < (uint32_t)s.K;
+                const bool unique = next > lim && best.m2 > lim && ((best.sets >> 24) & 1u) == 0u && in.single() && (uint32_t)j1 < (uint32_t)s.K;
                 int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
                 uint32_t todo = __ballot_sync(0xFFFFFFFFu, !deg && (scan_all || !unique));
                 while (todo) {
@@ -408,7 +404,7 @@ encode_split_kernel(const SplitParams p)
                         q = mp[lane * 128 + (src - lane)];
                     }
                     uint32_t inside = __ballot_sync(0xFFFFFFFFu, lane < ctas && q.m1 <= lim_s);
-                    all_s = all_s || __any_sync(0xFFFFFFFFu, ((inside >> lane) & 1u) && ((q.sets >> 22) & 1u));    // a third chunk somewhere
+                    all_s = all_s || __any_sync(0xFFFFFFFFu, ((inside >> lane) & 1u) && ((q.sets >> 24) & 1u));    // a third chunk somewhere
                     float bv = INFINITY;
                     int bi = 0x7FFFFFFF;
                     if (all_s) {

@@ -19,11 +19,11 @@
 //   - Epilogue threads read their row's 128 scores with four tcgen05.ld of 32
 //     columns issued together, hand the accumulator back to the issuer as soon
 //     as they have landed, and fold them afterwards while the next chain runs.
-//     The fold keeps running minima over four partitions of the stage's
-//     columns: by 128-column chunk (the two lowest chunks and the value of the third), by 32-column block of a chunk,
-//     by half of a block, and by place within a half (16 places): 36 minimum
-//     operations per 32 scores.  At the stage end the sets of chunks, blocks,
-//     halves and places whose minimum lies inside the window bound where the
+//     The fold keeps running minima over three partitions of the stage's
+//     columns: by 128-column chunk (the two lowest chunks and the value of the third), by 16-column block of a
+//     chunk, and by place within a block (16 places): 35 minimum
+//     operations per 32 scores.  At the stage end the sets of chunks, blocks
+//     and places whose minimum lies inside the window bound where the
 //     exact argmin can be: when each set has one member the column is known
 //     and only that codeword is fetched; otherwise the warp re-scores every
 //     column in the product of the sets exactly in float32 against the float32
@@ -392,12 +392,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kPitch] = z[i];
                 if (!EIGHT) w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
-                w.m1 = w.m2 = w.m3 = INFINITY;
-                w.c1 = w.c2 = 0;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) w.d[q] = INFINITY;
-                w.h[0] = w.h[1] = INFINITY;
-                w.bb[0] = w.bb[1] = w.bb[2] = w.bb[3] = INFINITY;
+                w.clear();
                 // (no entry reaches 60000 in half precision; none is above 2^14, where 64 times its remainder leaves the 8-bit range)
                 const bool force_scan = EIGHT ? !(w.zz < 2.68e8f) || !(prm.a < INFINITY) : !(w.zz < 3.6e9f) || !(w.win < INFINITY);
 
@@ -426,11 +421,12 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     tc_fence_before();
                     __syncwarp();
                     if (!LONE && lane == 0) mbar_arrive(BAR(kBarAccFree + tile));    // the accumulator may be overwritten
-                    const float c0 = fold_block(w, ua, 0);
-                    const float c1 = fold_block(w, ub, 1);
-                    const float c2 = fold_block(w, uc, 2);
-                    const float c3 = fold_block(w, ud, 3);
-                    rank_chunk(w, fminf(min3(c0, c1, c2), c3), c);
+                    float lowest;
+                    fold_block(w, ua, 0, lowest);
+                    fold_block(w, ub, 1, lowest);
+                    fold_block(w, uc, 2, lowest);
+                    fold_block(w, ud, 3, lowest);
+                    rank_chunk(w, lowest, c);
                 }
                 if (!ok) break;
                 // The column of the lowest score is the choice of nearly every row: its codeword is asked for before it is
@@ -443,8 +439,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 load_codeword(cbr + (size_t)jm * 32, ev);
 
                 // ---- stage end: the columns that can still be the exact argmin are those of a listed
-                // chunk, in a listed block of the chunk, in a listed half, at a listed place.  When each of
-                // the four lists has one entry (almost always) that column is the choice: every other
+                // chunk, in a listed block of the chunk, at a listed place.  When each of
+                // the three lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
                 const float lim = EIGHT ? threshold8(w, m1, sc[r]) : threshold(w, m1, sc[r]);
                 const Listed in = listed(w, lim);
