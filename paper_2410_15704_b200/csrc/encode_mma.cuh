@@ -363,17 +363,18 @@ __device__ __forceinline__ int bit_at(uint32_t bits, int k)
     return __ffs(bits) - 1;
 }
 
-// Exact comparison of the columns listed by `sets` (Listed::word) in chunk1 and, unless negative, chunk2, by a
-// whole warp for one row z: lane l takes the l-th column, so that their codewords arrive together (one after
+// Exact comparison of the columns listed by `sets` (Listed::word) in `chunks` chunks -- chunk1 and chunk2, or with more than two all
+// of a stage --, by STRIDE lanes for one row z: lane l takes the l-th column, so that their codewords arrive together (one after
 // the other they cost a trip to L2 each: 4400 cycles a row, measured).  The lane's best joins (bv, bi).
+template <int STRIDE>
 __device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
-                                               uint32_t sets, int chunk1, int chunk2, float &bv, int &bi)
+                                               uint32_t sets, int chunk1, int chunk2, int chunks, float &bv, int &bi)
 {
     const Listed in = listed_of(sets);
-    const int nc = __popc(in.places), nb = __popc(in.blocks), total = nc * nb * (chunk2 >= 0 ? 2 : 1);
-    for (int l = lane; l < total; l += 32) {
-        const int b = l / nc, second = b >= nb ? 1 : 0;
-        const int j = (second ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b - second * nb) * 16 + bit_at(in.places, l - b * nc);
+    const int nc = __popc(in.places), per = nc * __popc(in.blocks), total = per * chunks;
+    for (int l = lane; l < total; l += STRIDE) {
+        const int c = l / per, in_chunk = l - c * per, b = in_chunk / nc;
+        const int j = (chunks > 2 ? c : c ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b) * 16 + bit_at(in.places, in_chunk - b * nc);
         if (j < K) {
             const float d = exact_distance(z, cbr + (size_t)j * 32);
             if (d < bv || (d == bv && j < bi)) { bv = d; bi = j; }
@@ -390,11 +391,12 @@ __device__ __forceinline__ void compare_all(const float (&z)[32], const float *_
     }
 }
 
-// The warp's best: smallest distance, lowest index on ties.
-__device__ __forceinline__ void best_of_warp(float &bv, int &bi)
+// The best of every LANES neighbouring lanes, in all of them: smallest distance, lowest index on ties.
+template <int LANES>
+__device__ __forceinline__ void best_of(float &bv, int &bi)
 {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = LANES / 2; off > 0; off >>= 1) {
         const float ov = __shfl_xor_sync(0xFFFFFFFFu, bv, off);
         const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
         if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }

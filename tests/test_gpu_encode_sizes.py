@@ -74,6 +74,24 @@ def test_chunks_over_accumulators_and_ctas(tiles, K):
     assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
 
 
+@pytest.mark.parametrize("n,K,layout", [(5000, 1024, 1), (19000, 1024, 0), (900, 1024, 1), (500, 384, 0), (40, 2048, 1)])
+@pytest.mark.parametrize("copies", [2, 3, 8])
+def test_rows_with_many_candidates(n, K, layout, copies):
+    """Every codeword there several times, some copies moved a little: each row has candidates in two, three or all
+    chunks, and the rows of a warp are compared four at a time; the lowest index wins among equals."""
+    x, cb = batch(n, 128, K, 4, "bf16", n + copies)
+    step = K // copies
+    for c in range(1, copies):
+        cb[:, c * step:(c + 1) * step] = cb[:, :step] * (1.0 + 1e-6 * (c % 2))
+    cfg = rvq.make_config(128, 32, layout, 4, K, 16, rvq.BF16, 0)
+    b = rvq.alloc_buffers(cfg, n, cb)
+    exact = torch.empty_like(b.codes)
+    rvq.rvq_encode(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
+    torch.cuda.synchronize()
+    assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
+
+
 def test_against_the_oracle():
     x, cb = batch(24, 128, 1024, 8, "f32", 5)
     cfg = rvq.make_config(128, 32, 0, 8, 1024, 16, rvq.F32, 0)
