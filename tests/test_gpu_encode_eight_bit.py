@@ -1,5 +1,6 @@
 """The throughput encoder's chain with 8-bit corrections: contiguous groups, 1024 codes and more, more than four tiles of 128 group
-rows per SM (three from 1921 codes on), and codebooks without outliers.  Its error window is some fifty times that of the
+rows per SM (three from 1921 codes on), and codebooks without outliers; or any groups and codebooks, from 40 tiles per SM on at 2048
+codes and from 100 on with statistics.  Its error window is some fifty times that of the
 half-precision chain, so these cases aim at it: planted pairs of codewords at gaps on both sides of the window, the
 statistics taken in the same pass, and codebooks with outliers, which keep the half-precision chain at the same sizes."""
 import numpy as np
@@ -97,3 +98,40 @@ def test_codebooks_with_outliers(n, K):
     assert torch.equal(b.codes, exact)
     # (with 8-bit corrections 2-3 % of the rows and stages were compared exactly)
     assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * 4
+
+
+@pytest.mark.parametrize("tiles,K,R,layout,statistics", [(40, 2048, 3, 1, False), (40, 1921, 2, 0, False), (39, 2048, 2, 1, False), (100, 1024, 2, 1, True),
+                                                         (100, 1000, 2, 0, True)])
+def test_long_calls_take_it_whatever_the_codebooks(tiles, K, R, layout, statistics):
+    """Heavy-tailed keys and codebooks on both sides of the lines: the codes are the float32 kernel's, and statistics taken in the
+    pass are those of rvq_ema_stats."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = tiles * sms * 32 - (1 if tiles == 39 else 0)
+    gen = torch.Generator(device="cuda").manual_seed(tiles + K)
+    scale = 0.25 - torch.log(torch.rand(8, 128, generator=gen, device="cuda").clamp_min(1e-7))
+    scale[:, ::16] *= 20.0
+    x = (torch.randn((n + 7) // 8, 8, 128, generator=gen, device="cuda") * scale).view(-1, 128)[:n].contiguous()
+    x[11] = 0.0
+    unit = scale / scale.square().mean(dim=1, keepdim=True).sqrt()
+    groups = (unit.view(8, 32, 4).transpose(1, 2) if layout else unit.view(8, 4, 32)).reshape(-1, 32)
+    cb = torch.randn(R, K, 32, generator=gen, device="cuda") * groups[torch.randint(32, (R, K), generator=gen, device="cuda")]
+    cb[1:] *= 0.8
+    assert kurtosis(cb.cpu().numpy()).min() > 6.0
+    cfg = rvq.make_config(128, 32, layout, R, K, 16, rvq.F32, 0)
+    b = rvq.alloc_buffers(cfg, n, cb)
+    exact = torch.empty_like(b.codes)
+    got, want = [[torch.empty(R, K, device="cuda"), torch.empty(R, K, 32, device="cuda")] for _ in range(2)]
+    if statistics:
+        rvq.rvq_encode_stats(cfg, x, n, 128, b.codebooks, b.prepared, b.codes, b.std, *got, b.workspace, b.workspace_bytes, b.status)
+        rvq.rvq_ema_stats(cfg, x, n, 128, b.codes, b.codebooks, *want, b.workspace, b.workspace_bytes, None)
+        assert torch.equal(got[0], want[0])
+        # (float32 sums of a bin's rows in another order, entries up to some 10 a row: the bound is a few ulps per row)
+        assert ((got[1] - want[1]).abs() / want[0].clamp(min=1.0)[..., None]).max().item() <= 1e-4
+    else:
+        rvq.rvq_encode(cfg, x, n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    st = rvq.read_status(b.status)
+    rvq.rvq_encode_exact(cfg, x, n, 128, b.codebooks, b.prepared, exact, b.std, None)
+    torch.cuda.synchronize()
+    assert torch.equal(b.codes, exact) and st["wait_timeouts"] == 0
+    # (the wider window of the 8-bit corrections lists more rows: 2 % instead of some 0.05 %)
+    assert (st["rescored_rows"] > 0.004 * n * 4 * R) == (tiles >= 40)
