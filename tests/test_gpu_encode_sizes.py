@@ -92,6 +92,24 @@ def test_rows_with_many_candidates(n, K, layout, copies):
     assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
 
 
+@pytest.mark.parametrize("tiles", [149, 296, 400, 592, 740, 1030, 1184])
+@pytest.mark.parametrize("K,R,layout", [(100, 3, 1), (256, 8, 0), (600, 1, 0), (1024, 4, 1), (1500, 2, 0)])
+def test_rounds_of_two_and_three_tiles(tiles, K, R, layout):
+    """One to eight tiles per SM: rounds of three tiles, of two tiles on three accumulators, and one kind after the other, with chunk
+    counts that begin such rounds at any accumulator; a last tile that is not full."""
+    n = 32 * tiles - 5
+    x, cb = batch(n, 128, K, R, "bf16", tiles + K)
+    cfg = rvq.make_config(128, 32, layout, R, K, 16, rvq.BF16, 0)
+    b = rvq.alloc_buffers(cfg, n, cb)
+    exact = torch.empty_like(b.codes)
+    for _ in range(2):
+        b.codes.fill_(0xAA)
+        rvq.rvq_encode(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+        rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
+        torch.cuda.synchronize()
+        assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
+
+
 def test_against_the_oracle():
     x, cb = batch(24, 128, 1024, 8, "f32", 5)
     cfg = rvq.make_config(128, 32, 0, 8, 1024, 16, rvq.F32, 0)
