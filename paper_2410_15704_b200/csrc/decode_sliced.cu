@@ -456,15 +456,21 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
         if (F32) {
             // entry (code j, stage r) = elements 4 slice .. 4 slice + 3 of codeword j of stage r (rotary slices
             // of strided groups: 2 slice, 2 slice + 1 and the two 16 elements on)
+            // From the prepared block's float32 section, where the pieces of neighbouring codewords lie together: a warp's entries
+            // are 64 contiguous bytes of a stage, not 16 of each of 32 lines (of the float32 codebooks; rotated keys, whose slices take two half pieces
+            // per codeword: 136000 vectors 46.7 -> 42.3 us, 240008 72.6 -> 68.1; plain decodes, one whole piece: the same within 0.5 %).
+            const uint8_t *blocks = dsec + 256 + 2 * decode_table_bytes(s.K);
+            const uint32_t per_stage = (uint32_t)slots_per_stage(s.K) * (uint32_t)kFloatBlockBytes;
             for (uint32_t t = tid; t < (uint32_t)s.K * 8; t += kDecThreads) {
                 const uint32_t r = t & 7u, j = t >> 3;
-                const float *src = cb + ((size_t)r * s.K + j) * 32;
+                const uint8_t *src = blocks + r * per_stage + (j >> 7) * (uint32_t)kFloatBlockBytes + (j & 127u) * 16u;
                 if (SPLIT) {
-                    const uint2 a = __ldg(reinterpret_cast<const uint2 *>(src + 2 * slice));
-                    const uint2 b = __ldg(reinterpret_cast<const uint2 *>(src + 2 * slice + 16));
+                    const uint8_t *half = src + (slice >> 1) * 2048u + (slice & 1u) * 8u;
+                    const uint2 a = __ldg(reinterpret_cast<const uint2 *>(half));
+                    const uint2 b = __ldg(reinterpret_cast<const uint2 *>(half + 4u * 2048u));
                     dst[t] = make_uint4(a.x, a.y, b.x, b.y);
                 } else {
-                    dst[t] = __ldg(reinterpret_cast<const uint4 *>(src) + slice);
+                    dst[t] = __ldg(reinterpret_cast<const uint4 *>(src + slice * 2048u));
                 }
             }
         } else if (SPLIT) {
