@@ -678,16 +678,17 @@ att_combine_kernel(const float *part, const float2 *part_ml, int chunks, int lay
     __shared__ float f_s[kShortMaxChunks];
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int head = blockIdx.x, c = threadIdx.x;
-    if (c < chunks) ml_s[c] = part_ml[head * chunks + c];
-    __syncthreads();
-    float top = -INFINITY, sum = 0.0f, a = 0.0f;
-    for (int k = 0; k < chunks; ++k) top = fmaxf(top, ml_s[k].x);
-    if (c < chunks) f_s[c] = ml_s[c].x == -INFINITY ? 0.0f : exp2f(ml_s[c].x - top);
-    __syncthreads();
-    // (all parts asked for together)
+    // (all parts asked for together, before the maxima that weigh them are known: after them 3000 tokens took 24.7 us a call instead of 22.9, 9000 50.2 instead of 49.7)
     float v[kShortMaxChunks];
 #pragma unroll
     for (int k = 0; k < kShortMaxChunks; ++k) v[k] = k < chunks ? __ldcg(part + ((size_t)head * chunks + k) * 128 + c) : 0.0f;
+    if (c < kShortMaxChunks) ml_s[c] = c < chunks ? part_ml[head * chunks + c] : make_float2(-INFINITY, 0.0f);
+    __syncthreads();
+    float top = -INFINITY, sum = 0.0f, a = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kShortMaxChunks; ++k) top = fmaxf(top, ml_s[k].x);
+    if (c < chunks) f_s[c] = ml_s[c].x == -INFINITY ? 0.0f : exp2f(ml_s[c].x - top);
+    __syncthreads();
 #pragma unroll
     for (int k = 0; k < kShortMaxChunks; ++k)
         if (k < chunks) {
