@@ -12,7 +12,7 @@
 //     in TMEM.
 //     EIGHT: the two small products of the split (remainder x head) in e4m3, as two K=32 steps beside
 //     three K=16 ones: 327 cycles per chain instead of 455, at an error of up to 2^-13 |z||e| in the score that the
-//     window allows for (window8).  For eight or more chunks, by codebooks, groups and size (eight_mode says why).
+//     window allows for (window8).  For contiguous groups, eight or more chunks and even codebooks (eight_possible says why).
 //   - The B operand (128 codewords per slot) streams from the prepared block
 //     through a ring of shared-memory slots filled by cp.async.bulk; every
 //     slot serves all three tiles.
@@ -75,24 +75,21 @@ constexpr int kDeferMinSlots = 6;                                     // chunks 
 // not what a stage waits for, and the added work at the stage end is (values, us, half precision / 8 bits, tiles per SM at
 // most: 1024 codes 64 / 75 at two, 122 / 137 at four, 145 / 138 at five; 2048 codes 147 / 156 at three, 207 / 191 at four).
 // And it needs rows whose window stays narrow.  With outlier channels 2.2-2.9 % of the rows and stages have more than one
-// candidate instead of 0.5 %.  The data are not known on the host; the codebooks, which follow them, are
-// looked at when they are prepared (PreparedHeader::even), and the kernel reads there which chain to take.  131072 vectors,
-// us in a burst, by the kurtosis of the codewords' entries (1024 codes; 2048 codes; measured with candidates compared row by row): 3: 721 -> 722, 1265 -> 1165;
-// 4.1: 721 -> 744, 1261 -> 1204; 4.4: 720 -> 726, 1264 -> 1197; 7.8: 721 -> 762, 1261 -> 1230; 9.3: 718 -> 769, 1259 -> 1273; 13: 720 -> 768, 1270 -> 1314;
-// 24: 720 -> 807, 1280 -> 1343; 44: 722 -> 904, 1274 -> 1590.
-// Whatever the codebooks, and on strided groups too, where the call is so long that its rounds are full and the chip at its power limit, which the shorter chain
-// spares (heavy-tailed keys on strided groups; us in a burst / back to back, seven steps -> five).  2048 codes, from 40 tiles per SM on: 28 tiles 1273 -> 1302 /
-// 1461 -> 1409; 41 1868 -> 1872 / 2126 -> 2042; 55 2494 -> 2455 / 2839 -> 2705; 111 4955 -> 4752 / 5696 -> 5395.  With statistics, whose additions hide the comparisons,
-// from 100 on: 55 1564 -> 1584 / 1777 -> 1718; 111 3055 -> 3036 / 3462 -> 3360; 221 6058 -> 5965 / 6902 -> 6670.  Without them and with 1024 codes
-// 221 tiles lose in a burst what they gain back to back (5367 -> 5545 / 6163 -> 6050).
+// candidate instead of 0.5 %, and the more the farther the outliers stand out.  The data are not known on the host; the codebooks, which
+// follow them, are looked at when they are prepared (PreparedHeader::even), and the kernel reads there which chain to take.  131072 vectors,
+// us in a burst, by the kurtosis of the codewords' entries (1024 codes; 2048 codes; measured with candidates compared row by row): 3: 721 -> 722,
+// 1265 -> 1165; 4.1: 721 -> 744, 1261 -> 1204; 4.4: 720 -> 726, 1264 -> 1197; 7.8: 721 -> 762, 1261 -> 1230; 9.3: 718 -> 769, 1259 -> 1273;
+// 13: 720 -> 768, 1270 -> 1314; 24: 720 -> 807, 1280 -> 1343; 44: 722 -> 904, 1274 -> 1590.  (Under the power cap the shorter chain gains another 6-7 % on both.)
+// However long the call is: with candidates compared four rows at a time, long calls on heavy-tailed keys gain a little while the
+// outlier channels stay moderate, on either kind of groups, but no size bounds what they lose (2048 codes, 194176 vectors = 41 tiles per SM on
+// contiguous groups, us in a burst, rows compared, by the factor on eight outlier channels of 128: 5: 1885 -> 1729, 1.7 %; 20: 1890 -> 1913, 2.8 %;
+// 60: 1881 -> 2244, 4.7 %; 200: 1867 -> 3427, 9.9 %; 1000 on four channels: 1872 -> 64295, 45 %; strided groups 20: 1892 -> 1826, 60: 1881 -> 2105,
+// 1000: 1885 -> 44969; 1024 codes with statistics, 100 tiles per SM, 1000: 2768 -> 51737 and 2753 -> 27474).
 constexpr int kEightMinSlots = 8;
-enum class Eight { kNever, kEven, kAlways };
-inline Eight eight_mode(const Shape &s, int64_t tiles, int sms, bool statistics)
+inline bool eight_possible(const Shape &s, int64_t tiles, int sms)
 {
     const int slots = slots_per_stage(s.K);
-    if (slots < kEightMinSlots || s.raw) return Eight::kNever;
-    if (tiles >= (int64_t)sms * (slots >= 16 ? 40 : 100) && (slots >= 16 || statistics)) return Eight::kAlways;
-    return s.layout == RVQ_GROUP_CONTIGUOUS && tiles > (int64_t)sms * (slots >= 16 ? 3 : 4) ? Eight::kEven : Eight::kNever;
+    return slots >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw && tiles > (int64_t)sms * (slots >= 16 ? 3 : 4);
 }
 
 // barrier slots
@@ -114,7 +111,6 @@ struct Params {
     float *energy;      // optional [R]: sum over the rows of the squared norm of what each stage leaves
     uint32_t wait_limit;   // polls after which a wait gives up (kWaitLimit; smaller only in the timeout self-test)
     int drop_last_chain;   // timeout self-test: 1 = tile 0's issuer leaves out the CTA's very last chain; else 0
-    int eight;             // 1 = 8-bit corrections whatever the codebooks (encode_tensor_either_kernel)
     int defer_stats;       // 1 = the statistics of every stage but the last are added by the MMA issuer warps (below)
 };
 
@@ -557,10 +553,10 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_kernel(const __grid_constant__ Params p) { encode_tensor_body<false, false>(p); }
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_lone_kernel(const __grid_constant__ Params p) { encode_tensor_body<false, true>(p); }
 
-// Where the 8-bit corrections are possible: always, or by the codebooks.
+// Where the 8-bit corrections are possible: by the codebooks.
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_either_kernel(const __grid_constant__ Params p)
 {
-    if (p.eight || reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true, false>(p);
+    if (reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true, false>(p);
     else encode_tensor_body<false, false>(p);
 }
 
@@ -589,12 +585,11 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     if (tiles > 0x7FFFFFFF) return RVQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
-    const Eight eight = eight_mode(s, tiles, sms, stat_sum != nullptr);
     const bool lone = tiles <= sms && slots_per_stage(s.K) <= kTiles && !s.raw && !stat_sum;
-    auto kernel = lone ? encode_tensor_lone_kernel : eight != Eight::kNever ? encode_tensor_either_kernel : encode_tensor_kernel;
+    auto kernel = lone ? encode_tensor_lone_kernel : eight_possible(s, tiles, sms) ? encode_tensor_either_kernel : encode_tensor_kernel;
     if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles, stat_cnt, stat_sum,
-             energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain, eight == Eight::kAlways ? 1 : 0,
+             energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,
              stat_sum != nullptr && encode_tensor_deferred_stages(s) > 0 ? 1 : 0};
     const int grid = (int)(tiles < sms ? tiles : sms);        // (fewer tiles than three per SM: one or two in each, not three in some)
     kernel<<<grid, kThreads, kSmemBytes, stream>>>(p);

@@ -1,6 +1,5 @@
 """The throughput encoder's chain with 8-bit corrections: contiguous groups, 1024 codes and more, more than four tiles of 128 group
-rows per SM (three from 1921 codes on), and codebooks without outliers; or any groups and codebooks, from 40 tiles per SM on at 2048
-codes and from 100 on with statistics.  Its error window is some fifty times that of the
+rows per SM (three from 1921 codes on), and codebooks without outliers.  Its error window is some fifty times that of the
 half-precision chain, so these cases aim at it: planted pairs of codewords at gaps on both sides of the window, the
 statistics taken in the same pass, and codebooks with outliers, which keep the half-precision chain at the same sizes."""
 import numpy as np
@@ -100,16 +99,17 @@ def test_codebooks_with_outliers(n, K):
     assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * 4
 
 
-@pytest.mark.parametrize("tiles,K,R,layout,statistics", [(40, 2048, 3, 1, False), (40, 1921, 2, 0, False), (39, 2048, 2, 1, False), (100, 1024, 2, 1, True),
-                                                         (100, 1000, 2, 0, True)])
-def test_long_calls_take_it_whatever_the_codebooks(tiles, K, R, layout, statistics):
-    """Heavy-tailed keys and codebooks on both sides of the lines: the codes are the float32 kernel's, and statistics taken in the
-    pass are those of rvq_ema_stats."""
+@pytest.mark.parametrize("tiles,K,R,layout,statistics,factor", [(40, 2048, 3, 1, False, 20), (40, 1921, 2, 0, False, 20), (41, 2048, 2, 0, False, 1000),
+                                                                (39, 2048, 2, 1, False, 200), (100, 1024, 2, 1, True, 20), (100, 1000, 2, 0, True, 1000)])
+def test_long_calls_with_outliers(tiles, K, R, layout, statistics, factor):
+    """Heavy-tailed keys and codebooks that follow them keep the half-precision chain however long the call is (with 8-bit
+    corrections 45 % of the rows are compared at a factor of 1000, and the call takes 30 times as long): the codes are the
+    float32 kernel's, and statistics taken in the pass are those of rvq_ema_stats."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = tiles * sms * 32 - (1 if tiles == 39 else 0)
     gen = torch.Generator(device="cuda").manual_seed(tiles + K)
     scale = 0.25 - torch.log(torch.rand(8, 128, generator=gen, device="cuda").clamp_min(1e-7))
-    scale[:, ::16] *= 20.0
+    scale[:, ::16] *= factor
     x = (torch.randn((n + 7) // 8, 8, 128, generator=gen, device="cuda") * scale).view(-1, 128)[:n].contiguous()
     x[11] = 0.0
     unit = scale / scale.square().mean(dim=1, keepdim=True).sqrt()
@@ -133,5 +133,4 @@ def test_long_calls_take_it_whatever_the_codebooks(tiles, K, R, layout, statisti
     rvq.rvq_encode_exact(cfg, x, n, 128, b.codebooks, b.prepared, exact, b.std, None)
     torch.cuda.synchronize()
     assert torch.equal(b.codes, exact) and st["wait_timeouts"] == 0
-    # (the wider window of the 8-bit corrections lists more rows: 2 % instead of some 0.05 %)
-    assert (st["rescored_rows"] > 0.004 * n * 4 * R) == (tiles >= 40)
+    assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * R
