@@ -278,7 +278,7 @@ encode_split_kernel(const SplitParams p)
                     Sweep w;
                     if (!sweep_chunks(w, grp, P, base, cnt, acc, BAR(kSAccFull + grp), BAR(kSAccFree + grp), acc_par, BAR(kSEmpty), (uint32_t)(r * cnt), lane, abort_flag)) break;
                     w.zz = grp < cnt ? norm[row] : 0.0f;                  // (a group without chunks has nothing inside any window)
-                    w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);
+                    w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
                     const float lim = threshold(w, w.m1, prm);
                     local[(grp - 1) * 128] = Part{w.m1, w.m2, listed(w, lim).word() | (w.m3 <= lim ? 1u << 24 : 0u),
                                                   (uint32_t)w.c1 | ((uint32_t)w.c2 << 16)};
@@ -316,7 +316,7 @@ encode_split_kernel(const SplitParams p)
                 if (warp == 0 && lane == 0 && ctas > 1) mbar_expect_tx(BAR(kSArrived + par), (uint32_t)ctas * 128u * 16u);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kZPitch] = z[i];
-                w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);
+                w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
                 ok = sweep_chunks(w, 0, P, base, cnt, acc, BAR(kSAccFull), BAR(kSAccFree), acc_par, BAR(kSEmpty), (uint32_t)(r * cnt), lane, abort_flag);
                 if (!ok) break;
                 uint32_t sets;

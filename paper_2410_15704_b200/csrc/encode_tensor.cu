@@ -395,7 +395,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 // park the float32 residual in shared memory for the sweep
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kPitch] = z[i];
-                if (!EIGHT) w.win = 2.125f * (prm.a * rough_sqrt(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
+                if (!EIGHT) w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);    // 2 * bound, with slack for this arithmetic
                 w.clear();
                 // (no entry reaches 60000 in half precision; none is above 2^14, where 64 times its remainder leaves the 8-bit range)
                 const bool force_scan = EIGHT ? !(w.zz < 2.68e8f) || !(prm.a < INFINITY) : !(w.zz < 3.6e9f) || !(w.win < INFINITY);

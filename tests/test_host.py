@@ -75,3 +75,16 @@ def test_bad_pointers_are_rejected_before_launch():
     assert rvq.lib.rvq_kmeans_init(ctypes.byref(odd), 256, 4, 128, 256, 3, 256, 256, 256, 1 << 40, None, None) == -3
     assert rvq.lib.rvq_ema_update(c, 256, 4, 128, 256, None, 256, 256, None, 0.9, 1e-5, 256, 1 << 30, None, None) == -1
     assert rvq.lib.rvq_prepare_codebooks(c, None, 256, None) == -1
+
+
+def test_error_windows_are_computed_with_rounded_operations():
+    """What decides which columns are compared exactly is float32 arithmetic rounded to nearest: no approximate instruction and no
+    fast-math intrinsic in the encoders, and no flag that would turn the rounded ones into such."""
+    csrc = os.path.join(ROOT, "paper_2410_15704_b200", "csrc")
+    names = [n for n in sorted(os.listdir(csrc)) if n.startswith("encode")]
+    assert "encode_mma.cuh" in names and "encode_tensor.cu" in names
+    for name in names:
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        assert not re.search(r"\.approx|__fdividef|__f(sqrt|rsqrt|rcp|div)_r[duz]|rsqrtf", code), name
+    build = open(os.path.join(ROOT, "paper_2410_15704_b200", "build.py")).read()
+    assert not re.search(r"use_fast_math|prec-sqrt|prec-div|ftz", build)
