@@ -430,8 +430,8 @@ __device__ __forceinline__ uint2 transpose_group_elements(uint32_t w0, uint32_t 
 }
 
 // F32 (4 channels per slice): the table holds the float32 codeword channels themselves (16 bytes per
-// code and stage, the geometry of the 8-channel level tables), filled from the codebooks by the CTA;
-// exact float32 sums, no table error and no exact route.
+// code and stage, the geometry of the 8-channel level tables), filled by the CTA from the prepared block's
+// float32 section, which holds every shape of the quoted kernels; exact float32 sums, no table error and no exact route.
 template <int DT, int CH, int LAYOUT, int BITS, bool SUMMED, int ROPE = 0, bool F32 = false>
 __device__ __forceinline__ void
 decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_t *__restrict__ std16, int64_t n,
@@ -439,6 +439,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
                    int64_t stride, rvq_status *st, uint8_t *table, RopeArgs ra = RopeArgs())
 {
     static_assert(F32 ? CH == 4 && !SUMMED : CH == 8, "8-channel level slices or 4-channel float32 slices");
+    static_assert(!F32 || (kDecodeWideK <= kFloatMaxK && kFloatMaxStages == 8), "the float32 section holds up to kDecodeWideK codes at depth 8");
     // half-split pairs on strided groups: a slice is two runs of elements 16 apart (CH / 2 each), so that
     // both channels of a pair are in the thread
     constexpr bool SPLIT = ROPE == 1 && LAYOUT == RVQ_GROUP_STRIDED;
@@ -459,7 +460,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             // From the prepared block's float32 section, where the pieces of neighbouring codewords lie together: a warp's entries
             // are 64 contiguous bytes of a stage, not 16 of each of 32 lines (of the float32 codebooks; rotated keys, whose slices take two half pieces
             // per codeword: 136000 vectors 46.7 -> 42.3 us, 240008 72.6 -> 68.1; plain decodes, one whole piece: the same within 0.5 %).
-            const uint8_t *blocks = dsec + 256 + 2 * decode_table_bytes(s.K);
+            const uint8_t *blocks = dsec + decode_section_bytes(s.K);              // (float_blocks_offset)
             const uint32_t per_stage = (uint32_t)slots_per_stage(s.K) * (uint32_t)kFloatBlockBytes;
             for (uint32_t t = tid; t < (uint32_t)s.K * 8; t += kDecThreads) {
                 const uint32_t r = t & 7u, j = t >> 3;

@@ -59,7 +59,10 @@ constexpr int kDecodeWideK = 1536;                        // 128 bytes per code 
 constexpr int kDecodeMaxK = 3072;                         // 64 bytes per code per slice
 __host__ __device__ inline int decode_slice_channels(int K) { return K <= kDecodeWideK ? 8 : 4; }
 __host__ __device__ inline size_t decode_table_bytes(int K) { return (size_t)K * 512; }   // 32 channels x 8 stages x 2 bytes
-// the prepared block holds two such tables: levels scaled per stage, then levels summed per stage parity
+// the prepared block holds two such tables: levels scaled per stage, then levels summed per stage parity;
+// the section: DecodeParams in 256 bytes, then the tables
+__host__ __device__ inline size_t decode_section_bytes(int K) { return 256 + 2 * decode_table_bytes(K); }
+static_assert(sizeof(DecodeParams) <= 256, "the decoder's parameters have 256 bytes");
 constexpr int kDecodeExactWideK = 1792;                   // float32 tables: 128 bytes per code per 4-channel slice
 constexpr int kDecodeExactK = 3584;                       // ... 64 bytes per code per 2-channel slice
 // Which tables a shape can be decoded through (group_dim 32, a power-of-two number of groups up to 32, depth <= 8; of
@@ -111,7 +114,7 @@ __host__ __device__ inline size_t decode_section_offset(const Shape &s)
 }
 __host__ __device__ inline size_t float_blocks_offset(const Shape &s)
 {
-    return decode_section_offset(s) + (decode_levels_prepared(s) ? 256 + 2 * decode_table_bytes(s.K) : 0);
+    return decode_section_offset(s) + (decode_levels_prepared(s) ? decode_section_bytes(s.K) : 0);
 }
 __host__ __device__ inline size_t float_blocks_bytes(const Shape &s)
 {
