@@ -95,8 +95,8 @@ def test_rows_with_many_candidates(n, K, layout, copies):
 @pytest.mark.parametrize("tiles", [149, 296, 400, 592, 740, 1030, 1184])
 @pytest.mark.parametrize("K,R,layout", [(100, 3, 1), (256, 8, 0), (600, 1, 0), (1024, 4, 1), (1500, 2, 0)])
 def test_rounds_of_two_and_three_tiles(tiles, K, R, layout):
-    """One to eight tiles per SM: rounds of three tiles, of two tiles on three accumulators, and one kind after the other, with chunk
-    counts that begin such rounds at any accumulator; a last tile that is not full."""
+    """One to eight tiles per SM: rounds of one, two and three tiles and one kind after the other, among them calls in which some
+    CTAs have a tile more than others; codebooks of one to twelve chunks; a last tile that is not full."""
     n = 32 * tiles - 5
     x, cb = batch(n, 128, K, R, "bf16", tiles + K)
     cfg = rvq.make_config(128, 32, layout, R, K, 16, rvq.BF16, 0)
@@ -108,6 +108,25 @@ def test_rounds_of_two_and_three_tiles(tiles, K, R, layout):
         rvq.rvq_encode_exact(cfg, x.cuda(), n, 128, b.codebooks, b.prepared, exact, b.std, b.status)
         torch.cuda.synchronize()
         assert torch.equal(b.codes, exact) and rvq.read_status(b.status)["wait_timeouts"] == 0
+
+
+@pytest.mark.parametrize("n,dim,K,R,layout,dtype", [(14209, 128, 256, 2, 1, "bf16"), (20003, 128, 1024, 3, 1, "f32"), (19001, 128, 1024, 2, 0, "f16"),
+                                                    (7150, 256, 600, 2, 0, "f32"), (60001, 32, 300, 2, 0, "bf16"), (1801, 1024, 400, 2, 1, "bf16")])
+@pytest.mark.parametrize("gap", [0, 16, 1000])
+def test_rows_of_the_rounds_to_come(n, dim, K, R, layout, dtype, gap):
+    """More than three tiles per SM, so that every CTA, or some, ask for the rows of a second round while the first runs: as one run where
+    the rows lie without gaps, vector by vector where they do not, up to a last round that ends inside a tile.  Rows with gaps are the
+    last thing in their allocation."""
+    x, cb = batch(n, dim, K, R, dtype, n + gap)
+    cfg = rvq.make_config(dim, 32, layout, R, K, 16, DT[dtype], 0)
+    stride = dim + gap
+    xd = torch.full(((n - 1) * stride + dim,), float("nan"), dtype=x.dtype, device="cuda").as_strided((n, dim), (stride, 1))
+    xd.copy_(x)
+    b, e = rvq.alloc_buffers(cfg, n, cb), rvq.alloc_buffers(cfg, n, cb)
+    rvq.rvq_encode(cfg, xd, n, stride, b.codebooks, b.prepared, b.codes, b.std, b.workspace, b.workspace_bytes, b.status)
+    rvq.rvq_encode_exact(cfg, x.cuda(), n, dim, e.codebooks, e.prepared, e.codes, e.std, e.status)
+    torch.cuda.synchronize()
+    assert torch.equal(b.codes, e.codes) and torch.equal(b.std, e.std) and rvq.read_status(b.status)["wait_timeouts"] == 0
 
 
 def test_against_the_oracle():
