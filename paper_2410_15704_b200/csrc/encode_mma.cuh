@@ -136,7 +136,7 @@ __device__ __forceinline__ float min3(float a, float b, float c)
     "r"(u[24]), "r"(u[25]), "r"(u[26]), "r"(u[27]), "r"(u[28]), "r"(u[29]), "r"(u[30]), "r"(u[31])
 
 // Start loading 32 consecutive TMEM columns of this thread's lane.  The
-// registers are not valid until tmem_ld_wait() has been given the same array.
+// registers are not valid until a wait has been given the same array.
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "

@@ -24,11 +24,12 @@
 //     chunk, and by place within a block (16 places): 35 minimum
 //     operations per 32 scores.  At the stage end the sets of chunks, blocks
 //     and places whose minimum lies inside the window bound where the
-//     exact argmin can be: when each set has one member the column is known
-//     and only that codeword is fetched; otherwise the warp re-scores every
-//     column in the product of the sets exactly in float32 against the float32
-//     codebook (direct form, lowest index on ties), and a full exact scan
-//     covers a third chunk inside the window.  The emitted code is the exact-L2 choice.
+//     exact argmin can be: when each set has one member the column is known,
+//     and its codeword already on the way; otherwise the columns in the product of
+//     the sets are compared exactly in float32 against the float32 codebook (direct
+//     form, lowest index on ties), four rows of a warp at a time with eight lanes to each; with
+//     a third chunk inside the window, in the listed blocks and places of all chunks.  A full exact scan
+//     covers rows whose scores say nothing.  The emitted code is the exact-L2 choice.
 //   - The A operand (the residual split into half-precision head and remainder)
 //     lives in TMEM next to its tile's scores, so the tensor core fetches only B
 //     from shared memory; the constant (1 1 1 0 ...) rows that pick up the
@@ -62,7 +63,7 @@ constexpr int kOffB = 0;
 constexpr int kOffZ = kOffB + kRing * kSlotBytes;                     // parked residuals, float [32][kPitch]
 constexpr int kPitch = kRowsPerPass + 1;                              // (odd: scatter_piece)
 constexpr int kOffCodes = kOffZ + 32 * kPitch * 4;
-constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;          
+constexpr int kOffBars = kOffCodes + kRowsPerPass * 16 * 2;
 constexpr int kOffFlags = kOffBars + 256;                             // per row of the round: 1 for a vector's, 0 past the last
 constexpr int kOffStages = kOffFlags + kRowsPerPass;                  // StageConst[16]
 constexpr int kSmemBytes = kOffStages + 16 * (int)sizeof(StageConst);
@@ -194,8 +195,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     __syncthreads();
     tc_fence_after();
 
-    // The four role warps run one lane each and need few registers; their share goes to the
-    // epilogue warps, which hold three 32-column blocks of scores at a time
+    // The four role warps need few registers; their share goes to the
+    // epilogue warps, which hold the four 32-column blocks of a chunk's scores at a time
     // (12 warps x 32 x 152 + 4 warps x 32 x 40 = 63488 of the 65536 the block was launched with).
     if (warp >= kEpiThreads / 32) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
@@ -234,7 +235,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
         }
     } else {
         // ------------------------------------------------------------ MMA issuer of tile t
-        // One thread per tile, each in a warp of its own so that the tiles' waits overlap.
+        // A warp per tile, so that the tiles' waits overlap.
         // Whatever it does between two tcgen05.mma chains delays its tile, so descriptors
         // are built once and all counters advance by increments.
         // (The whole warp runs the loop with warp-uniform values and one lane issues: operands that the
