@@ -146,11 +146,6 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&u)[32
 }
 // Waits for every tcgen05.ld of this thread; the arrays pass through so that no
 // use of them can be scheduled ahead of the wait.
-__device__ __forceinline__ void tmem_ld_wait2(uint32_t (&u)[32], uint32_t (&v)[32])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
-    asm volatile("" : RVQ_INOUT32(v) : : "memory");
-}
 __device__ __forceinline__ void tmem_ld_wait4(uint32_t (&u)[32], uint32_t (&v)[32], uint32_t (&w)[32], uint32_t (&x)[32])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
