@@ -8,7 +8,8 @@
 namespace rvq {
 
 constexpr uint32_t kWaitLimit = 4u * 1000u * 1000u;
-constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // f16 x f16 or e4m3 x e4m3 -> f32, M = N = 128
+// f16 x f16 or e4m3 x e4m3 -> f32, M = N = 128
+constexpr uint32_t kChainDesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -61,8 +62,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 }
 
 // Wait, when a role ends, for what it has left in flight (a phase of `bar` that a copy or a chain of MMAs will
-// complete): shared memory and TMEM stay the CTA's until then, also when its other waits have given up.  With nothing in
-// flight, as always at a regular end, this is one test of the barrier.
+// complete): shared memory and TMEM stay the CTA's until then, also when its other waits have given up.  With nothing
+// in flight, as always at a regular end, this is one test of the barrier.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity)
 {
     uint32_t ok = 0u;
@@ -172,7 +173,7 @@ __device__ __forceinline__ void tmem_ones(uint32_t taddr)
 // Per-row state of one stage's sweep over the scores.
 struct Sweep {
     float win;               // error window
-    float zz, ll;            // squared norms of the scaled residual (m1 + zz is the best squared distance) and of its remainder
+    float zz, ll;  // squared norms of the scaled residual (m1 + zz is the best squared distance) and of its remainder
     float m1, m2, m3;        // the three lowest chunk minima ...
     int c1, c2;              // ... and the chunks of the first two
     float hb[8];             // minimum per block of 16 columns inside its 128-column chunk
@@ -216,17 +217,18 @@ __device__ __forceinline__ void fold_block(Sweep &w, const uint32_t (&u)[32], in
     chunk = b == 0 ? fminf(hm[0], hm[1]) : min3(chunk, hm[0], hm[1]);
 }
 
-// What a stage's rows need to know of its codebook (prepare.cu), copied to shared memory at the start: asked for in the
-// prepared block when it was needed, every stage end waited for it.
+// What a stage's rows need to know of its codebook (prepare.cu), copied to shared memory at the start: asked for in
+// the prepared block when it was needed, every stage end waited for it.
 struct StageConst {
     float scale, a, b;                      // operand scale; |score error| <= a ||Z|| + b
-    float emax, eerr, elo;                  // norms, the stage's largest: codeword, what its two halves miss, its remainder half
+    float emax, eerr, elo;       // norms, the stage's largest: codeword, what its two halves miss, its remainder half
 };
 __device__ __forceinline__ void load_stage_consts(const uint8_t *prepared, int R, int tid, StageConst *out)
 {
     if (tid < R) {
         const StageParams q = reinterpret_cast<const StageParams *>(prepared + kPreparedParamsOffset)[tid];
-        const uint4 m = __ldg(reinterpret_cast<const uint4 *>(prepared + kPreparedMaximaOffset) + tid);     // StageMaxima
+        // StageMaxima
+        const uint4 m = __ldg(reinterpret_cast<const uint4 *>(prepared + kPreparedMaximaOffset) + tid);
         out[tid] = StageConst{q.scale, q.a, q.b, __uint_as_float(m.x), __uint_as_float(m.y), __uint_as_float(m.w)};
     }
 }
@@ -239,13 +241,14 @@ __device__ __forceinline__ void load_stage_consts(const uint8_t *prepared, int R
 // approximate winner's squared distance, at most m1 + zz + win; so their norms are at most E = ||Z|| + rho,
 // and the error bound of prepare.cu, which allows every codeword the largest norm of the stage, is taken
 // with E where that is smaller.
-// (Roots are the rounded ones: approximate ones save 0.8-2 % on small calls, 300 tokens' keys 46.3 -> 45.4 us, 512 float32 tokens at 256 codes
-// 26.05 -> 25.8, and 0.3 % on 4096 tokens' keys, 191.3 -> 190.7; they are less exact.)
+// (Roots are the rounded ones: approximate ones save 0.8-2 % on small calls, 300 tokens' keys 46.3 -> 45.4 us, 512
+// float32 tokens at 256 codes 26.05 -> 25.8, and 0.3 % on 4096 tokens' keys, 191.3 -> 190.7; they are less exact.)
 __device__ __forceinline__ float threshold(const Sweep &w, float m1, const StageConst &sb)
 {
     const float nz = sqrtf(w.zz) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
     const float e = fminf(sb.emax, (nz + sqrtf(d2 + w.win)) * 1.0001f);
-    const float elo = fminf(sb.elo, 4.8828125e-4f * e + 1.7e-7f), eerr = fminf(sb.eerr, 2.384185791015625e-7f * e + 1.7e-7f);
+    const float elo = fminf(sb.elo, 4.8828125e-4f * e + 1.7e-7f),
+                eerr = fminf(sb.eerr, 2.384185791015625e-7f * e + 1.7e-7f);
     const float a = 2.0f * (4.8828125e-4f * elo + 2.384185791015625e-7f * e + eerr) + 3.814697265625e-6f * e;
     const float b = e * (1.9073486328125e-6f * e + 4.76837158203125e-7f);
     const float win = fminf(w.win, 2.125f * (a * nz + b));
@@ -257,9 +260,9 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1, const Stage
 // above, the dot product is off by at most
 //   |z_lo.e - [64 z_lo][e/64]|        <= ||z_lo|| (cE + (1 + c)(cE + 64 sqrt(32) 2^-10)) + sqrt(32) 2^-16 (1 + c) E
 //   |z_hi.e_lo - [z_hi/64][64 e_lo]|  <= (cN + 0.354) L + ((1 + c) N + 0.354)(cL + sqrt(32) 2^-16)
-// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (prepare.cu; five instructions
-// of two kinds add up no worse than seven of one).  That comes to some 2^-13 |z||e|; the worst of 6.3 million
-// chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.
+// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (prepare.cu; five
+// instructions of two kinds add up no worse than seven of one).  That comes to some 2^-13 |z||e|; the worst of 6.3
+// million chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.
 __device__ __forceinline__ float window8(float nz, float nl, float e, const StageConst &sb)
 {
     constexpr float c = 0.0595f;
@@ -350,9 +353,10 @@ __device__ __forceinline__ int bit_at(uint32_t bits, int k)
     return __ffs(bits) - 1;
 }
 
-// Exact comparison of the columns listed by `sets` (Listed::word) in `chunks` chunks -- chunk1 and chunk2, or with more than two all
-// of a stage --, by STRIDE lanes for one row z: lane l takes the l-th column, so that their codewords arrive together (one after
-// the other they cost a trip to L2 each: 4400 cycles a row, measured).  The lane's best joins (bv, bi).
+// Exact comparison of the columns listed by `sets` (Listed::word) in `chunks` chunks -- chunk1 and chunk2, or with
+// more than two all of a stage --, by STRIDE lanes for one row z: lane l takes the l-th column, so that their
+// codewords arrive together (one after the other they cost a trip to L2 each: 4400 cycles a row, measured).  The
+// lane's best joins (bv, bi).
 template <int STRIDE>
 __device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
                                                uint32_t sets, int chunk1, int chunk2, int chunks, float &bv, int &bi)
@@ -361,7 +365,8 @@ __device__ __forceinline__ void compare_listed(const float (&z)[32], const float
     const int nc = __popc(in.places), per = nc * __popc(in.blocks), total = per * chunks;
     for (int l = lane; l < total; l += STRIDE) {
         const int c = l / per, in_chunk = l - c * per, b = in_chunk / nc;
-        const int j = (chunks > 2 ? c : c ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b) * 16 + bit_at(in.places, in_chunk - b * nc);
+        const int j = (chunks > 2 ? c : c ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b) * 16 +
+                      bit_at(in.places, in_chunk - b * nc);
         if (j < K) {
             const float d = exact_distance(z, cbr + (size_t)j * 32);
             if (d < bv || (d == bv && j < bi)) { bv = d; bi = j; }
@@ -370,7 +375,8 @@ __device__ __forceinline__ void compare_listed(const float (&z)[32], const float
 }
 
 // Exact comparison of all columns.
-__device__ __forceinline__ void compare_all(const float (&z)[32], const float *__restrict__ cbr, int K, int lane, float &bv, int &bi)
+__device__ __forceinline__ void compare_all(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
+                                            float &bv, int &bi)
 {
     for (int j = lane; j < K; j += 32) {
         const float d = exact_distance(z, cbr + (size_t)j * 32);
@@ -416,8 +422,8 @@ __device__ __forceinline__ void issue_chain8(uint32_t acc, uint32_t a0, uint64_t
     mma_f16_ts(acc, ones, bd, kChainDesc, 1);               // (1 1 1 0 .. 0) . norm cell 4 (and cell 5 . 0)
 }
 
-// The elements of 16-byte piece `off` of a head vector, widened, to where its group rows stand: element i of group g at
-// zv[i * PITCH + g].  PITCH is odd, so that neither the pieces of a vector nor its rows share banks.
+// The elements of 16-byte piece `off` of a head vector, widened, to where its group rows stand: element i of group g
+// at zv[i * PITCH + g].  PITCH is odd, so that neither the pieces of a vector nor its rows share banks.
 template <int PITCH, int N>
 __device__ __forceinline__ void scatter_piece(const Shape &s, const float (&val)[N], int off, float *zv)
 {
@@ -460,15 +466,16 @@ __device__ __forceinline__ void scatter_piece(const Shape &s, uint4 raw, int off
     }
 }
 // Piece `off` of head vector v; zeros past the last.
-__device__ __forceinline__ uint4 load_piece(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride, int64_t v, int off)
+__device__ __forceinline__ uint4 load_piece(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride,
+                                            int64_t v, int off)
 {
     if (v >= n) return make_uint4(0u, 0u, 0u, 0u);
     return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(x) + v * stride * s.elem_bytes) + off);
 }
 
-// The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces, four loads in flight per lane;
-// lane l gets the 32 elements of group l % G of vector l / G, zeros past the last vector.  `rows`: element 0 of the
-// warp's first row in a scratch area [32][PITCH].
+// The warp's 32 / G head vectors (1024 elements), from vector v_first on, come in as 16-byte pieces, four loads in
+// flight per lane; lane l gets the 32 elements of group l % G of vector l / G, zeros past the last vector.  `rows`:
+// element 0 of the warp's first row in a scratch area [32][PITCH].
 template <int PITCH>
 __device__ __forceinline__ void load_group_rows(const Shape &s, const void *__restrict__ x, int64_t n, int64_t stride,
                                                 int64_t v_first, int lane, float *rows, float (&z)[32])
@@ -525,7 +532,8 @@ __device__ __forceinline__ void divide_row(float (&z)[32], float dev, bool deg)
         lo = min(lo, twice - 1u);                                         // (zeros count as large)
         hi = max(hi, twice);
     }
-    const bool ordinary = lo >= 2u * 0x21800000u - 1u && hi <= 2u * 0x5D800000u && dev >= 9.094947e-13f && dev <= 1.0995116e12f;
+    const bool ordinary = lo >= 2u * 0x21800000u - 1u && hi <= 2u * 0x5D800000u &&
+                          dev >= 9.094947e-13f && dev <= 1.0995116e12f;
     if (__all_sync(0xFFFFFFFFu, ordinary || deg)) {                       // 2^-60 .. 2^60 over 2^-40 .. 2^40
         const float b = deg ? 1.0f : dev, y = __frcp_rn(b);
 #pragma unroll
@@ -573,7 +581,8 @@ __device__ __forceinline__ uint32_t e4m3x2(__half2 v)
     asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(d) : "r"(*reinterpret_cast<const uint32_t *>(&v)));
     return d;
 }
-__device__ __forceinline__ void split_operand8(const float (&z)[32], float scale, uint32_t (&ab)[32], float &zz, float &ll)
+__device__ __forceinline__ void split_operand8(const float (&z)[32], float scale, uint32_t (&ab)[32], float &zz,
+                                                float &ll)
 {
     zz = ll = 0.0f;
     const __half2 up = __floats2half2_rn(64.0f, 64.0f), down = __floats2half2_rn(0.015625f, 0.015625f);
@@ -616,15 +625,18 @@ __device__ __forceinline__ void emit_codes(const Shape &s, const uint16_t *codes
     } else {
         // the warp holds 32 / G whole head vectors; one 32-bit word per lane and step
         const int words = s.code_bytes / 4, vec_per_warp = 32 / G;
-        // quotients as products with 2^20 / d, rounded up: exact while the dividend is below 2^20 / d (here 512 codes of a vector by
-        // up to 16 stages, 8192 + 31 bits by up to 16, 256 words by 256); divisions were most of this loop
-        const uint32_t by_words = (1u << 20) / (uint32_t)words + 1u, by_bits = (1u << 20) / (uint32_t)s.bits + 1u, by_R = (1u << 20) / (uint32_t)s.R + 1u;
+        // quotients as products with 2^20 / d, rounded up: exact while the dividend is below 2^20 / d (here 512 codes
+        // of a vector by up to 16 stages, 8192 + 31 bits by up to 16, 256 words by 256); divisions were most of this
+        // loop
+        const uint32_t by_words = (1u << 20) / (uint32_t)words + 1u, by_bits = (1u << 20) / (uint32_t)s.bits + 1u,
+                       by_R = (1u << 20) / (uint32_t)s.R + 1u;
         for (int t = lane; t < vec_per_warp * words; t += 32) {
             const int vl = (int)((uint32_t)t * by_words >> 20), w = t - vl * words;
             const int64_t vv = v_first + vl;
             if (vv >= n) continue;
             uint32_t word = 0;
-            const int k_lo = (int)((uint32_t)(32 * w) * by_bits >> 20), k_hi = min(s.per_vector - 1, (int)((uint32_t)(32 * w + 31) * by_bits >> 20));
+            const int k_lo = (int)((uint32_t)(32 * w) * by_bits >> 20),
+                      k_hi = min(s.per_vector - 1, (int)((uint32_t)(32 * w + 31) * by_bits >> 20));
             for (int k = k_lo; k <= k_hi; ++k) {
                 const int gg = (int)((uint32_t)k * by_R >> 20), rr = k - gg * s.R;
                 const uint32_t val = codes_s[(vl * G + gg) * 16 + rr];
