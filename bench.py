@@ -50,17 +50,16 @@ def workload_name(tokens):
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant kernels, from ncu captures of the
 # kernels as they stand, keyed by (kernel, workload, tokens): an entry holds for that launch only, any other size
 # reports null.  An entry is taken out when its kernel changes.
-# (a batch of this size takes the chain with 8-bit corrections: five K-steps, two useful)
-ENCODE_KERNEL = "encode_tensor_either_kernel"
+ENCODE_KERNEL = "encode_tensor_kernel"
 DRAM_TRAFFIC = {
-    # encode with the EMA statistics fused in: 273.2 MB read + 55.9 MB written over 1,048,576 head vectors
-    (ENCODE_KERNEL, "ema_learning", 131072): 273177600 + 55933696,
-    # decode, contiguous layout: 72.4 MB read + 213.1 MB written (the rest of the 268 MB output still sat in L2
+    # encode with the EMA statistics fused in: 272.5 MB read + 56.1 MB written over 1,048,576 head vectors
+    (ENCODE_KERNEL, "ema_learning", 131072): 272471040 + 56119552,
+    # decode, contiguous layout: 73.4 MB read + 217.1 MB written (the rest of the 268 MB output still sat in L2
     # when the kernel ended)
-    ("decode_quoted_kernel", "decode_bandwidth", 131072): 72387584 + 213052160,
+    ("decode_quoted_kernel", "decode_bandwidth", 131072): 73449216 + 217148672,
 }
 # share of the tensor pipe's cycles that one launch keeps busy (%), from the same captures
-TENSOR_PIPE_PCT = {(ENCODE_KERNEL, "ema_learning", 131072): 41.4}
+TENSOR_PIPE_PCT = {(ENCODE_KERNEL, "ema_learning", 131072): 66.2}
 
 
 def algorithmic_numbers(w, bits=None):
@@ -480,8 +479,7 @@ def run_ours(args):
     enc_tflops = alg["encode_flops"] / (enc_ms * 1e-3) / 1e12
     # the encode kernel runs for milliseconds at a time, back to back for seconds: the sustained peak applies
     tensor_peak = peaks["bf16_tflops_sustained"]
-    # K-steps of a score chain, of which two are useful: with statistics five from 100 tiles of 128 group rows per SM on
-    chain_steps = 5 if n * 4 // 128 >= 100 * torch.cuda.get_device_properties(0).multi_processor_count else 7
+    chain_steps = 7                                           # K-steps of a score chain, of which two are useful
     traffic = DRAM_TRAFFIC.get((ENCODE_KERNEL, "ema_learning", args.tokens))
     line = {
         "metric": METRIC, "value": n * world * args.steps / (total_ms * 1e-3) / 1e6, "unit": UNIT,
