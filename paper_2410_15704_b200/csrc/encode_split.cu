@@ -12,12 +12,12 @@
 // parts of its rows -- one part with one column inside the window: the choice is certified; otherwise the listed
 // columns are compared exactly in float32 -- and takes the residual to the next stage.  All CTAs of a
 // cluster make the same choice from the same parts.
-// What bounds it: the chain of the stages.  One of 5200 cycles at 20 tiles and 2048 codes (7 CTAs of three chunks):
+// What bounds it: the chain of the stages.  One of 5200 cycles at 20 tiles and 2048 codes (6 CTAs of two or three chunks):
 // operand 400, first accumulator 900 later, the third and its fold 1900 after that, the joined part 300, the exchange
 // 500-800, merge and window 550, the codeword, asked for as soon as a candidate is known, 900.  us with parts sent by
 // every group, one issuer that waited before each chain and the codeword fetched at the end, and now: 616 values at
-// 2048 codes 43.1 / 36.9, 2400 keys at 1024 53.4 / 45.6, 4720 at 2048 (one CTA per tile) 80.3 / 65.1, 4720 at 512
-// 43.4 / 38.3.
+// 2048 codes 45.7 / 39.0, 2400 keys at 1024 54.5 / 46.6, 4720 at 2048 (one CTA per tile) 82.6 / 66.1, 4720 at 512
+// 45.2 / 39.0.  (The cycles were read with approximate roots in the window; the rounded ones add some 250.)
 #include "encode_mma.cuh"
 
 namespace rvq {
