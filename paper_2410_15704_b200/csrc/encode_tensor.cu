@@ -79,8 +79,8 @@ constexpr int kDeferMinSlots = 6;                       // chunks a stage needs 
 // three, 207 / 191 at four).
 // And it needs rows whose window stays narrow.  With outlier channels 2.2-2.9 % of the rows and stages have more than
 // one candidate instead of 0.5 %, and the more the farther the outliers stand out.  The data are not known on the
-// host; the codebooks, which follow them, are looked at when they are prepared (PreparedHeader::even), and the kernel
-// reads there which chain to take.  131072 vectors, us in a burst, by the kurtosis of the codewords' entries (1024
+// host; the codebooks, which follow them, are looked at when they are prepared (PreparedHeader::even: outliers, and
+// codewords far smaller than the largest, kMostInverse), and the kernel reads there which chain to take.  131072 vectors, us in a burst, by the kurtosis of the codewords' entries (1024
 // codes; 2048 codes; measured with candidates compared row by row): 3: 721 -> 722, 1265 -> 1165; 4.1: 721 -> 744,
 // 1261 -> 1204; 4.4: 720 -> 726, 1264 -> 1197; 7.8: 721 -> 762, 1261 -> 1230; 9.3: 718 -> 769, 1259 -> 1273; 13: 720
 // -> 768, 1270 -> 1314; 24: 720 -> 807, 1280 -> 1343; 44: 722 -> 904, 1274 -> 1590.  (Under the power cap the shorter

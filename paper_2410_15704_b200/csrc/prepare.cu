@@ -9,8 +9,8 @@
 // are split into a half-precision head and a half-precision remainder and the
 // contraction keeps the three leading products:
 //     z.e  ~  z_hi.e_hi + z_hi.e_lo + z_lo.e_hi        (error ~ 2^-22 |z||e|),
-// or, where a sweep is long enough to make up for more rows with several candidates and the codewords' energy is
-// not in a few outliers, the two small products in 8 bits (e4m3, twice the depth per step; error up to ~ 2^-13 |z||e|):
+// or, where a sweep is long enough to make up for more rows with several candidates and neither the codewords' energy is
+// in a few outliers nor many of them far smaller than the largest, the two small products in 8 bits (e4m3, twice the depth per step; error up to ~ 2^-13 |z||e|):
 //     z.e  ~  z_hi.e_hi + [64 z_lo]_8.[e / 64]_8 + [z_hi / 64]_8.[64 e_lo]_8.
 // Per stage r the block holds
 //   - a power-of-two scale 2^k chosen so that the largest scaled squared norm
@@ -179,12 +179,12 @@ prepare_params_kernel(Shape s, const StagePartial *part, PreparedHeader *hdr, St
         sp[r].a = INFINITY;
         sp[r].b = INFINITY;
         sp[r].unsafe = (!isfinite(maxn) || ldexp(maxn, 2 * k) > 8200.0) ? 1.0f : 0.0f;
-        mx[r].emax = 0u; mx[r].eerr = 0u; mx[r].nmax = 0u; mx[r].elomax = 0u;
+        mx[r].emax = 0u; mx[r].eerr = 0u; mx[r].inverse = 0u; mx[r].elomax = 0u;
         if (r < 8) { s_lo[r] = lo; s_step[r] = hi > lo ? (hi - lo) / 65535.0f : 0.0f; }     // finest unit the range allows
     }
     const int evens = __popc(__ballot_sync(0xFFFFFFFFu, even));
     if (r == 0) {
-        hdr->even = 2 * evens >= s.R ? 1u : 0u;
+        hdr->even = 2 * evens >= s.R ? 1u : 0u;                 // (prepare_finish_kernel has the last word)
         hdr->magic = kPreparedMagic; hdr->R = s.R; hdr->K = s.K; hdr->gd = s.gd;
         hdr->slots = slots_per_stage(s.K);
         hdr->decode_offset = decode_levels_prepared(s)
@@ -253,7 +253,7 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
     for (int c = 0; c < 9; ++c)
 #pragma unroll
         for (int i = 0; i < 8; ++i) cell[c][i] = __float2half_rn(0.0f);
-    float emax = 0.f, eerr = 0.f, nmax = 0.f, elomax = 0.f;
+    float emax = 0.f, eerr = 0.f, elomax = 0.f;
     float e[32];
     if (j < s.K) {
         const float4 *src = reinterpret_cast<const float4 *>(cb + ((size_t)r * s.K + j) * 32);
@@ -283,7 +283,7 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
         cell[4][0] = n_hi; cell[4][1] = n_lo; cell[4][2] = __double2half(r2);
         // round the maxima up so that the bound stays a bound in float32
         emax = __double2float_ru(sqrt(n2)); eerr = __double2float_ru(sqrt(d2));
-        nmax = __double2float_ru(n2); elomax = __double2float_ru(sqrt(l2));
+        elomax = __double2float_ru(sqrt(l2));
     } else {
         cell[4][0] = __float2half_rn(60000.0f);           // padding never wins
     }
@@ -296,13 +296,15 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
 #pragma unroll
         for (int q = 0; q < 8; ++q) o[q * kSlotCodewords] = j < s.K ? make_float4(e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3]) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
     }
+    // (a codeword of zeros says nothing of its rows)
+    const float excess = emax > 0.0f ? fminf(fmaxf(__frcp_rn(emax) - kInverseFree, 0.0f), kInverseCap) : 0.0f;
     // non-negative floats order like their bit patterns (a NaN's is above all); one addition to the maxima per warp
     const uint32_t b0 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(emax)), b1 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(eerr));
-    const uint32_t b2 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(nmax)), b3 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(elomax));
+    const uint32_t b2 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(excess * 2048.0f)), b3 = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(elomax));
     if ((jj & 31) == 0) {
         atomicMax(&mx[r].emax, b0);
         atomicMax(&mx[r].eerr, b1);
-        atomicMax(&mx[r].nmax, b2);
+        if (b2 != 0u) atomicAdd(&mx[r].inverse, b2);          // (65535 codes: below 2^32; whole numbers: the same in any order)
         atomicMax(&mx[r].elomax, b3);
     }
 }
@@ -314,23 +316,30 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
 //   |.| <= ||Z|| (2^-11 elomax + 2^-22 emax + eerr) + sqrt(32) 2^-25 emax
 //   (the last term: a subnormal Zl is off by at most 2^-25 per channel),
 //   times 2 for the factor -2 of the score; plus the accumulation of 115 terms
-//   in the tensor core, taken as 2^-19 of nmax + 2 ||Z|| emax, which bounds the
+//   in the tensor core, taken as 2^-19 of nmax + 2 ||Z|| emax (nmax = emax^2, rounded up), which bounds the
 //   sum of the terms' magnitudes.  The hardware's accumulation is not
 //   documented; measured on B200 against float64 sums of the very operands, 6.3
 //   million chains each, the error was at most 2^-20.7 of the sum of magnitudes on
 //   normal data and 2^-20.0 with x20 outlier channels, so 2^-19 leaves a factor of
 //   2 (the chain with 8-bit corrections: 2^-22.3 and 2^-20.9); the tests
 //   compare tens of millions of choices with the all-float32 kernel's.
-__global__ void prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxima *mx)
+__global__ void __launch_bounds__(32)
+prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxima *mx, PreparedHeader *hdr)
 {
     follow_previous();
     const int r = threadIdx.x;
-    if (r >= s.R) return;
-    const float emax = __uint_as_float(mx[r].emax), eerr = __uint_as_float(mx[r].eerr);
-    const float nmax = __uint_as_float(mx[r].nmax), elomax = __uint_as_float(mx[r].elomax);
-    if (sp[r].unsafe != 0.0f) return;                      // a, b stay infinite: every row is scanned exactly
-    sp[r].a = 2.0f * (4.8828125e-4f * elomax + 2.384185791015625e-7f * emax + eerr) + 3.814697265625e-6f * emax;
-    sp[r].b = 1.9073486328125e-6f * nmax + 4.76837158203125e-7f * emax;
+    uint32_t inverse = 0u;
+    if (r < s.R) {
+        inverse = mx[r].inverse >> 4;                      // (16 stages of 65535 codes: below 2^32)
+        const float emax = __uint_as_float(mx[r].emax), eerr = __uint_as_float(mx[r].eerr);
+        const float nmax = emax * emax * 1.000001f, elomax = __uint_as_float(mx[r].elomax);
+        if (sp[r].unsafe == 0.0f) {                        // else a, b stay infinite: every row is scanned exactly
+            sp[r].a = 2.0f * (4.8828125e-4f * elomax + 2.384185791015625e-7f * emax + eerr) + 3.814697265625e-6f * emax;
+            sp[r].b = 1.9073486328125e-6f * nmax + 4.76837158203125e-7f * emax;
+        }
+    }
+    inverse = __reduce_add_sync(0xFFFFFFFFu, inverse);
+    if (r == 0 && (float)inverse > kMostInverse * 128.0f * (float)s.K * (float)s.R) hdr->even = 0u;
 }
 
 int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream, bool chained)
@@ -351,7 +360,7 @@ int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t
         rc = launch_chained(true, prepare_image_kernel, dim3(slots_per_stage(s.K), s.R), kSlotCodewords, 0, stream, s, cb, sp, mx, p + kPreparedImageOffset,
                             float_blocks_prepared(s) ? reinterpret_cast<float4 *>(p + float_blocks_offset(s)) : nullptr);
         if (rc != RVQ_OK) return rc;
-        if ((rc = launch_chained(true, prepare_finish_kernel, dim3(1), 32, 0, stream, s, sp, mx)) != RVQ_OK) return rc;
+        if ((rc = launch_chained(true, prepare_finish_kernel, dim3(1), 32, 0, stream, s, sp, mx, hdr)) != RVQ_OK) return rc;
     }
     if (dec)
         return launch_chained(true, decode_table_kernel, dim3((s.K * 8 + 255) / 256, 4), 256, 0, stream, s, cb, dp, lo,

@@ -24,12 +24,25 @@ constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 24;   // operand image, 
 struct PreparedHeader {
     uint32_t magic, R, K, gd, slots;
     uint32_t decode_offset;   // byte offset of the decoder section, 0 if absent
-    uint32_t even;            // 1: the codewords' energy is spread over their entries (kEvenKurtosis), 0: outliers carry it
+    uint32_t even;            // 1: the codebooks suit the 8-bit corrections (kEvenKurtosis, kMostInverse)
 };
 // A stage's codewords count as even when the fourth moment of their entries is at most this many times the square of the
-// second (3 for a normal distribution); the block does when at least half of its stages do.  The throughput encoder
-// takes the 8-bit corrections by it (encode_tensor.cu).
+// second (3 for a normal distribution); the block does when at least half of its stages do and its codewords are not
+// too small for the steps of the 8-bit operands.  The throughput encoder takes the 8-bit corrections by it (encode_tensor.cu).
 constexpr float kEvenKurtosis = 6.0f;
+// The 8-bit operands have a smallest step, so a row's window has a part that does not shrink with the row (window8): of
+// the rows, whose norms follow the codewords', some 0.5 % + 5 % / norm have several candidates, the norm in the operands'
+// scale (the largest of a stage is 45 ... 90), and each of them costs the more the smaller it is.  So a codeword counts by
+// what 1 / norm has over kInverseFree, and the block by the mean.  (A fourth moment does not see it: with one group of
+// four 1000 times smaller than the others it is 4.1.)  us with seven steps -> with five, by the mean; 194176 vectors on
+// contiguous groups, 2048 codes unless said:
+//   all groups alike 0: 1831 -> 1596; one of four 10 times smaller 0.04: 1843 -> 1652, 30 times 0.16: 1850 -> 1779, 100
+//   times 0.57: 1852 -> 2361, 300 times 1.8: 1898 -> 5163, 1000 times 4: 1973 -> 41109;
+//   outlier channels in one stage of eight, x200 0.08: 1815 -> 1734 (1024 codes 997 -> 1010), x1000 0.56: 1805 -> 10447;
+//   in two, x60 0.09: 1821 -> 1684, x200 with 1024 codes 0.13: 992 -> 1044;
+//   in four, x20 0.08: 1841 -> 1691 (1024 codes 0.05: 1012 -> 1027), x60 0.15: 1819 -> 1874, x1000 2.2: 1818 -> 36012.
+// Back to back, under the power cap, five steps take 3-9 % less than that beside seven.
+constexpr float kMostInverse = 0.1f, kInverseFree = 0.0625f, kInverseCap = 16.0f;
 
 // Decoder section (group_dim 32, R <= 8, K <= kDecodeMaxK): per stage an affine
 // map value = lo_r + q * scale_r * base with q a 16-bit level, scale_r an integer in
@@ -134,7 +147,9 @@ struct StagePartial {
 };
 
 struct StageMaxima {
-    uint32_t emax, eerr, nmax, elomax;   // float bit patterns (non-negative), filled with atomicMax
+    uint32_t emax, eerr;                 // float bit patterns (non-negative), filled with atomicMax
+    uint32_t inverse;                    // the codewords' sum of what 1 / norm has over kInverseFree, in units of 2^-11
+    uint32_t elomax;                     // as emax
 };
 
 __host__ __device__ inline int slots_per_stage(int K) { return (K + kSlotCodewords - 1) / kSlotCodewords; }

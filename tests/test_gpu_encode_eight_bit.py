@@ -1,5 +1,5 @@
 """The throughput encoder's chain with 8-bit corrections: contiguous groups, 1024 codes and more, more than four tiles of 128 group
-rows per SM (three from 1921 codes on), and codebooks without outliers.  Its error window is some fifty times that of the
+rows per SM (three from 1921 codes on), and codebooks without outliers and of codewords of like sizes.  Its error window is some fifty times that of the
 half-precision chain, so these cases aim at it: planted pairs of codewords at gaps on both sides of the window, the
 statistics taken in the same pass, and codebooks with outliers, which keep the half-precision chain at the same sizes."""
 import numpy as np
@@ -97,6 +97,29 @@ def test_codebooks_with_outliers(n, K):
     assert torch.equal(b.codes, exact)
     # (with 8-bit corrections 2-3 % of the rows and stages were compared exactly)
     assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * 4
+
+
+@pytest.mark.parametrize("n,K", [(18945, 1024), (14219, 2048)])
+@pytest.mark.parametrize("kind,eight", [("group 10", True), ("group 1000", False), ("stages 1000", False)])
+def test_codewords_of_different_sizes(n, K, kind, eight):
+    """One of four groups smaller than the others, by 10 or 1000, in rows and codewords; half of the stages with outlier channels, the
+    others even.  Rows far smaller than the largest codeword have many candidates under the 8-bit
+    corrections (24 % and 22 % of the rows and stages, 20 times the time), so such codebooks keep the half-precision chain."""
+    g = np.random.default_rng(n)
+    R, what = 4, kind.split()
+    scale = np.ones((R, 4, 32))
+    if what[0] == "group":
+        scale[:, 1] /= float(what[1])
+    if what[0] == "stages":
+        scale[:2, 0, :6] *= float(what[1])
+    x = (g.normal(size=(n, 128)) * scale[0].reshape(-1)).astype(np.float32)
+    scale /= np.sqrt((scale ** 2).mean(axis=(1, 2), keepdims=True))
+    cb = np.stack([g.normal(size=(K, 32)) * scale[r, g.integers(0, 4, size=K)] * 0.8 ** r for r in range(R)]).astype(np.float32)
+    assert np.sort(kurtosis(cb))[R // 2 - 1] < 6.0              # (even in at least half of the stages)
+    _, b, _, exact, st = encode_both(x, cb, R, K)
+    assert torch.equal(b.codes, exact)
+    share = (st["rescored_rows"] + st["exhaustive_rows"]) / (n * 4 * R)
+    assert 0.005 < share < 0.02 if eight else share < 0.01
 
 
 @pytest.mark.parametrize("tiles,K,R,layout,statistics,factor", [(40, 2048, 3, 1, False, 20), (40, 1921, 2, 0, False, 20), (41, 2048, 2, 0, False, 1000),
