@@ -353,18 +353,21 @@ __device__ __forceinline__ int bit_at(uint32_t bits, int k)
     return __ffs(bits) - 1;
 }
 
+// a / b, rounded down, for 0 <= a < 2^16 and 1 <= b <= 128: the quotient of the halves between has an error far below
+// the 1 / 256 that separates it from a whole number.  (An integer division takes some 200 cycles.)
+__device__ __forceinline__ int small_quotient(int a, int b) { return (int)__fdividef((float)a + 0.5f, (float)b); }
+
 // Exact comparison of the columns listed by `sets` (Listed::word) in `chunks` chunks -- chunk1 and chunk2, or with
-// more than two all of a stage --, by STRIDE lanes for one row z: lane l takes the l-th column, so that their
+// more than two all of a stage --, by `stride` lanes for one row z: lane l takes the l-th column, so that their
 // codewords arrive together (one after the other they cost a trip to L2 each: 4400 cycles a row, measured).  The
 // lane's best joins (bv, bi).
-template <int STRIDE>
-__device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane,
+__device__ __forceinline__ void compare_listed(const float (&z)[32], const float *__restrict__ cbr, int K, int lane, int stride,
                                                uint32_t sets, int chunk1, int chunk2, int chunks, float &bv, int &bi)
 {
     const Listed in = listed_of(sets);
     const int nc = __popc(in.places), per = nc * __popc(in.blocks), total = per * chunks;
-    for (int l = lane; l < total; l += STRIDE) {
-        const int c = l / per, in_chunk = l - c * per, b = in_chunk / nc;
+    for (int l = lane; l < total; l += stride) {
+        const int c = small_quotient(l, per), in_chunk = l - c * per, b = small_quotient(in_chunk, nc);
         const int j = (chunks > 2 ? c : c ? chunk2 : chunk1) * 128 + bit_at(in.blocks, b) * 16 +
                       bit_at(in.places, in_chunk - b * nc);
         if (j < K) {
@@ -384,12 +387,10 @@ __device__ __forceinline__ void compare_all(const float (&z)[32], const float *_
     }
 }
 
-// The best of every LANES neighbouring lanes, in all of them: smallest distance, lowest index on ties.
-template <int LANES>
-__device__ __forceinline__ void best_of(float &bv, int &bi)
+// The best of every `lanes` neighbouring lanes (a power of two), in all of them: smallest distance, lowest index on ties.
+__device__ __forceinline__ void best_of(int lanes, float &bv, int &bi)
 {
-#pragma unroll
-    for (int off = LANES / 2; off > 0; off >>= 1) {
+    for (int off = lanes / 2; off > 0; off >>= 1) {
         const float ov = __shfl_xor_sync(0xFFFFFFFFu, bv, off);
         const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
         if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }

@@ -440,13 +440,13 @@ encode_split_kernel(const SplitParams p)
                             const int second = q.m2 <= lim_s ? (int)(q.chunks >> 16) : -1;
                             for (; inside; inside &= inside - 1u) {
                                 const int k = __ffs(inside) - 1;
-                                compare_listed<32>(zs, cbr, s.K, lane, __shfl_sync(0xFFFFFFFFu, q.sets, k),
+                                compare_listed(zs, cbr, s.K, lane, 32, __shfl_sync(0xFFFFFFFFu, q.sets, k),
                                                (int)(__shfl_sync(0xFFFFFFFFu, q.chunks, k) & 0xFFFFu),
                                                __shfl_sync(0xFFFFFFFFu, second, k),
                                                __shfl_sync(0xFFFFFFFFu, second >= 0 ? 2 : 1, k), bv, bi);
                             }
                         }
-                        best_of<32>(bv, bi);
+                        best_of(32, bv, bi);
                         if (lane == src) {
                             bj = bi < s.K ? bi : 0;
                             if (rank == 0) { if (all_s) ++n_exhaustive; else ++n_rescored; }

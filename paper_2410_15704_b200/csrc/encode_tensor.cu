@@ -28,7 +28,7 @@
 //     exact argmin can be: when each set has one member the column is known,
 //     and its codeword already on the way; otherwise the columns in the product of
 //     the sets are compared exactly in float32 against the float32 codebook (direct
-//     form, lowest index on ties), four rows of a warp at a time with eight lanes to each; with
+//     form, lowest index on ties), up to four rows of a warp at a time with eight lanes or more to each; with
 //     a third chunk inside the window, in the listed blocks and places of all chunks.  A full exact scan
 //     covers rows whose scores say nothing.  The emitted code is the exact-L2 choice.
 //   - The A operand (the residual split into half-precision head and remainder)
@@ -490,9 +490,10 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
                 // Rows with more than one candidate: their candidate columns are compared
                 // exactly in float32, direct form: smallest distance, lowest index on ties.  Four rows at a time,
-                // eight lanes to a row; rows whose scores say nothing one by one, all columns, by the whole warp.
+                // eight lanes to a row, more with fewer rows; rows whose scores say nothing one by one, all columns, by the whole warp.
                 // (One row at a time, and all columns also where a third chunk came inside the window: 32768 keys 219
-                // -> 215 us, 262144 values 2515 -> 2495.)
+                // -> 215 us, 262144 values 2515 -> 2495.  All lanes for a single row, half for two, and no integer
+                // divisions: 65536 values with one group of four 10 times smaller 609 -> 570, in a burst.)
                 uint32_t scans = __ballot_sync(0xFFFFFFFFu, flagged && scan_all);
                 uint32_t todo = __ballot_sync(0xFFFFFFFFu, flagged) & ~scans;
                 while (todo | scans) {
@@ -504,23 +505,24 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 #pragma unroll
                         for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kPitch + (src - lane)];
                         compare_all(zs, cbr, s.K, lane, bv, bi);
-                        best_of<32>(bv, bi);
+                        best_of(32, bv, bi);
                         if (lane == src) { bj = bi < s.K ? bi : 0; ++n_exhaustive; }
                         continue;
                     }
-                    // this lane's row: the (lane / 8)-th of the list, or the last
+                    // a warp's lanes for one row, half of them each for two, a quarter each for more: this lane's row
+                    const int share = (todo & (todo - 1u)) == 0u ? 5 : __popc(todo) == 2 ? 4 : 3;
                     int src = __ffs(todo) - 1;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        if (k <= (lane >> 3) && todo) src = __ffs(todo) - 1;
+                        if (k <= (lane >> share) && todo) src = __ffs(todo) - 1;
                         todo &= todo - 1u;
                     }
 #pragma unroll
                     for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kPitch + (src - lane)];
-                    compare_listed<8>(zs, cbr, s.K, lane & 7, __shfl_sync(0xFFFFFFFFu, in.word(), src),
-                                      __shfl_sync(0xFFFFFFFFu, w.c1, src), __shfl_sync(0xFFFFFFFFu, w.c2, src),
-                                      __shfl_sync(0xFFFFFFFFu, chunks, src), bv, bi);
-                    best_of<8>(bv, bi);
+                    compare_listed(zs, cbr, s.K, lane & ((1 << share) - 1), 1 << share, __shfl_sync(0xFFFFFFFFu, in.word(), src),
+                                   __shfl_sync(0xFFFFFFFFu, w.c1, src), __shfl_sync(0xFFFFFFFFu, w.c2, src),
+                                   __shfl_sync(0xFFFFFFFFu, chunks, src), bv, bi);
+                    best_of(1 << share, bv, bi);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int row = __shfl_sync(0xFFFFFFFFu, src, 8 * k), best = __shfl_sync(0xFFFFFFFFu, bi, 8 * k);
