@@ -152,6 +152,25 @@ __device__ __forceinline__ void tmem_ld_wait4(uint32_t (&u)[32], uint32_t (&v)[3
     asm volatile("" : RVQ_INOUT32(w) : : "memory");
     asm volatile("" : RVQ_INOUT32(x) : : "memory");
 }
+__device__ __forceinline__ void tmem_ld_wait2(uint32_t (&u)[32], uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : RVQ_INOUT32(u) : : "memory");
+    asm volatile("" : RVQ_INOUT32(v) : : "memory");
+}
+// The low halves of 64 consecutive columns, two to a register.
+__device__ __forceinline__ void tmem_ld64_packed_issue(uint32_t taddr, uint32_t (&u)[32])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.pack::16b.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : RVQ_OUT32(u) : "r"(taddr));
+}
+// (the wait for it is tmem_st32's)
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 u)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 : : "r"(taddr), "r"(u.x), "r"(u.y), "r"(u.z), "r"(u.w) : "memory");
+}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -176,6 +195,12 @@ struct Sweep {
     float zz, ll;  // squared norms of the scaled residual (m1 + zz is the best squared distance) and of its remainder
     float m1, m2, m3;        // the three lowest chunk minima ...
     int c1, c2;              // ... and the chunks of the first two
+    static constexpr float kPadded = 59000.0f;      // (a padded column scores 60000)
+    __device__ __forceinline__ float lowest() const { return m1; }
+    __device__ __forceinline__ float second() const { return m2; }
+    __device__ __forceinline__ float third() const { return m3; }
+    __device__ __forceinline__ int chunk1() const { return c1; }
+    __device__ __forceinline__ int chunk2() const { return c2; }
     float hb[8];             // minimum per block of 16 columns inside its 128-column chunk
     float d[16];             // minimum per column position inside its block
 
@@ -260,22 +285,22 @@ __device__ __forceinline__ float threshold(const Sweep &w, float m1, const Stage
 // above, the dot product is off by at most
 //   |z_lo.e - [64 z_lo][e/64]|        <= ||z_lo|| (cE + (1 + c)(cE + 64 sqrt(32) 2^-10)) + sqrt(32) 2^-16 (1 + c) E
 //   |z_hi.e_lo - [z_hi/64][64 e_lo]|  <= (cN + 0.354) L + ((1 + c) N + 0.354)(cL + sqrt(32) 2^-16)
-// with N = ||z||, L = ||e_lo||; twice that for the score, plus the accumulation as before (prepare.cu; five
+// with N = ||z||, L = ||e_lo||, z the row's operand; twice that for the score, plus the accumulation as before (prepare.cu; five
 // instructions of two kinds add up no worse than seven of one).  That comes to some 2^-13 |z||e|; the worst of 6.3
-// million chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.
-__device__ __forceinline__ float window8(float nz, float nl, float e, const StageConst &sb)
+// million chains was 3.1e-5 |z||e| on normal data and 1.13e-4 (2^-13.1) with x20 outlier channels.  (c_norm: what multiplies the norm).
+__device__ __forceinline__ float window8(float nz, float nl, float e, float c_norm, const StageConst &sb)
 {
     constexpr float c = 0.0595f;
     const float elo = fminf(sb.elo + sb.eerr, 4.8828125e-4f * e + 1.7e-7f);
     const float t1 = nl * (c * e + (1.0f + c) * (c * e + 0.354f)) + 8.7e-5f * 1.06f * e;
     const float t2 = (c * nz + 0.354f) * elo + ((1.0f + c) * nz + 0.354f) * (c * elo + 8.7e-5f);
-    return 2.125f * (2.0f * (t1 + t2) + 1.9073486328125e-6f * e * (e + 2.0f * nz) + 4.76837158203125e-7f * e);
+    return 2.125f * (2.0f * (t1 + t2) + 1.9073486328125e-6f * e * (c_norm * e + 2.0f * nz) + 4.76837158203125e-7f * e);
 }
 __device__ __forceinline__ float threshold8(const Sweep &w, float m1, const StageConst &sb)
 {
     const float nz = sqrtf(w.zz) * 1.0001f, nl = sqrtf(w.ll) * 1.0001f, d2 = fmaxf(m1 + w.zz, 0.0f);
-    const float full = window8(nz, nl, sb.emax, sb);
-    const float win = fminf(full, window8(nz, nl, fminf(sb.emax, (nz + sqrtf(d2 + full)) * 1.0001f), sb));
+    const float full = window8(nz, nl, sb.emax, 1.0f, sb);
+    const float win = fminf(full, window8(nz, nl, fminf(sb.emax, (nz + sqrtf(d2 + full)) * 1.0001f), 1.0f, sb));
     return m1 + win + 5.4e-6f * (d2 + win);
 }
 
@@ -310,6 +335,116 @@ __device__ __forceinline__ void rank_chunk(Sweep &w, float v, int c)
     w.m2 = fminf(w.m2, fmaxf(w.m1, v));
     w.c1 = first ? c : w.c1;
     w.m1 = fminf(w.m1, v);
+}
+
+// ---- Scores as 16-bit whole numbers, for the chain with 8-bit corrections.
+// The chain's last step, the norm's, also adds 1.5 * 2^22, so that the accumulator's unit is 1/2 and the low sixteen bits
+// of its word are the score in that unit: tcgen05.ld packs them in pairs (columns 2k and 2k + 1 in a register), and
+// one three-input minimum of pairs folds in four scores.  For that the scores of a row have to lie within [0, 2^15): the
+// row's operand and the constants that multiply the norm are scaled by c, and `off` lifts the lowest score
+// that the row can have, -c ||Z||^2, to 20 (a score is within c (-||Z||^2 ... emax^2 + 2 ||Z|| emax) of a codeword).
+constexpr float kPackedRange = 32000.0f;
+// What the last step loses: it cuts its addends to 1/4 and the sum to 1/2, towards zero.  With four addends that are no multiples of
+// it the errors of two scores differ by at most 1.5; measured on B200 against float64 sums of the very operands, 9.4
+// million chains with 8-bit corrections and without, they lay within -0.81 ... 0.25.
+constexpr float kPackedCut = 1.5f;
+
+__device__ __forceinline__ float squared_norm(const float (&z)[32])
+{
+    float q[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int i = 0; i < 32; ++i) q[i & 3] = fmaf(z[i], z[i], q[i & 3]);
+    return (q[0] + q[1]) + (q[2] + q[3]);
+}
+
+struct PackedSweep {
+    static constexpr uint32_t kPadded = 64800u;      // (a padded column scores 65504, no other one above 64100)
+    float zz, ll;            // squared norms of the scaled residual, and of the remainder of its operand
+    float c, off;            // row scale (a half) and lift (a half)
+    uint32_t v1, v2, v3;     // the three lowest chunk minima, each above its chunk's number
+    uint32_t hb[8];          // minima per block of 16 columns: of its even columns, and of its odd ones above
+    uint32_t d[8];           // minima of places 2k, and of 2k + 1 above
+
+    __device__ __forceinline__ void start(const float (&z)[32], const StageConst &prm)
+    {
+        zz = squared_norm(z) * prm.scale * prm.scale;
+        const float t = prm.emax + sqrtf(zz) * 1.0001f;
+        c = __half2float(__float2half_rd(fminf(kPackedRange / (t * t), 16.0f)));
+        off = __half2float(__float2half_ru(c * zz + 20.0f));
+    }
+    // (c c) (c 2048) (off 1) (c 0): what multiplies the norm's three halves, 3072, 1, and a padded column's entries
+    __device__ __forceinline__ uint4 row_constants() const
+    {
+        const uint32_t hc = __half_as_ushort(__float2half_rn(c)), ho = __half_as_ushort(__float2half_rn(off));
+        return make_uint4(hc | (hc << 16), hc | (0x6800u << 16), ho | (0x3C00u << 16), hc);
+    }
+    __device__ __forceinline__ void clear()
+    {
+        v1 = v2 = v3 = 0xFFFFFFFFu;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) d[q] = hb[q] = 0xFFFFFFFFu;
+    }
+    // The minima `low` of chunk k (even columns, odd ones) join the three lowest.
+    __device__ __forceinline__ void rank(uint32_t low, int k)
+    {
+        const uint32_t v = min((low << 16) | (uint32_t)k, (low & 0xFFFF0000u) | (uint32_t)k);
+        v3 = min(v3, max(v2, v));
+        v2 = min(v2, max(v1, v));
+        v1 = min(v1, v);
+    }
+    __device__ __forceinline__ uint32_t lowest() const { return v1 >> 16; }
+    __device__ __forceinline__ uint32_t second() const { return v2 >> 16; }
+    __device__ __forceinline__ uint32_t third() const { return v3 >> 16; }
+    __device__ __forceinline__ int chunk1() const { return (int)(v1 & 0xFFFFu); }
+    __device__ __forceinline__ int chunk2() const { return (int)(v2 & 0xFFFFu); }
+};
+
+__device__ __forceinline__ uint32_t threshold8(const PackedSweep &w, uint32_t m1, const StageConst &sb)
+{
+    const float rz = sqrtf(w.zz) * 1.0001f, nz = w.c * rz, nl = sqrtf(w.ll) * 1.0001f;
+    const float d2 = fmaxf(0.5f * (float)m1 - w.off + w.c * w.zz, 0.0f) + 2.0f;
+    const float full = window8(nz, nl, sb.emax, w.c, sb) + kPackedCut;
+    const float e = fminf(sb.emax, (rz + sqrtf((d2 + full) / w.c)) * 1.0001f);
+    const float win = fminf(full, window8(nz, nl, e, w.c, sb) + kPackedCut);
+    return min(m1 + (uint32_t)fminf(ceilf(2.0f * (win + 5.4e-6f * (d2 + win))), 65534.0f), 65534u);
+}
+
+// 64 columns of scores (half `h` of their chunk) in pairs, folded into the same partitions as in fold_block: 38 minimum
+// operations instead of 70.
+__device__ __forceinline__ void fold_packed(PackedSweep &w, const uint32_t (&u)[32], int h, uint32_t &chunk)
+{
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        w.d[k] = __vimin3_u16x2(w.d[k], u[k], u[k + 8]);
+        w.d[k] = __vimin3_u16x2(w.d[k], u[k + 16], u[k + 24]);
+    }
+    uint32_t m[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const uint32_t *v = u + 8 * b;
+        m[b] = __vimin3_u16x2(__vimin3_u16x2(v[0], v[1], v[2]), __vimin3_u16x2(v[3], v[4], v[5]), __vminu2(v[6], v[7]));
+        w.hb[4 * h + b] = __vminu2(w.hb[4 * h + b], m[b]);
+    }
+    chunk = __vimin3_u16x2(__vimin3_u16x2(chunk, m[0], m[1]), m[2], m[3]);
+}
+
+// Members whose minimum is at most `limit` (below 65535).
+__device__ __forceinline__ Listed listed(const PackedSweep &w, uint32_t limit)
+{
+    const uint32_t above = (limit + 1u) * 0x10001u;
+    // 1 in the half word of a member that is listed
+    auto flags = [&](uint32_t v) { return __vminu2(above - __vminu2(v, above), 0x10001u); };
+    uint32_t q = 0u, b = 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q += flags(w.d[k]) << k;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        b += flags(__vminu2(__byte_perm(w.hb[k], w.hb[k + 4], 0x5410), __byte_perm(w.hb[k], w.hb[k + 4], 0x7632))) << k;
+    // even places in the low half word, odd ones in the high one: interleaved
+    q = (q | (q << 4)) & 0x0F0F0F0Fu;
+    q = (q | (q << 2)) & 0x33333333u;
+    q = (q | (q << 1)) & 0x55555555u;
+    return {(q & 0xFFFFu) | (q >> 15), (b & 0xFu) | (b >> 12)};
 }
 
 // 32-byte read-only global load: a codeword row costs four of these, and for
@@ -575,17 +710,16 @@ __device__ __forceinline__ float split_operand(const float (&z)[32], float scale
 }
 
 // The same for the chain with 8-bit corrections: 16 words of head, 8 of 64 times the remainder, 8 of a 64th of the
-// head; zz, ll: squared norms of the scaled residual and of the remainder.
+// head; returns the squared norm of the remainder.
 __device__ __forceinline__ uint32_t e4m3x2(__half2 v)
 {
     uint16_t d;
     asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(d) : "r"(*reinterpret_cast<const uint32_t *>(&v)));
     return d;
 }
-__device__ __forceinline__ void split_operand8(const float (&z)[32], float scale, uint32_t (&ab)[32], float &zz,
-                                                float &ll)
+__device__ __forceinline__ float split_operand8(const float (&z)[32], float scale, uint32_t (&ab)[32])
 {
-    zz = ll = 0.0f;
+    float ll = 0.0f;
     const __half2 up = __floats2half2_rn(64.0f, 64.0f), down = __floats2half2_rn(0.015625f, 0.015625f);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -593,7 +727,6 @@ __device__ __forceinline__ void split_operand8(const float (&z)[32], float scale
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float z0 = z[4 * i + 2 * h] * scale, z1 = z[4 * i + 2 * h + 1] * scale;
-            zz = fmaf(z0, z0, zz); zz = fmaf(z1, z1, zz);
             const __half2 h2 = __floats2half2_rn(z0, z1);
             const float2 hf = __half22float2(h2);
             const float l0 = z0 - hf.x, l1 = z1 - hf.y;
@@ -605,6 +738,7 @@ __device__ __forceinline__ void split_operand8(const float (&z)[32], float scale
         ab[16 + i] = __byte_perm(lo8[0], lo8[1], 0x5410);
         ab[24 + i] = __byte_perm(hi8[0], hi8[1], 0x5410);
     }
+    return ll;
 }
 
 // Codes of the warp's 32 rows (first vector v_first), from codes_s[row of the warp][16], to global memory in

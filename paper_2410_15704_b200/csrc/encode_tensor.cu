@@ -12,8 +12,11 @@
 //     in TMEM.
 //     EIGHT: the two small products of the split (remainder x head) in e4m3, as two K=32 steps beside
 //     three K=16 ones: 327 cycles per chain instead of 455, at an error of up to 2^-13 |z||e| in the score that the
-//     window allows for (window8).  For contiguous groups, eight or more chunks and even codebooks (eight_possible
+//     window allows for (window8).  For contiguous groups, eight or more chunks and even codebooks (eight_from
 //     says why).
+//     PACKED: these chains with scores that are read and folded as 16-bit whole numbers, two to a register (PackedSweep):
+//     84 minimum operations per chunk and row instead of 140, at an error of 1.5 units of 2^-15 of the range that a
+//     row's scores can have.  262144 values, 2048 codes: 2090 -> 1965 us in a burst.
 //   - The B operand (128 codewords per slot) streams from the prepared block
 //     through a ring of shared-memory slots filled by cp.async.bulk; every
 //     slot serves all three tiles.
@@ -43,10 +46,12 @@
 //     two chains of that sweep (count x codeword is added back by the caller's finishing kernel); the
 //     last stage's input is added by the epilogue warps.
 // TMEM columns of tile t: scores [160 t, 160 t + 128), A operand
-// [160 t + 128, 160 t + 160) (16 columns of head, 16 of remainder); the constant operand [480, 488).
+// [160 t + 128, 160 t + 160) (16 columns of head, 16 of remainder); the constant operand [480, 488) (PACKED: of tile t, [480 + 8 t, 488 + 8 t)).
 // Every wait is bounded; a wait that gives up sets status->wait_timeouts, and
 // the kernel waits (bounded as well) for its copies and chains in flight and returns.
 #include "encode_mma.cuh"
+
+#include <type_traits>
 
 namespace rvq {
 
@@ -76,7 +81,9 @@ constexpr int kDeferMinSlots = 6;                       // chunks a stage needs 
 // It also needs rounds of three tiles, whose chains queue up at the tensor core: with fewer tiles per SM a chain's
 // length is not what a stage waits for, and the added work at the stage end is (values, us, half precision / 8 bits,
 // tiles per SM at most: 1024 codes 64 / 75 at two, 122 / 137 at four, 145 / 138 at five; 2048 codes 147 / 156 at
-// three, 207 / 191 at four).
+// three, 207 / 191 at four).  With packed scores earlier: 1024 codes 73 / 73 at two, 93 / 90 at three, 129 / 129 at four,
+// 145 / 140 at five, 495 / 465 at twenty; 2048 codes 72 / 78 at one, 112 / 107 at two, 143 / 135 at three, 233 / 209 at
+// five; 768 codes 110 / 113 at four, 408 / 406 at twenty; 512 codes 51 / 57 at two, 327 / 346 at twenty.
 // And it needs rows whose window stays narrow.  With outlier channels 2.2-2.9 % of the rows and stages have more than
 // one candidate instead of 0.5 %, and the more the farther the outliers stand out.  The data are not known on the
 // host; the codebooks, which follow them, are looked at when they are prepared (PreparedHeader::even: outliers, and
@@ -92,12 +99,16 @@ constexpr int kDeferMinSlots = 6;                       // chunks a stage needs 
 // 3427, 9.9 %; 1000 on four channels: 1872 -> 64295, 45 %; strided groups 20: 1892 -> 1826, 60: 1881 -> 2105, 1000:
 // 1885 -> 44969; 1024 codes with statistics, 100 tiles per SM, 1000: 2768 -> 51737 and 2753 -> 27474).
 constexpr int kEightMinSlots = 8;
-inline bool eight_possible(const Shape &s, int64_t tiles, int sms)
+// The smallest PreparedHeader::even with which a call takes them (2: packed scores); 3: none.
+inline uint32_t eight_from(const Shape &s, int64_t tiles, int sms)
 {
     const int slots = slots_per_stage(s.K);
-    return slots >= kEightMinSlots && s.layout == RVQ_GROUP_CONTIGUOUS && !s.raw &&
-           tiles > (int64_t)sms * (slots >= 16 ? 3 : 4);
+    if (slots < kEightMinSlots || s.layout != RVQ_GROUP_CONTIGUOUS || s.raw) return 3u;
+    return tiles > (int64_t)sms * (slots >= 16 ? 3 : 4) ? 1u : tiles > (int64_t)sms * (slots >= 16 ? 1 : 2) ? 2u : 3u;
 }
+
+// Seven steps in half precision; five, with the small products in 8 bits; five, and scores as 16-bit whole numbers.
+enum Chain { kHalf, kEight, kPacked };
 
 // barrier slots
 constexpr int kBarFull = 0, kBarEmpty = kRing, kBarAReady = 2 * kRing, kBarAccFull = 2 * kRing + kTiles,
@@ -118,6 +129,7 @@ struct Params {
     float *energy;      // optional [R]: sum over the rows of the squared norm of what each stage leaves
     uint32_t wait_limit;   // polls after which a wait gives up (kWaitLimit; smaller only in the timeout self-test)
     int drop_last_chain;   // timeout self-test: 1 = tile 0's issuer leaves out the CTA's very last chain; else 0
+    uint32_t eight_from;   // encode_tensor_either_kernel: eight_from
     int defer_stats;       // 1 = the statistics of every stage but the last are added by the MMA issuer warps (below)
 };
 
@@ -139,9 +151,10 @@ struct Work {
 // take part in the way in.
 // (4096 float32 vectors at 256 codes 27.8 -> 24.9 us, at 384 34.1 -> 30.5.  The split encoder with a CTA per tile
 // takes 30.8 and 35.7: with up to three chunks the parts' join costs more than the folds that it puts side by side.)
-template <bool EIGHT, bool LONE>
+template <int CHAIN, bool LONE>
 __device__ __forceinline__ void encode_tensor_body(const Params &p)
 {
+    constexpr bool EIGHT = CHAIN != kHalf, PACKED = CHAIN == kPacked;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBars);
     uint32_t *tmem_word = reinterpret_cast<uint32_t *>(smem + kOffBars + kNumBars * 8);
@@ -196,7 +209,8 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
     tc_fence_after();
     const uint32_t tmem = *tmem_word;
     // the constant A operand, shared by all tiles (the issuers hear of it with their first A operand)
-    if (warp < 4) tmem_ones(tmem + ((uint32_t)(warp * 32) << 16) + kOnesCol);
+    // (PACKED: a tile's own, written again in every stage)
+    if (warp < (PACKED ? 4 * kTiles : 4)) tmem_ones(tmem + ((uint32_t)((warp & 3) * 32) << 16) + kOnesCol + 8 * (warp >> 2));
     if (LONE) {
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
@@ -330,7 +344,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     // epilogue's wait for it runs out with no copy or MMA of this CTA still in flight)
                     if (p.drop_last_chain && t == 0 && q == total - 1) break;
                     if (elect_one()) {
-                        if (EIGHT) issue_chain8(acc, a0, bd, tmem + kOnesCol);
+                        if (EIGHT) issue_chain8(acc, a0, bd, tmem + kOnesCol + (PACKED ? 8 * t : 0));
                         else issue_chain(acc, a0, bd, tmem + kOnesCol);
                         mma_commit(bar_acc);
                         mma_commit(BAR(kBarEmpty + slot));
@@ -413,9 +427,17 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 const float *cbr = p.cb + (size_t)r * s.K * 32;
                 // scaled half-precision copy of the residual -> A operand row; error window of this row
                 uint32_t ab[32];
-                Sweep w;
-                if (EIGHT) split_operand8(z, prm.scale, ab, w.zz, w.ll);
-                else w.zz = split_operand(z, prm.scale, ab);
+                std::conditional_t<PACKED, PackedSweep, Sweep> w;
+                if constexpr (PACKED) {
+                    w.start(z, prm);
+                    w.ll = split_operand8(z, prm.scale * w.c, ab);
+                    tmem_st4(tmem + ((uint32_t)(q4 * 32) << 16) + kOnesCol + 8 * tile, w.row_constants());
+                } else if (EIGHT) {
+                    w.zz = squared_norm(z) * prm.scale * prm.scale;
+                    w.ll = split_operand8(z, prm.scale, ab);
+                } else {
+                    w.zz = split_operand(z, prm.scale, ab);
+                }
                 tmem_st32(taddr + 128, ab);
                 tc_fence_before();
                 __syncwarp();
@@ -424,12 +446,13 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 #pragma unroll
                 for (int i = 0; i < 32; ++i) z_park[i * kPitch] = z[i];
                 // 2 * bound, with slack for this arithmetic
-                if (!EIGHT) w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
+                if constexpr (!EIGHT) w.win = 2.125f * (prm.a * sqrtf(w.zz) * 1.0001f + prm.b);
                 w.clear();
                 // (no entry reaches 60000 in half precision; none is above 2^14, where 64 times its remainder leaves
                 // the 8-bit range)
-                const bool force_scan = EIGHT ? !(w.zz < 2.68e8f) || !(prm.a < INFINITY)
-                                              : !(w.zz < 3.6e9f) || !(w.win < INFINITY);
+                bool force_scan;
+                if constexpr (EIGHT) force_scan = !(w.zz < 2.68e8f) || !(prm.a < INFINITY);
+                else force_scan = !(w.zz < 3.6e9f) || !(w.win < INFINITY);
 
 #pragma unroll 1
                 for (int c = 0; c < S && ok; ++c) {
@@ -447,30 +470,44 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                     // the MMA issuer as soon as they have landed: the reduction below runs while the
                     // next chain computes.
                     const uint32_t acc = LONE ? taddr + (uint32_t)(c * kTileCols) : taddr;
-                    uint32_t ua[32], ub[32], uc[32], ud[32];
-                    tmem_ld32_issue(acc, ua);
-                    tmem_ld32_issue(acc + 32, ub);
-                    tmem_ld32_issue(acc + 64, uc);
-                    tmem_ld32_issue(acc + 96, ud);
-                    tmem_ld_wait4(ua, ub, uc, ud);
-                    tc_fence_before();
-                    __syncwarp();
-                    // the accumulator may be overwritten
-                    if (!LONE && lane == 0) mbar_arrive(BAR(kBarAccFree + tile));
-                    float lowest;
-                    fold_block(w, ua, 0, lowest);
-                    fold_block(w, ub, 1, lowest);
-                    fold_block(w, uc, 2, lowest);
-                    fold_block(w, ud, 3, lowest);
-                    rank_chunk(w, lowest, c);
+                    if constexpr (PACKED) {
+                        uint32_t ua[32], ub[32];
+                        tmem_ld64_packed_issue(acc, ua);
+                        tmem_ld64_packed_issue(acc + 64, ub);
+                        tmem_ld_wait2(ua, ub);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(BAR(kBarAccFree + tile));      // the accumulator may be overwritten
+                        uint32_t lowest = 0xFFFFFFFFu;
+                        fold_packed(w, ua, 0, lowest);
+                        fold_packed(w, ub, 1, lowest);
+                        w.rank(lowest, c);
+                    } else {
+                        uint32_t ua[32], ub[32], uc[32], ud[32];
+                        tmem_ld32_issue(acc, ua);
+                        tmem_ld32_issue(acc + 32, ub);
+                        tmem_ld32_issue(acc + 64, uc);
+                        tmem_ld32_issue(acc + 96, ud);
+                        tmem_ld_wait4(ua, ub, uc, ud);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (!LONE && lane == 0) mbar_arrive(BAR(kBarAccFree + tile));
+                        float lowest;
+                        fold_block(w, ua, 0, lowest);
+                        fold_block(w, ub, 1, lowest);
+                        fold_block(w, uc, 2, lowest);
+                        fold_block(w, ud, 3, lowest);
+                        rank_chunk(w, lowest, c);
+                    }
                 }
                 if (!ok) break;
                 // The column of the lowest score is the choice of nearly every row: its codeword is asked for before
                 // it is known to be (the trip to L2 takes as long as the rest of the stage end: asked for after it,
                 // 225 -> 217 us on 32768 keys, 30.7 -> 28.2 on 4096 float32 vectors with 256 codes; a prefetch of the
                 // running winner into L1 before the last chunk, on top of this, costs 1.2 %).
-                const float m1 = w.m1;
-                const int jm = min(max(w.c1 * 128 + listed(w, m1).column(), 0), s.K - 1);
+                const auto m1 = w.lowest();
+                const int c1 = w.chunk1(), c2 = w.chunk2();
+                const int jm = min(max(c1 * 128 + listed(w, m1).column(), 0), s.K - 1);
                 float ev[32];
                 load_codeword(cbr + (size_t)jm * 32, ev);
 
@@ -478,19 +515,22 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
                 // chunk, in a listed block of the chunk, at a listed place.  When each of
                 // the three lists has one entry (almost always) that column is the choice: every other
                 // column is farther than the approximation and float32 evaluation errors can bridge.
-                const float lim = EIGHT ? threshold8(w, m1, sc[r]) : threshold(w, m1, sc[r]);
+                const auto lim = [&] {
+                    if constexpr (EIGHT) return threshold8(w, m1, sc[r]);
+                    else return threshold(w, m1, sc[r]);
+                }();
                 const Listed in = listed(w, lim);
-                const int j1 = w.c1 * 128 + in.column();
-                // (a padded column scores 60000: if nothing real scored less, scan everything)
-                const bool scan_all = force_scan || !(m1 < 59000.0f);
+                const int j1 = c1 * 128 + in.column();
+                // (if nothing real scored less than a padded column, scan everything)
+                const bool scan_all = force_scan || !(m1 < w.kPadded);
                 // with columns inside the window (three or more: taken as all)
-                const int chunks = w.m3 <= lim ? S : w.m2 <= lim ? 2 : 1;
+                const int chunks = w.third() <= lim ? S : w.second() <= lim ? 2 : 1;
                 const bool unique = chunks == 1 && in.single() && (uint32_t)j1 < (uint32_t)s.K;
                 const bool flagged = !deg && (scan_all || !unique);
                 int bj = (uint32_t)j1 < (uint32_t)s.K ? j1 : 0;
                 // Rows with more than one candidate: their candidate columns are compared
                 // exactly in float32, direct form: smallest distance, lowest index on ties.  Four rows at a time,
-                // eight lanes to a row, more with fewer rows; rows whose scores say nothing one by one, all columns, by the whole warp.
+                // eight lanes to a row, or fewer with more; rows whose scores say nothing one by one, all columns, by the whole warp.
                 // (One row at a time, and all columns also where a third chunk came inside the window: 32768 keys 219
                 // -> 215 us, 262144 values 2515 -> 2495.  All lanes for a single row, half for two, and no integer
                 // divisions: 65536 values with one group of four 10 times smaller 609 -> 570, in a burst.)
@@ -520,7 +560,7 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 #pragma unroll
                     for (int i = 0; i < 32; ++i) zs[i] = z_park[i * kPitch + (src - lane)];
                     compare_listed(zs, cbr, s.K, lane & ((1 << share) - 1), 1 << share, __shfl_sync(0xFFFFFFFFu, in.word(), src),
-                                   __shfl_sync(0xFFFFFFFFu, w.c1, src), __shfl_sync(0xFFFFFFFFu, w.c2, src),
+                                   __shfl_sync(0xFFFFFFFFu, c1, src), __shfl_sync(0xFFFFFFFFu, c2, src),
                                    __shfl_sync(0xFFFFFFFFu, chunks, src), bv, bi);
                     best_of(1 << share, bv, bi);
 #pragma unroll
@@ -590,18 +630,20 @@ __device__ __forceinline__ void encode_tensor_body(const Params &p)
 
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_kernel(const __grid_constant__ Params p)
 {
-    encode_tensor_body<false, false>(p);
+    encode_tensor_body<kHalf, false>(p);
 }
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_lone_kernel(const __grid_constant__ Params p)
 {
-    encode_tensor_body<false, true>(p);
+    encode_tensor_body<kHalf, true>(p);
 }
 
 // Where the 8-bit corrections are possible: by the codebooks.
 __global__ void __launch_bounds__(kThreads, 1) encode_tensor_either_kernel(const __grid_constant__ Params p)
 {
-    if (reinterpret_cast<const PreparedHeader *>(p.prepared)->even) encode_tensor_body<true, false>(p);
-    else encode_tensor_body<false, false>(p);
+    const uint32_t even = reinterpret_cast<const PreparedHeader *>(p.prepared)->even;
+    if (even < p.eight_from) encode_tensor_body<kHalf, false>(p);
+    else if (even == 1u) encode_tensor_body<kEight, false>(p);
+    else encode_tensor_body<kPacked, false>(p);
 }
 
 }  // namespace
@@ -630,11 +672,12 @@ int launch_encode_tensor(const Shape &s, const void *x, int64_t n, int64_t strid
     const int sms = sm_count();
     if (sms <= 0) return RVQ_ERR_DEVICE;
     const bool lone = tiles <= sms && slots_per_stage(s.K) <= kTiles && !s.raw && !stat_sum;
+    const uint32_t from = eight_from(s, tiles, sms);
     auto kernel = lone ? encode_tensor_lone_kernel
-                : eight_possible(s, tiles, sms) ? encode_tensor_either_kernel : encode_tensor_kernel;
+                : from < 3u ? encode_tensor_either_kernel : encode_tensor_kernel;
     if (!allow_shared_memory(reinterpret_cast<const void *>(kernel), kSmemBytes)) return RVQ_ERR_LAUNCH;
     Params p{s, x, n, stride, cb, reinterpret_cast<const uint8_t *>(prepared), codes, std16, st, (int)tiles,
-             stat_cnt, stat_sum, energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain,
+             stat_cnt, stat_sum, energy, wait_limit ? wait_limit : kWaitLimit, drop_last_chain, from,
              stat_sum != nullptr && encode_tensor_deferred_stages(s) > 0 ? 1 : 0};
     // (fewer tiles than three per SM: one or two in each, not three in some)
     const int grid = (int)(tiles < sms ? tiles : sms);

@@ -18,11 +18,13 @@
 //   - the B operand image of tcgen05.mma: for every slot of 128 codewords thirteen
 //     "cells" (16 bytes per codeword per cell, K-major, no swizzle): cells 0-3
 //     hold -2 e_lo (8 halves each), cell 4 the scaled squared norm split into
-//     three halves (hi, lo, lo2) then zeros, cells 5-8 hold -2 e_hi, cells 9-10
+//     three halves (hi, lo, lo2) then what packed scores need (below), cells 5-8 hold -2 e_hi, cells 9-10
 //     -2 e / 64 and cells 11-12 -2 * 64 e_lo (16 e4m3 each).  The A operand
 //     carries Z_hi and Z_lo, or Z_hi and the 8-bit 64 Z_lo and Z_hi / 64, and (1 1
 //     1 0 ... 0) for the norm, whose K = 16 step takes cells 4 and 5 (A is zero
-//     where cell 5 stands): seven or five steps make the accumulator the score;
+//     where cell 5 stands): seven or five steps make the accumulator the score.  Packed scores (encode_mma.cuh) take a
+//     row with its constants instead, (c c c 2048 off 1 c 0 ... 0), whose last four meet (3072 1 0 0), or for a padding
+//     codeword (3072 0 32752 -60000): 1.5 * 2^22, the row's lift, and padding above everything at any c;
 //   - the float32 codewords again, in blocks of 128 (prepared.cuh), for the encoder of a few vectors;
 //   - two numbers (a, b) such that |score error| <= a * ||Z|| + b, from the
 //     actual rounding errors of this codebook (see prepare_finish_kernel).
@@ -281,11 +283,14 @@ prepare_image_kernel(Shape s, const float *cb, const StageParams *sp,
         const __half n_lo = __double2half(r1);
         const double r2 = r1 - (double)__half2float(n_lo);
         cell[4][0] = n_hi; cell[4][1] = n_lo; cell[4][2] = __double2half(r2);
+        cell[4][3] = __float2half_rn(3072.0f); cell[4][4] = __float2half_rn(1.0f);
         // round the maxima up so that the bound stays a bound in float32
         emax = __double2float_ru(sqrt(n2)); eerr = __double2float_ru(sqrt(d2));
         elomax = __double2float_ru(sqrt(l2));
     } else {
-        cell[4][0] = __float2half_rn(60000.0f);           // padding never wins
+        // padding never wins
+        cell[4][0] = __float2half_rn(60000.0f);
+        cell[4][3] = __float2half_rn(3072.0f); cell[4][5] = __float2half_rn(32752.0f); cell[4][6] = __float2half_rn(-60000.0f);
     }
 #pragma unroll
     for (int c = 0; c < 13; ++c)
@@ -339,7 +344,10 @@ prepare_finish_kernel(Shape s, StageParams *sp, const StageMaxima *mx, PreparedH
         }
     }
     inverse = __reduce_add_sync(0xFFFFFFFFu, inverse);
-    if (r == 0 && (float)inverse > kMostInverse * 128.0f * (float)s.K * (float)s.R) hdr->even = 0u;
+    if (r == 0 && hdr->even != 0u) {
+        const float mean = (float)inverse / (128.0f * (float)s.K * (float)s.R);
+        hdr->even = mean > kMostInverse ? 0u : mean > kPackedInverse ? 1u : 2u;
+    }
 }
 
 int launch_prepare(const Shape &s, const float *cb, void *prepared, cudaStream_t stream, bool chained)

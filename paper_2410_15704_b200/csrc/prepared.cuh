@@ -24,7 +24,7 @@ constexpr size_t kPreparedImageOffset = 768 + 16 * 16 * 24;   // operand image, 
 struct PreparedHeader {
     uint32_t magic, R, K, gd, slots;
     uint32_t decode_offset;   // byte offset of the decoder section, 0 if absent
-    uint32_t even;            // 1: the codebooks suit the 8-bit corrections (kEvenKurtosis, kMostInverse)
+    uint32_t even;            // 1: the codebooks suit the 8-bit corrections (kEvenKurtosis, kMostInverse); 2: packed scores as well (kPackedInverse)
 };
 // A stage's codewords count as even when the fourth moment of their entries is at most this many times the square of the
 // second (3 for a normal distribution); the block does when at least half of its stages do and its codewords are not
@@ -42,7 +42,11 @@ constexpr float kEvenKurtosis = 6.0f;
 //   in two, x60 0.09: 1821 -> 1684, x200 with 1024 codes 0.13: 992 -> 1044;
 //   in four, x20 0.08: 1841 -> 1691 (1024 codes 0.05: 1012 -> 1027), x60 0.15: 1819 -> 1874, x1000 2.2: 1818 -> 36012.
 // Back to back, under the power cap, five steps take 3-9 % less than that beside seven.
-constexpr float kMostInverse = 0.1f, kInverseFree = 0.0625f, kInverseCap = 16.0f;
+// Packed scores have a unit that does not shrink with the row either, 2^-16 of the range of a row against the largest
+// codeword, and twice to four times the window.  65536 vectors, 2048 codes, us as they are / packed and share of the rows and stages
+// with several candidates, one of four groups smaller than the others: alike 543 / 485, 1.0 %; 3 times 587 / 526, 1.7 %; 5 times
+// (mean 0.009) 593 / 534, 2.2 %; 10 times (0.04) 570 / 691, 4.0 %.
+constexpr float kMostInverse = 0.1f, kPackedInverse = 0.015f, kInverseFree = 0.0625f, kInverseCap = 16.0f;
 
 // Decoder section (group_dim 32, R <= 8, K <= kDecodeMaxK): per stage an affine
 // map value = lo_r + q * scale_r * base with q a 16-bit level, scale_r an integer in

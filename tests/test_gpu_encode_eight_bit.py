@@ -157,3 +157,29 @@ def test_long_calls_with_outliers(tiles, K, R, layout, statistics, factor):
     torch.cuda.synchronize()
     assert torch.equal(b.codes, exact) and st["wait_timeouts"] == 0
     assert st["rescored_rows"] + st["exhaustive_rows"] < 0.005 * n * 4 * R
+
+
+@pytest.mark.parametrize("n,K,R", [(4737, 2048, 2), (4737, 1921, 1), (9473, 1024, 2), (9473, 1030, 1), (9473, 2047, 2), (14209, 2048, 8)])
+def test_packed_scores(n, K, R):
+    """Codewords of like norms: scores in 16 bits, from two tiles per SM on (three with up to 1920 codes), also beside padding codewords.
+    One codeword in four has a copy at 0 ... 1e-2 of its norm, which the window (some 2e-2 of a squared distance) cannot tell from
+    it, and the rows' norms reach from 1e-3 to 2e4 times the codewords'."""
+    g = np.random.default_rng(n + K)
+    x = g.normal(size=(n, 128)).astype(np.float32)
+    cb = np.stack([g.normal(scale=0.8 ** r, size=(K, 32)) for r in range(R)]).astype(np.float32)
+    twin = g.permutation(K)[:2 * (K // 8)].reshape(2, -1)
+    off = g.normal(size=(R, twin.shape[1], 32)) * np.exp(g.uniform(np.log(1e-6), np.log(2e-3), size=(1, twin.shape[1], 1)))
+    cb[:, twin[1]] = cb[:, twin[0]] + (off * (g.random((1, twin.shape[1], 1)) < 0.9) * 0.8 ** np.arange(R)[:, None, None]).astype(np.float32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert n * 4 > sms * 128 * (1 if K > 1920 else 2)
+    _, b, _, exact, st = encode_both(x, cb, R, K)
+    assert torch.equal(b.codes, exact) and st["rescored_rows"] > 0.1 * n * 4 * R
+    # (the first group of every third row carries next to all of its energy, or next to none)
+    x[::3, :32] *= np.exp(g.uniform(np.log(1e-3), np.log(1e3), size=(len(x[::3]), 1))).astype(np.float32)
+    for scale in (1.0, 1e-3, 20.0, 2e-4):
+        _, b, _, exact, _ = encode_both(x, (cb * scale).astype(np.float32), R, K)
+        assert torch.equal(b.codes, exact)
+    # (exact ties: the lowest index)
+    cb[:, twin[1]] = cb[:, twin[0]]
+    _, b, _, exact, _ = encode_both(x, cb, R, K)
+    assert torch.equal(b.codes, exact)
