@@ -138,19 +138,25 @@ encode_small_kernel(const SmallParams p)
     const uint32_t to_arrived = map_to(arrived0, (uint32_t)min(lane, ctas - 1));
     constexpr uint32_t kRowKeys = kSmallMaxCluster * 8 * 8, kAllKeys = kSmallRows * kRowKeys;      // bytes
     bool ok = true;
-    int buffer = 0;
-    uint32_t full_par = 0;
+    int buffer = 0, next_buffer = 0;
+    uint32_t full_par = 0;                                        // of next_buffer
     int r = 0;
+    // this thread's codeword of the next stage
+    float4 e[8];
+    auto take_codeword = [&] {
+        const bool there = mbar_wait(smem_u32(&w.full[next_buffer]), full_par, &w.abort_flag);
+        const float4 *mine4 = reinterpret_cast<const float4 *>(table + (size_t)next_buffer * kStageBytes) + (c >> 7) * 1024 + (c & 127);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) e[q] = mine4[q * 128];
+        if (++next_buffer == kBuffers) { next_buffer = 0; full_par ^= 1u; }
+        return there;
+    };
+    ok = take_codeword();
 #pragma unroll 1
     for (; r < R; ++r) {
         const uint32_t par = (uint32_t)r & 1u;
         if (tid == 0) mbar_expect_tx(arrived0 + 8u * par, (uint32_t)(p.rows * slots * 8));
-        ok = mbar_wait(smem_u32(&w.full[buffer]), full_par, &w.abort_flag);
         const uint8_t *stage = table + (size_t)buffer * kStageBytes;
-        const float4 *mine4 = reinterpret_cast<const float4 *>(stage) + (c >> 7) * 1024 + (c & 127);
-        float4 e[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) e[q] = mine4[q * 128];
 #pragma unroll 1
         for (int row = first; row < p.rows; row += next) {
             float d[kSmallAtOnce] = {};
@@ -181,6 +187,8 @@ encode_small_kernel(const SmallParams p)
                                  ::"r"(to_keys + par * kAllKeys + (uint32_t)(row + k) * kRowKeys), "l"(key), "r"(to_arrived + 8u * par) : "memory");
             }
         }
+        // (while the minima travel: read at the stage's start, 16 warps' codewords were 512 cycles of its distances)
+        if (r + 1 < R) ok = take_codeword() && ok;
         ok = mbar_wait(arrived0 + 8u * par, (uint32_t)(r >> 1) & 1u, &w.abort_flag) && ok;
         const bool subtract = r + 1 < R || p.energy != nullptr;
         float e2 = 0.0f;
@@ -214,7 +222,7 @@ encode_small_kernel(const SmallParams p)
         // Every CTA has read this CTA's codewords of stage r - 1 (it could not have sent its minima of stage r
         // before): their place is free.
         if (PER == 2 && tid == 0 && r >= 1 && r - 1 + kBuffers < R) copy_stage(r - 1 + kBuffers, r - 1);
-        if (++buffer == kBuffers) { buffer = 0; full_par ^= 1u; }
+        if (++buffer == kBuffers) buffer = 0;
     }
     if (!ok && tid == 0) {
         // (the stages from here on are still coming in)
