@@ -7,8 +7,9 @@
 // into registers and computes its exact distances to the cluster's rows (direct form, the scalar
 // kernel's operation order, so the codes are the same).  The minima of all warps meet in every CTA's
 // shared memory (st.async, counted by an mbarrier), every CTA picks the winner for itself and reads its
-// codeword from the CTA that holds it.
-// What bounds it: the chain of the stages.  Measured for 4 rows at 1024 codes: distances and
+// codeword from the CTA that holds it.  For a token or two a cluster takes one or two groups of a vector (small_share_plan).
+// What bounds it: the chain of the stages.  Measured for 4 rows at 1024 codes, when a stage began with reading the
+// codewords and not while the minima of the one before travel: distances and
 // minima 1050 cycles of a stage, the exchange 260, winner and residual 500, the barrier and the next
 // stage's table 300.
 #include "encode_mma.cuh"
@@ -17,11 +18,11 @@ namespace rvq {
 
 namespace {
 
-constexpr int kSmallAtOnce = 2;                   // rows that a thread takes at a time
 constexpr int kSmallThreads = 512;
 constexpr int kSmallRows = 32;                    // group rows per cluster at most
 constexpr int kSmallMaxCluster = 8;
-constexpr int kSmallTableBytes = 10 * kFloatBlockBytes;   // eight stages of one block, or five of two
+// stages in shared memory at a time, by the blocks of 128 codewords that a CTA has of each
+template <int PER> constexpr int kSmallBuffers = PER == 1 ? kFloatMaxStages : PER == 2 ? 5 : 3;
 
 struct SmallParams {
     Shape s;
@@ -33,37 +34,44 @@ struct SmallParams {
     rvq_status *st;
     float *energy;
     int vectors;        // head vectors per cluster
-    int rows;           // their group rows
+    int rows;           // group rows per cluster: theirs, or a share of the only one's
+    int shares;         // clusters per head vector, each with `rows` of its groups (1: whole vectors)
     int blocks_per_stage;
 };
 
+// ROWS: group rows of a cluster at most.
+template <int ROWS>
 struct SmallWork {
     // (distance bits, code) of the best of every warp's 32 codewords, from every CTA of the cluster
-    unsigned long long keys[2][kSmallRows][kSmallMaxCluster * 8];
-    float z[kSmallRows + kSmallAtOnce][32];
+    unsigned long long keys[2][ROWS][kSmallMaxCluster * 8];
+    float z[ROWS + 1][32];
     float xs[kSmallRows * 32];
     float dev[kSmallRows];
-    uint16_t codes[kSmallRows][kFloatMaxStages];
+    uint16_t codes[ROWS][kFloatMaxStages];
     uint64_t full[kFloatMaxStages], arrived[2];
     volatile uint32_t abort_flag;
 };
-constexpr int kSmallSharedBytes = kSmallTableBytes + (int)sizeof(SmallWork);
+template <int PER> constexpr int kSmallMostRows = PER == 4 ? 2 : kSmallRows;
+template <int PER> constexpr int kSmallSharedBytes = kSmallBuffers<PER> * PER * kFloatBlockBytes + (int)sizeof(SmallWork<kSmallMostRows<PER>>);
 
-// blockDim.x = PER * 128 threads for every kSmallAtOnce rows of the cluster, up to kSmallThreads.
-template <int PER>                                                // blocks of 128 codewords per CTA and stage
+// PER: blocks of 128 codewords per CTA and stage.  AT_ONCE: rows that a thread takes at a time.
+// blockDim.x = PER * 128 threads for every AT_ONCE rows of the cluster, up to kSmallThreads.
+template <int PER, int AT_ONCE>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 encode_small_kernel(const SmallParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t *table = smem;                                        // [buffers][PER blocks]
-    SmallWork &w = *reinterpret_cast<SmallWork *>(smem + kSmallTableBytes);
-    constexpr int kBuffers = PER == 1 ? kFloatMaxStages : 5;
+    constexpr int kBuffers = kSmallBuffers<PER>, kRows = kSmallMostRows<PER>;
     constexpr uint32_t kStageBytes = PER * kFloatBlockBytes;
+    SmallWork<kRows> &w = *reinterpret_cast<SmallWork<kRows> *>(smem + kBuffers * kStageBytes);
     const Shape &s = p.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x;
     const int G = s.G, R = s.R, dim = s.dim;
     const int rank = (int)cluster_rank(), ctas = (int)gridDim.y;  // CTA of the cluster, CTAs of a cluster
-    const int64_t v0 = (int64_t)blockIdx.x * p.vectors;           // first head vector of this cluster
+    // first head vector of this cluster, and the first of its groups
+    const int64_t v0 = p.shares > 1 ? (int64_t)blockIdx.x / p.shares : (int64_t)blockIdx.x * p.vectors;
+    const int g0 = p.shares > 1 ? (int)blockIdx.x % p.shares * p.rows : 0;
     const int mine = min(PER, p.blocks_per_stage - rank * PER);   // (the last CTA of an odd number of blocks: one of two)
     const uint8_t *src = p.blocks + (size_t)rank * kStageBytes;
     const size_t src_stage = (size_t)p.blocks_per_stage * kFloatBlockBytes;
@@ -85,7 +93,7 @@ encode_small_kernel(const SmallParams p)
         if (lane < kBuffers && lane < R) copy_stage(lane, lane);
     }
     if (ctas > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
-    for (int t = tid; t < p.rows * 32; t += threads) {
+    for (int t = tid; t < p.vectors * dim; t += threads) {
         const int v = t / dim;
         w.xs[t] = v < live ? load_as_float(p.x, (v0 + v) * p.stride + (t - v * dim), s.dtype) : 0.0f;
     }
@@ -93,7 +101,7 @@ encode_small_kernel(const SmallParams p)
     if (warp == 0) {
         // deviations (the scalar kernel's order of additions): one lane per row
         const int vl = lane / G, g = lane - vl * G, base = lane - g;
-        const bool row = lane < p.rows;
+        const bool row = lane < p.vectors * G;
         const float *xr = w.xs + (row ? vl * dim + (s.layout == RVQ_GROUP_STRIDED ? g : g * 32) : 0);
         const int step = s.layout == RVQ_GROUP_STRIDED ? G : 1;
         float c[32], a = 0.0f, mu = 0.0f, sum = 0.0f;
@@ -110,7 +118,7 @@ encode_small_kernel(const SmallParams p)
         const float dev = sqrtf(sum / (float)(dim - s.ddof));
         const bool deg = vl >= live || deviation_is_degenerate(dev);
         if (row) w.dev[lane] = deg ? 0.0f : dev;                  // (0: codes 0, residual 0)
-        if (row && rank == 0 && vl < live && g == 0) {
+        if (row && rank == 0 && vl < live && g == 0 && g0 == 0) {
             const uint16_t hb = deg ? (uint16_t)0 : __half_as_ushort(__float2half_rn(dev));
             p.std16[v0 + vl] = hb;
             if (p.st) {
@@ -121,26 +129,26 @@ encode_small_kernel(const SmallParams p)
     }
     __syncthreads();
     for (int t = tid; t < p.rows * 32; t += threads) {
-        const int row = t >> 5, v = row / G;
+        const int row = (t >> 5) + g0, v = row / G;
         const float dev = w.dev[row];
-        w.z[row][t & 31] = dev == 0.0f ? 0.0f : w.xs[v * dim + channel_of(s.layout, G, 32, row - v * G, t & 31)] / dev;
+        w.z[t >> 5][t & 31] = dev == 0.0f ? 0.0f : w.xs[v * dim + channel_of(s.layout, G, 32, row - v * G, t & 31)] / dev;
     }
     if (ctas > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // every CTA's barriers are set up
     __syncthreads();
 
-    // thread: codeword c of this CTA, kSmallAtOnce rows from `first` on, then those `next` further on
-    const int c = tid & (PER * 128 - 1), first = kSmallAtOnce * (tid / (PER * 128)), next = kSmallAtOnce * (threads / (PER * 128));
+    // thread: codeword c of this CTA, AT_ONCE rows from `first` on, then those `next` further on
+    const int c = tid & (PER * 128 - 1), first = AT_ONCE * (tid / (PER * 128)), next = AT_ONCE * (threads / (PER * 128));
     const int slots = ctas * PER * 4;                             // warps of a cluster that have codewords of one row
     const int slot = rank * PER * 4 + (c >> 5);
     const bool real = (c >> 7) < mine;
     const uint32_t arrived0 = smem_u32(&w.arrived[0]);
     const uint32_t to_keys = map_to(smem_u32(&w.keys[0][0][slot]), (uint32_t)min(lane, ctas - 1));    // in CTA `lane`
     const uint32_t to_arrived = map_to(arrived0, (uint32_t)min(lane, ctas - 1));
-    constexpr uint32_t kRowKeys = kSmallMaxCluster * 8 * 8, kAllKeys = kSmallRows * kRowKeys;      // bytes
+    constexpr uint32_t kRowKeys = kSmallMaxCluster * 8 * 8, kAllKeys = kRows * kRowKeys;      // bytes
     bool ok = true;
     int buffer = 0, next_buffer = 0;
     uint32_t full_par = 0;                                        // of next_buffer
-    int r = 0;
+    int r = 0, copies = min(R, kBuffers);                         // stages asked for (thread 0)
     // this thread's codeword of the next stage
     float4 e[8];
     auto take_codeword = [&] {
@@ -159,11 +167,11 @@ encode_small_kernel(const SmallParams p)
         const uint8_t *stage = table + (size_t)buffer * kStageBytes;
 #pragma unroll 1
         for (int row = first; row < p.rows; row += next) {
-            float d[kSmallAtOnce] = {};
+            float d[AT_ONCE] = {};
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
 #pragma unroll
-                for (int k = 0; k < kSmallAtOnce; ++k) {
+                for (int k = 0; k < AT_ONCE; ++k) {
                     const float4 u = *reinterpret_cast<const float4 *>(&w.z[row + k][4 * q]);
                     float t;
                     t = u.x - e[q].x; d[k] = fmaf(t, t, d[k]); t = u.y - e[q].y; d[k] = fmaf(t, t, d[k]);
@@ -171,16 +179,16 @@ encode_small_kernel(const SmallParams p)
                 }
             }
             // non-negative floats order like their bit patterns; a distance that is infinite or NaN never wins
-            uint32_t bits[kSmallAtOnce], m[kSmallAtOnce], who[kSmallAtOnce];
+            uint32_t bits[AT_ONCE], m[AT_ONCE], who[AT_ONCE];
 #pragma unroll
-            for (int k = 0; k < kSmallAtOnce; ++k) bits[k] = real ? __float_as_uint(d[k]) : 0xFFFFFFFFu;
+            for (int k = 0; k < AT_ONCE; ++k) bits[k] = real ? __float_as_uint(d[k]) : 0xFFFFFFFFu;
 #pragma unroll
-            for (int k = 0; k < kSmallAtOnce; ++k) m[k] = __reduce_min_sync(0xFFFFFFFFu, bits[k]);
+            for (int k = 0; k < AT_ONCE; ++k) m[k] = __reduce_min_sync(0xFFFFFFFFu, bits[k]);
 #pragma unroll
-            for (int k = 0; k < kSmallAtOnce; ++k) who[k] = __ballot_sync(0xFFFFFFFFu, bits[k] == m[k]);
+            for (int k = 0; k < AT_ONCE; ++k) who[k] = __ballot_sync(0xFFFFFFFFu, bits[k] == m[k]);
             // this warp's best of these rows, to every CTA of the cluster: lane l to CTA l
 #pragma unroll
-            for (int k = 0; k < kSmallAtOnce; ++k) {
+            for (int k = 0; k < AT_ONCE; ++k) {
                 const unsigned long long key = ((unsigned long long)m[k] << 32) | (uint32_t)(rank * PER * 128 + (c & ~31) + __ffs(who[k]) - 1);
                 if (lane < ctas && row + k < p.rows)
                     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
@@ -190,15 +198,21 @@ encode_small_kernel(const SmallParams p)
         // (while the minima travel: read at the stage's start, 16 warps' codewords were 512 cycles of its distances)
         if (r + 1 < R) ok = take_codeword() && ok;
         ok = mbar_wait(arrived0 + 8u * par, (uint32_t)(r >> 1) & 1u, &w.abort_flag) && ok;
+        // Every CTA has read this CTA's codewords of stage r - 1 (it could not have sent its minima of stage r
+        // before): their place is free.
+        if (PER > 1 && tid == 0 && ok && r >= 1 && copies < R) {
+            copy_stage(copies, copies % kBuffers);
+            ++copies;
+        }
         const bool subtract = r + 1 < R || p.energy != nullptr;
         float e2 = 0.0f;
 #pragma unroll 1
         for (int row = warp; row < p.rows; row += threads / 32) {
             unsigned long long k = lane < slots ? w.keys[par][row][lane] : ~0ull;
-            if (PER == 2 && lane + 32 < slots) k = min(k, w.keys[par][row][lane + 32]);
+            if (PER > 1 && lane + 32 < slots) k = min(k, w.keys[par][row][lane + 32]);
             const uint32_t hi = (uint32_t)(k >> 32), best = __reduce_min_sync(0xFFFFFFFFu, hi);
             uint32_t j = __reduce_min_sync(0xFFFFFFFFu, hi == best ? (uint32_t)k : 0xFFFFFFFFu);
-            const float dev = w.dev[row];
+            const float dev = w.dev[g0 + row];
             if (best >= 0x7F800000u || dev == 0.0f) j = 0;
             if (lane == 0) w.codes[row][r] = (uint16_t)j;
             if (subtract) {
@@ -219,14 +233,11 @@ encode_small_kernel(const SmallParams p)
         if (!ok) w.abort_flag = 1u;
         __syncthreads();
         if (w.abort_flag) { ok = false; break; }
-        // Every CTA has read this CTA's codewords of stage r - 1 (it could not have sent its minima of stage r
-        // before): their place is free.
-        if (PER == 2 && tid == 0 && r >= 1 && r - 1 + kBuffers < R) copy_stage(r - 1 + kBuffers, r - 1);
         if (++buffer == kBuffers) buffer = 0;
     }
     if (!ok && tid == 0) {
         // (the stages from here on are still coming in)
-        for (int k = r; k < R && k < kBuffers + max(r - 1, 0); ++k)
+        for (int k = r; k < copies; ++k)
             mbar_drain(smem_u32(&w.full[k % kBuffers]), (uint32_t)(k / kBuffers) & 1u);
         if (p.st) atomicAdd(&p.st->wait_timeouts, 1u);
     }
@@ -235,7 +246,18 @@ encode_small_kernel(const SmallParams p)
     if (rank != 0) return;
 
     // codes out (Section 3.2 storage)
-    if (s.bits == 16) {
+    if (p.shares > 1) {
+        // (a row's codes are whole bytes, and those of a vector whole words: small_plan)
+        const int row_bytes = R * s.bits / 8;
+        uint8_t *o = reinterpret_cast<uint8_t *>(p.codes) + v0 * s.code_bytes + g0 * row_bytes;
+        for (int t = tid; t < p.rows * row_bytes; t += threads) {
+            const int row = t / row_bytes, bit = 8 * (t - row * row_bytes);
+            uint32_t byte = 0;
+            for (int k = bit / s.bits, at = k * s.bits - bit; at < 8 && k < R; ++k, at += s.bits)
+                byte |= at >= 0 ? (uint32_t)w.codes[row][k] << at : (uint32_t)w.codes[row][k] >> -at;
+            o[t] = (uint8_t)byte;
+        }
+    } else if (s.bits == 16) {
         uint16_t *o = reinterpret_cast<uint16_t *>(p.codes) + v0 * G * R;
         for (int t = tid; t < live * G * R; t += threads) { const int row = t / R; o[t] = w.codes[row][t - row * R]; }
     } else {
@@ -255,47 +277,78 @@ encode_small_kernel(const SmallParams p)
 }
 
 struct SmallPlan {
-    const void *kernel;
-    int per_cta, ctas, at_once;
+    const void *kernel;                        // null: not for this encoder
+    int ctas, vectors, rows, shares, threads, smem;
+    int64_t clusters;
 };
 
-// How a shape is split, and how many clusters of that split the current device runs at a time (0: none).
-SmallPlan small_plan(const Shape &s)
+template <int PER, int AT_ONCE>
+void small_kernel(SmallPlan &plan)
 {
-    const int blocks = slots_per_stage(s.K), per = blocks <= kSmallMaxCluster ? 1 : 2;
-    SmallPlan plan{per == 1 ? reinterpret_cast<const void *>(encode_small_kernel<1>) : reinterpret_cast<const void *>(encode_small_kernel<2>),
-                   per, (blocks + per - 1) / per, 0};
-    plan.at_once = resident_clusters(plan.kernel, plan.ctas, kSmallThreads, kSmallSharedBytes);
-    return plan;
+    plan.kernel = reinterpret_cast<const void *>(encode_small_kernel<PER, AT_ONCE>);
+    plan.smem = kSmallSharedBytes<PER>;
+    const int threads = PER * 128 * ((plan.rows + AT_ONCE - 1) / AT_ONCE);
+    plan.threads = threads < kSmallThreads ? threads : kSmallThreads;
 }
 
-}  // namespace
+// A vector of whose groups several clusters of up to four CTAs take one or two each, where all of these run at a time: a
+// token's or two.  (Clusters of eight CTAs with all rows of a vector leave half of the SMs idle, and have twice the
+// distances each: 8 vectors, 2048 codes 16.4 -> 14.35 us, 1024 codes 12.3 -> 12.3, 16 vectors 20.5 -> 16.4 and 16.4 ->
+// 14.35.  Calls back to back come in steps of 2.05 us.)
+SmallPlan small_share_plan(const Shape &s, int64_t n)
+{
+    SmallPlan plan{};
+    const int blocks = slots_per_stage(s.K), per = blocks <= 4 ? 1 : blocks <= 8 ? 2 : 4;
+    // (codes are written by bytes)
+    if (s.G < 2 || s.R * s.bits % 8 != 0 || s.per_vector * s.bits % 32 != 0) return plan;
+    for (int rows = 1; rows <= 2 && rows < s.G; ++rows) {
+        SmallPlan t{};
+        t.ctas = (blocks + per - 1) / per; t.vectors = 1; t.rows = rows; t.shares = s.G / rows; t.clusters = n * t.shares;
+        if (rows == 1) {
+            if (per == 1) small_kernel<1, 1>(t); else if (per == 2) small_kernel<2, 1>(t); else small_kernel<4, 1>(t);
+        } else {
+            if (per == 1) small_kernel<1, 2>(t); else if (per == 2) small_kernel<2, 2>(t); else small_kernel<4, 2>(t);
+        }
+        if (t.clusters <= resident_clusters(t.kernel, t.ctas, kSmallThreads, t.smem)) return t;
+    }
+    return plan;
+}
 
 // Group rows per cluster up to which this encoder is faster than tiles of 128 rows: a row costs about 1.6 us at two blocks per CTA and
 // 1 us at one, a tile's stages about the same for one row as for 128.  us, this encoder / tiles: 2048 codes 16 rows 32.6 / 32.9, 20 39.1 / 33.3; 1024 codes 20 rows
 // 27.5 / 28.1, 24 29.8 / 28.1; 512 codes 20 rows 25.6 / 26.1, 24 27.7 / 26.1; at depth 4, 1024 codes, 24 rows 16.6 / 17.7.  Up to three chunks, where
 // a tile is one CTA's (encode_tensor.cu): 256 codes 16 rows 20.4 / 22.0, 20 25.0 / 22.0.
-bool encode_small_wanted(const Shape &s, int64_t n)
+SmallPlan small_plan(const Shape &s, int64_t n)
 {
-    if (!float_blocks_prepared(s) || s.raw || s.G > kSmallRows || n < 1 || n > 4096) return false;
-    const SmallPlan plan = small_plan(s);
-    const int64_t vectors = plan.at_once > 0 ? (n + plan.at_once - 1) / plan.at_once : 0;
-    const int most = plan.per_cta == 2 || slots_per_stage(s.K) <= 3 ? 16 : s.R <= 4 ? 24 : 20;
-    return vectors == 1 || (vectors > 0 && vectors * s.G <= most);
+    SmallPlan plan{};
+    if (!float_blocks_prepared(s) || s.raw || s.G > kSmallRows || n < 1 || n > 4096) return plan;
+    plan = small_share_plan(s, n);
+    if (plan.kernel) return plan;
+    const int blocks = slots_per_stage(s.K), per = blocks <= kSmallMaxCluster ? 1 : 2;
+    plan.ctas = (blocks + per - 1) / per;
+    const int at_once = resident_clusters(per == 1 ? reinterpret_cast<const void *>(encode_small_kernel<1, 2>) : reinterpret_cast<const void *>(encode_small_kernel<2, 2>),
+                                          plan.ctas, kSmallThreads, per == 1 ? kSmallSharedBytes<1> : kSmallSharedBytes<2>);
+    const int64_t vectors = at_once > 0 ? (n + at_once - 1) / at_once : 0;
+    const int most = per == 2 || blocks <= 3 ? 16 : s.R <= 4 ? 24 : 20;
+    if (vectors == 0 || (vectors > 1 && vectors * s.G > most)) return plan;
+    plan.vectors = (int)vectors; plan.rows = (int)vectors * s.G; plan.shares = 1; plan.clusters = (n + vectors - 1) / vectors;
+    if (per == 1) small_kernel<1, 2>(plan); else small_kernel<2, 2>(plan);
+    return plan;
 }
+
+}  // namespace
+
+bool encode_small_wanted(const Shape &s, int64_t n) { return small_plan(s, n).kernel != nullptr; }
 
 int launch_encode_small(const Shape &s, const void *x, int64_t n, int64_t stride, const void *prepared, void *codes,
                         uint16_t *std16, rvq_status *st, cudaStream_t stream, float *energy)
 {
-    const SmallPlan plan = small_plan(s);
-    if (plan.at_once <= 0 || !allow_shared_memory(plan.kernel, kSmallSharedBytes)) return RVQ_ERR_LAUNCH;
-    const int vectors = (int)((n + plan.at_once - 1) / plan.at_once);
+    const SmallPlan plan = small_plan(s, n);
+    if (!plan.kernel || !allow_shared_memory(plan.kernel, plan.smem)) return RVQ_ERR_LAUNCH;
     SmallParams p{s, x, n, stride, reinterpret_cast<const uint8_t *>(prepared) + float_blocks_offset(s), codes, std16, st, energy,
-                  vectors, vectors * s.G, slots_per_stage(s.K)};
-    int threads = plan.per_cta * 128 * ((p.rows + kSmallAtOnce - 1) / kSmallAtOnce);
-    if (threads > kSmallThreads) threads = kSmallThreads;
+                  plan.vectors, plan.rows, plan.shares, slots_per_stage(s.K)};
     void *args[] = {&p};
-    return launch_clusters(plan.kernel, (int)((n + vectors - 1) / vectors), plan.ctas, threads, kSmallSharedBytes, stream, args);
+    return launch_clusters(plan.kernel, (int)plan.clusters, plan.ctas, plan.threads, plan.smem, stream, args);
 }
 
 }  // namespace rvq

@@ -51,6 +51,16 @@ def test_few_vectors(n, K, R, layout, bits, dtype):
     check(n, 128, K, R, layout, bits, dtype, n + K)
 
 
+@pytest.mark.parametrize("n", [1, 3, 5, 8, 15, 16, 17, 33])
+@pytest.mark.parametrize("dim,K,R,layout,bits,dtype", [(128, 2048, 8, 1, "packed", "bf16"), (128, 1300, 8, 0, 16, "f32"), (256, 600, 4, 0, "packed", "f16"),
+                                                       (128, 2, 8, 1, "packed", "f32"), (128, 16, 2, 0, "packed", "f32"), (64, 1025, 8, 1, 16, "bf16"),
+                                                       (512, 1024, 8, 1, "packed", "bf16"), (1024, 512, 8, 0, "packed", "f32")])
+def test_groups_of_a_vector_shared_out(n, dim, K, R, layout, bits, dtype):
+    """Clusters that take one or two of a head vector's groups each, in as many as run at a time and beyond, and write the
+    bytes of their rows' codes: one to eleven bits a code, one to sixteen blocks of codewords."""
+    check(n, dim, K, R, layout, bits, dtype, n + K, stride=dim + 16)
+
+
 @pytest.mark.parametrize("n,dim,K", [(5, 256, 2048), (70, 256, 1024), (301, 64, 512), (9, 32, 2048), (40, 96, 300), (3, 512, 129),
                                      (13000, 128, 512), (150, 128, 5000), (4, 1024, 2049)])
 def test_other_head_sizes_and_row_strides(n, dim, K):
