@@ -314,10 +314,11 @@ SmallPlan small_share_plan(const Shape &s, int64_t n)
     return plan;
 }
 
-// Group rows per cluster up to which this encoder is faster than tiles of 128 rows: a row costs about 1.6 us at two blocks per CTA and
-// 1 us at one, a tile's stages about the same for one row as for 128.  us, this encoder / tiles: 2048 codes 16 rows 32.6 / 32.9, 20 39.1 / 33.3; 1024 codes 20 rows
-// 27.5 / 28.1, 24 29.8 / 28.1; 512 codes 20 rows 25.6 / 26.1, 24 27.7 / 26.1; at depth 4, 1024 codes, 24 rows 16.6 / 17.7.  Up to three chunks, where
-// a tile is one CTA's (encode_tensor.cu): 256 codes 16 rows 20.4 / 22.0, 20 25.0 / 22.0.
+// Group rows per cluster up to which this encoder is faster than tiles of 128 rows: a row costs about 1.5 us at two blocks per CTA and
+// 1 us at one, a tile's stages about the same for one row as for 128.  us, this encoder / tiles: 2048 codes 16 rows 32.1 / 34.8, 20 38.9 / 34.8;
+// 1536 codes 20 rows 30.7 / 32.8, 24 36.9 / 34.8; 1024 codes 20 rows 26.7 / 30.8, 24 28.7 / 28.7, 28 32.8 / 29.4; 512 codes 24 rows 26.7 / 28.7, 28 30.7 / 28.7; at
+// depth 4, 1024 codes, 24 rows 16.9 / 18.4.  Up to three chunks, where a tile is one CTA's (encode_tensor.cu): 384 codes 20 rows 24.6 / 26.6, 24 26.7 / 26.6;
+// 256 codes 16 rows 20.5 / 24.6, 20 24.6 / 24.6, 24 26.7 / 24.4.
 SmallPlan small_plan(const Shape &s, int64_t n)
 {
     SmallPlan plan{};
@@ -329,7 +330,7 @@ SmallPlan small_plan(const Shape &s, int64_t n)
     const int at_once = resident_clusters(per == 1 ? reinterpret_cast<const void *>(encode_small_kernel<1, 2>) : reinterpret_cast<const void *>(encode_small_kernel<2, 2>),
                                           plan.ctas, kSmallThreads, per == 1 ? kSmallSharedBytes<1> : kSmallSharedBytes<2>);
     const int64_t vectors = at_once > 0 ? (n + at_once - 1) / at_once : 0;
-    const int most = per == 2 || blocks <= 3 ? 16 : s.R <= 4 ? 24 : 20;
+    const int most = blocks > 12 ? 16 : blocks > 8 || blocks <= 3 ? 20 : 24;
     if (vectors == 0 || (vectors > 1 && vectors * s.G > most)) return plan;
     plan.vectors = (int)vectors; plan.rows = (int)vectors * s.G; plan.shares = 1; plan.clusters = (n + vectors - 1) / vectors;
     if (per == 1) small_kernel<1, 2>(plan); else small_kernel<2, 2>(plan);
