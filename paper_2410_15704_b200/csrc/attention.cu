@@ -134,7 +134,8 @@ __device__ __forceinline__ void att_cut(const Shape &s, const AttCodes &ac, AttR
 }
 
 // Sum over the stages of the four channels of this thread's row: STEPS 16-byte reads, stage
-// (rot + k) mod STEPS at step k.  PACKED: two additions per instruction -- us of the kernel, single / packed, scores 267 / 260, with four steps 114 / 107
+// rot ^ k (its last two bits with four steps) at step k.  (With stage rot + k, eight operations more, and two more per step for its address, the
+// call over 131072 tokens takes 466 us instead of 438.)  PACKED: two additions per instruction -- us of the kernel, single / packed, scores 267 / 260, with four steps 114 / 107
 // (60000 tokens); values 187 / 191 (register pairs cost moves), with four steps 72 / 67.  Codes past the codebook are read as code 0 and counted.
 template <int STEPS, bool PACKED>
 __device__ __forceinline__ void att_gather(const AttRow &a, uint32_t K, uint32_t rot, uint32_t smem_table,
@@ -154,27 +155,15 @@ __device__ __forceinline__ void att_gather(const AttRow &a, uint32_t K, uint32_t
             }
         }
     }
-    // rotate the halves left by `rot` so that step k finds its code at a fixed place
-    if (STEPS == 4) {
-        if (rot & 2u) { const uint32_t t0 = c0; c0 = c1; c1 = t0; }
-        if (rot & 1u) { const uint32_t b0 = __funnelshift_r(c0, c1, 16); c1 = __funnelshift_r(c1, c0, 16); c0 = b0; }
-    }
-    if (STEPS == 8 && (rot & 4u)) { const uint32_t t0 = c0, t1 = c1; c0 = c2; c1 = c3; c2 = t0; c3 = t1; }
-    if (STEPS == 8 && (rot & 2u)) { const uint32_t t0 = c0; c0 = c1; c1 = c2; c2 = c3; c3 = t0; }
-    if (STEPS == 8 && (rot & 1u)) {
-        const uint32_t b0 = __funnelshift_r(c0, c1, 16), b1 = __funnelshift_r(c1, c2, 16);
-        const uint32_t b2 = __funnelshift_r(c2, c3, 16), b3 = __funnelshift_r(c3, c0, 16);
-        c0 = b0; c1 = b1; c2 = b2; c3 = b3;
-    }
+    exchange_codes<STEPS>(rot, c0, c1, c2, c3);
     const uint32_t cw[4] = {c0, c1, c2, c3};
     uint64_t s01 = 0, s23 = 0;
     acc[0] = acc[1] = acc[2] = acc[3] = 0.0f;
 #pragma unroll
     for (int k = 0; k < STEPS; ++k) {
-        const uint32_t w = cw[k >> 1];
-        const uint32_t line = (k & 1) ? ((w >> 9) & (0xFFFFu << 7)) : ((w << 7) & (0xFFFFu << 7));
-        const uint32_t slot = STEPS == 8 ? (rot + k) & 7u : ((rot + k) & 3u) | (rot & 4u);
-        const uint32_t addr = smem_table + (line | (slot * 16u));
+        const uint32_t w = cw[k >> 1], code = (k & 1) ? w >> 16 : w & 0xFFFFu;
+        const uint32_t slot = STEPS == 8 ? rot ^ k : ((rot ^ k) & 3u) | (rot & 4u);
+        const uint32_t addr = code * 128u + (smem_table + slot * 16u);
         if (PACKED) {
             uint64_t f01, f23;
             asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(f01), "=l"(f23) : "r"(addr));

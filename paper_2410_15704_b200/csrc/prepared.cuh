@@ -156,6 +156,26 @@ struct StageMaxima {
     uint32_t elomax;                     // as emax
 };
 
+#ifdef __CUDACC__
+// A row's eight (STEPS 4: four) codes as halves of words, stage by stage, into the order in which a lane visits its stages: at
+// step k stage rot ^ k, so that the eight lanes of a quarter warp, whose rot are 0 ... 7, read eight different bank groups.
+// (A rotation, stage rot + k, takes eight operations more.)
+template <int STEPS>
+__device__ __forceinline__ void exchange_codes(uint32_t rot, uint32_t &c0, uint32_t &c1, uint32_t &c2, uint32_t &c3)
+{
+    auto swap_if = [](bool yes, uint32_t &a, uint32_t &b) { const uint32_t t = yes ? b : a; b = yes ? a : b; a = t; };
+    const uint32_t halves = (rot & 1u) ? 0x1032u : 0x3210u;
+    swap_if(rot & 2u, c0, c1);
+    c0 = __byte_perm(c0, 0u, halves); c1 = __byte_perm(c1, 0u, halves);
+    if (STEPS == 8) {
+        swap_if(rot & 2u, c2, c3);
+        c2 = __byte_perm(c2, 0u, halves); c3 = __byte_perm(c3, 0u, halves);
+        swap_if(rot & 4u, c0, c2);
+        swap_if(rot & 4u, c1, c3);
+    }
+}
+#endif
+
 __host__ __device__ inline int slots_per_stage(int K) { return (K + kSlotCodewords - 1) / kSlotCodewords; }
 
 }  // namespace rvq
