@@ -489,16 +489,22 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             for (uint32_t t = tid; t < (uint32_t)s.K * CH; t += kDecThreads) dst[t] = __ldg(src + t);
         }
     }
-    // this thread visits stage (rot + k) & 7 at step k (the 8 lanes of a quarter warp then touch 8
-    // different bank groups): the scale of that stage in bytes 0 and 3, and the byte offset of its entry
+    // this thread visits stage (rot + k) & 7, or rot ^ k (exchange_codes), at step k (the 8 lanes of a quarter warp then touch 8
+    // different bank groups): the scale of that stage in bytes 0 and 3, and the byte offset of its entry (kFromTable: with the
+    // table's address).  us, (rot + k) & 7 / rot ^ k, 1 M vectors: level tables, strided 132 / 124, 10-bit codes 149.8 / 145.4;
+    // float32 tables, strided, with the address added once 210 / 201.  16-bit codes on contiguous groups, at the data pipe's
+    // limit, 133.3 / 134.6; rotated 240008 vectors 69.8 / 71.2, 1 M with 10-bit codes 295 / 309 (64 registers).
+    constexpr bool kExchange = ROPE == 0 && (LAYOUT == RVQ_GROUP_STRIDED || BITS != 16), kFromTable = kExchange && F32;
     uint32_t scale[SUMMED ? 2 : 8], unit[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         if (!SUMMED || k < 2) {
-            const uint32_t sc = SUMMED ? dp->pscale[(rot + k) & 1u] : dp->scale[(rot + k) & 7u];
+            const uint32_t sc = kExchange ? SUMMED ? dp->pscale[(rot ^ k) & 1u] : dp->scale[rot ^ k]
+                                          : SUMMED ? dp->pscale[(rot + k) & 1u] : dp->scale[(rot + k) & 7u];
             scale[SUMMED ? (k & 1) : k] = sc | (sc << 24);
         }
-        unit[k] = ((rot + k) & 7u) * kEntry;
+        unit[k] = (kExchange ? rot ^ k : (rot + k) & 7u) * kEntry;
+        if (kFromTable) unit[k] += (uint32_t)__cvta_generic_to_shared(table);
     }
     const float bias = dp->bias, base = SUMMED ? dp->pbase : dp->base;
     const float terr = SUMMED ? dp->perr : dp->err;
@@ -566,13 +572,17 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             c0 = cw[0]; c1 = cw[1]; c2 = cw[2]; c3 = cw[3];
         }
         const uint32_t n0 = c0, n1 = c1, n2 = c2, n3 = c3;          // natural order, for the exact route
-        // rotate the 8 halves left by `rot` so that step k finds its code at a fixed place
-        if (rot & 4u) { const uint32_t t0 = c0, t1 = c1; c0 = c2; c1 = c3; c2 = t0; c3 = t1; }
-        if (rot & 2u) { const uint32_t t0 = c0; c0 = c1; c1 = c2; c2 = c3; c3 = t0; }
-        if (rot & 1u) {
-            const uint32_t b0 = __funnelshift_r(c0, c1, 16), b1 = __funnelshift_r(c1, c2, 16);
-            const uint32_t b2 = __funnelshift_r(c2, c3, 16), b3 = __funnelshift_r(c3, c0, 16);
-            c0 = b0; c1 = b1; c2 = b2; c3 = b3;
+        if (kExchange) {
+            exchange_codes<8>(rot, c0, c1, c2, c3);
+        } else {
+            // rotate the 8 halves left by `rot` so that step k finds its code at a fixed place
+            if (rot & 4u) { const uint32_t t0 = c0, t1 = c1; c0 = c2; c1 = c3; c2 = t0; c3 = t1; }
+            if (rot & 2u) { const uint32_t t0 = c0; c0 = c1; c1 = c2; c2 = c3; c3 = t0; }
+            if (rot & 1u) {
+                const uint32_t b0 = __funnelshift_r(c0, c1, 16), b1 = __funnelshift_r(c1, c2, 16);
+                const uint32_t b2 = __funnelshift_r(c2, c3, 16), b3 = __funnelshift_r(c3, c0, 16);
+                c0 = b0; c1 = b1; c2 = b2; c3 = b3;
+            }
         }
         // codes out of range (never produced by the encoder): counted, read as code 0
         {
@@ -604,7 +614,7 @@ decode_levels_fast(const Shape &s, const void *__restrict__ codes, const uint16_
             // byte offset of the table line of this step's code: (code << kShift) | unit
             const uint32_t w = cwk[k >> 1];
             const uint32_t line = (k & 1) ? ((w >> (16 - kShift)) & (0xFFFFu << kShift)) : ((w << kShift) & (0xFFFFu << kShift));
-            const uint32_t a = smem_table + (line | unit[k]);
+            const uint32_t a = kFromTable ? (((k & 1) ? w >> 16 : w & 0xFFFFu) << kShift) + unit[k] : smem_table + (line | unit[k]);
             uint32_t e[CH / 2];
             if (F32) {
                 if (ROPE == 0) {
